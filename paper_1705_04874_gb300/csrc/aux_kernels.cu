@@ -278,11 +278,11 @@ cudaError_t launch_nonfinite(float* const* fields, size_t n, int* flag, cudaStre
     return cudaGetLastError();
 }
 
-// slab[cell in slab] = copy ? total[cell] : 0
+// slab[cell in slab] = copy ? total[cell] : 0 (0 in an x slab's unused cells)
 __global__ void fill_slab_kernel(const float* total, float* slab, int axis, int nx, int ny, int nz, int L,
                                  int copy)
 {
-    const int S = 2 * L + 1;
+    const int S = slab_width(axis, L);
     const int n = axis == 0 ? nx : (axis == 1 ? ny : nz);
     const size_t cnt = (size_t)nx * ny * nz / n * S;
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < cnt; i += (size_t)gridDim.x * blockDim.x) {
@@ -290,7 +290,11 @@ __global__ void fill_slab_kernel(const float* total, float* slab, int axis, int 
         if (axis == 0) { sp = (int)(i % S); size_t l = i / S; y = (int)(l % ny); z = (int)(l / ny); x = 0; }
         else if (axis == 1) { x = (int)(i % nx); size_t l = i / nx; sp = (int)(l % S); z = (int)(l / S); y = 0; }
         else { x = (int)(i % nx); size_t l = i / nx; y = (int)(l % ny); sp = (int)(l / ny); z = 0; }
-        const int pos = sp < L ? sp : sp - L + (n - 1 - L);
+        const int pos = sp < L ? sp : sp - S + n;
+        if (sp >= L && pos < n - 1 - L) {
+            slab[i] = 0.f;
+            continue;
+        }
         if (axis == 0) x = pos; else if (axis == 1) y = pos; else z = pos;
         slab[i] = copy ? total[(size_t)x + (size_t)nx * ((size_t)y + (size_t)ny * z)] : 0.f;
     }

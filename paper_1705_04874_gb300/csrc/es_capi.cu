@@ -384,7 +384,7 @@ bool stag_along(int f, int a)
     }
 }
 int axis_len(const es_model* m, int a) { return a == 0 ? m->nx : (a == 1 ? m->ny : m->nz); }
-size_t slab_count(const es_model* m, int a) { return m->L > 0 ? m->ncell / axis_len(m, a) * (2 * m->L + 1) : 0; }
+size_t slab_count(const es_model* m, int a) { return m->ncell / axis_len(m, a) * slab_width(a, m->L); }
 
 int upload_sources(es_model* m, double dt)
 {
@@ -594,6 +594,7 @@ PassParams make_pass(const es_model* m, int axis, bool stress, float dt)
     p.pc = m->pc[axis];
     p.ps = m->ps[axis];
     p.L = m->L;
+    p.S = slab_width(axis, m->L);
     p.dt = dt;
     p.nsim = m->nsim;
     p.fstride = (long long)m->ncell;

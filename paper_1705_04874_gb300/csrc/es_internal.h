@@ -34,6 +34,17 @@ constexpr int NEAR_PAIRS = NEAR_TAPS / 2;
 // first tap offset o: D(+) (result at i + 1/2) reads i-4 .. i+5, D(-) reads i-5 .. i+4
 __host__ __device__ constexpr int near_ofs(int sign) { return sign > 0 ? -4 : -5; }
 
+// Storage of the split parts inside a PML slab: [0, L) and [n-1-L, n) along the
+// axis, every point whose whole- or half-index factor differs from 1.  y and z
+// slabs keep exactly these 2 L + 1 rows; x slabs keep whole quads at both ends
+// (unused cells between), so that the x pass moves them 16 bytes at a time.
+__host__ __device__ constexpr int slab_width(int axis, int L)
+{
+    return L <= 0 ? 0 : (axis == 0 ? (L + 3) / 4 * 4 + (L + 4) / 4 * 4 : 2 * L + 1);
+}
+// slab coordinate of a position in the slab (S = slab_width)
+__host__ __device__ constexpr int slab_pos(int pos, int n, int L, int S) { return pos < L ? pos : pos - n + S; }
+
 struct PassJob {
     const float* src;     // field differentiated (total)
     float* tgt[3];        // target totals
@@ -87,7 +98,8 @@ struct PassParams {
                           // previous pass finishes (the epilogue waits); 2 wait before any read
     const float* pc;      // PML factors at whole indices along the axis
     const float* ps;      // PML factors at half indices along the axis
-    int L;                // PML cells per face (slab width 2L+1, none if 0)
+    int L;                // PML cells per face
+    int S;                // slab_width(axis, L)
     float dt;
     int nsim;             // independent simulations sharing the materials
     long long fstride;    // elements between consecutive simulations' field arrays
@@ -142,10 +154,12 @@ int plan_current(int kind, int n, int* ra, int* rb);
 int plan_select(int kind, int n, int ra, int rb);
 // Launches one pass (all jobs) along p.axis.  Returns a cudaError_t.
 cudaError_t launch_pass(const PassParams& p, cudaStream_t st);
-// The y / z FFT pass for an odd nx with stage radices ra, rb, rc (rc = 1: two
-// stages; pass_kernels_odd.cu), and its shared-memory opt-in.
-cudaError_t launch_strided_odd(int ra, int rb, int rc, dim3 grid, const PassParams& p, cudaStream_t st);
-cudaError_t prepare_strided_odd();
+// The y / z FFT pass with stage radices ra, rb, rc (rc = 1: two stages) and 2 (nx even) or
+// 1 floats per access (pass_strided2.cu, pass_strided1.cu), and its shared-memory opt-in.
+cudaError_t launch_strided2(int ra, int rb, int rc, int ntiles, const PassParams& p, cudaStream_t st);
+cudaError_t launch_strided1(int ra, int rb, int rc, int ntiles, const PassParams& p, cudaStream_t st);
+cudaError_t prepare_strided2();
+cudaError_t prepare_strided1();
 // Longest axis the circulant pass takes (shared tiles of 2 x 32 x pad(n) floats).
 constexpr int CIRC_MAX_N = 512;
 // From this length on, the CUDA-core circulant passes along y and z run their epilogue from

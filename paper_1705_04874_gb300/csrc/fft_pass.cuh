@@ -2,13 +2,13 @@
 // arXiv 1705.04874: Fourier-domain spatial derivatives on a staggered grid).
 //
 // One CTA owns a tile of 32 real pencils along the pass axis, packed two at a
-// time into 16 complex lines (line c = pencil 2c + i * pencil 2c+1).  For
-// each job it runs: forward FFT along the axis -> multiply by
-// i kappa exp(+/- i kappa d / 2) / n -> inverse FFT -> field-update epilogue.
-// Because the multiplier is Hermitian (a real field has a real derivative,
-// including at the Nyquist bin, where it is the real number -/+ pi / d), the
-// real and imaginary parts of the result are the derivatives of the two
-// packed pencils.
+// time into 16 complex lines (line c = pencil 2c + i * pencil 2c+1; y and z
+// passes with an odd nx: pencil c + i * pencil 16+c).  For
+// each job it runs: near stencil -> forward FFT along the axis -> multiply by
+// (H - H_near) / n -> inverse FFT -> field-update epilogue.  Because the
+// multiplier is Hermitian (a real field has a real derivative, including at
+// the Nyquist bin, where it is the real number -/+ pi / d), the real and
+// imaginary parts of the result are the derivatives of the two packed pencils.
 //
 // The transform of length n = RA * RB is a two-stage Stockham autosort FFT
 // (radix RA with stride n/RA, then radix RB with twiddles exp(-2 pi i k r / n)).
@@ -21,28 +21,39 @@
 // Three-stage plans (Core3: 125 = 5 x 5 x 5, 75 = 3 x 5 x 5) run their middle
 // stages through shared memory and keep the same first / last-stage layout.
 //
-// Strided passes (y, z): a tile is 32 consecutive x (128-byte rows) by the
-// whole pencil; every global access of a warp is a full row segment (an odd
-// nx moves the x-adjacent pairs as two floats).  The x pass stages 32 whole
-// x-lines (contiguous in memory) through shared memory with float4 accesses
-// (float accesses, and a per-line copy of the source for the near stencil,
-// when the length is not a multiple of 16) and runs the same FFT core on the
-// staged tile.
+// Near part.  Each derivative is a near part plus a far part (es_internal.h):
+// the multiplier tables hold H_far / n, and the NEAR_TAPS-point stencil is
+// formed first, from the staged source tile, several consecutive positions per
+// thread with the window sliding through registers (1 + 9 / 16 shared loads
+// per output along y and z instead of 10).  It waits in tensor memory, which
+// nothing else here uses, until the inverse transform is done.  In exact
+// arithmetic the sum is the spectral derivative itself; in FP32 the FFT's
+// roundoff, which is spread over the whole pencil, is scaled down by
+// |H_far| / |H| (about 1 %), so far-away receivers no longer see the FP32
+// noise of the pencil's largest values.
 //
-// Each derivative is evaluated as a near part plus a far part (es_internal.h):
-// the multiplier tables hold H_far / n, and once the last inverse stage has
-// read the shared buffer, the source tile comes back into it (cp.async from
-// L2, where the tile's first read left it, with wrap-around copies of the
-// first and last rows); the epilogue adds the NEAR_TAPS-point near stencil
-// from there (the x pass reads it from the staged lines' L1 / L2 copies, or
-// from its per-line copy).  In exact arithmetic the sum is the spectral
-// derivative itself; in FP32 the FFT's roundoff, which is spread
-// over the whole pencil, is scaled down by |H_far| / |H| (about 1 %), so
-// far-away receivers no longer see the FP32 noise of the pencil's largest
-// values.
+// The passes are persistent: while a CTA works on one tile, the next one's
+// source arrives in shared memory (cp.async), so that the 3 CTAs an SM holds at
+// n = 256 (72 KB each) have 6 tiles in hand.  What bounds them is memory: at
+// 256^3 (one GB300, 6.68 TB/s copy rate) the y / z velocity passes move 844 MB
+// in 0.158 / 0.163 ms (5.3 TB/s), the stress passes 1.21 GB in 0.213 / 0.217 ms
+// (5.7 TB/s), the x passes the same bytes in 0.182 and 0.227 ms.  One tile per
+// CTA (four CTAs per SM, the source read straight into registers and fetched
+// again from L2 for the stencil) took 0.188 / 0.203, 0.245 / 0.258, 0.191 and
+// 0.242 ms: a chain of load, transform, reload and update with nothing to
+// overlap it but the other CTAs.  Tried on the way and dropped: four pencils
+// per thread (half the instructions, 12 warps per SM: 0.191 ms, latency-bound);
+// the near parts in a third shared tile and one tile per CTA (0.188 ms); slab
+// rows left to the warps that own them (0.231 ms, the others wait).
+//
+// Strided passes (y, z): a tile is 32 consecutive x (128-byte rows) by the
+// whole pencil.  The x pass stages 32 whole x-lines (contiguous in memory),
+// turns them around into the same [position][pencil] rows, and reads the far
+// parts back from there line by line.
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
+#include <algorithm>
 #include <type_traits>
 #include <utility>
 
@@ -75,6 +86,74 @@ __host__ __device__ constexpr double ce_sin_frac(long m, long r)
     return ce_cos_frac(4 * m - r, 4 * r);  // sin(t) = cos(t - pi/2)
 }
 
+template <int... Is, class F>
+__device__ __forceinline__ void sfor_impl(std::integer_sequence<int, Is...>, F&& f)
+{
+    (f(std::integral_constant<int, Is>{}), ...);
+}
+template <int N, class F>
+__device__ __forceinline__ void sfor(F&& f)
+{
+    sfor_impl(std::make_integer_sequence<int, N>{}, f);
+}
+
+// Packed FP32 pairs (PTX f32x2): two operations in one instruction, each
+// component rounded exactly as the scalar operation
+__device__ __forceinline__ float2 add2(float2 a, float2 b)
+{
+    float2 d;
+    asm("{\n.reg .b64 ra, rb, rd;\nmov.b64 ra, {%2, %3};\nmov.b64 rb, {%4, %5};\n"
+        "add.rn.f32x2 rd, ra, rb;\nmov.b64 {%0, %1}, rd;\n}"
+        : "=f"(d.x), "=f"(d.y)
+        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return d;
+}
+__device__ __forceinline__ float2 sub2(float2 a, float2 b)
+{
+    float2 d;
+    asm("{\n.reg .b64 ra, rb, rd;\nmov.b64 ra, {%2, %3};\nmov.b64 rb, {%4, %5};\n"
+        "sub.rn.f32x2 rd, ra, rb;\nmov.b64 {%0, %1}, rd;\n}"
+        : "=f"(d.x), "=f"(d.y)
+        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return d;
+}
+__device__ __forceinline__ float2 mul2(float2 a, float2 b)
+{
+    float2 d;
+    asm("{\n.reg .b64 ra, rb, rd;\nmov.b64 ra, {%2, %3};\nmov.b64 rb, {%4, %5};\n"
+        "mul.rn.f32x2 rd, ra, rb;\nmov.b64 {%0, %1}, rd;\n}"
+        : "=f"(d.x), "=f"(d.y)
+        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return d;
+}
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c)
+{
+    float2 d;
+    asm("{\n.reg .b64 ra, rb, rc, rd;\nmov.b64 ra, {%2, %3};\nmov.b64 rb, {%4, %5};\nmov.b64 rc, {%6, %7};\n"
+        "fma.rn.f32x2 rd, ra, rb, rc;\nmov.b64 {%0, %1}, rd;\n}"
+        : "=f"(d.x), "=f"(d.y)
+        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
+    return d;
+}
+__device__ __forceinline__ float2 rep2(float s) { return make_float2(s, s); }
+
+__device__ __forceinline__ float2 cadd(float2 a, float2 b) { return add2(a, b); }
+__device__ __forceinline__ float2 csub(float2 a, float2 b) { return sub2(a, b); }
+// a - i b and a + i b
+__device__ __forceinline__ float2 csub_i(float2 a, float2 b)
+{
+    return make_float2(__fadd_rn(a.x, b.y), __fsub_rn(a.y, b.x));
+}
+__device__ __forceinline__ float2 cadd_i(float2 a, float2 b)
+{
+    return make_float2(__fsub_rn(a.x, b.y), __fadd_rn(a.y, b.x));
+}
+__device__ __forceinline__ float2 cmul(float2 a, float2 b)
+{
+    return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
+}
+
+// v W_R^M, a compile-time constant
 template <int R, int M>
 __device__ __forceinline__ float2 twc(float2 v)
 {
@@ -93,36 +172,6 @@ __device__ __forceinline__ float2 twc(float2 v)
     }
 }
 
-template <int... Is, class F>
-__device__ __forceinline__ void sfor_impl(std::integer_sequence<int, Is...>, F&& f)
-{
-    (f(std::integral_constant<int, Is>{}), ...);
-}
-template <int N, class F>
-__device__ __forceinline__ void sfor(F&& f)
-{
-    sfor_impl(std::make_integer_sequence<int, N>{}, f);
-}
-
-__device__ __forceinline__ float2 cadd(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
-__device__ __forceinline__ float2 csub(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
-__device__ __forceinline__ float2 cmul(float2 a, float2 b)
-{
-    return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
-}
-__device__ __forceinline__ float2 mul_mi(float2 a) { return make_float2(a.y, -a.x); }  // -i a
-
-// Packed FP32 pairs (fma.rn.f32x2 / add.rn.f32x2): two multiply-adds or adds
-// in one instruction, each component rounded exactly as fmaf / __fadd_rn
-__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c)
-{
-    float2 d;
-    asm("{\n.reg .b64 ra, rb, rc, rd;\nmov.b64 ra, {%2, %3};\nmov.b64 rb, {%4, %5};\nmov.b64 rc, {%6, %7};\n"
-        "fma.rn.f32x2 rd, ra, rb, rc;\nmov.b64 {%0, %1}, rd;\n}"
-        : "=f"(d.x), "=f"(d.y)
-        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
-    return d;
-}
 // Index check of the bounds-checked build (ES_BOUNDS, es_internal.h): true
 // when 0 <= i < n; otherwise the first such index is recorded with the source
 // line and the caller skips the access.  Always true in the release build.
@@ -141,16 +190,6 @@ __device__ __forceinline__ bool inb(unsigned long long* bad, long long i, long l
 #endif
 }
 #define ES_INB(p, i, n) inb((p).bad, (long long)(i), (long long)(n), __LINE__)
-
-__device__ __forceinline__ float2 add2(float2 a, float2 b)
-{
-    float2 d;
-    asm("{\n.reg .b64 ra, rb, rd;\nmov.b64 ra, {%2, %3};\nmov.b64 rb, {%4, %5};\n"
-        "add.rn.f32x2 rd, ra, rb;\nmov.b64 {%0, %1}, rd;\n}"
-        : "=f"(d.x), "=f"(d.y)
-        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
-    return d;
-}
 
 // ---------------------------------------------------------------------------
 // forward DFTs of small sizes in registers: a[k] <- sum_j a[j] W_R^(jk)
@@ -172,10 +211,9 @@ template <> struct Dft<3> {
         constexpr float h = 0.86602540378443864676f;  // sqrt(3) / 2
         float2 t1 = cadd(a[1], a[2]), t2 = csub(a[1], a[2]);
         float2 m = make_float2(a[0].x - 0.5f * t1.x, a[0].y - 0.5f * t1.y);
-        float2 s = mul_mi(make_float2(h * t2.x, h * t2.y));
         a[0] = cadd(a[0], t1);
-        a[1] = cadd(m, s);
-        a[2] = csub(m, s);
+        a[1] = make_float2(m.x + h * t2.y, m.y - h * t2.x);  // m - i h t2
+        a[2] = make_float2(m.x - h * t2.y, m.y + h * t2.x);  // m + i h t2
     }
 };
 
@@ -183,11 +221,11 @@ template <> struct Dft<4> {
     static __device__ __forceinline__ void run(float2* a)
     {
         float2 s02 = cadd(a[0], a[2]), d02 = csub(a[0], a[2]);
-        float2 s13 = cadd(a[1], a[3]), d13 = mul_mi(csub(a[1], a[3]));
+        float2 s13 = cadd(a[1], a[3]), d13 = csub(a[1], a[3]);
         a[0] = cadd(s02, s13);
         a[2] = csub(s02, s13);
-        a[1] = cadd(d02, d13);
-        a[3] = csub(d02, d13);
+        a[1] = csub_i(d02, d13);
+        a[3] = cadd_i(d02, d13);
     }
 };
 
@@ -202,13 +240,13 @@ template <> struct Dft<5> {
         float2 t3 = csub(a[1], a[4]), t4 = csub(a[2], a[3]);
         float2 b1 = make_float2(a[0].x + c1 * t1.x + c2 * t2.x, a[0].y + c1 * t1.y + c2 * t2.y);
         float2 b2 = make_float2(a[0].x + c2 * t1.x + c1 * t2.x, a[0].y + c2 * t1.y + c1 * t2.y);
-        float2 e1 = mul_mi(make_float2(s1 * t3.x + s2 * t4.x, s1 * t3.y + s2 * t4.y));
-        float2 e2 = mul_mi(make_float2(s2 * t3.x - s1 * t4.x, s2 * t3.y - s1 * t4.y));
+        float2 e1 = make_float2(s1 * t3.x + s2 * t4.x, s1 * t3.y + s2 * t4.y);
+        float2 e2 = make_float2(s2 * t3.x - s1 * t4.x, s2 * t3.y - s1 * t4.y);
         a[0] = cadd(a[0], cadd(t1, t2));
-        a[1] = cadd(b1, e1);
-        a[4] = csub(b1, e1);
-        a[2] = cadd(b2, e2);
-        a[3] = csub(b2, e2);
+        a[1] = csub_i(b1, e1);
+        a[4] = cadd_i(b1, e1);
+        a[2] = csub_i(b2, e2);
+        a[3] = cadd_i(b2, e2);
     }
 };
 
@@ -244,12 +282,6 @@ template <> struct Dft<25> : DftPQ<5, 5> {};
 // ---------------------------------------------------------------------------
 // epilogues
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ int slab_pos(int pos, int n, int L)
-{
-    // slab storage covers [0, L) and [n-1-L, n): every point whose whole- or
-    // half-index PML factor differs from 1
-    return pos < L ? pos : pos - (n - 1 - L) + L;
-}
 __device__ __forceinline__ bool in_slab(int pos, int n, int L)
 {
     return L > 0 && (pos < L || pos >= n - 1 - L);
@@ -285,105 +317,47 @@ __device__ __forceinline__ float normal_coef(float lam, float mu, bool diag) { r
 // increment, and passes are stream-ordered, so the result is the plain
 // rounded sum, deterministic, while the epilogue never waits for the old
 // value.
-
-// Epilogue for a pair of x-adjacent cells (x even) at position `pos` along
-// the axis: q = linear index of the first cell, (x, y, z) its coordinates;
-// off / soff = this simulation's offset into the field / slab arrays
-// (materials are shared by all simulations).
-__device__ __forceinline__ void epilogue_pair(const PassParams& p, const PassJob& J, size_t q, int pos,
-                                              int x, int y, int z, float d0, float d1, size_t off, size_t soff)
+// ---- y / z epilogue: two cells per thread and position ----
+// A thread's pencil pair is x0 + 2c, x0 + 2c + 1 with an even nx (V = 2: 8-byte
+// accesses); with an odd one, whose rows start anywhere, x0 + c and x0 + D + c
+// (V = 1, D pairs per row: two 4-byte accesses, each coalesced over the row's
+// half).  two: whether the second cell exists (V = 1; V = 2 has both).
+template <int V, int D>
+__device__ __forceinline__ float2 ld_pair(const float* q, bool two)
 {
-    if (!ES_INB(p, off + q + 1, p.ext_f)) return;
-    if (J.kind == JOB_STORE) {
-        *reinterpret_cast<float2*>(J.tgt[0] + off + q) = make_float2(d0, d1);
-        return;
-    }
-    if (!ES_INB(p, q + 1, p.ext_c)) return;
-    const float dt = p.dt;
-    const bool slab = in_slab(pos, p.n, p.L);
-    const int S = 2 * p.L + 1;
-    if (J.kind == JOB_SINGLE) {
-        const float2 c = __ldg(reinterpret_cast<const float2*>(J.coef[0] + q));
-        float2 inc = make_float2(increment(dt, c.x, d0), increment(dt, c.y, d1));
-        if (slab) {
-            const float P = __ldg((J.stag ? p.ps : p.pc) + pos);
-            const size_t si = slab_index(p.axis, x, y, z, slab_pos(pos, p.n, p.L), p.nx, p.ny, S);
-            if (!ES_INB(p, soff + si + 1, p.ext_s)) return;
-            inc.x = split_delta(J.slab[0], soff + si, P, inc.x);
-            inc.y = split_delta(J.slab[0], soff + si + 1, P, inc.y);
-        }
-        atomicAdd(reinterpret_cast<float2*>(J.tgt[0] + off + q), inc);
+    if constexpr (V == 2) return *reinterpret_cast<const float2*>(q);
+    return make_float2(q[0], two ? q[D] : 0.f);
+}
+// the same from memory no kernel writes (the coefficients)
+template <int V, int D>
+__device__ __forceinline__ float2 ldg_pair(const float* q, bool two)
+{
+    if constexpr (V == 2) return __ldg(reinterpret_cast<const float2*>(q));
+    return make_float2(__ldg(q), two ? __ldg(q + D) : 0.f);
+}
+template <int V, int D>
+__device__ __forceinline__ void st_pair(float* q, float2 v, bool two)
+{
+    if constexpr (V == 2) {
+        *reinterpret_cast<float2*>(q) = v;
     } else {
-        const float2 lam = __ldg(reinterpret_cast<const float2*>(J.coef[0] + q));
-        const float2 mu = __ldg(reinterpret_cast<const float2*>(J.coef[1] + q));
-        const float P = slab ? __ldg(p.pc + pos) : 1.f;
-        const size_t si = slab ? slab_index(p.axis, x, y, z, slab_pos(pos, p.n, p.L), p.nx, p.ny, S) : 0;
-        if (slab && !ES_INB(p, soff + si + 1, p.ext_s)) return;
-#pragma unroll
-        for (int t = 0; t < 3; ++t) {
-            const float2 c = make_float2(normal_coef(lam.x, mu.x, t == J.diag), normal_coef(lam.y, mu.y, t == J.diag));
-            float2 inc = make_float2(increment(dt, c.x, d0), increment(dt, c.y, d1));
-            if (slab) {
-                inc.x = split_delta(J.slab[t], soff + si, P, inc.x);
-                inc.y = split_delta(J.slab[t], soff + si + 1, P, inc.y);
-            }
-            atomicAdd(reinterpret_cast<float2*>(J.tgt[t] + off + q), inc);
-        }
+        q[0] = v.x;
+        if (two) q[D] = v.y;
     }
 }
-
-// Epilogue for 4 x-consecutive cells of one x line (x pass): q0 = linear
-// index of the first, pos0 its x, line = y + ny z (the x slabs' row index),
-// d[] the derivatives.
-__device__ __forceinline__ void epilogue_quad(const PassParams& p, const PassJob& J, size_t q0, int pos0,
-                                              int line, const float* d, size_t off, size_t soff)
+template <int V, int D>
+__device__ __forceinline__ void red_pair(float* q, float2 v, bool two)
 {
-    if (!ES_INB(p, off + q0 + 3, p.ext_f)) return;
-    if (J.kind == JOB_STORE) {
-        *reinterpret_cast<float4*>(J.tgt[0] + off + q0) = make_float4(d[0], d[1], d[2], d[3]);
-        return;
-    }
-    // the coefficients, and this line's row of the x slabs (S cells)
-    if (!ES_INB(p, q0 + 3, p.ext_c)) return;
-    if (p.L > 0 && !ES_INB(p, soff + (size_t)(2 * p.L + 1) * (line + 1) - 1, p.ext_s)) return;
-    const float dt = p.dt;
-    const int S = 2 * p.L + 1;
-    const size_t srow = soff + (size_t)S * (size_t)line;  // slab_index(0, ...) without the division
-    if (J.kind == JOB_SINGLE) {
-        const float4 c4 = __ldg(reinterpret_cast<const float4*>(J.coef[0] + q0));
-        const float cv[4] = {c4.x, c4.y, c4.z, c4.w};
-        float iv[4];
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            const int pos = pos0 + e;
-            iv[e] = increment(dt, cv[e], d[e]);
-            if (in_slab(pos, p.n, p.L))
-                iv[e] = split_delta(J.slab[0], srow + slab_pos(pos, p.n, p.L), __ldg((J.stag ? p.ps : p.pc) + pos),
-                                    iv[e]);
-        }
-        atomicAdd(reinterpret_cast<float4*>(J.tgt[0] + off + q0), make_float4(iv[0], iv[1], iv[2], iv[3]));
+    if constexpr (V == 2) {
+        atomicAdd(reinterpret_cast<float2*>(q), v);
     } else {
-        const float4 l4 = __ldg(reinterpret_cast<const float4*>(J.coef[0] + q0));
-        const float4 m4 = __ldg(reinterpret_cast<const float4*>(J.coef[1] + q0));
-        const float lv[4] = {l4.x, l4.y, l4.z, l4.w};
-        const float mv[4] = {m4.x, m4.y, m4.z, m4.w};
-#pragma unroll
-        for (int t = 0; t < 3; ++t) {
-            float iv[4];
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const int pos = pos0 + e;
-                iv[e] = increment(dt, normal_coef(lv[e], mv[e], t == J.diag), d[e]);
-                if (in_slab(pos, p.n, p.L))
-                    iv[e] = split_delta(J.slab[t], srow + slab_pos(pos, p.n, p.L), __ldg(p.pc + pos), iv[e]);
-            }
-            atomicAdd(reinterpret_cast<float4*>(J.tgt[t] + off + q0), make_float4(iv[0], iv[1], iv[2], iv[3]));
-        }
+        atomicAdd(q, v.x);
+        if (two) atomicAdd(q + D, v.y);
     }
 }
 
 // Epilogue for one cell (odd nx in the y / z passes, any length in the x pass,
-// the circulant passes): the same arithmetic as epilogue_pair / epilogue_quad,
+// the circulant passes): the same arithmetic as the pass epilogues,
 // one cell at a time.
 __device__ __forceinline__ void epilogue_one(const PassParams& p, const PassJob& J, size_t q, int pos, int x, int y,
                                              int z, float d, size_t off, size_t soff)
@@ -396,12 +370,12 @@ __device__ __forceinline__ void epilogue_one(const PassParams& p, const PassJob&
     if (!ES_INB(p, q, p.ext_c)) return;
     const float dt = p.dt;
     const bool slab = in_slab(pos, p.n, p.L);
-    const int S = 2 * p.L + 1;
+    const int S = p.S;
     if (J.kind == JOB_SINGLE) {
         float inc = increment(dt, __ldg(J.coef[0] + q), d);
         if (slab) {
             const float P = __ldg((J.stag ? p.ps : p.pc) + pos);
-            const size_t si = slab_index(p.axis, x, y, z, slab_pos(pos, p.n, p.L), p.nx, p.ny, S);
+            const size_t si = slab_index(p.axis, x, y, z, slab_pos(pos, p.n, p.L, p.S), p.nx, p.ny, S);
             if (!ES_INB(p, soff + si, p.ext_s)) return;
             inc = split_delta(J.slab[0], soff + si, P, inc);
         }
@@ -409,7 +383,7 @@ __device__ __forceinline__ void epilogue_one(const PassParams& p, const PassJob&
     } else {
         const float lam = __ldg(J.coef[0] + q), mu = __ldg(J.coef[1] + q);
         const float P = slab ? __ldg(p.pc + pos) : 1.f;
-        const size_t si = slab ? slab_index(p.axis, x, y, z, slab_pos(pos, p.n, p.L), p.nx, p.ny, S) : 0;
+        const size_t si = slab ? slab_index(p.axis, x, y, z, slab_pos(pos, p.n, p.L, p.S), p.nx, p.ny, S) : 0;
         if (slab && !ES_INB(p, soff + si, p.ext_s)) return;
 #pragma unroll
         for (int t = 0; t < 3; ++t) {
@@ -421,93 +395,112 @@ __device__ __forceinline__ void epilogue_one(const PassParams& p, const PassJob&
 }
 
 // ---------------------------------------------------------------------------
-// FFT core on the shared [pos][line] layout (one buffer, updated in place:
-// every stage reads all its inputs, the block synchronises, then it writes)
+// FFT core on the shared [pos][quad] rows (one buffer, updated in place:
+// every stage reads all its inputs, the block synchronises, then it writes).
+// Thread (j, c): j = tid / PAIRS, quad c = tid % PAIRS.
 // ---------------------------------------------------------------------------
-template <int RA, int RB, int CPAD>
+constexpr int PAIRS = 16;  // pencil pairs per row of a tile (32 pencils, 128 bytes)
+
+// the butterfly of a stage of B dealt over T threads: past the last one the last
+// one again (the same values go to the same places, which costs less than
+// branches around register arrays: those spill)
+template <int B, int T>
+__device__ __forceinline__ int butterfly(int b)
+{
+    return B % T == 0 ? b : min(b, B - 1);
+}
+
+template <int RA, int RB, int T_>
 struct Core {
     static constexpr int N = RA * RB;
-    static constexpr int BA = N / RA;   // stage-A butterflies = threads per line
+    static constexpr int R1 = RA;
+    static constexpr int BA = N / RA;   // stage-A butterflies
     static constexpr int BB = N / RB;   // stage-B butterflies
-    static constexpr int T = BA;
-    static constexpr int MB = (BB + T - 1) / T;
+    static constexpr int T = T_;        // threads per pair
+    static constexpr int MA = (BA + T - 1) / T, MB = (BB + T - 1) / T;  // butterflies per thread
 
-    // stage A (radix RA, Stockham Ns = 1): a[] holds elements j + r BA; the
-    // result goes to element j RA + q
-    static __device__ __forceinline__ void stageA_store(const float2* a, float2* buf, int j, int c)
+    // first forward stage (radix RA, Stockham Ns = 1) on elements b + r BA, b = j + m T; row(e)
+    // reads source element e
+    template <class Row>
+    static __device__ __forceinline__ void stageA(float2 (&a)[MA][RA], int j, Row row)
     {
 #pragma unroll
-        for (int q = 0; q < RA; ++q) buf[(j * RA + q) * CPAD + c] = a[q];
+        for (int m = 0; m < MA; ++m) {
+            const int b = butterfly<BA, T>(j + m * T);
+#pragma unroll
+            for (int r = 0; r < RA; ++r) a[m][r] = row(b + r * BA);
+            Dft<RA>::run(a[m]);
+        }
+    }
+    // its results to elements b RA + q
+    static __device__ __forceinline__ void stageA_store(const float2 (&a)[MA][RA], float2* buf, int j, int c)
+    {
+#pragma unroll
+        for (int m = 0; m < MA; ++m) {
+            const int b = butterfly<BA, T>(j + m * T);
+#pragma unroll
+            for (int q = 0; q < RA; ++q) buf[(b * RA + q) * PAIRS + c] = a[m][q];
+        }
     }
 
     // stage B (radix RB, Ns = RA), spectral multiply, conjugate, first inverse
     // stage (radix RB, Ns = 1), all in registers
-    static __device__ __forceinline__ void stageB_compute(const float2* buf, float2 (&v)[MB][RB], const float2* tw,
-                                                          const float2* H, int j, int c)
-    {
-#pragma unroll
-        for (int m = 0; m < MB; ++m) {
-            const int b = j + m * T;
-            if (BB % T == 0 || b < BB) {
-                const int k = b % RA;
-#pragma unroll
-                for (int r = 0; r < RB; ++r) {
-                    const float2 x = buf[(b + r * BB) * CPAD + c];
-                    v[m][r] = r == 0 ? x : cmul(x, tw[k * r]);
-                }
-                Dft<RB>::run(v[m]);
-#pragma unroll
-                for (int q = 0; q < RB; ++q) {
-                    const float2 y = cmul(H[b + q * BB], v[m][q]);
-                    v[m][q] = make_float2(y.x, -y.y);
-                }
-                Dft<RB>::run(v[m]);
-            }
-        }
-    }
-    static __device__ __forceinline__ void stageB_store(float2* buf, const float2 (&v)[MB][RB], int j, int c)
-    {
-#pragma unroll
-        for (int m = 0; m < MB; ++m) {
-            const int b = j + m * T;
-            if (BB % T == 0 || b < BB) {
-#pragma unroll
-                for (int q = 0; q < RB; ++q) buf[(b * RB + q) * CPAD + c] = v[m][q];
-            }
-        }
-    }
-
-    // last inverse stage (radix RA, Ns = RB): a[q] = conj(result) at element
-    // j + q BA, so a[q].x / a[q].y are the derivatives of pencils 2c / 2c+1
-    static __device__ __forceinline__ void stageA_inv_load(const float2* buf, const float2* tw, float2* a, int j,
-                                                           int c)
-    {
-        const int k = j % RB;
-#pragma unroll
-        for (int r = 0; r < RA; ++r) {
-            const float2 x = buf[(j + r * BA) * CPAD + c];
-            a[r] = r == 0 ? x : cmul(x, tw[k * r]);
-        }
-    }
-    static __device__ __forceinline__ void stageA_inv_finish(float2* a)
-    {
-        Dft<RA>::run(a);
-#pragma unroll
-        for (int q = 0; q < RA; ++q) a[q].y = -a[q].y;
-    }
-    static __device__ __forceinline__ void stageA_inv(const float2* buf, const float2* tw, float2* a, int j, int c)
-    {
-        stageA_inv_load(buf, tw, a, j, c);
-        stageA_inv_finish(a);
-    }
-
-    // everything between the first forward and the last inverse stage
     static __device__ __forceinline__ void middle(float2* buf, const float2* tw, const float2* H, int j, int c)
     {
         float2 v[MB][RB];
-        stageB_compute(buf, v, tw, H, j, c);
+#pragma unroll
+        for (int m = 0; m < MB; ++m) {
+            const int b = butterfly<BB, T>(j + m * T);
+            const int k = b % RA;
+#pragma unroll
+            for (int r = 0; r < RB; ++r) {
+                const float2 x = buf[(b + r * BB) * PAIRS + c];
+                v[m][r] = r == 0 ? x : cmul(x, tw[k * r]);
+            }
+            Dft<RB>::run(v[m]);
+#pragma unroll
+            for (int q = 0; q < RB; ++q) {
+                const float2 y = cmul(H[b + q * BB], v[m][q]);
+                v[m][q] = make_float2(y.x, -y.y);
+            }
+            Dft<RB>::run(v[m]);
+        }
         __syncthreads();
-        stageB_store(buf, v, j, c);
+#pragma unroll
+        for (int m = 0; m < MB; ++m) {
+            const int b = butterfly<BB, T>(j + m * T);
+#pragma unroll
+            for (int q = 0; q < RB; ++q) buf[(b * RB + q) * PAIRS + c] = v[m][q];
+        }
+    }
+
+    // last inverse stage (radix RA, Ns = RB): conj(a[m][q]) = the result at
+    // element b + q BA
+    static __device__ __forceinline__ void stageA_inv(const float2* buf, const float2* tw, float2 (&a)[MA][RA], int j,
+                                                      int c)
+    {
+#pragma unroll
+        for (int m = 0; m < MA; ++m) {
+            const int b = butterfly<BA, T>(j + m * T);
+            const int k = b % RB;
+#pragma unroll
+            for (int r = 0; r < RA; ++r) {
+                const float2 x = buf[(b + r * BA) * PAIRS + c];
+                a[m][r] = r == 0 ? x : cmul(x, tw[k * r]);
+            }
+            Dft<RA>::run(a[m]);
+        }
+    }
+    // put(e, v) for every element e this thread's last stage ends on
+    template <class Put>
+    static __device__ __forceinline__ void results(const float2 (&a)[MA][RA], int j, Put put)
+    {
+#pragma unroll
+        for (int m = 0; m < MA; ++m) {
+            const int b = butterfly<BA, T>(j + m * T);
+#pragma unroll
+            for (int q = 0; q < RA; ++q) put(b + q * BA, a[m][q]);
+        }
     }
 };
 
@@ -519,18 +512,31 @@ struct Core {
 // stages whose radices multiply to Ns: butterfly b (k = b mod Ns) reads
 // elements b + r n/R times W_(Ns R)^(k r), runs the R-point DFT and writes
 // element (b / Ns) Ns R + k + q Ns.  All stages but the first and the last
-// run on the shared buffer; n/R1 threads per line, every butterfly of a
-// stage by one thread.
-template <int R1, int R2, int R3, int CPAD>
+// run on the shared buffer, every butterfly of a stage by one thread.
+template <int R1_, int R2, int R3, int T_>
 struct Core3 {
+    static constexpr int R1 = R1_;
     static constexpr int N = R1 * R2 * R3;
-    static constexpr int BA = N / R1;  // first / last stage butterflies = threads per line
-    static constexpr int T = BA;
-
-    static __device__ __forceinline__ void stageA_store(const float2* a, float2* buf, int j, int c)
+    static constexpr int BA = N / R1;  // first / last stage butterflies
+    static constexpr int T = T_;       // threads per pair
+    static constexpr int MA = BA / T;  // first / last stage butterflies per thread
+    static_assert(BA % T == 0, "the first stage deals its butterflies evenly");
+    template <class Row>
+    static __device__ __forceinline__ void stageA(float2 (&a)[MA][R1], int j, Row row)
     {
 #pragma unroll
-        for (int q = 0; q < R1; ++q) buf[(j * R1 + q) * CPAD + c] = a[q];
+        for (int m = 0; m < MA; ++m) {
+#pragma unroll
+            for (int r = 0; r < R1; ++r) a[m][r] = row(j + m * T + r * BA);
+            Dft<R1>::run(a[m]);
+        }
+    }
+    static __device__ __forceinline__ void stageA_store(const float2 (&a)[MA][R1], float2* buf, int j, int c)
+    {
+#pragma unroll
+        for (int m = 0; m < MA; ++m)
+#pragma unroll
+            for (int q = 0; q < R1; ++q) buf[((j + m * T) * R1 + q) * PAIRS + c] = a[m][q];
     }
 
     // one stage of radix R after radices multiplying to NS, shared buffer to
@@ -542,26 +548,22 @@ struct Core3 {
         float2 v[M][R];
 #pragma unroll
         for (int m = 0; m < M; ++m) {
-            const int b = j + m * T;
-            if (B % T == 0 || b < B) {
-                const int k = b % NS;
+            const int b = butterfly<B, T>(j + m * T);
+            const int k = b % NS;
 #pragma unroll
-                for (int r = 0; r < R; ++r) {
-                    const float2 x = buf[(b + r * B) * CPAD + c];
-                    v[m][r] = r == 0 ? x : cmul(x, tw[k * r * TS]);
-                }
-                Dft<R>::run(v[m]);
+            for (int r = 0; r < R; ++r) {
+                const float2 x = buf[(b + r * B) * PAIRS + c];
+                v[m][r] = r == 0 ? x : cmul(x, tw[k * r * TS]);
             }
+            Dft<R>::run(v[m]);
         }
         __syncthreads();
 #pragma unroll
         for (int m = 0; m < M; ++m) {
-            const int b = j + m * T;
-            if (B % T == 0 || b < B) {
-                const int k = b % NS, o = (b / NS) * NS * R + k;
+            const int b = butterfly<B, T>(j + m * T);
+            const int k = b % NS, o = (b / NS) * NS * R + k;
 #pragma unroll
-                for (int q = 0; q < R; ++q) buf[(o + q * NS) * CPAD + c] = v[m][q];
-            }
+            for (int q = 0; q < R; ++q) buf[(o + q * NS) * PAIRS + c] = v[m][q];
         }
     }
 
@@ -576,112 +578,184 @@ struct Core3 {
             float2 v[M][R3];
 #pragma unroll
             for (int m = 0; m < M; ++m) {
-                const int b = j + m * T;
-                if (B % T == 0 || b < B) {
+                const int b = butterfly<B, T>(j + m * T);
 #pragma unroll
-                    for (int r = 0; r < R3; ++r) {
-                        const float2 x = buf[(b + r * B) * CPAD + c];
-                        v[m][r] = r == 0 ? x : cmul(x, tw[b * r]);
-                    }
-                    Dft<R3>::run(v[m]);
-#pragma unroll
-                    for (int q = 0; q < R3; ++q) {
-                        const float2 y = cmul(H[b + q * B], v[m][q]);
-                        v[m][q] = make_float2(y.x, -y.y);
-                    }
-                    Dft<R3>::run(v[m]);
+                for (int r = 0; r < R3; ++r) {
+                    const float2 x = buf[(b + r * B) * PAIRS + c];
+                    v[m][r] = r == 0 ? x : cmul(x, tw[b * r]);
                 }
+                Dft<R3>::run(v[m]);
+#pragma unroll
+                for (int q = 0; q < R3; ++q) {
+                    const float2 y = cmul(H[b + q * B], v[m][q]);
+                    v[m][q] = make_float2(y.x, -y.y);
+                }
+                Dft<R3>::run(v[m]);
             }
             __syncthreads();
 #pragma unroll
             for (int m = 0; m < M; ++m) {
-                const int b = j + m * T;
-                if (B % T == 0 || b < B) {
+                const int b = butterfly<B, T>(j + m * T);
 #pragma unroll
-                    for (int q = 0; q < R3; ++q) buf[(b * R3 + q) * CPAD + c] = v[m][q];
-                }
+                for (int q = 0; q < R3; ++q) buf[(b * R3 + q) * PAIRS + c] = v[m][q];
             }
         }
         __syncthreads();
         stage<R2, R3>(buf, tw, j, c);
     }
 
-    // last inverse stage (radix R1, Ns = n/R1, so k = j); a[q] = conj(result)
-    // at element j + q BA
-    static __device__ __forceinline__ void stageA_inv(const float2* buf, const float2* tw, float2* a, int j, int c)
+    // last inverse stage (radix R1, Ns = n/R1, so k = b): conj(a[m][q]) = the
+    // result at element b + q BA, b = j + m T
+    static __device__ __forceinline__ void stageA_inv(const float2* buf, const float2* tw, float2 (&a)[MA][R1], int j,
+                                                      int c)
     {
 #pragma unroll
-        for (int r = 0; r < R1; ++r) {
-            const float2 x = buf[(j + r * BA) * CPAD + c];
-            a[r] = r == 0 ? x : cmul(x, tw[j * r]);
-        }
-        Dft<R1>::run(a);
+        for (int m = 0; m < MA; ++m) {
+            const int b = j + m * T;
 #pragma unroll
-        for (int q = 0; q < R1; ++q) a[q].y = -a[q].y;
+            for (int r = 0; r < R1; ++r) {
+                const float2 x = buf[(b + r * BA) * PAIRS + c];
+                a[m][r] = r == 0 ? x : cmul(x, tw[b * r]);
+            }
+            Dft<R1>::run(a[m]);
+        }
+    }
+    template <class Put>
+    static __device__ __forceinline__ void results(const float2 (&a)[MA][R1], int j, Put put)
+    {
+#pragma unroll
+        for (int m = 0; m < MA; ++m)
+#pragma unroll
+            for (int q = 0; q < R1; ++q) put(j + m * T + q * BA, a[m][q]);
     }
 };
 
 // the FFT core of a plan (RC = 1: two stages)
-template <int RA, int RB, int RC, int CPAD>
-using CoreOf = std::conditional_t<RC == 1, Core<RA, RB, CPAD>, Core3<RA, RB, RC, CPAD>>;
+template <int RA, int RB, int RC, int T>
+using CoreOf = std::conditional_t<RC == 1, Core<RA, RB, T>, Core3<RA, RB, RC, T>>;
 
-// asynchronous 8-byte global -> shared copy (cp.async, through L1); no
-// register is held while it is in flight
-__device__ __forceinline__ void cp_async8(void* dst, const void* src)
+// asynchronous BYTES-byte global -> shared copy (cp.async); ok == false writes
+// zeros and reads nothing
+template <int BYTES>
+__device__ __forceinline__ void cp_async(void* dst, const void* src, bool ok)
 {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"((unsigned)__cvta_generic_to_shared(dst)),
-                 "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async4(void* dst, const void* src)
-{
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"((unsigned)__cvta_generic_to_shared(dst)),
-                 "l"(src) : "memory");
+    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+    const int n = ok ? BYTES : 0;
+    if constexpr (BYTES == 16)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(d), "l"(src), "r"(n) : "memory");
+    else
+        asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;\n" ::"r"(d), "l"(src), "n"(BYTES), "r"(n)
+                     : "memory");
 }
 __device__ __forceinline__ void cp_async_commit_wait_all()
 {
     asm volatile("cp.async.commit_group;\ncp.async.wait_all;\n" ::: "memory");
 }
 
-constexpr int CP = 16;  // complex lines (pencil pairs) per CTA
+template <int T>
+__host__ __device__ constexpr int pass_threads() { return T * PAIRS; }
 
-template <int RA, int RB, int RC>
-__host__ __device__ constexpr int pass_threads() { return RB * RC * CP; }
-
-// blocks per SM the register budget is sized for (about 1024 threads per SM;
-// 1200 for the three-stage plans, whose butterflies hold fewer registers)
-template <int RA, int RB, int RC>
-__host__ __device__ constexpr int pass_min_blocks()
+// blocks per SM the register budget is sized for, from the pairs a thread
+// carries through its largest stage (80 registers up to 16 pairs: measured on
+// the two-stage plans, where a spill costs more than the CTA it buys)
+template <int RA, int RB, int RC, int T>
+__host__ __device__ constexpr int pass_min_blocks(int small = 1024)
 {
-    return pass_threads<RA, RB, RC>() >= 1024 ? 1 : (RC == 1 ? 1024 : 1200) / pass_threads<RA, RB, RC>();
+    constexpr int N = RA * RB * RC;
+    auto held = [](int r) { return (N / r + T - 1) / T * r; };
+    constexpr int top = held(RA) > held(RB) ? (held(RA) > held(RC) ? held(RA) : held(RC))
+                                            : (held(RB) > held(RC) || RC == 1 ? held(RB) : held(RC));
+    // `small`: threads per SM for plans that hold 10 pairs or fewer
+    const int per_sm = top > 16 ? 640 : (top > 10 ? 768 : small);
+    const int b = per_sm / ((pass_threads<T>() + 31) / 32 * 32);
+    return b < 1 ? 1 : (b > 24 ? 24 : b);
 }
 
-// rows of wrap-around copies on each side of the strided passes' reloaded
-// source tile
-constexpr int HALO = 5;
-static_assert(-near_ofs(-1) <= HALO && near_ofs(+1) + NEAR_TAPS - 1 <= HALO, "near taps reach beyond the halo");
+// Whether the near parts wait in tensor memory (2 n / T columns of 32 bits per
+// warp) instead of a third shared tile: from 12 positions per thread on, three
+// tiles per CTA, not the registers, would limit the CTAs on an SM.  tcgen05.st /
+// ld work on whole warps, four of them side by side in the tensor memory's lanes.
+template <int N, int T>
+__host__ __device__ constexpr bool near_in_tmem()
+{
+    return N / T >= 12 && N / T % 4 == 0 && pass_threads<T>() % 32 == 0;
+}
+// columns to allocate: a power of two, at least 32
+template <int N, int T>
+__host__ __device__ constexpr unsigned tmem_columns()
+{
+    constexpr unsigned n = 2 * (N / T) * ((pass_threads<T>() / 32 + 3) / 4);
+    return n <= 32 ? 32 : (n <= 64 ? 64 : (n <= 128 ? 128 : 256));
+}
+// positions whose near parts move to or from tensor memory (and whose
+// coefficients are in flight) at once
+template <int RN>
+__host__ __device__ constexpr int epi_batch()
+{
+    return RN % 4 == 0 ? 4 : (RN % 5 == 0 ? 5 : (RN % 3 == 0 ? 3 : 2));
+}
 
-// shared bytes: one buffer [N + 2 HALO][CP] (FFT, then the source tile) + tables (y, z passes)
-template <int RA, int RB, int RC>
+// shared bytes of the y / z passes: two tiles [N][PAIRS] (the current one,
+// source then FFT buffer; the next one, arriving), the near parts where they
+// are not in tensor memory, twiddles and both multipliers
+template <int N, int T>
 __host__ __device__ constexpr size_t pass_smem_strided()
 {
-    return sizeof(float2) * ((size_t)(RA * RB * RC + 2 * HALO) * CP + 3 * (size_t)RA * RB * RC);
+    return (near_in_tmem<N, T>() ? 2 : 3) * sizeof(float2) * N * PAIRS + 3 * sizeof(float2) * N;
 }
-// x pass, lengths that are not a multiple of 16: cells per near-stencil item
-// (a divisor of n) and the halo of the per-line copy of the source tile
-template <int N>
-__host__ __device__ constexpr int xseg()
-{
-    return N % 5 == 0 ? 5 : (N % 4 == 0 ? 4 : (N % 3 == 0 ? 3 : (N % 2 == 0 ? 2 : 1)));
-}
-constexpr int XHALO = 5;
-// FFT buffer [N][CP + 1] + tables (x pass); for a length that is not a
-// multiple of 16 also the source tile, line by line with XHALO wrap-around
-// copies on each side
-template <int RA, int RB, int RC>
+// of the x pass: the same (the tile as it is in memory, the next one's place,
+// and its turned-around rows); lengths that are not a multiple of 16: the
+// rows, the near parts, twiddles and multiplier
+template <int N, int T>
 __host__ __device__ constexpr size_t pass_smem_x()
 {
-    constexpr size_t N = (size_t)RA * RB * RC;
-    return sizeof(float2) * (N * (CP + 1) + 3 * N) + (N % 16 ? sizeof(float) * 2 * CP * (N + 2 * XHALO) : 0);
+    return N % 16 == 0 ? pass_smem_strided<N, T>() : 2 * sizeof(float2) * N * PAIRS + 2 * sizeof(float2) * N;
+}
+
+// tensor memory as a per-thread store: K consecutive columns of the thread's lane
+template <int K>
+__device__ __forceinline__ void tmem_st(uint32_t addr, const float* v)
+{
+    static_assert(K == 4 || K == 8, "");
+    if constexpr (K == 8)
+        asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"r"(addr),
+                     "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7])
+                     : "memory");
+    else
+        asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "f"(v[0]), "f"(v[1]),
+                     "f"(v[2]), "f"(v[3])
+                     : "memory");
+}
+__device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+template <int K>
+__device__ __forceinline__ void tmem_ld(uint32_t addr, float* v)
+{
+    static_assert(K == 4 || K == 8, "");
+    if constexpr (K == 8)
+        asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];\n"
+                     "tcgen05.wait::ld.sync.aligned;"
+                     : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7])
+                     : "r"(addr)
+                     : "memory");
+    else
+        asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];\ntcgen05.wait::ld.sync.aligned;"
+                     : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3])
+                     : "r"(addr)
+                     : "memory");
+}
+// warp 0 takes the CTA's columns (it waits while other CTAs hold them: they
+// give them back without waiting for this one) and publishes the address
+__device__ __forceinline__ void tmem_alloc(uint32_t* slot, unsigned columns)
+{
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                     (uint32_t)__cvta_generic_to_shared(slot)),
+                 "r"(columns)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void tmem_free(uint32_t addr, unsigned columns)
+{
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(addr), "r"(columns) : "memory");
 }
 
 // Programmatic dependent launch (a pass launched with PDL while the previous
@@ -705,9 +779,9 @@ __device__ __forceinline__ void pdl_begin(int pdl)
 
 // Launch of a pass kernel, with the programmatic-stream-serialization
 // attribute when p.pdl is set (the kernel then waits as p.pdl says).
-template <class K>
+template <class K, class... Args>
 inline cudaError_t launch_pass_kernel(K kernel, dim3 grid, int threads, size_t smem, cudaStream_t st,
-                                      const PassParams& p)
+                                      const PassParams& p, Args... args)
 {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
@@ -719,7 +793,33 @@ inline cudaError_t launch_pass_kernel(K kernel, dim3 grid, int threads, size_t s
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = p.pdl ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, kernel, p);
+    return cudaLaunchKernelEx(&cfg, kernel, p, args...);
+}
+
+// CTAs of a persistent launch over `units` tiles: what the device holds at
+// once (by shared memory, registers and threads), or fewer so that all of them
+// take the same number of tiles
+template <class K>
+inline cudaError_t persistent_grid(K kernel, int threads, size_t smem, int units, int* grid)
+{
+    int dev = 0, sms = 0, sm_smem = 0, sm_regs = 0, sm_threads = 0, reserved = 0;
+    cudaFuncAttributes fa;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sm_smem, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sm_regs, cudaDevAttrMaxRegistersPerMultiprocessor, dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sm_threads, cudaDevAttrMaxThreadsPerMultiProcessor, dev);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, kernel);
+    if (e != cudaSuccess) return e;
+    const int warps = (threads + 31) / 32;
+    const int per_warp = (fa.numRegs + 7) / 8 * 8 * 32;  // registers are given out in eights per thread
+    int per = std::min(sm_threads / (32 * warps), sm_regs / (per_warp * warps));
+    per = std::min(per, (int)(sm_smem / (smem + fa.sharedSizeBytes + reserved)));
+    const int most = sms * std::max(1, per);
+    const int rounds = (units + most - 1) / most;
+    *grid = (units + rounds - 1) / rounds;
+    return cudaSuccess;
 }
 
 // Fused point sources and receivers of this CTA (PassParams::sp_mode): once
@@ -730,9 +830,9 @@ inline cudaError_t launch_pass_kernel(K kernel, dim3 grid, int threads, size_t s
 // and recording kernels (inject_kernel, record_kernel).  job = the CTA's job
 // (blockIdx.y): the velocity z pass's job c updates v_c, the stress y pass's
 // job 1 sxy, the stress z pass's job 0 sxx syy szz, job 1 sxz, job 2 syz.
-__device__ __forceinline__ void special_phase(const PassParams& p, const PassJob& J, int job)
+__device__ __forceinline__ void special_phase(const PassParams& p, const PassJob& J, int job, int tile)
 {
-    const int b0 = p.sp_off[blockIdx.x], b1 = p.sp_off[blockIdx.x + 1];
+    const int b0 = p.sp_off[tile], b1 = p.sp_off[tile + 1];
     if (b0 == b1) return;  // the same for every thread of the CTA
     const int n = *p.step_now - 1;
     __syncthreads();
@@ -790,213 +890,408 @@ __device__ __forceinline__ void prefetch_l2(const void* p)
 {
     asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
 }
-
+// twiddles and the multiplier of this job's direction into shared memory
 template <int N>
-__device__ __forceinline__ void load_tables(const PassParams& p, float2* s_tw, float2* s_hp, float2* s_hm, int tid,
+__device__ __forceinline__ void load_tables(const PassParams& p, const PassJob& J, float2* s_tw, float2* s_h, int tid,
                                             int nthreads)
 {
+    const float2* h = J.sign > 0 ? p.hp : p.hm;
     for (int i = tid; i < N; i += nthreads) {
-        s_tw[i] = p.tw[i];
-        s_hp[i] = p.hp[i];
-        s_hm[i] = p.hm[i];
+        s_tw[i] = __ldg(p.tw + i);
+        s_h[i] = __ldg(h + i);
     }
 }
 
-// y and z passes: blockIdx.x = tile (32 consecutive x at one z (y pass) or
-// one y (z pass)), blockIdx.y = job.  ODD: nx is odd, so a pencil pair does not
-// start on an 8-byte boundary in every row; the pair then moves as two floats
-// (the second one absent at x = nx - 1), with the same arithmetic.
-template <int RA, int RB, int RC, bool ODD>
-__global__ void __launch_bounds__(pass_threads<RA, RB, RC>(), pass_min_blocks<RA, RB, RC>())
-pass_strided(const __grid_constant__ PassParams p)
+// Near part of the rows RA j .. RA j + RA - 1 of pair c: the NEAR_TAPS taps in
+// order from the first offset, the window of rows sliding through registers,
+// wrapped along the axis.  row(e) reads source row e of this pair, put(q, s)
+// takes the result of row RA j + q.
+template <int N, int RA, class Row, class Put>
+__device__ __forceinline__ void near_part(const PassJob& J, int j, Row row, Put put)
 {
-    using C = CoreOf<RA, RB, RC, CP>;
-    constexpr int N = C::N, BA = C::BA, T = C::T;
-    extern __shared__ float2 smem[];
-    float2* buf = smem;  // FFT rows 0 .. N-1; then the source tile at rows HALO + pos (wrapped)
-    float2* s_tw = buf + (N + 2 * HALO) * CP;
+    const int ofs = near_ofs(J.sign);
+    float2 g[NEAR_TAPS];
+#pragma unroll
+    for (int t = 0; t < NEAR_TAPS; ++t) g[t] = rep2(J.g[t]);
+    float2 w[RA + NEAR_TAPS - 1];
+#pragma unroll
+    for (int k = 0; k < RA + NEAR_TAPS - 1; ++k) {
+        int e = RA * j + ofs + k;
+        if (k < 5) e = e < 0 ? e + N : e;             // the first rows of the axis look back over its end,
+        if (k >= RA + 4) e = e >= N ? e - N : e;      // the last ones past it (ofs is -4 or -5)
+        w[k] = row(e);
+        if (k >= NEAR_TAPS - 1) {
+            const int q = k - (NEAR_TAPS - 1);
+            float2 s = make_float2(0.f, 0.f);
+#pragma unroll
+            for (int t = 0; t < NEAR_TAPS; ++t) s = fma2(g[t], w[q + t], s);
+            put(q, s);
+        }
+    }
+}
+
+// A tile of a y or z pass: 32 consecutive x at one z (y pass) or one y (z
+// pass) of one simulation, and the job done on it.
+struct StridedTile {
+    int job, list;   // list: index of the tile in the special-cell lists
+    int x0, outer;
+    size_t base;     // linear index of its first cell
+    size_t off, soff;
+};
+__device__ __forceinline__ StridedTile strided_tile(const PassParams& p, int w, int ntiles)
+{
+    StridedTile t;
+    t.job = 0;
+    while (w >= ntiles) {  // at most njobs - 1 times
+        w -= ntiles;
+        ++t.job;
+    }
+    t.list = w;
+    // simulations run fastest: the CTAs of one tile are adjacent and read that
+    // tile's material rows through L2
+    int sim = 0;
+    if (p.nsim > 1) {
+        sim = w % p.nsim;
+        w /= p.nsim;
+    }
+    const int ntx = (p.nx + 2 * PAIRS - 1) / (2 * PAIRS);
+    t.outer = w / ntx;
+    t.x0 = (w - t.outer * ntx) * 2 * PAIRS;
+    t.base = (size_t)t.x0 + (size_t)p.nx * (p.axis == 1 ? (size_t)p.ny * t.outer : (size_t)t.outer);
+    t.off = (size_t)sim * p.fstride;
+    t.soff = (size_t)sim * p.sstride;
+    return t;
+}
+
+// the tile's source into shared rows, W floats per asynchronous copy, zeros
+// past the last column
+template <int N, int NT, int W>
+__device__ __forceinline__ void stage_strided(const PassParams& p, const StridedTile& t, float2* buf, unsigned est)
+{
+    constexpr int CH = W == 1 ? PAIRS : 2 * PAIRS / W;  // threads per row
+    static_assert(NT % CH == 0, "a thread keeps its columns");
+    const float* src = p.job[t.job].src + t.off + t.base;
+    const int e0 = threadIdx.x / CH, k = threadIdx.x % CH;
+    // floats of a row this thread copies: W from x0 + W k on; W = 1: x0 + k and x0 + PAIRS + k, the
+    // two pencils of pair k
+    const int x = W * k;
+    unsigned o = (unsigned)e0 * est + x;
+    float* d = reinterpret_cast<float*>(buf + e0 * PAIRS) + (W == 1 ? 2 * k : x);
+#pragma unroll 4
+    for (int e = e0; e < N; e += NT / CH, o += NT / CH * est, d += NT / CH * 2 * PAIRS) {
+#pragma unroll
+        for (int f = 0; f < (W == 1 ? 2 : 1); ++f) {
+            const bool ok = t.x0 + x + f * PAIRS < p.nx && ES_INB(p, t.off + t.base + o + f * PAIRS + W - 1, p.ext_f);
+            cp_async<4 * W>(d + f, ok ? src + o + f * PAIRS : src, ok);
+        }
+    }
+}
+
+// Epilogue of a tile of a y or z pass: each thread takes RN consecutive
+// positions of its pair, EB at a time with the next batch's coefficients in
+// flight; the far parts come from the shared rows, the near parts from tensor
+// memory (TM) or their shared rows.  Addresses are a tile's base plus a 32-bit
+// offset.
+//
+// The PML slab rows (the first L and the last L + 1 positions) would all fall to
+// the first and the last warps, which would keep the others waiting while they
+// fetch the old splits: there the derivative goes back into the shared row, and
+// afterwards the CTA takes the slab's (row, pair) items evenly (run_slab).
+template <int RN, int V, bool TM>
+struct StridedEpilogue {
+    static constexpr int EB = epi_batch<RN>();
+    const PassParams& p;
+    const PassJob& J;
+    const StridedTile& t;
+    const unsigned est;
+    float2* const rows;   // the far parts (source tile's rows)
+    const float2* const near;
+    const uint32_t tm;
+    const int c, pos0;
+    const bool valid, two;
+    const float *co0, *co1;
+    unsigned o;
+    float2 c0[EB], c1[EB];
+
+    __device__ __forceinline__ StridedEpilogue(const PassParams& p_, const PassJob& J_, const StridedTile& t_,
+                                               unsigned est_, float2* buf, const float2* nearp, uint32_t tm_)
+        : p(p_), J(J_), t(t_), est(est_), rows(buf), near(nearp), tm(tm_), c((int)threadIdx.x % PAIRS),
+          pos0(RN * ((int)threadIdx.x / PAIRS)), valid(t_.x0 + V * c < p_.nx), two(V == 2 || t_.x0 + PAIRS + c < p_.nx)
+    {
+        co0 = J.coef[0] + t.base;
+        co1 = J.coef[1] + t.base;
+        o = (unsigned)pos0 * est + V * c;
+    }
+    __device__ __forceinline__ void coefs(unsigned oc, bool normal)
+    {
+#pragma unroll
+        for (int e = 0; e < EB; ++e) {
+            const unsigned oe = oc + e * est;
+            if (!valid || !ES_INB(p, t.base + oe + last(), p.ext_c)) continue;
+            c0[e] = ldg_pair<V, PAIRS>(co0 + oe, two);
+            if (normal) c1[e] = ldg_pair<V, PAIRS>(co1 + oe, two);
+        }
+    }
+    __device__ __forceinline__ void first_coefs()
+    {
+        if (J.kind != JOB_STORE) coefs(o, J.kind == JOB_NORMAL);
+    }
+    // offset of the pair's last cell (index checks)
+    __device__ __forceinline__ int last() const { return V == 2 ? 1 : (two ? PAIRS : 0); }
+    // SLAB: slab rows may be among this warp's positions
+    template <int KIND, bool SLAB>
+    __device__ __forceinline__ void run()
+    {
+        constexpr int NT = KIND == JOB_NORMAL ? 3 : 1;
+        float* tgt[NT];
+#pragma unroll
+        for (int k = 0; k < NT; ++k) tgt[k] = J.tgt[k] + t.off + t.base;
+        const float dt = p.dt;
+#pragma unroll 1
+        for (int k0 = 0; k0 < RN; k0 += EB) {
+            float s[2 * EB];
+            if constexpr (TM) tmem_ld<2 * EB>(tm + (uint32_t)(2 * k0), s);
+            float2 d0[EB], d1[EB];
+#pragma unroll
+            for (int e = 0; e < EB; ++e) {
+                d0[e] = c0[e];
+                d1[e] = c1[e];
+            }
+            if (KIND != JOB_STORE && k0 + EB < RN) coefs(o + EB * est, KIND == JOB_NORMAL);
+#pragma unroll
+            for (int e = 0; e < EB; ++e, o += est) {
+                const int pos = pos0 + k0 + e;
+                float2* const row = rows + pos * PAIRS + c;
+                const float2 f = *row;
+                const float2 n = TM ? make_float2(s[2 * e], s[2 * e + 1]) : near[pos * PAIRS + c];
+                const float2 d = make_float2(__fadd_rn(f.x, n.x), __fsub_rn(n.y, f.y));  // far (conj) + near
+                const bool ok = valid && ES_INB(p, t.off + t.base + o + last(), p.ext_f);
+                if (KIND == JOB_STORE) {
+                    if (ok) st_pair<V, PAIRS>(tgt[0] + o, d, two);
+                    continue;
+                }
+#if ES_BOUNDS
+                if (!ok || !ES_INB(p, t.base + o + last(), p.ext_c)) continue;
+#endif
+                if (SLAB && in_slab(pos, p.n, p.L)) {
+                    *row = d;
+                    continue;
+                }
+#pragma unroll
+                for (int k = 0; k < NT; ++k) {
+                    const bool diag = k == J.diag;
+                    const float cx = KIND == JOB_NORMAL ? normal_coef(d0[e].x, d1[e].x, diag) : d0[e].x;
+                    const float cy = KIND == JOB_NORMAL ? normal_coef(d0[e].y, d1[e].y, diag) : d0[e].y;
+                    const float2 inc = make_float2(increment(dt, cx, d.x), increment(dt, cy, d.y));
+                    if (ok) red_pair<V, PAIRS>(tgt[k] + o, inc, two);
+                }
+            }
+        }
+    }
+    // the slab rows, (row, pair) items dealt over the CTA's NTHR threads
+    template <int KIND, int NTHR>
+    __device__ __forceinline__ void run_slab()
+    {
+        constexpr int NT = KIND == JOB_NORMAL ? 3 : 1;
+        const int S = 2 * p.L + 1;
+        const float* prof = J.stag ? p.ps : p.pc;
+        // slab rows have the field's stride along the axis
+        const size_t s0 = t.soff + t.x0 + (p.axis == 1 ? (size_t)p.nx * S * t.outer : (size_t)p.nx * t.outer);
+        if (!valid) return;
+#pragma unroll 1
+        for (int sp = threadIdx.x / PAIRS; sp < S; sp += NTHR / PAIRS) {
+            const int pos = sp < p.L ? sp : sp - p.L + p.n - 1 - p.L;
+            const unsigned q = (unsigned)pos * est + V * c, so = (unsigned)sp * est + V * c;
+            if (!ES_INB(p, t.off + t.base + q + last(), p.ext_f) ||
+                !ES_INB(p, t.base + q + last(), p.ext_c) || !ES_INB(p, s0 + so + last(), p.ext_s))
+                continue;
+            const float2 d = rows[pos * PAIRS + c];
+            const float2 k0 = ldg_pair<V, PAIRS>(co0 + q, two);
+            const float2 k1 = KIND == JOB_NORMAL ? ldg_pair<V, PAIRS>(co1 + q, two) : k0;
+            const float P = __ldg(prof + pos);
+            float2 sv[NT];
+#pragma unroll
+            for (int k = 0; k < NT; ++k) sv[k] = ld_pair<V, PAIRS>(J.slab[k] + s0 + so, two);
+#pragma unroll
+            for (int k = 0; k < NT; ++k) {
+                const bool diag = k == J.diag;
+                const float cx = KIND == JOB_NORMAL ? normal_coef(k0.x, k1.x, diag) : k0.x;
+                const float cy = KIND == JOB_NORMAL ? normal_coef(k0.y, k1.y, diag) : k0.y;
+                float2 inc = make_float2(increment(p.dt, cx, d.x), increment(p.dt, cy, d.y));
+                // split-field update s <- P (P s + inc); the total takes the split's change
+                const float2 sn = make_float2(__fmul_rn(P, __fmaf_rn(P, sv[k].x, inc.x)),
+                                              __fmul_rn(P, __fmaf_rn(P, sv[k].y, inc.y)));
+                st_pair<V, PAIRS>(J.slab[k] + s0 + so, sn, two);
+                inc = make_float2(__fsub_rn(sn.x, sv[k].x), __fsub_rn(sn.y, sv[k].y));
+                red_pair<V, PAIRS>(J.tgt[k] + t.off + t.base + q, inc, two);
+            }
+        }
+    }
+};
+
+// y and z passes, persistent: CTA b takes tiles b, b + gridDim.x, ... of
+// njobs x ntiles (job slowest), and while it works on one, the next one's source
+// arrives in the other half of its shared memory.  V: floats per access of the
+// epilogue (2: nx even; 1: nx odd).
+template <int RA, int RB, int RC, int T, int V>
+__global__ void __launch_bounds__(pass_threads<T>(), pass_min_blocks<RA, RB, RC, T>())
+pass_strided(const __grid_constant__ PassParams p, int ntiles)
+{
+    using C = CoreOf<RA, RB, RC, T>;
+    constexpr int N = C::N, RN = N / T, NT = T * PAIRS;
+    constexpr bool TM = near_in_tmem<N, T>();
+    constexpr int EB = epi_batch<RN>();
+    extern __shared__ __align__(16) float2 smem[];
+    __shared__ uint32_t tmem_slot;
+    float2* nearp = smem + 2 * N * PAIRS;  // near parts (not TM)
+    float2* s_tw = nearp + (TM ? 0 : N * PAIRS);
     float2* s_hp = s_tw + N;
     float2* s_hm = s_hp + N;
     const int tid = threadIdx.x;
-    const int c = tid % CP, j = tid / CP;
-    const PassJob& J = p.job[blockIdx.y];
+    const int c = tid % PAIRS, j = tid / PAIRS;
+    uint32_t tm = 0;
+    // the columns are taken before dependents may launch: a dependent kernel's
+    // CTAs, which may hold columns while they wait for this kernel, then never
+    // keep them from it
+    if (TM) {
+        if (tid < 32) tmem_alloc(&tmem_slot, tmem_columns<N, T>());
+        __syncthreads();
+        tm = tmem_slot + ((uint32_t)(tid / 32 % 4) << 21) + (uint32_t)(tid / 128 * 2 * RN);
+    }
     pdl_begin(p.pdl);
-    // simulations run fastest in blockIdx.x: the CTAs of one tile are adjacent
-    // and read that tile's material rows through L2
-    const int sim = blockIdx.x % p.nsim, tile = blockIdx.x / p.nsim;
-    const size_t off = (size_t)sim * p.fstride, soff = (size_t)sim * p.sstride;
-    const int ntx = (p.nx + 2 * CP - 1) / (2 * CP);
-    const int tx = tile % ntx, outer = tile / ntx;
-    const int x = tx * 2 * CP + 2 * c;
-    const bool valid = x < p.nx;
-    const bool valid1 = x + 1 < p.nx;  // the second pencil of the pair (ODD)
-    size_t base, est;
-    int y = 0, z = 0;
-    if (p.axis == 1) {
-        z = outer;
-        base = (size_t)x + (size_t)p.nx * p.ny * z;
-        est = (size_t)p.nx;
-    } else {
-        y = outer;
-        base = (size_t)x + (size_t)p.nx * y;
-        est = (size_t)p.nx * p.ny;
+    // stride along the axis; offsets within a tile fit 32 bits (an axis has at most 512 cells)
+    const unsigned est = p.axis == 1 ? (unsigned)p.nx : (unsigned)p.nx * p.ny;
+    const int total = ntiles * p.njobs;
+    auto stage = [&](const StridedTile& t, float2* buf) {
+        if (V == 1) stage_strided<N, NT, 1>(p, t, buf, est);
+        else if (p.nx % 4 == 0) stage_strided<N, NT, 4>(p, t, buf, est);
+        else stage_strided<N, NT, 2>(p, t, buf, est);
+    };
+    stage(strided_tile(p, blockIdx.x, ntiles), smem);
+    for (int i = tid; i < N; i += NT) {
+        s_tw[i] = __ldg(p.tw + i);
+        s_hp[i] = __ldg(p.hp + i);
+        s_hm[i] = __ldg(p.hm + i);
     }
-    const float* src = J.src + off + base;
-    float2 a[RA];
-    if constexpr (ODD) {
-#pragma unroll
-        for (int r = 0; r < RA; ++r) {
-            const float* g = src + (size_t)(j + r * BA) * est;
-            a[r].x = valid && ES_INB(p, off + base + (size_t)(j + r * BA) * est, p.ext_f) ? __ldg(g) : 0.f;
-            a[r].y = valid1 && ES_INB(p, off + base + (size_t)(j + r * BA) * est + 1, p.ext_f) ? __ldg(g + 1) : 0.f;
-        }
-    } else {
-#pragma unroll
-        for (int r = 0; r < RA; ++r)
-            a[r] = valid && ES_INB(p, off + base + (size_t)(j + r * BA) * est + 1, p.ext_f)
-                       ? __ldg(reinterpret_cast<const float2*>(src + (size_t)(j + r * BA) * est))
-                       : make_float2(0.f, 0.f);
-    }
-    // coefficient rows of this tile (128 bytes each) into L2 for the epilogue
-    if (tid < N && J.coef[0] && tx * 2 * CP < p.nx) {
-        const size_t row = base - 2 * c + (size_t)tid * est;
-        if (ES_INB(p, row, p.ext_c)) {
-            prefetch_l2(J.coef[0] + row);
-            if (J.coef[1]) prefetch_l2(J.coef[1] + row);
-        }
-    }
-    load_tables<N>(p, s_tw, s_hp, s_hm, tid, T * CP);
-    Dft<RA>::run(a);
-    C::stageA_store(a, buf, j, c);
-    __syncthreads();
-    C::middle(buf, s_tw, J.sign > 0 ? s_hp : s_hm, j, c);
-    __syncthreads();
-    C::stageA_inv(buf, s_tw, a, j, c);
-    __syncthreads();
-    if (valid) {
-        const float* g = src + (size_t)j * est;
-        float2* sb = buf + (j + HALO) * CP + c;
-        const size_t gstep = (size_t)BA * est;
-#pragma unroll 1
-        for (int r = 0; r < RA; ++r, g += gstep, sb += BA * CP) {
-#if ES_BOUNDS
-            if (!ES_INB(p, off + base + (size_t)(j + r * BA) * est + (ODD && !valid1 ? 0 : 1), p.ext_f)) {
-                *sb = make_float2(0.f, 0.f);
-                continue;
+    bool waited = p.pdl != 1;
+    int half = 0;
+    for (int w = blockIdx.x; w < total; w += gridDim.x, half ^= 1) {
+        const PassJob& J = p.job[w / ntiles];
+        float2* buf = smem + half * N * PAIRS;
+        cp_async_commit_wait_all();
+        __syncthreads();  // the tile is there; the other half is no longer read
+        if (w + (int)gridDim.x < total)
+            stage(strided_tile(p, w + gridDim.x, ntiles), smem + (half ^ 1) * N * PAIRS);
+        // coefficient and PML slab rows of this tile (128 bytes each) into L2 for the epilogue
+        if (J.coef[0]) {
+            const StridedTile t = strided_tile(p, w, ntiles);
+            for (int i = tid; i < N; i += NT) {
+                const unsigned o = (unsigned)i * est;
+                if (ES_INB(p, t.base + o, p.ext_c)) {
+                    prefetch_l2(J.coef[0] + t.base + o);
+                    if (J.coef[1]) prefetch_l2(J.coef[1] + t.base + o);
+                }
             }
-#endif
-            if constexpr (ODD) {
-                cp_async4(&sb->x, g);
-                if (valid1) cp_async4(&sb->y, g + 1);
-                else sb->y = 0.f;
-            } else {
-                cp_async8(sb, g);
+            const int S = p.L > 0 ? 2 * p.L + 1 : 0;
+            const size_t s0 = t.soff + t.x0 + (p.axis == 1 ? (size_t)p.nx * S * t.outer : (size_t)p.nx * t.outer);
+            for (int i = tid; i < S; i += NT) {
+                const unsigned o = (unsigned)i * est;
+                if (ES_INB(p, s0 + o, p.ext_s)) {
+                    prefetch_l2(J.slab[0] + s0 + o);
+                    if (J.coef[1]) {
+                        prefetch_l2(J.slab[1] + s0 + o);
+                        prefetch_l2(J.slab[2] + s0 + o);
+                    }
+                }
             }
         }
-    }
-    for (int i = tid; i < 2 * HALO * CP; i += T * CP) {
-        const int h = i / CP, cc = i % CP;
-        const int xc = tx * 2 * CP + 2 * cc;
-        if (xc >= p.nx) continue;
-        const int pos = h < HALO ? N - HALO + h : h - HALO;
-        float2* d = buf + (h < HALO ? h : N + h) * CP + cc;
-        const float* g = J.src + off + base - 2 * c + 2 * cc + (size_t)pos * est;
-#if ES_BOUNDS
-        if (!ES_INB(p, off + base - 2 * c + 2 * cc + (size_t)pos * est + (ODD && xc + 1 >= p.nx ? 0 : 1), p.ext_f)) {
-            *d = make_float2(0.f, 0.f);
-            continue;
-        }
-#endif
-        if constexpr (ODD) {
-            cp_async4(&d->x, g);
-            if (xc + 1 < p.nx) cp_async4(&d->y, g + 1);
-            else d->y = 0.f;
+        if constexpr (TM) {
+            float v[2 * EB];
+            near_part<N, RN>(
+                J, j, [&](int e) { return buf[e * PAIRS + c]; },
+                [&](int q, float2 s) {
+                    v[2 * (q % EB)] = s.x;
+                    v[2 * (q % EB) + 1] = s.y;
+                    if (q % EB == EB - 1) tmem_st<2 * EB>(tm + (uint32_t)(2 * (q - EB + 1)), v);
+                });
         } else {
-            cp_async8(d, g);
+            near_part<N, RN>(
+                J, j, [&](int e) { return buf[e * PAIRS + c]; },
+                [&](int q, float2 s) { nearp[(RN * j + q) * PAIRS + c] = s; });
         }
+        {
+            float2 a[C::MA][RA];
+            C::stageA(a, j, [&](int e) { return buf[e * PAIRS + c]; });
+            __syncthreads();  // the source rows have been read
+            C::stageA_store(a, buf, j, c);
+            __syncthreads();
+            C::middle(buf, s_tw, J.sign > 0 ? s_hp : s_hm, j, c);
+            __syncthreads();
+            C::stageA_inv(buf, s_tw, a, j, c);
+            __syncthreads();  // the FFT's rows have been read
+            C::results(a, j, [&](int e, float2 v) { buf[e * PAIRS + c] = v; });
+        }
+        if (TM) tmem_st_wait();
+        // epilogue of the positions RN j .. RN j + RN - 1 of the thread's pair: one variant per kind
+        // of job and, for whole warps, with or without PML slab rows among their positions
+        const StridedTile t = strided_tile(p, w, ntiles);
+        StridedEpilogue<RN, V, TM> ep(p, J, t, est, buf, nearp, tm);
+        const int r0 = RN * (tid / 32 * (32 / PAIRS)), r1 = r0 + RN * (32 / PAIRS);  // rows of this warp
+        const bool slab = p.L > 0 && (r0 < p.L || r1 > p.n - 1 - p.L);
+        ep.first_coefs();
+        __syncthreads();  // the far parts are there
+        if (!waited) {
+            pdl_wait();  // the previous pass's updates of the targets come first
+            waited = true;
+        }
+        if (J.kind == JOB_STORE) ep.template run<JOB_STORE, false>();
+        else if (J.kind == JOB_SINGLE && !slab) ep.template run<JOB_SINGLE, false>();
+        else if (J.kind == JOB_SINGLE) ep.template run<JOB_SINGLE, true>();
+        else if (!slab) ep.template run<JOB_NORMAL, false>();
+        else ep.template run<JOB_NORMAL, true>();
+        if (p.L > 0 && J.kind != JOB_STORE) {
+            __syncthreads();
+            if (J.kind == JOB_SINGLE) ep.template run_slab<JOB_SINGLE, NT>();
+            else ep.template run_slab<JOB_NORMAL, NT>();
+        }
+        if (p.sp_mode != SP_NONE) special_phase(p, J, t.job, t.list);
     }
-    cp_async_commit_wait_all();
-    __syncthreads();
-    if (valid) {
-        // near part: the 10 taps in order from the first offset, then one add to the far part
-        const int o = HALO + near_ofs(J.sign);
-#pragma unroll
-        for (int q = 0; q < RA; ++q) {
-            const float2* w = buf + (j + q * BA + o) * CP + c;
-            float2 s = make_float2(0.f, 0.f);
-#pragma unroll
-            for (int t = 0; t < NEAR_TAPS; ++t) s = fma2(make_float2(J.g[t], J.g[t]), w[t * CP], s);
-            a[q] = add2(a[q], s);
-        }
-        if (p.pdl == 1) pdl_wait();  // the previous pass's updates of the targets come first
-#pragma unroll
-        for (int q = 0; q < RA; ++q) {
-            const int pos = j + q * BA;
-            if (p.axis == 1) y = pos; else z = pos;
-            const size_t qc = base + (size_t)pos * est;
-            if constexpr (ODD) {
-                epilogue_one(p, J, qc, pos, x, y, z, a[q].x, off, soff);
-                if (valid1) epilogue_one(p, J, qc + 1, pos, x + 1, y, z, a[q].y, off, soff);
-            } else {
-                epilogue_pair(p, J, qc, pos, x, y, z, a[q].x, a[q].y, off, soff);
-            }
-        }
+    if (TM) {
+        __syncthreads();
+        if (tid < 32) tmem_free(tmem_slot, tmem_columns<N, T>());
     }
-    if (p.sp_mode != SP_NONE) special_phase(p, J, blockIdx.y);
 }
 
-// x pass epilogue: the far derivative from the turned-around FFT buffer (bf,
-// [x][line]) plus the near stencil over the source line, read again from
-// global memory (L1 / L2: the CTA read the whole tile at its start), then the
-// field update, four consecutive x of one line per item.  OFS = first tap
-// offset.
-template <int N, int CPAD, int OFS, int NT>
-__device__ __forceinline__ void pass_x_epilogue(const PassParams& p, const PassJob& J, const float* bf,
-                                                const float* src, int line0, int nlines, size_t off, size_t soff)
+// x pass: cell (position x, line r of the tile) of a turned-around tile is
+// float x_at(x, r): row x, the line exchanged within the row (whole pairs) so
+// that the turning accesses of a warp, x_chunks 4-cell chunks of 32 / x_chunks
+// lines (lengths that are a multiple of 16) or 8 cells of 4 lines (others), hit
+// 32 banks.
+template <int N>
+__host__ __device__ constexpr int x_chunks()
 {
-    constexpr int LINES = 2 * CP;
-    constexpr int ITEMS = LINES * N / 4;
+    return N % 32 == 0 ? 8 : 4;
+}
+template <int N>
+__device__ __forceinline__ int x_swz(int x)
+{
+    return N % 32 == 0 ? ((x >> 2) & 7) << 1 : (N % 16 == 0 ? ((x >> 2) & 3) << 2 : (x & 7) << 1);
+}
+template <int N>
+__device__ __forceinline__ int x_at(int x, int r)
+{
+    return x * 2 * PAIRS + (r ^ (x_swz<N>(x) << 1));
+}
 
-    // x = xx - 8 .. xx + 11 in five float4 chunks (wrapped along the line); the
-    // taps of the four outputs reach xx + OFS .. xx + 3 + OFS + NEAR_TAPS - 1
-    static_assert(8 + OFS >= 0 && 8 + 3 + OFS + NEAR_TAPS - 1 < 20, "near taps outside the window");
-#pragma unroll 2
-    for (int i = 0; i < (ITEMS + NT - 1) / NT; ++i) {
-        const int it = (int)threadIdx.x + i * NT;
-        if (ITEMS % NT != 0 && it >= ITEMS) break;
-        const int lo = it & 3, r = (it >> 2) & (LINES - 1), hi = it >> 7;
-        const int xx = (hi * 4 + lo) * 4;
-        const int line = line0 + r;
-        if (line >= nlines) continue;
-        const float* ln = src + (size_t)line * N;
-        float w[20];  // w[m] = f at x = xx - 8 + m
-#pragma unroll
-        for (int m = 0; m < 5; ++m) {
-            const int x0 = (xx - 8 + 4 * m + N) % N;
-            if (4 * m + 3 < 8 + OFS || 4 * m > 8 + 3 + OFS + NEAR_TAPS - 1) continue;  // chunk unused
-#if ES_BOUNDS
-            if (!ES_INB(p, off + (size_t)line * N + x0 + 3, p.ext_f)) return;
-#endif
-            const float4 v = __ldg(reinterpret_cast<const float4*>(ln + x0));
-            w[4 * m] = v.x;
-            w[4 * m + 1] = v.y;
-            w[4 * m + 2] = v.z;
-            w[4 * m + 3] = v.w;
-        }
-        // outputs xx, xx + 1 and xx + 2, xx + 3 as packed pairs
-        float2 s01 = make_float2(0.f, 0.f), s23 = make_float2(0.f, 0.f);
-#pragma unroll
-        for (int t = 0; t < NEAR_TAPS; ++t) {
-            const float2 g2 = make_float2(J.g[t], J.g[t]);
-            s01 = fma2(g2, make_float2(w[8 + OFS + t], w[9 + OFS + t]), s01);
-            s23 = fma2(g2, make_float2(w[10 + OFS + t], w[11 + OFS + t]), s23);
-        }
-        const float sn[4] = {s01.x, s01.y, s23.x, s23.y};
-        float d[4];
-#pragma unroll
-        for (int e = 0; e < 4; ++e) d[e] = __fadd_rn(bf[((xx + e) * CPAD) * 2 + r], sn[e]);
-        epilogue_quad(p, J, (size_t)line * N + xx, xx, line, d, off, soff);
-    }
+// An item of the x pass (lengths that are a multiple of 16): four consecutive
+// cells xx .. xx + 3 of line r of the tile
+template <int N>
+__device__ __forceinline__ void x_item(int it, int* r, int* xx)
+{
+    constexpr int CL = x_chunks<N>();
+    const int lo = it % CL;
+    *r = (it / CL) % (2 * PAIRS);
+    *xx = 4 * (it / (CL * 2 * PAIRS) * CL + lo);
 }
 
 // Epilogue for 4 consecutive cells of an x-pass tile in memory order (f0 =
@@ -1015,7 +1310,7 @@ __device__ __forceinline__ void epilogue_quad_flat(const PassParams& p, const Pa
     if (!ES_INB(p, q0 + 3, p.ext_c)) return;
     const float d[4] = {d4.x, d4.y, d4.z, d4.w};
     const float dt = p.dt;
-    const int S = 2 * p.L + 1;
+    const int S = p.S;
     int xs[4];
     size_t srow[4];
 #pragma unroll
@@ -1033,7 +1328,7 @@ __device__ __forceinline__ void epilogue_quad_flat(const PassParams& p, const Pa
         for (int e = 0; e < 4; ++e) {
             iv[e] = increment(dt, cv[e], d[e]);
             if (in_slab(xs[e], p.n, p.L))
-                iv[e] = split_delta(J.slab[0], srow[e] + slab_pos(xs[e], p.n, p.L),
+                iv[e] = split_delta(J.slab[0], srow[e] + slab_pos(xs[e], p.n, p.L, p.S),
                                     __ldg((J.stag ? p.ps : p.pc) + xs[e]), iv[e]);
         }
         atomicAdd(reinterpret_cast<float4*>(J.tgt[0] + off + q0), make_float4(iv[0], iv[1], iv[2], iv[3]));
@@ -1049,67 +1344,343 @@ __device__ __forceinline__ void epilogue_quad_flat(const PassParams& p, const Pa
             for (int e = 0; e < 4; ++e) {
                 iv[e] = increment(dt, normal_coef(lv[e], mv[e], t == J.diag), d[e]);
                 if (in_slab(xs[e], p.n, p.L))
-                    iv[e] = split_delta(J.slab[t], srow[e] + slab_pos(xs[e], p.n, p.L), __ldg(p.pc + xs[e]), iv[e]);
+                    iv[e] = split_delta(J.slab[t], srow[e] + slab_pos(xs[e], p.n, p.L, p.S), __ldg(p.pc + xs[e]), iv[e]);
             }
             atomicAdd(reinterpret_cast<float4*>(J.tgt[t] + off + q0), make_float4(iv[0], iv[1], iv[2], iv[3]));
         }
     }
 }
 
-// x pass epilogue for a length that is not a multiple of 16.  The derivative
-// of every cell is formed one cell per thread in memory order over the tile
-// (the far part from the turned-around buffer, the near taps read one by one
-// and wrapped along the line: the arithmetic of pass_x_epilogue), written
-// back to the buffer in memory order, and the update then takes four cells
-// per thread with 16-byte coefficient loads and reductions (the tile, 32 n
-// floats from line 32 k, starts on a 16-byte boundary).
-template <int N, int CPAD, int OFS, int NT>
-__device__ __forceinline__ void pass_x_epilogue_any(const PassParams& p, const PassJob& J, float* bf,
-                                                    const float* srcs, int line0, int nlines, size_t off,
-                                                    size_t soff)
+// Epilogue of a tile of the x pass (lengths that are a multiple of 16): item by
+// item, the next item's coefficients in flight; every access is a whole quad,
+// the split parts of the PML slabs included.
+template <int N, int NT, int PER, bool TM, int KIND>
+__device__ __forceinline__ void x_epilogue(const PassParams& p, const PassJob& J, float* bf, const float* nearp,
+                                           uint32_t tm, int line0, int nl, int sim)
 {
-    static_assert(XHALO + OFS >= 0 && XHALO + OFS + NEAR_TAPS - 1 <= 2 * XHALO, "near taps outside the halo");
-    constexpr int LINES = 2 * CP;
-    constexpr int XS = xseg<N>(), NS = N / XS, W = N + 2 * XHALO;
-    constexpr int ITER = (LINES * NS + NT - 1) / NT;
-    static_assert(LINES * N <= 2 * N * CPAD, "the tile's derivatives fit the buffer");
-    const int nl = min(LINES, nlines - line0);
-    const int nf = nl * N;
+    constexpr int LINES = 2 * PAIRS, ITEMS = LINES * N / 4, TG = KIND == JOB_NORMAL ? 3 : 1;
     const int tid = threadIdx.x;
-    // item = XS consecutive cells of one line: a window of XS + NEAR_TAPS - 1
-    // source values from the line's copy, the near taps in order from the
-    // first offset, then one add to the far part
-    float dv[ITER][XS];
+    const size_t cell0 = (size_t)line0 * N, off = (size_t)sim * p.fstride + cell0;
+    const float *co0 = J.coef[0] + cell0, *co1 = J.coef[1] + cell0;
+    float* tgt[TG];
 #pragma unroll
-    for (int i = 0; i < ITER; ++i) {
+    for (int k = 0; k < TG; ++k) tgt[k] = J.tgt[k] + off;
+    const float dt = p.dt;
+    const int S = p.S;
+    const size_t s0 = (size_t)sim * p.sstride + (size_t)line0 * S;
+    const float* prof = J.stag ? p.ps : p.pc;
+    float4 c0 = make_float4(0.f, 0.f, 0.f, 0.f), c1 = c0;
+    auto coefs = [&](int it) {
+        if (KIND == JOB_STORE || (ITEMS % NT != 0 && it >= ITEMS)) return;
+        int r, xx;
+        x_item<N>(it, &r, &xx);
+        if (r >= nl || !ES_INB(p, cell0 + r * N + xx + 3, p.ext_c)) return;
+        c0 = __ldg(reinterpret_cast<const float4*>(co0 + r * N + xx));
+        if (KIND == JOB_NORMAL) c1 = __ldg(reinterpret_cast<const float4*>(co1 + r * N + xx));
+    };
+    coefs(tid);
+#pragma unroll 1
+    for (int i = 0; i < PER; ++i) {
         const int it = tid + i * NT;
-        const int r = it / NS, x0 = (it - r * NS) * XS;
-        if (r < nl) {
-            const float* wrow = srcs + r * W + XHALO + OFS + x0;
-            float w[XS + NEAR_TAPS - 1];
+        if (ITEMS % NT != 0 && it >= ITEMS) break;
+        int r, xx;
+        x_item<N>(it, &r, &xx);
+        float n[4];
+        if constexpr (TM) {
+            tmem_ld<4>(tm + (uint32_t)(4 * i), n);
+        } else {
+            const float4 v = reinterpret_cast<const float4*>(nearp)[it];
+            n[0] = v.x;
+            n[1] = v.y;
+            n[2] = v.z;
+            n[3] = v.w;
+        }
+        const float4 d0 = c0, d1 = c1;
+        if (i + 1 < PER) coefs(it + NT);
+        if (r >= nl || !ES_INB(p, off + r * N + xx + 3, p.ext_f)) continue;
+        float* f = bf + x_at<N>(xx, r);
+        float d[4];
 #pragma unroll
-            for (int k = 0; k < XS + NEAR_TAPS - 1; ++k) w[k] = wrow[k];
+        for (int e = 0; e < 4; ++e) d[e] = __fadd_rn(f[e * LINES], n[e]);
+        const unsigned o = r * N + xx;
+        if (KIND == JOB_STORE) {
+            *reinterpret_cast<float4*>(tgt[0] + o) = make_float4(d[0], d[1], d[2], d[3]);
+            continue;
+        }
+        const float a[4] = {d0.x, d0.y, d0.z, d0.w}, b[4] = {d1.x, d1.y, d1.z, d1.w};
+        const bool slab = p.L > 0 && (xx < p.L || xx + 3 >= N - 1 - p.L);
+        float4 P, old[TG];
+        size_t so = 0;
+        if (slab) {  // the quad's split parts (storage whole quads wide, slab_width)
+            so = s0 + (size_t)r * S + (xx < p.L ? xx : xx - N + S);
+            if (!ES_INB(p, so + 3, p.ext_s)) continue;
+            P = __ldg(reinterpret_cast<const float4*>(prof + xx));
 #pragma unroll
-            for (int e = 0; e < XS; ++e) {
-                float s = 0.f;
+            for (int k = 0; k < TG; ++k) old[k] = *reinterpret_cast<const float4*>(J.slab[k] + so);
+        }
 #pragma unroll
-                for (int t = 0; t < NEAR_TAPS; ++t) s = fmaf(J.g[t], w[e + t], s);
-                dv[i][e] = __fadd_rn(bf[((x0 + e) * CPAD) * 2 + r], s);
+        for (int k = 0; k < TG; ++k) {
+            float v[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+                v[e] = increment(dt, KIND == JOB_NORMAL ? normal_coef(a[e], b[e], k == J.diag) : a[e], d[e]);
+            if (slab) {
+                const float P4[4] = {P.x, P.y, P.z, P.w}, s4[4] = {old[k].x, old[k].y, old[k].z, old[k].w};
+                float n4[4];
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    n4[e] = __fmul_rn(P4[e], __fmaf_rn(P4[e], s4[e], v[e]));  // s <- P (P s + inc)
+                    if (in_slab(xx + e, N, p.L)) v[e] = __fsub_rn(n4[e], s4[e]);
+                }
+                *reinterpret_cast<float4*>(J.slab[k] + so) = make_float4(n4[0], n4[1], n4[2], n4[3]);
+            }
+            atomicAdd(reinterpret_cast<float4*>(tgt[k] + o), make_float4(v[0], v[1], v[2], v[3]));
+        }
+    }
+}
+
+// x pass for lengths that are a multiple of 16, persistent as the y and z
+// passes: a tile is 32 consecutive x-lines (line = y + ny z), one contiguous
+// block of memory, which arrives as it is (raw) while the previous tile is
+// worked on.  Items (four consecutive cells of a line) form the near parts
+// along their line and turn the tile around into the FFT's [position][pencil]
+// rows; at the end they read the far parts back from the turned-around rows, so
+// every access to memory is four consecutive cells of 4 (or 8) lines per warp.
+template <int RA, int RB, int RC, int T>
+__global__ void __launch_bounds__(pass_threads<T>(), pass_min_blocks<RA, RB, RC, T>())
+pass_x(const __grid_constant__ PassParams p, int ntiles)
+{
+    using C = CoreOf<RA, RB, RC, T>;
+    constexpr int N = C::N, RN = N / T, NT = T * PAIRS;
+    constexpr bool TM = near_in_tmem<N, T>();
+    constexpr int LINES = 2 * PAIRS;
+    constexpr int ITEMS = LINES * N / 4, PER = (ITEMS + NT - 1) / NT;  // items, and per thread
+    static_assert(!TM || ITEMS % NT == 0, "tensor memory is read by whole warps");
+    extern __shared__ __align__(16) float2 smem[];
+    __shared__ uint32_t tmem_slot;
+    float* raw = reinterpret_cast<float*>(smem);  // the tile as it is in memory
+    float2* buf = smem + N * PAIRS;               // turned around: the FFT's rows
+    float* nearp = reinterpret_cast<float*>(buf + N * PAIRS);  // near parts, item by item (not TM)
+    float2* s_tw = buf + N * PAIRS + (TM ? 0 : N * PAIRS);
+    float2* s_hp = s_tw + N;
+    float2* s_hm = s_hp + N;
+    float* bf = reinterpret_cast<float*>(buf);
+    const int tid = threadIdx.x;
+    const int c = tid % PAIRS, j = tid / PAIRS;
+    uint32_t tm = 0;
+    if (TM) {  // before dependents may launch (see pass_strided)
+        if (tid < 32) tmem_alloc(&tmem_slot, tmem_columns<N, T>());
+        __syncthreads();
+        tm = tmem_slot + ((uint32_t)(tid / 32 % 4) << 21) + (uint32_t)(tid / 128 * 2 * RN);
+    }
+    pdl_begin(p.pdl);
+    // the first pass of a fused time step advances the step counter
+    if (p.step_counter && blockIdx.x == 0 && tid == 0) *p.step_counter += 1;
+    const int nlines = p.ny * p.nz, total = ntiles * p.njobs;
+    auto decode = [&](int w, int* sim) {  // first line of a tile
+        w %= ntiles;
+        *sim = p.nsim > 1 ? w % p.nsim : 0;
+        return (p.nsim > 1 ? w / p.nsim : w) * LINES;
+    };
+    auto stage = [&](int w) {
+        int sim;
+        const int line0 = decode(w, &sim);
+        const int nf = min(LINES, nlines - line0) * N;
+        const size_t q = (size_t)sim * p.fstride + (size_t)line0 * N;
+        const float* src = p.job[w / ntiles].src + q;
+#pragma unroll 4
+        for (int f = 4 * tid; f < LINES * N; f += 4 * NT) {
+            const bool ok = f < nf && ES_INB(p, q + f + 3, p.ext_f);
+            cp_async<16>(raw + f, ok ? src + f : src, ok);
+        }
+    };
+    stage(blockIdx.x);
+    for (int i = tid; i < N; i += NT) {
+        s_tw[i] = __ldg(p.tw + i);
+        s_hp[i] = __ldg(p.hp + i);
+        s_hm[i] = __ldg(p.hm + i);
+    }
+    bool waited = p.pdl != 1;
+    for (int w = blockIdx.x; w < total; w += gridDim.x) {
+        const PassJob& J = p.job[w / ntiles];
+        int sim;
+        const int line0 = decode(w, &sim), nl = min(LINES, nlines - line0);
+        cp_async_commit_wait_all();
+        __syncthreads();  // the tile is there; the previous tile's rows are no longer read
+        // the tile's coefficient and slab lines (contiguous) into L2
+        if (J.coef[0]) {
+            const size_t q = (size_t)line0 * N, end = (size_t)nlines * N;
+            for (int i = tid; i < N; i += NT)
+                if (q + (size_t)i * 32 < end) {
+                    prefetch_l2(J.coef[0] + q + (size_t)i * 32);
+                    if (J.coef[1]) prefetch_l2(J.coef[1] + q + (size_t)i * 32);
+                }
+            if (p.L > 0) {
+                const int S = p.S, ns = nl * S;
+                const size_t s0 = (size_t)sim * p.sstride + (size_t)line0 * S;
+                for (int f = 32 * tid; f < ns; f += 32 * NT) {
+                    prefetch_l2(J.slab[0] + s0 + f);
+                    if (J.coef[1]) {
+                        prefetch_l2(J.slab[1] + s0 + f);
+                        prefetch_l2(J.slab[2] + s0 + f);
+                    }
+                }
+            }
+        }
+        // near parts along the lines, and the turn into the FFT's rows
+        auto items = [&](auto sign) {
+            constexpr int OFS = near_ofs(decltype(sign)::value);
+            // x = xx - 8 .. xx + 11 in five chunks (wrapped along the line); the taps of the four
+            // outputs reach xx + OFS .. xx + 3 + OFS + NEAR_TAPS - 1
+            static_assert(8 + OFS >= 0 && 8 + 3 + OFS + NEAR_TAPS - 1 < 20, "near taps outside the window");
+#pragma unroll 2
+            for (int i = 0; i < PER; ++i) {
+                const int it = tid + i * NT;
+                if (ITEMS % NT != 0 && it >= ITEMS) break;
+                int r, xx;
+                x_item<N>(it, &r, &xx);
+                const float* ln = raw + r * N;
+                float v[20];
+#pragma unroll
+                for (int m = 0; m < 5; ++m) {
+                    if (4 * m + 3 < 8 + OFS || 4 * m > 8 + 3 + OFS + NEAR_TAPS - 1) continue;  // chunk unused
+                    int x0 = xx - 8 + 4 * m;
+                    if (m < 2) x0 = x0 < 0 ? x0 + N : x0;
+                    if (m > 2) x0 = x0 >= N ? x0 - N : x0;
+                    const float4 f = *reinterpret_cast<const float4*>(ln + x0);
+                    v[4 * m] = f.x;
+                    v[4 * m + 1] = f.y;
+                    v[4 * m + 2] = f.z;
+                    v[4 * m + 3] = f.w;
+                }
+                float* d = bf + x_at<N>(xx, r);  // rows xx .. xx + 3 share the exchange
+#pragma unroll
+                for (int e = 0; e < 4; ++e) d[e * LINES] = v[8 + e];
+                // outputs xx, xx + 1 and xx + 2, xx + 3 as packed pairs
+                float2 s01 = make_float2(0.f, 0.f), s23 = make_float2(0.f, 0.f);
+#pragma unroll
+                for (int t = 0; t < NEAR_TAPS; ++t) {
+                    const float2 g = rep2(J.g[t]);
+                    s01 = fma2(g, make_float2(v[8 + OFS + t], v[9 + OFS + t]), s01);
+                    s23 = fma2(g, make_float2(v[10 + OFS + t], v[11 + OFS + t]), s23);
+                }
+                if constexpr (TM) {
+                    const float s[4] = {s01.x, s01.y, s23.x, s23.y};
+                    tmem_st<4>(tm + (uint32_t)(4 * i), s);
+                } else {
+                    reinterpret_cast<float4*>(nearp)[it] = make_float4(s01.x, s01.y, s23.x, s23.y);
+                }
+            }
+        };
+        if (J.sign > 0) items(std::integral_constant<int, 1>{});
+        else items(std::integral_constant<int, -1>{});
+        __syncthreads();  // the rows are there; the raw tile has been read
+        if (w + (int)gridDim.x < total) stage(w + gridDim.x);
+        auto at = [&](int e) { return e * PAIRS + (c ^ x_swz<N>(e)); };
+        {
+            float2 a[C::MA][RA];
+            C::stageA(a, j, [&](int e) { return buf[at(e)]; });
+            __syncthreads();  // the turned-around rows have been read
+            C::stageA_store(a, buf, j, c);
+            __syncthreads();
+            C::middle(buf, s_tw, J.sign > 0 ? s_hp : s_hm, j, c);
+            __syncthreads();
+            C::stageA_inv(buf, s_tw, a, j, c);
+            __syncthreads();  // the FFT's rows have been read
+            C::results(a, j, [&](int e, float2 v) { buf[at(e)] = make_float2(v.x, -v.y); });
+        }
+        if (TM) tmem_st_wait();
+        __syncthreads();  // the far parts are there
+        if (!waited) {
+            pdl_wait();  // the previous pass's updates of the targets come first
+            waited = true;
+        }
+        if (J.kind == JOB_STORE) x_epilogue<N, NT, PER, TM, JOB_STORE>(p, J, bf, nearp, tm, line0, nl, sim);
+        else if (J.kind == JOB_SINGLE) x_epilogue<N, NT, PER, TM, JOB_SINGLE>(p, J, bf, nearp, tm, line0, nl, sim);
+        else x_epilogue<N, NT, PER, TM, JOB_NORMAL>(p, J, bf, nearp, tm, line0, nl, sim);
+    }
+    if (TM) {
+        __syncthreads();
+        if (tid < 32) tmem_free(tmem_slot, tmem_columns<N, T>());
+    }
+}
+
+// x pass for other lengths: blockIdx.x = tile of 32 consecutive x-lines,
+// blockIdx.y = job.  After the inverse transform the derivatives are turned
+// around through shared memory into memory order (the tile, 32 n floats from
+// line 32 k, starts on a 16-byte boundary), and a thread updates four
+// consecutive cells with 16-byte accesses where every array allows it.
+template <int RA, int RB, int RC, int T>
+__global__ void __launch_bounds__(pass_threads<T>(), pass_min_blocks<RA, RB, RC, T>(1250))
+pass_x_any(const __grid_constant__ PassParams p)
+{
+    using C = CoreOf<RA, RB, RC, T>;
+    constexpr int N = C::N, RN = N / T, NT = T * PAIRS;
+    constexpr int LINES = 2 * PAIRS;
+    extern __shared__ float2 smem[];
+    float2* buf = smem;
+    float2* nearp = buf + N * PAIRS;
+    float2* s_tw = nearp + N * PAIRS;
+    float2* s_h = s_tw + N;
+    float* bf = reinterpret_cast<float*>(buf);
+    const int tid = threadIdx.x;
+    const int c = tid % PAIRS, j = tid / PAIRS;
+    const PassJob& J = p.job[blockIdx.y];
+    pdl_begin(p.pdl);
+    // the first pass of a fused time step advances the step counter
+    if (p.step_counter && blockIdx.x == 0 && blockIdx.y == 0 && tid == 0) *p.step_counter += 1;
+    const int nlines = p.ny * p.nz;
+    const int sim = blockIdx.x % p.nsim;
+    const size_t off = (size_t)sim * p.fstride, soff = (size_t)sim * p.sstride;
+    const int line0 = (blockIdx.x / p.nsim) * LINES;
+    const int nl = min(LINES, nlines - line0);
+    const float* src = J.src + off;
+    constexpr int XB = (N + 7) / 8, CELLS = LINES * XB * 8;
+#pragma unroll
+    for (int i = 0; i < (CELLS + NT - 1) / NT; ++i) {
+        const int it = tid + i * NT;
+        if (CELLS % NT != 0 && it >= CELLS) break;
+        const int r = 4 * ((it >> 5) & 7) + ((it >> 3) & 3), xx = 8 * (it >> 8) + (it & 7);
+        if (xx >= N) continue;
+        float v = 0.f;
+        if (r < nl && ES_INB(p, off + (size_t)(line0 + r) * N + xx, p.ext_f))
+            v = __ldg(src + (size_t)(line0 + r) * N + xx);
+        bf[x_at<N>(xx, r)] = v;
+    }
+    // the tile's coefficient lines (contiguous, N lines of 128 bytes) into L2
+    if (J.coef[0]) {
+        for (int i = tid; i < N; i += NT) {
+            const size_t o = (size_t)line0 * N + (size_t)i * 32;
+            if (o < (size_t)nlines * N) {
+                prefetch_l2(J.coef[0] + o);
+                if (J.coef[1]) prefetch_l2(J.coef[1] + o);
             }
         }
     }
+    load_tables<N>(p, J, s_tw, s_h, tid, NT);
     __syncthreads();
-#pragma unroll
-    for (int i = 0; i < ITER; ++i) {
-        const int it = tid + i * NT;
-        const int r = it / NS, x0 = (it - r * NS) * XS;
-        if (r < nl) {
-#pragma unroll
-            for (int e = 0; e < XS; ++e) bf[r * N + x0 + e] = dv[i][e];
-        }
-    }
+    auto at = [&](int e) { return e * PAIRS + (c ^ x_swz<N>(e)); };
+    near_part<N, RN>(
+        J, j, [&](int e) { return buf[at(e)]; }, [&](int q, float2 s) { nearp[at(RN * j + q)] = s; });
+    float2 a[C::MA][RA];
+    C::stageA(a, j, [&](int e) { return buf[at(e)]; });
+    __syncthreads();  // the staged rows have been read; the near parts are visible
+    C::stageA_store(a, buf, j, c);
     __syncthreads();
+    C::middle(buf, s_tw, s_h, j, c);
+    __syncthreads();
+    C::stageA_inv(buf, s_tw, a, j, c);
+    __syncthreads();  // the FFT rows have been read
+    C::results(a, j, [&](int e, float2 v) {
+        const float2 s = nearp[at(e)];
+        float* o = bf + (2 * c) * N + e;  // lines 2c, 2c + 1 in memory order
+        o[0] = __fadd_rn(v.x, s.x);
+        o[N] = __fsub_rn(s.y, v.y);
+    });
+    __syncthreads();
+    if (p.pdl == 1) pdl_wait();
     const size_t q0 = (size_t)line0 * N;
+    const int nf = nl * N;
     // 16-byte chunks need every array they touch on a 16-byte boundary at the
     // tile (the tile's own offset q0 is a multiple of 4 cells): the targets
     // at this simulation's offset (an odd cell count per simulation leaves
@@ -1121,118 +1692,11 @@ __device__ __forceinline__ void pass_x_epilogue_any(const PassParams& p, const P
     if (J.kind != JOB_STORE) vec = vec && a16(J.coef[0]);
     const int nq = vec ? nf / 4 : 0;
     for (int i = tid; i < nq; i += NT)
-        epilogue_quad_flat<N>(p, J, q0 + 4 * (size_t)i, 4 * i, line0, reinterpret_cast<const float4*>(bf)[i], off,
-                              soff);
+        epilogue_quad_flat<N>(p, J, q0 + 4 * (size_t)i, 4 * i, line0, reinterpret_cast<const float4*>(bf)[i], off, soff);
     // what is left: a last, partial tile's cells past its last full chunk
     for (int f = 4 * nq + tid; f < nf; f += NT) {
         const int r = f / N, x = f - r * N, line = line0 + r;
         epilogue_one(p, J, q0 + f, x, x, line % p.ny, line / p.ny, bf[f], off, soff);
-    }
-}
-
-// x pass: blockIdx.x = tile of 32 consecutive x-lines (line = y + ny z, so
-// the tile is one contiguous block of memory), blockIdx.y = job.  The FFT
-// result is turned around in the shared buffer so that a thread owns four
-// consecutive x of one line (an item) in the epilogue.
-template <int RA, int RB, int RC>
-__global__ void __launch_bounds__(pass_threads<RA, RB, RC>(), pass_min_blocks<RA, RB, RC>())
-pass_x(const __grid_constant__ PassParams p)
-{
-    constexpr int CPAD = CP + 1;  // row padding: the staging transposes stay conflict-free
-    using C = CoreOf<RA, RB, RC, CPAD>;
-    constexpr int N = C::N, BA = C::BA, NT = C::T * CP;
-    constexpr int LINES = 2 * CP;
-    constexpr int ITEMS = LINES * N / 4;  // float4 chunks in the tile (N a multiple of 16)
-    extern __shared__ float2 smem[];
-    float2* buf = smem;
-    float2* s_tw = buf + N * CPAD;
-    float2* s_hp = s_tw + N;
-    float2* s_hm = s_hp + N;
-    const int tid = threadIdx.x;
-    const int c = tid % CP, j = tid / CP;
-    const PassJob& J = p.job[blockIdx.y];
-    pdl_begin(p.pdl);
-    // the first pass of a fused time step advances the step counter
-    if (p.step_counter && blockIdx.x == 0 && blockIdx.y == 0 && tid == 0) *p.step_counter += 1;
-    const int nlines = p.ny * p.nz;
-    const int sim = blockIdx.x % p.nsim;
-    const size_t off = (size_t)sim * p.fstride, soff = (size_t)sim * p.sstride;
-    const int line0 = (blockIdx.x / p.nsim) * LINES;
-    const float* src = J.src + off;
-    // chunk it -> line r = (it / 4) % 32, x = 4 (4 (it / 128) + it % 4): a warp
-    // covers 8 lines x 64 contiguous bytes, and its shared stores hit 32 banks
-    float* bf = reinterpret_cast<float*>(buf);
-    // the tile's coefficient lines (contiguous, N lines of 128 bytes) into L2
-    if (J.coef[0] && tid < N) {
-        const size_t off = (size_t)line0 * N + (size_t)tid * 32;
-        if (off < (size_t)nlines * N) {
-            prefetch_l2(J.coef[0] + off);
-            if (J.coef[1]) prefetch_l2(J.coef[1] + off);
-        }
-    }
-    if constexpr (N % 16 == 0) {
-#pragma unroll
-        for (int i = 0; i < (ITEMS + NT - 1) / NT; ++i) {
-            const int it = tid + i * NT;
-            if (ITEMS % NT != 0 && it >= ITEMS) break;
-            const int lo = it & 3, r = (it >> 2) & (LINES - 1), hi = it >> 7;
-            const int xx = (hi * 4 + lo) * 4;
-            const int line = line0 + r;
-            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (line < nlines && ES_INB(p, off + (size_t)line * N + xx + 3, p.ext_f))
-                v = __ldg(reinterpret_cast<const float4*>(src + (size_t)line * N + xx));
-            bf[((xx + 0) * CPAD) * 2 + r] = v.x;
-            bf[((xx + 1) * CPAD) * 2 + r] = v.y;
-            bf[((xx + 2) * CPAD) * 2 + r] = v.z;
-            bf[((xx + 3) * CPAD) * 2 + r] = v.w;
-        }
-    } else {
-        // any length: the tile is one contiguous run of 32 N floats, read in
-        // order; each value also goes to the per-line source copy (row r at
-        // r (N + 2 XHALO), x at XHALO + x, the ends wrapped on both sides)
-        const float* tile = src + (size_t)line0 * N;
-        const int nf = min(LINES, nlines - line0) * N;
-        float* srcs = reinterpret_cast<float*>(s_hm + N);
-        constexpr int W = N + 2 * XHALO;
-        constexpr int ITER = (LINES * N + NT - 1) / NT;
-#pragma unroll
-        for (int i = 0; i < ITER; ++i) {
-            const int f = tid + i * NT;
-            if (f < LINES * N) {
-                const int r = f / N, xx = f - r * N;
-                const float v = f < nf && ES_INB(p, off + (size_t)line0 * N + f, p.ext_f) ? __ldg(tile + f) : 0.f;
-                bf[(xx * CPAD) * 2 + r] = v;
-                float* row = srcs + r * W + XHALO;
-                row[xx] = v;
-                if (xx < XHALO) row[N + xx] = v;
-                if (xx >= N - XHALO) row[xx - N] = v;
-            }
-        }
-    }
-    load_tables<N>(p, s_tw, s_hp, s_hm, tid, NT);
-    __syncthreads();
-    float2 a[RA];
-#pragma unroll
-    for (int r = 0; r < RA; ++r) a[r] = buf[(j + r * BA) * CPAD + c];
-    Dft<RA>::run(a);
-    __syncthreads();
-    C::stageA_store(a, buf, j, c);
-    __syncthreads();
-    C::middle(buf, s_tw, J.sign > 0 ? s_hp : s_hm, j, c);
-    __syncthreads();
-    C::stageA_inv(buf, s_tw, a, j, c);
-    __syncthreads();
-#pragma unroll
-    for (int q = 0; q < RA; ++q) buf[(j + q * BA) * CPAD + c] = a[q];
-    __syncthreads();
-    if (p.pdl == 1) pdl_wait();  // the previous pass's updates of the targets come first
-    if constexpr (N % 16 == 0) {
-        if (J.sign > 0) pass_x_epilogue<N, CPAD, near_ofs(+1), NT>(p, J, bf, src, line0, nlines, off, soff);
-        else pass_x_epilogue<N, CPAD, near_ofs(-1), NT>(p, J, bf, src, line0, nlines, off, soff);
-    } else {
-        const float* srcs = reinterpret_cast<const float*>(s_hm + N);
-        if (J.sign > 0) pass_x_epilogue_any<N, CPAD, near_ofs(+1), NT>(p, J, bf, srcs, line0, nlines, off, soff);
-        else pass_x_epilogue_any<N, CPAD, near_ofs(-1), NT>(p, J, bf, srcs, line0, nlines, off, soff);
     }
 }
 

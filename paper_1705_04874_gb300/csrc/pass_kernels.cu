@@ -12,7 +12,7 @@ struct PlanRow {
     int n, ra, rb, rc;
 };
 const PlanRow kPlans[] = {
-#define ES_ROW(n, a, b, c) {n, a, b, c},
+#define ES_ROW(n, a, b, c, t) {n, a, b, c},
     ES_PLANS(ES_ROW)
 #undef ES_ROW
 };
@@ -65,40 +65,49 @@ int plan_current(int kind, int n, int* ra, int* rb)
     return 1;
 }
 
-template <int RA, int RB, int RC>
+template <int RA, int RB, int RC, int T>
 static cudaError_t launch_one(const PassParams& p, cudaStream_t st)
 {
-    constexpr int threads = pass_threads<RA, RB, RC>();
+    constexpr int W = 2 * PAIRS;  // pencils per tile
     if (p.axis == 0) {
-        const int lines = p.ny * p.nz;
-        dim3 grid((lines + 2 * CP - 1) / (2 * CP) * p.nsim, p.njobs);
-        return launch_pass_kernel(pass_x<RA, RB, RC>, grid, threads, pass_smem_x<RA, RB, RC>(), st, p);
+        const int ntiles = (p.ny * p.nz + W - 1) / W * p.nsim;
+        constexpr int threads = pass_threads<T>();
+        constexpr size_t smem = pass_smem_x<RA * RB * RC, T>();
+        if constexpr (RA * RB * RC % 16 == 0) {
+            int grid = 0;
+            const cudaError_t e = persistent_grid(pass_x<RA, RB, RC, T>, threads, smem, ntiles * p.njobs, &grid);
+            if (e != cudaSuccess) return e;
+            return launch_pass_kernel(pass_x<RA, RB, RC, T>, dim3((unsigned)grid), threads, smem, st, p, ntiles);
+        } else {
+            return launch_pass_kernel(pass_x_any<RA, RB, RC, T>, dim3((unsigned)ntiles, (unsigned)p.njobs), threads, smem,
+                                      st, p);
+        }
     }
-    const int ntx = (p.nx + 2 * CP - 1) / (2 * CP);
+    const int ntx = (p.nx + W - 1) / W;
     const int outer = p.axis == 1 ? p.nz : p.ny;
-    dim3 grid(ntx * outer * p.nsim, p.njobs);
-    if (p.nx % 2) return launch_strided_odd(RA, RB, RC, grid, p, st);
-    return launch_pass_kernel(pass_strided<RA, RB, RC, false>, grid, threads, pass_smem_strided<RA, RB, RC>(), st,
-                              p);
+    const int ntiles = ntx * outer * p.nsim;
+    if (p.nx % 2 == 0) return launch_strided2(RA, RB, RC, ntiles, p, st);
+    return launch_strided1(RA, RB, RC, ntiles, p, st);
 }
 
-template <int RA, int RB, int RC>
+template <int RA, int RB, int RC, int T>
 static cudaError_t prepare_one()
 {
-    cudaError_t e = cudaFuncSetAttribute(pass_x<RA, RB, RC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)pass_smem_x<RA, RB, RC>());
-    if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(pass_strided<RA, RB, RC, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)pass_smem_strided<RA, RB, RC>());
+    constexpr int smem = (int)pass_smem_x<RA * RB * RC, T>();
+    if constexpr (RA * RB * RC % 16 == 0)
+        return cudaFuncSetAttribute(pass_x<RA, RB, RC, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    else
+        return cudaFuncSetAttribute(pass_x_any<RA, RB, RC, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
 }
 
 cudaError_t prepare_pass_kernels()
 {
     cudaError_t e;
-#define ES_PREP(n, a, b, c) if ((e = prepare_one<a, b, c>()) != cudaSuccess) return e;
+#define ES_PREP(n, a, b, c, t) if ((e = prepare_one<a, b, c, t>()) != cudaSuccess) return e;
     ES_PLANS(ES_PREP)
 #undef ES_PREP
-    if ((e = prepare_strided_odd()) != cudaSuccess) return e;
+    if ((e = prepare_strided2()) != cudaSuccess) return e;
+    if ((e = prepare_strided1()) != cudaSuccess) return e;
     return prepare_circ_kernels();
 }
 
@@ -109,7 +118,7 @@ cudaError_t launch_pass(const PassParams& p, cudaStream_t st)
     const int kind = p.axis == 0 ? 0 : 1;
     if (p.n < 1 || p.n > 256 || g_choice[kind][p.n] < 0) return cudaErrorInvalidValue;
     const PlanRow& r = kPlans[g_choice[kind][p.n]];
-#define ES_CASE(n, a, b, c) if (r.ra == a && r.rb == b && r.rc == c) return launch_one<a, b, c>(p, st);
+#define ES_CASE(n, a, b, c, t) if (r.ra == a && r.rb == b && r.rc == c) return launch_one<a, b, c, t>(p, st);
     ES_PLANS(ES_CASE)
 #undef ES_CASE
     return cudaErrorInvalidValue;
