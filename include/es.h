@@ -21,12 +21,13 @@
  *   finished; into a device buffer, it is complete in stream order.
  * - A model is not thread-safe: one thread at a time per model.
  * - Axis lengths run from 3 to 512; anything else is ES_ERR_SIZE.  The
- *   lengths 16, 32, 48, 64, 80, 96, 128, 160, 192 and 256 take the fused FFT
- *   passes (two-stage plans R1 x R2, R1, R2 in {4,5,6,8,10,12,16}; along y
- *   and z only when nx is even); every other length -- odd or non-smooth
- *   ones such as the paper's 125 x 75 x 301 grid (Sec. III) -- takes the
- *   circulant passes, which apply the same staggered spectral derivative as
- *   an exact periodic convolution with O(n) work per element.
+ *   lengths 16, 32, 48, 64, 75, 80, 96, 125, 128, 160, 192 and 256 take the
+ *   fused FFT passes (two-stage plans R1 x R2, three-stage ones for 75 and
+ *   125); every other length from 16 on -- odd or non-smooth ones such as the
+ *   301 of the paper's 125 x 75 x 301 grid (Sec. III) -- takes the same
+ *   passes as a zero-padded convolution through a longer FFT, and the
+ *   shortest axes a direct sum; both apply the same staggered spectral
+ *   derivative as an exact periodic convolution.
  */
 #ifndef ES_H
 #define ES_H
@@ -65,19 +66,21 @@ int es_model_create(const float* rho, const float* cp, const float* cs, int nx, 
  * ES_PREC_FP32 (default): fused FFT passes where an axis has a plan (each
  * derivative as a 10-point near stencil in FP32 plus the FFT of the rest of
  * the operator, which confines FP32 FFT roundoff to about 1 % of its plain
- * size), FP32 circulant passes on the CUDA cores elsewhere.
+ * size), elsewhere the same derivative as a zero-padded convolution (direct
+ * circulant sums below 16 cells).
  * ES_PREC_COMPENSATED: every axis through the circulant passes with
  * error-free transformations (each product split exactly by one FMA, Knuth's
  * TwoSum on the running sum, the kernel row as FP32 high plus low parts), so
  * each derivative is accurate to about twice FP32's precision and only the
  * FP32 storage of the fields limits the traces (O(n) work per element, about
  * 10 FP32 operations per multiply-add).  ES_PREC_FP32_TC: as ES_PREC_FP32, but
- * circulant axes of 192 to 512 cells run as GEMMs on the tensor cores (the
+ * axes of 192 to 512 cells without an FFT plan run as GEMMs on the tensor cores (the
  * field and the kernel matrix split in three BF16 parts each, six products
  * accumulated in FP32; the near stencil stays on the CUDA cores).  The paper
- * has no tensor-core step: this mode is an opt-in speed-up for long odd axes
- * such as the paper's 301.  Applies from the next es_run.  ES_ERR_ARG for any
- * other mode. */
+ * has no tensor-core step: this mode is an opt-in alternative for long odd axes
+ * such as the paper's 301 (the default mode's passes take 0.078 / 0.084 ms
+ * there, this one's 0.106 / 0.112).  Applies from the next es_run.  ES_ERR_ARG
+ * for any other mode. */
 #define ES_PREC_FP32 0
 #define ES_PREC_COMPENSATED 1
 #define ES_PREC_FP32_TC 2

@@ -1,6 +1,6 @@
-// Staggered spectral derivative passes for axis lengths without an FFT plan
-// (odd or non-smooth lengths such as 75, 125 or 301 = 7 * 43, the paper's
-// own grid; Sec. III).  Along a periodic axis the operator
+// Staggered spectral derivative passes as direct circulant sums: the axes too
+// short for the convolution passes (conv_pass.cuh, n < CONV_MIN_N), and every
+// axis in the compensated mode.  Along a periodic axis the operator
 //   D(+/-) f = IFFT( i kappa exp(+/- i kappa d / 2) FFT(f) )
 // is a real circulant matrix: (D f)_i = sum_j c[(i - j) mod n] f_j with
 // c_l = sum_m H_m exp(2 pi i m l / n), computed once on the host in FP64
@@ -164,7 +164,7 @@ __device__ __forceinline__ void load_kernel_row(float* cw, const float* c, int n
     }
 }
 
-// Long axes (n >= CIRC_DIRECT_N, es_internal.h) give every warp several 16-output chunks:
+// Long axes (n >= CIRC_DIRECT_N, es_internal.h; compensated mode) give every warp several output chunks:
 // the y and z passes then run the epilogue straight from the registers (no output tile,
 // half the shared memory, twice the resident CTAs); shorter axes keep the output tile so
 // that all warps share the epilogue.
@@ -301,7 +301,6 @@ cudaError_t prepare_circ_kernels()
     opt(circ_x<false>);
     opt(circ_x<true>);
     opt(circ_strided<false, false>);
-    opt(circ_strided<false, true>);
     opt(circ_strided<true, false>);
     opt(circ_strided<true, true>);
     return e;
@@ -322,11 +321,9 @@ cudaError_t launch_circ(const PassParams& p, cudaStream_t st)
     const int ntx = (p.nx + TP - 1) / TP;
     const int outer = p.axis == 1 ? p.nz : p.ny;
     dim3 grid((unsigned)(ntx * outer) * p.nsim, p.njobs);
-    const bool direct = p.n >= CIRC_DIRECT_N;
+    const bool direct = p.comp && p.n >= CIRC_DIRECT_N;
     const size_t smem = circ_smem(p.n, p.comp != 0, !direct);
-    if (direct)
-        return launch_pass_kernel(p.comp ? circ_strided<true, true> : circ_strided<false, true>, grid, threads, smem,
-                                  st, p);
+    if (direct) return launch_pass_kernel(circ_strided<true, true>, grid, threads, smem, st, p);
     return launch_pass_kernel(p.comp ? circ_strided<true, false> : circ_strided<false, false>, grid, threads, smem,
                               st, p);
 }

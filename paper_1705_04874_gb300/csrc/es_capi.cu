@@ -211,7 +211,8 @@ int ensure_prepared()
     return ES_OK;
 }
 
-// Axis lengths: an FFT plan (pass_plans.h), else the circulant pass up to
+// Axis lengths: an FFT plan (pass_plans.h), else a convolution pass (conv_plans.h) or, below
+// CONV_MIN_N cells and in the compensated mode, the circulant pass, up to
 // CIRC_MAX_N (circ_pass.cu).  With an odd nx the y and z FFT passes move their
 // x-adjacent pencil pairs as single floats (pass_kernels_odd.cu).
 bool fft_plan(int n) { int a, b; return plan_radices(n, &a, &b) != 0; }
@@ -226,21 +227,33 @@ bool fft_axis(int n, int) { return fft_plan(n); }
 // near + far equals D exactly up to the rounding of the tables.  Axes of NEAR_TAPS cells
 // or fewer keep the whole multiplier (g = 0).  For a circulant axis also the kernels
 // c_l = sum_m H_m / n exp(2 pi i m l / n) (real: H is Hermitian, Nyquist included).
-void axis_tables(int n, double d, std::vector<float2>& tw, std::vector<float2>& hp, std::vector<float2>& hm,
+// For a convolution pass (m > 0) the tables have m entries: tw the m-point twiddles, and the
+// multipliers the m-point transforms / m of the far kernels (c less the taps) laid out over the lags
+// -(n-1) .. n-1.  Angles that are multiples of 2 pi / n (or / m) come from one table of cosines
+// and sines, the same FP64 calls as at each use.
+struct Circle {
+    std::vector<double> c, s;  // cos, sin of 2 pi k / n
+    explicit Circle(int n) : c(n), s(n)
+    {
+        for (int k = 0; k < n; ++k) {
+            const double a = 2.0 * 3.14159265358979323846 * (double)k / (double)n;
+            c[k] = std::cos(a);
+            s[k] = std::sin(a);
+        }
+    }
+};
+
+void axis_tables(int n, double d, int m_conv, std::vector<float2>& tw, std::vector<float2>& hp, std::vector<float2>& hm,
                  float* gp, float* gm, std::vector<double>* ckp = nullptr, std::vector<double>* ckm = nullptr)
 {
     const double pi = 3.14159265358979323846;
-    tw.resize(n);
-    hp.resize(n);
-    hm.resize(n);
+    const Circle cn(n);
     std::vector<double> hr[2], hi[2];
     for (int s = 0; s < 2; ++s) {
         hr[s].resize(n);
         hi[s].resize(n);
     }
     for (int m = 0; m < n; ++m) {
-        const double a = 2.0 * pi * (double)m / (double)n;
-        tw[m] = make_float2((float)std::cos(a), (float)(-std::sin(a)));
         const int mk = (2 * m < n) ? m : m - n;  // even n: bin n/2 -> -n/2
         const double kap = 2.0 * pi * (double)mk / ((double)n * d);
         for (int s = 0; s < 2; ++s) {
@@ -252,17 +265,16 @@ void axis_tables(int n, double d, std::vector<float2>& tw, std::vector<float2>& 
     // c_l of D(+) (s = 0) or D(-) (s = 1), angles reduced exactly in integers
     auto kernel_entry = [&](int s, int l) {
         double acc = 0.0;
-        for (int m = 0; m < n; ++m) {
-            const long long ml = ((long long)m * l) % n;
-            const double a = 2.0 * pi * (double)ml / (double)n;
-            acc += hr[s][m] * std::cos(a) - hi[s][m] * std::sin(a);
+        for (int m = 0, ml = 0; m < n; ++m) {
+            acc += hr[s][m] * cn.c[ml] - hi[s][m] * cn.s[ml];
+            ml += l;
+            if (ml >= n) ml -= n;
         }
         return acc;
     };
     for (int s = 0; s < 2; ++s) {
         float* g = s == 0 ? gp : gm;
         const int ofs = near_ofs(s == 0 ? +1 : -1);
-        std::vector<double> nr(n, 0.0), ni(n, 0.0);  // H_near / n
         // the taps in antisymmetric pairs, g[NEAR_TAPS - 1 - t] = -g[t] (exact for the staggered
         // kernel up to FP64 roundoff; enforced here so the passes can sum differences)
         for (int t = 0; t < NEAR_PAIRS; ++t) {
@@ -273,25 +285,60 @@ void axis_tables(int n, double d, std::vector<float2>& tw, std::vector<float2>& 
             g[t] = (float)(0.5 * (lo - hi));
             g[NEAR_TAPS - 1 - t] = -g[t];
         }
+    }
+    if (ckp && ckm) {
+        ckp->resize(n);
+        ckm->resize(n);
+        for (int l = 0; l < n; ++l) {
+            (*ckp)[l] = kernel_entry(0, l);
+            (*ckm)[l] = kernel_entry(1, l);
+        }
+    }
+    const int len = m_conv > 0 ? m_conv : n;
+    tw.resize(len);
+    hp.resize(len);
+    hm.resize(len);
+    if (m_conv > 0) {
+        const Circle cm(len);
+        for (int k = 0; k < len; ++k) tw[k] = make_float2((float)cm.c[k], (float)(-cm.s[k]));
+        for (int s = 0; s < 2; ++s) {
+            std::vector<double> far = s == 0 ? *ckp : *ckm;
+            const float* g = s == 0 ? gp : gm;
+            for (int t = 0; t < NEAR_TAPS; ++t) {
+                const int delta = near_ofs(s == 0 ? +1 : -1) + t;  // (N f)_i gains g_t f_{i + delta}
+                far[((-delta) % n + n) % n] -= (double)g[t];
+            }
+            // lags 0 .. n-1 at 0 .. n-1, lags -1 .. -(n-1) at len-1 .. len-(n-1)
+            for (int k = 0; k < len; ++k) {
+                double re = far[0], im = 0.0;
+                for (int l = 1, kl = k; l < n; ++l) {
+                    // exp(-2 pi i k l / len) for lag l, its conjugate for lag -l
+                    re += (far[l] + far[n - l]) * cm.c[kl];
+                    im -= (far[l] - far[n - l]) * cm.s[kl];
+                    kl += k;
+                    if (kl >= len) kl -= len;
+                }
+                (s == 0 ? hp : hm)[k] = make_float2((float)(re / len), (float)(im / len));
+            }
+        }
+        return;
+    }
+    for (int m = 0; m < n; ++m) tw[m] = make_float2((float)cn.c[m], (float)(-cn.s[m]));
+    for (int s = 0; s < 2; ++s) {
+        const float* g = s == 0 ? gp : gm;
+        std::vector<double> nr(n, 0.0), ni(n, 0.0);  // H_near / n
         for (int t = 0; t < NEAR_TAPS; ++t) {
             if (n <= NEAR_TAPS) continue;
-            const int delta = ofs + t;                      // (N f)_i gains g_t f_{i + delta}
-            for (int m = 0; m < n; ++m) {
-                const long long md = (((long long)m * delta) % n + n) % n;
-                const double a = 2.0 * pi * (double)md / (double)n;
-                nr[m] += (double)g[t] * std::cos(a) / n;
-                ni[m] += (double)g[t] * std::sin(a) / n;
+            const int delta = ((near_ofs(s == 0 ? +1 : -1) + t) % n + n) % n;  // (N f)_i gains g_t f_{i + delta}
+            for (int m = 0, md = 0; m < n; ++m) {
+                nr[m] += (double)g[t] * cn.c[md] / n;
+                ni[m] += (double)g[t] * cn.s[md] / n;
+                md += delta;
+                if (md >= n) md -= n;
             }
         }
         for (int m = 0; m < n; ++m)
             (s == 0 ? hp : hm)[m] = make_float2((float)(hr[s][m] - nr[m]), (float)(hi[s][m] - ni[m]));
-    }
-    if (!ckp || !ckm) return;
-    ckp->resize(n);
-    ckm->resize(n);
-    for (int l = 0; l < n; ++l) {
-        (*ckp)[l] = kernel_entry(0, l);
-        (*ckm)[l] = kernel_entry(1, l);
     }
 }
 
@@ -444,7 +491,8 @@ cudaError_t upload_axis_tables(es_model* m, int a)
     std::vector<float2> tw, hp, hm;
     std::vector<double> ckp, ckm;
     const bool circ = circ_axis(m, a);
-    axis_tables(n, m->d[a], tw, hp, hm, m->gp[a], m->gm[a], circ ? &ckp : nullptr, circ ? &ckm : nullptr);
+    axis_tables(n, m->d[a], circ ? conv_length(n) : 0, tw, hp, hm, m->gp[a], m->gm[a], circ ? &ckp : nullptr,
+                circ ? &ckm : nullptr);
     cudaError_t e = cudaMemcpy(m->tw[a], tw.data(), tw.size() * 8, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(m->hp[a], hp.data(), hp.size() * 8, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(m->hm[a], hm.data(), hm.size() * 8, cudaMemcpyHostToDevice);
@@ -591,6 +639,7 @@ PassParams make_pass(const es_model* m, int axis, bool stress, float dt)
     p.scratch = m->prec == ES_PREC_FP32_TC ? m->ctc_scratch : nullptr;
     p.circ = circ_axis(m, axis) ? 1 : 0;
     p.comp = m->prec == ES_PREC_COMPENSATED ? 1 : 0;
+    p.m = !p.circ ? p.n : (p.comp ? 0 : conv_length(p.n));
     p.pc = m->pc[axis];
     p.ps = m->ps[axis];
     p.L = m->L;
@@ -870,17 +919,22 @@ cudaError_t derivative_pass(const float* f, int nx, int ny, int nz, int axis, do
     std::vector<float2> tw, hp, hm;
     std::vector<double> ckp64, ckm64;
     float gp[NEAR_TAPS], gm[NEAR_TAPS];
-    axis_tables(n, d, tw, hp, hm, gp, gm, circ ? &ckp64 : nullptr, circ ? &ckm64 : nullptr);
-    std::vector<float> ckp(ckp64.begin(), ckp64.end()), ckm(ckm64.begin(), ckm64.end());
-    float2* tab = nullptr;
-    cudaError_t e = dev_alloc(&tab, 3 * n * 8 + 2 * n * 4);
+    const int m = circ ? conv_length(n) : n;
+    axis_tables(n, d, circ ? m : 0, tw, hp, hm, gp, gm, circ ? &ckp64 : nullptr, circ ? &ckm64 : nullptr);
+    // one buffer: twiddles, the two multipliers, the two circulant kernels
+    const size_t len = tw.size();
+    std::vector<float> h(6 * len + (circ ? 2 * (size_t)n : 0));
+    std::memcpy(h.data(), tw.data(), len * 8);
+    std::memcpy(h.data() + 2 * len, hp.data(), len * 8);
+    std::memcpy(h.data() + 4 * len, hm.data(), len * 8);
+    for (int l = 0; circ && l < n; ++l) {
+        h[6 * len + l] = (float)ckp64[l];
+        h[6 * len + n + l] = (float)ckm64[l];
+    }
+    float* tab = nullptr;
+    cudaError_t e = dev_alloc(&tab, h.size() * 4);
     if (e != cudaSuccess) return e;
-    float* ck = reinterpret_cast<float*>(tab + 3 * n);
-    e = cudaMemcpy(tab, tw.data(), n * 8, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(tab + n, hp.data(), n * 8, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(tab + 2 * n, hm.data(), n * 8, cudaMemcpyHostToDevice);
-    if (circ && e == cudaSuccess) e = cudaMemcpy(ck, ckp.data(), n * 4, cudaMemcpyHostToDevice);
-    if (circ && e == cudaSuccess) e = cudaMemcpy(ck + n, ckm.data(), n * 4, cudaMemcpyHostToDevice);
+    e = cudaMemcpyAsync(tab, h.data(), h.size() * 4, cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) {
         PassParams p;
         std::memset(&p, 0, sizeof p);
@@ -889,14 +943,15 @@ cudaError_t derivative_pass(const float* f, int nx, int ny, int nz, int axis, do
         p.nz = nz;
         p.axis = axis;
         p.n = n;
+        p.m = m;
         p.njobs = 1;
         p.nsim = 1;
         p.dt = 1.f;
-        p.tw = tab;
-        p.hp = tab + n;
-        p.hm = tab + 2 * n;
-        p.ckp = ck;
-        p.ckm = ck + n;
+        p.tw = reinterpret_cast<const float2*>(tab);
+        p.hp = p.tw + len;
+        p.hm = p.tw + 2 * len;
+        p.ckp = tab + 6 * len;
+        p.ckm = p.ckp + n;
         p.circ = circ ? 1 : 0;
         p.ext_f = p.ext_c = (long long)nx * ny * nz;
         p.bad = bounds_word();
@@ -1028,7 +1083,9 @@ int es_model_create(const float* rho, const float* cp, const float* cs, int nx, 
     const size_t A = 256;
     auto up = [&](size_t b) { return (b + A - 1) / A * A; };
     size_t bytes = up(n * 4) * NMAT;
-    for (int a = 0; a < 3; ++a) bytes += 3 * up(axis_len(m, a) * 8) + 6 * up(axis_len(m, a) * 4);
+    // an FFT's tables have the axis length, a convolution pass's the padded length
+    auto table_len = [&](int a) { return (size_t)std::max(axis_len(m, a), conv_length(axis_len(m, a))); };
+    for (int a = 0; a < 3; ++a) bytes += 3 * up(table_len(a) * 8) + 6 * up(axis_len(m, a) * 4);
     bytes += up(16) + up(NFIELD * sizeof(float*));
     cudaError_t e = dev_alloc(&m->pool, bytes);
     if (e != cudaSuccess) {
@@ -1039,9 +1096,9 @@ int es_model_create(const float* rho, const float* cp, const float* cs, int nx, 
     auto take = [&](size_t b) { char* p = cur; cur += up(b); return p; };
     for (int k = 0; k < NMAT; ++k) m->mat[k] = (float*)take(n * 4);
     for (int a = 0; a < 3; ++a) {
-        m->tw[a] = (float2*)take(axis_len(m, a) * 8);
-        m->hp[a] = (float2*)take(axis_len(m, a) * 8);
-        m->hm[a] = (float2*)take(axis_len(m, a) * 8);
+        m->tw[a] = (float2*)take(table_len(a) * 8);
+        m->hp[a] = (float2*)take(table_len(a) * 8);
+        m->hm[a] = (float2*)take(table_len(a) * 8);
         m->ckp[a] = (float*)take(axis_len(m, a) * 4);
         m->ckm[a] = (float*)take(axis_len(m, a) * 4);
         m->ckp_lo[a] = (float*)take(axis_len(m, a) * 4);

@@ -85,7 +85,8 @@ struct PassParams {
     int n;                // length along the axis
     int njobs;
     PassJob job[3];
-    const float2* tw;     // tw[m] = exp(-2 pi i m / n)
+    int m;                // length of the FFT: n, or a convolution pass's padded length (circ = 1; 0: none)
+    const float2* tw;     // tw[k] = exp(-2 pi i k / m)
     const float2* hp;     // (H - H_near) / n for D(+), H = i kappa exp(+i kappa d/2)
     const float2* hm;     // the same for D(-), H = i kappa exp(-i kappa d/2)
     const float* ckp;     // circulant kernel of D(+) along the axis (lengths without an FFT plan)
@@ -160,9 +161,21 @@ cudaError_t launch_strided2(int ra, int rb, int rc, int ntiles, const PassParams
 cudaError_t launch_strided1(int ra, int rb, int rc, int ntiles, const PassParams& p, cudaStream_t st);
 cudaError_t prepare_strided2();
 cudaError_t prepare_strided1();
+// Axis lengths without a plan, FP32 mode: zero-padded convolution passes (conv_pass.cuh) with
+// transforms of conv_length(n) points (0: none, the circulant pass), from CONV_MIN_N cells on:
+// below, the near stencil's window would wrap round the axis more than once, and 17 cells
+// already take the same time either way (2.5 against 2.5-2.7 ms per 17 M cells along z).
+constexpr int CONV_MIN_N = 16;
+int conv_length(int n);
+cudaError_t launch_conv(const PassParams& p, cudaStream_t st);
+cudaError_t launch_conv_strided1(const PassParams& p, cudaStream_t st);  // nx odd
+cudaError_t launch_conv_strided2(const PassParams& p, cudaStream_t st);  // nx even
+cudaError_t prepare_conv_kernels();
+cudaError_t prepare_conv_strided1();
+cudaError_t prepare_conv_strided2();
 // Longest axis the circulant pass takes (shared tiles of 2 x 32 x pad(n) floats).
 constexpr int CIRC_MAX_N = 512;
-// From this length on, the CUDA-core circulant passes along y and z run their epilogue from
+// From this length on, the compensated circulant passes along y and z run their epilogue from
 // the registers.
 constexpr int CIRC_DIRECT_N = 192;
 // From this length on, circulant passes in FP32 mode run on the tensor cores (circ_tc.cu):

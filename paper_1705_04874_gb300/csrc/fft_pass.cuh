@@ -410,7 +410,7 @@ __device__ __forceinline__ int butterfly(int b)
     return B % T == 0 ? b : min(b, B - 1);
 }
 
-template <int RA, int RB, int T_>
+template <int RA, int RB, int T_, int PR = PAIRS>
 struct Core {
     static constexpr int N = RA * RB;
     static constexpr int R1 = RA;
@@ -439,7 +439,7 @@ struct Core {
         for (int m = 0; m < MA; ++m) {
             const int b = butterfly<BA, T>(j + m * T);
 #pragma unroll
-            for (int q = 0; q < RA; ++q) buf[(b * RA + q) * PAIRS + c] = a[m][q];
+            for (int q = 0; q < RA; ++q) buf[(b * RA + q) * PR + c] = a[m][q];
         }
     }
 
@@ -454,7 +454,7 @@ struct Core {
             const int k = b % RA;
 #pragma unroll
             for (int r = 0; r < RB; ++r) {
-                const float2 x = buf[(b + r * BB) * PAIRS + c];
+                const float2 x = buf[(b + r * BB) * PR + c];
                 v[m][r] = r == 0 ? x : cmul(x, tw[k * r]);
             }
             Dft<RB>::run(v[m]);
@@ -470,7 +470,7 @@ struct Core {
         for (int m = 0; m < MB; ++m) {
             const int b = butterfly<BB, T>(j + m * T);
 #pragma unroll
-            for (int q = 0; q < RB; ++q) buf[(b * RB + q) * PAIRS + c] = v[m][q];
+            for (int q = 0; q < RB; ++q) buf[(b * RB + q) * PR + c] = v[m][q];
         }
     }
 
@@ -485,7 +485,7 @@ struct Core {
             const int k = b % RB;
 #pragma unroll
             for (int r = 0; r < RA; ++r) {
-                const float2 x = buf[(b + r * BA) * PAIRS + c];
+                const float2 x = buf[(b + r * BA) * PR + c];
                 a[m][r] = r == 0 ? x : cmul(x, tw[k * r]);
             }
             Dft<RA>::run(a[m]);
@@ -513,7 +513,7 @@ struct Core {
 // elements b + r n/R times W_(Ns R)^(k r), runs the R-point DFT and writes
 // element (b / Ns) Ns R + k + q Ns.  All stages but the first and the last
 // run on the shared buffer, every butterfly of a stage by one thread.
-template <int R1_, int R2, int R3, int T_>
+template <int R1_, int R2, int R3, int T_, int PR = PAIRS>
 struct Core3 {
     static constexpr int R1 = R1_;
     static constexpr int N = R1 * R2 * R3;
@@ -536,7 +536,7 @@ struct Core3 {
 #pragma unroll
         for (int m = 0; m < MA; ++m)
 #pragma unroll
-            for (int q = 0; q < R1; ++q) buf[((j + m * T) * R1 + q) * PAIRS + c] = a[m][q];
+            for (int q = 0; q < R1; ++q) buf[((j + m * T) * R1 + q) * PR + c] = a[m][q];
     }
 
     // one stage of radix R after radices multiplying to NS, shared buffer to
@@ -552,7 +552,7 @@ struct Core3 {
             const int k = b % NS;
 #pragma unroll
             for (int r = 0; r < R; ++r) {
-                const float2 x = buf[(b + r * B) * PAIRS + c];
+                const float2 x = buf[(b + r * B) * PR + c];
                 v[m][r] = r == 0 ? x : cmul(x, tw[k * r * TS]);
             }
             Dft<R>::run(v[m]);
@@ -563,7 +563,7 @@ struct Core3 {
             const int b = butterfly<B, T>(j + m * T);
             const int k = b % NS, o = (b / NS) * NS * R + k;
 #pragma unroll
-            for (int q = 0; q < R; ++q) buf[(o + q * NS) * PAIRS + c] = v[m][q];
+            for (int q = 0; q < R; ++q) buf[(o + q * NS) * PR + c] = v[m][q];
         }
     }
 
@@ -581,7 +581,7 @@ struct Core3 {
                 const int b = butterfly<B, T>(j + m * T);
 #pragma unroll
                 for (int r = 0; r < R3; ++r) {
-                    const float2 x = buf[(b + r * B) * PAIRS + c];
+                    const float2 x = buf[(b + r * B) * PR + c];
                     v[m][r] = r == 0 ? x : cmul(x, tw[b * r]);
                 }
                 Dft<R3>::run(v[m]);
@@ -597,7 +597,7 @@ struct Core3 {
             for (int m = 0; m < M; ++m) {
                 const int b = butterfly<B, T>(j + m * T);
 #pragma unroll
-                for (int q = 0; q < R3; ++q) buf[(b * R3 + q) * PAIRS + c] = v[m][q];
+                for (int q = 0; q < R3; ++q) buf[(b * R3 + q) * PR + c] = v[m][q];
             }
         }
         __syncthreads();
@@ -614,7 +614,7 @@ struct Core3 {
             const int b = j + m * T;
 #pragma unroll
             for (int r = 0; r < R1; ++r) {
-                const float2 x = buf[(b + r * BA) * PAIRS + c];
+                const float2 x = buf[(b + r * BA) * PR + c];
                 a[m][r] = r == 0 ? x : cmul(x, tw[b * r]);
             }
             Dft<R1>::run(a[m]);
@@ -631,8 +631,8 @@ struct Core3 {
 };
 
 // the FFT core of a plan (RC = 1: two stages)
-template <int RA, int RB, int RC, int T>
-using CoreOf = std::conditional_t<RC == 1, Core<RA, RB, T>, Core3<RA, RB, RC, T>>;
+template <int RA, int RB, int RC, int T, int PR = PAIRS>
+using CoreOf = std::conditional_t<RC == 1, Core<RA, RB, T, PR>, Core3<RA, RB, RC, T, PR>>;
 
 // asynchronous BYTES-byte global -> shared copy (cp.async); ok == false writes
 // zeros and reads nothing
@@ -938,6 +938,7 @@ struct StridedTile {
     size_t base;     // linear index of its first cell
     size_t off, soff;
 };
+template <int PR = PAIRS>
 __device__ __forceinline__ StridedTile strided_tile(const PassParams& p, int w, int ntiles)
 {
     StridedTile t;
@@ -954,9 +955,9 @@ __device__ __forceinline__ StridedTile strided_tile(const PassParams& p, int w, 
         sim = w % p.nsim;
         w /= p.nsim;
     }
-    const int ntx = (p.nx + 2 * PAIRS - 1) / (2 * PAIRS);
+    const int ntx = (p.nx + 2 * PR - 1) / (2 * PR);
     t.outer = w / ntx;
-    t.x0 = (w - t.outer * ntx) * 2 * PAIRS;
+    t.x0 = (w - t.outer * ntx) * 2 * PR;
     t.base = (size_t)t.x0 + (size_t)p.nx * (p.axis == 1 ? (size_t)p.ny * t.outer : (size_t)t.outer);
     t.off = (size_t)sim * p.fstride;
     t.soff = (size_t)sim * p.sstride;
@@ -965,24 +966,25 @@ __device__ __forceinline__ StridedTile strided_tile(const PassParams& p, int w, 
 
 // the tile's source into shared rows, W floats per asynchronous copy, zeros
 // past the last column
-template <int N, int NT, int W>
-__device__ __forceinline__ void stage_strided(const PassParams& p, const StridedTile& t, float2* buf, unsigned est)
+template <int NT, int W, int PR = PAIRS>
+__device__ __forceinline__ void stage_strided(const PassParams& p, const StridedTile& t, float2* buf, unsigned est,
+                                              int n)
 {
-    constexpr int CH = W == 1 ? PAIRS : 2 * PAIRS / W;  // threads per row
+    constexpr int CH = W == 1 ? PR : 2 * PR / W;  // threads per row
     static_assert(NT % CH == 0, "a thread keeps its columns");
     const float* src = p.job[t.job].src + t.off + t.base;
     const int e0 = threadIdx.x / CH, k = threadIdx.x % CH;
-    // floats of a row this thread copies: W from x0 + W k on; W = 1: x0 + k and x0 + PAIRS + k, the
+    // floats of a row this thread copies: W from x0 + W k on; W = 1: x0 + k and x0 + PR + k, the
     // two pencils of pair k
     const int x = W * k;
     unsigned o = (unsigned)e0 * est + x;
-    float* d = reinterpret_cast<float*>(buf + e0 * PAIRS) + (W == 1 ? 2 * k : x);
+    float* d = reinterpret_cast<float*>(buf + e0 * PR) + (W == 1 ? 2 * k : x);
 #pragma unroll 4
-    for (int e = e0; e < N; e += NT / CH, o += NT / CH * est, d += NT / CH * 2 * PAIRS) {
+    for (int e = e0; e < n; e += NT / CH, o += NT / CH * est, d += NT / CH * 2 * PR) {
 #pragma unroll
         for (int f = 0; f < (W == 1 ? 2 : 1); ++f) {
-            const bool ok = t.x0 + x + f * PAIRS < p.nx && ES_INB(p, t.off + t.base + o + f * PAIRS + W - 1, p.ext_f);
-            cp_async<4 * W>(d + f, ok ? src + o + f * PAIRS : src, ok);
+            const bool ok = t.x0 + x + f * PR < p.nx && ES_INB(p, t.off + t.base + o + f * PR + W - 1, p.ext_f);
+            cp_async<4 * W>(d + f, ok ? src + o + f * PR : src, ok);
         }
     }
 }
@@ -991,13 +993,14 @@ __device__ __forceinline__ void stage_strided(const PassParams& p, const Strided
 // positions of its pair, EB at a time with the next batch's coefficients in
 // flight; the far parts come from the shared rows, the near parts from tensor
 // memory (TM) or their shared rows.  Addresses are a tile's base plus a 32-bit
-// offset.
+// offset.  FULL: the threads' positions are exactly the axis (else they may pass
+// its end).
 //
 // The PML slab rows (the first L and the last L + 1 positions) would all fall to
 // the first and the last warps, which would keep the others waiting while they
 // fetch the old splits: there the derivative goes back into the shared row, and
 // afterwards the CTA takes the slab's (row, pair) items evenly (run_slab).
-template <int RN, int V, bool TM>
+template <int RN, int V, bool TM, bool FULL = true, int PR = PAIRS>
 struct StridedEpilogue {
     static constexpr int EB = epi_batch<RN>();
     const PassParams& p;
@@ -1015,29 +1018,31 @@ struct StridedEpilogue {
 
     __device__ __forceinline__ StridedEpilogue(const PassParams& p_, const PassJob& J_, const StridedTile& t_,
                                                unsigned est_, float2* buf, const float2* nearp, uint32_t tm_)
-        : p(p_), J(J_), t(t_), est(est_), rows(buf), near(nearp), tm(tm_), c((int)threadIdx.x % PAIRS),
-          pos0(RN * ((int)threadIdx.x / PAIRS)), valid(t_.x0 + V * c < p_.nx), two(V == 2 || t_.x0 + PAIRS + c < p_.nx)
+        : p(p_), J(J_), t(t_), est(est_), rows(buf), near(nearp), tm(tm_), c((int)threadIdx.x % PR),
+          pos0(RN * ((int)threadIdx.x / PR)), valid(t_.x0 + V * c < p_.nx), two(V == 2 || t_.x0 + PR + c < p_.nx)
     {
         co0 = J.coef[0] + t.base;
         co1 = J.coef[1] + t.base;
         o = (unsigned)pos0 * est + V * c;
     }
-    __device__ __forceinline__ void coefs(unsigned oc, bool normal)
+    // whether this thread updates its k-th position
+    __device__ __forceinline__ bool in(int k) const { return valid && (FULL || pos0 + k < p.n); }
+    __device__ __forceinline__ void coefs(int oc0, unsigned oc, bool normal)
     {
 #pragma unroll
         for (int e = 0; e < EB; ++e) {
             const unsigned oe = oc + e * est;
-            if (!valid || !ES_INB(p, t.base + oe + last(), p.ext_c)) continue;
-            c0[e] = ldg_pair<V, PAIRS>(co0 + oe, two);
-            if (normal) c1[e] = ldg_pair<V, PAIRS>(co1 + oe, two);
+            if (!in(oc0 + e) || !ES_INB(p, t.base + oe + last(), p.ext_c)) continue;
+            c0[e] = ldg_pair<V, PR>(co0 + oe, two);
+            if (normal) c1[e] = ldg_pair<V, PR>(co1 + oe, two);
         }
     }
     __device__ __forceinline__ void first_coefs()
     {
-        if (J.kind != JOB_STORE) coefs(o, J.kind == JOB_NORMAL);
+        if (J.kind != JOB_STORE) coefs(0, o, J.kind == JOB_NORMAL);
     }
     // offset of the pair's last cell (index checks)
-    __device__ __forceinline__ int last() const { return V == 2 ? 1 : (two ? PAIRS : 0); }
+    __device__ __forceinline__ int last() const { return V == 2 ? 1 : (two ? PR : 0); }
     // SLAB: slab rows may be among this warp's positions
     template <int KIND, bool SLAB>
     __device__ __forceinline__ void run()
@@ -1057,24 +1062,26 @@ struct StridedEpilogue {
                 d0[e] = c0[e];
                 d1[e] = c1[e];
             }
-            if (KIND != JOB_STORE && k0 + EB < RN) coefs(o + EB * est, KIND == JOB_NORMAL);
+            if (KIND != JOB_STORE && k0 + EB < RN) coefs(k0 + EB, o + EB * est, KIND == JOB_NORMAL);
 #pragma unroll
             for (int e = 0; e < EB; ++e, o += est) {
                 const int pos = pos0 + k0 + e;
-                float2* const row = rows + pos * PAIRS + c;
+                float2* const row = rows + pos * PR + c;
                 const float2 f = *row;
-                const float2 n = TM ? make_float2(s[2 * e], s[2 * e + 1]) : near[pos * PAIRS + c];
+                // (past the axis's end the near parts have no row)
+                const float2 n = TM ? make_float2(s[2 * e], s[2 * e + 1])
+                                    : (FULL || pos < p.n ? near[pos * PR + c] : make_float2(0.f, 0.f));
                 const float2 d = make_float2(__fadd_rn(f.x, n.x), __fsub_rn(n.y, f.y));  // far (conj) + near
-                const bool ok = valid && ES_INB(p, t.off + t.base + o + last(), p.ext_f);
+                const bool ok = in(k0 + e) && ES_INB(p, t.off + t.base + o + last(), p.ext_f);
                 if (KIND == JOB_STORE) {
-                    if (ok) st_pair<V, PAIRS>(tgt[0] + o, d, two);
+                    if (ok) st_pair<V, PR>(tgt[0] + o, d, two);
                     continue;
                 }
 #if ES_BOUNDS
                 if (!ok || !ES_INB(p, t.base + o + last(), p.ext_c)) continue;
 #endif
                 if (SLAB && in_slab(pos, p.n, p.L)) {
-                    *row = d;
+                    if (FULL || pos < p.n) *row = d;
                     continue;
                 }
 #pragma unroll
@@ -1083,7 +1090,7 @@ struct StridedEpilogue {
                     const float cx = KIND == JOB_NORMAL ? normal_coef(d0[e].x, d1[e].x, diag) : d0[e].x;
                     const float cy = KIND == JOB_NORMAL ? normal_coef(d0[e].y, d1[e].y, diag) : d0[e].y;
                     const float2 inc = make_float2(increment(dt, cx, d.x), increment(dt, cy, d.y));
-                    if (ok) red_pair<V, PAIRS>(tgt[k] + o, inc, two);
+                    if (ok) red_pair<V, PR>(tgt[k] + o, inc, two);
                 }
             }
         }
@@ -1099,19 +1106,19 @@ struct StridedEpilogue {
         const size_t s0 = t.soff + t.x0 + (p.axis == 1 ? (size_t)p.nx * S * t.outer : (size_t)p.nx * t.outer);
         if (!valid) return;
 #pragma unroll 1
-        for (int sp = threadIdx.x / PAIRS; sp < S; sp += NTHR / PAIRS) {
+        for (int sp = threadIdx.x / PR; sp < S; sp += NTHR / PR) {
             const int pos = sp < p.L ? sp : sp - p.L + p.n - 1 - p.L;
             const unsigned q = (unsigned)pos * est + V * c, so = (unsigned)sp * est + V * c;
             if (!ES_INB(p, t.off + t.base + q + last(), p.ext_f) ||
                 !ES_INB(p, t.base + q + last(), p.ext_c) || !ES_INB(p, s0 + so + last(), p.ext_s))
                 continue;
-            const float2 d = rows[pos * PAIRS + c];
-            const float2 k0 = ldg_pair<V, PAIRS>(co0 + q, two);
-            const float2 k1 = KIND == JOB_NORMAL ? ldg_pair<V, PAIRS>(co1 + q, two) : k0;
+            const float2 d = rows[pos * PR + c];
+            const float2 k0 = ldg_pair<V, PR>(co0 + q, two);
+            const float2 k1 = KIND == JOB_NORMAL ? ldg_pair<V, PR>(co1 + q, two) : k0;
             const float P = __ldg(prof + pos);
             float2 sv[NT];
 #pragma unroll
-            for (int k = 0; k < NT; ++k) sv[k] = ld_pair<V, PAIRS>(J.slab[k] + s0 + so, two);
+            for (int k = 0; k < NT; ++k) sv[k] = ld_pair<V, PR>(J.slab[k] + s0 + so, two);
 #pragma unroll
             for (int k = 0; k < NT; ++k) {
                 const bool diag = k == J.diag;
@@ -1121,9 +1128,9 @@ struct StridedEpilogue {
                 // split-field update s <- P (P s + inc); the total takes the split's change
                 const float2 sn = make_float2(__fmul_rn(P, __fmaf_rn(P, sv[k].x, inc.x)),
                                               __fmul_rn(P, __fmaf_rn(P, sv[k].y, inc.y)));
-                st_pair<V, PAIRS>(J.slab[k] + s0 + so, sn, two);
+                st_pair<V, PR>(J.slab[k] + s0 + so, sn, two);
                 inc = make_float2(__fsub_rn(sn.x, sv[k].x), __fsub_rn(sn.y, sv[k].y));
-                red_pair<V, PAIRS>(J.tgt[k] + t.off + t.base + q, inc, two);
+                red_pair<V, PR>(J.tgt[k] + t.off + t.base + q, inc, two);
             }
         }
     }
@@ -1163,9 +1170,9 @@ pass_strided(const __grid_constant__ PassParams p, int ntiles)
     const unsigned est = p.axis == 1 ? (unsigned)p.nx : (unsigned)p.nx * p.ny;
     const int total = ntiles * p.njobs;
     auto stage = [&](const StridedTile& t, float2* buf) {
-        if (V == 1) stage_strided<N, NT, 1>(p, t, buf, est);
-        else if (p.nx % 4 == 0) stage_strided<N, NT, 4>(p, t, buf, est);
-        else stage_strided<N, NT, 2>(p, t, buf, est);
+        if (V == 1) stage_strided<NT, 1>(p, t, buf, est, N);
+        else if (p.nx % 4 == 0) stage_strided<NT, 4>(p, t, buf, est, N);
+        else stage_strided<NT, 2>(p, t, buf, est, N);
     };
     stage(strided_tile(p, blockIdx.x, ntiles), smem);
     for (int i = tid; i < N; i += NT) {
@@ -1294,59 +1301,68 @@ __device__ __forceinline__ void x_item(int it, int* r, int* xx)
     *xx = 4 * (it / (CL * 2 * PAIRS) * CL + lo);
 }
 
-// Epilogue for 4 consecutive cells of an x-pass tile in memory order (f0 =
-// the first one's offset from the tile start, q0 its linear index, 16-byte
-// aligned): a chunk may span two lines, so every cell takes its own x and
-// line for the PML split (slab row S line); the arithmetic of epilogue_one.
-template <int N>
-__device__ __forceinline__ void epilogue_quad_flat(const PassParams& p, const PassJob& J, size_t q0, int f0,
-                                                   int line0, float4 d4, size_t off, size_t soff)
+// Update of nq chunks of 4 consecutive cells of an x-pass tile in memory order
+// (16-byte aligned from linear index q0 on), the next chunk's coefficients in
+// flight.  A chunk may span two lines, so every cell takes its own x and line for
+// the PML split.
+template <int NT, int KIND, class LineOf>
+__device__ __forceinline__ void x_quads_flat(const PassParams& p, const PassJob& J, const float* bf, size_t q0, int line0,
+                                             int nq, int n, size_t off, size_t soff, LineOf line_of)
 {
-    if (!ES_INB(p, off + q0 + 3, p.ext_f)) return;
-    if (J.kind == JOB_STORE) {
-        *reinterpret_cast<float4*>(J.tgt[0] + off + q0) = d4;
-        return;
-    }
-    if (!ES_INB(p, q0 + 3, p.ext_c)) return;
-    const float d[4] = {d4.x, d4.y, d4.z, d4.w};
-    const float dt = p.dt;
-    const int S = p.S;
-    int xs[4];
-    size_t srow[4];
+    constexpr int TG = KIND == JOB_NORMAL ? 3 : 1;
+    const float *co0 = J.coef[0] + q0, *co1 = J.coef[1] + q0;
+    const float* prof = J.stag ? p.ps : p.pc;
+    float* tgt[TG];
 #pragma unroll
-    for (int e = 0; e < 4; ++e) {
-        const int r = (f0 + e) / N;
-        xs[e] = f0 + e - r * N;
-        srow[e] = soff + (size_t)S * (size_t)(line0 + r);
-        if (p.L > 0 && !ES_INB(p, srow[e] + S - 1, p.ext_s)) return;
-    }
-    if (J.kind == JOB_SINGLE) {
-        const float4 c4 = __ldg(reinterpret_cast<const float4*>(J.coef[0] + q0));
-        const float cv[4] = {c4.x, c4.y, c4.z, c4.w};
-        float iv[4];
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            iv[e] = increment(dt, cv[e], d[e]);
-            if (in_slab(xs[e], p.n, p.L))
-                iv[e] = split_delta(J.slab[0], srow[e] + slab_pos(xs[e], p.n, p.L, p.S),
-                                    __ldg((J.stag ? p.ps : p.pc) + xs[e]), iv[e]);
+    for (int k = 0; k < TG; ++k) tgt[k] = J.tgt[k] + off + q0;
+    float4 c0 = make_float4(0.f, 0.f, 0.f, 0.f), c1 = c0;
+    auto coefs = [&](int i) {
+        if (KIND == JOB_STORE || i >= nq || !ES_INB(p, q0 + 4 * i + 3, p.ext_c)) return;
+        c0 = __ldg(reinterpret_cast<const float4*>(co0) + i);
+        if (KIND == JOB_NORMAL) c1 = __ldg(reinterpret_cast<const float4*>(co1) + i);
+    };
+    coefs(threadIdx.x);
+#pragma unroll 1
+    for (int i = threadIdx.x; i < nq; i += NT) {
+        const float4 d4 = reinterpret_cast<const float4*>(bf)[i], a4 = c0, b4 = c1;
+        coefs(i + NT);
+        if (!ES_INB(p, off + q0 + 4 * i + 3, p.ext_f)) continue;
+        if (KIND == JOB_STORE) {
+            reinterpret_cast<float4*>(tgt[0])[i] = d4;
+            continue;
         }
-        atomicAdd(reinterpret_cast<float4*>(J.tgt[0] + off + q0), make_float4(iv[0], iv[1], iv[2], iv[3]));
-    } else {
-        const float4 l4 = __ldg(reinterpret_cast<const float4*>(J.coef[0] + q0));
-        const float4 m4 = __ldg(reinterpret_cast<const float4*>(J.coef[1] + q0));
-        const float lv[4] = {l4.x, l4.y, l4.z, l4.w};
-        const float mv[4] = {m4.x, m4.y, m4.z, m4.w};
-#pragma unroll
-        for (int t = 0; t < 3; ++t) {
-            float iv[4];
+        const float d[4] = {d4.x, d4.y, d4.z, d4.w}, a[4] = {a4.x, a4.y, a4.z, a4.w}, b[4] = {b4.x, b4.y, b4.z, b4.w};
+        // the cells' split parts, all on their way before the first is used
+        size_t si[4];
+        float P[4], old[TG][4];
+        unsigned slab = 0;
+        if (p.L > 0) {
+            const int f = 4 * i, r = line_of(f), x = f - r * n;
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
-                iv[e] = increment(dt, normal_coef(lv[e], mv[e], t == J.diag), d[e]);
-                if (in_slab(xs[e], p.n, p.L))
-                    iv[e] = split_delta(J.slab[t], srow[e] + slab_pos(xs[e], p.n, p.L, p.S), __ldg(p.pc + xs[e]), iv[e]);
+                const int xe = x + e < n ? x + e : x + e - n, re = x + e < n ? r : r + 1;
+                if (!in_slab(xe, n, p.L)) continue;
+                si[e] = soff + (size_t)p.S * (line0 + re) + slab_pos(xe, n, p.L, p.S);
+                if (!ES_INB(p, si[e], p.ext_s)) continue;
+                slab |= 1u << e;
+                P[e] = __ldg(prof + xe);
+#pragma unroll
+                for (int k = 0; k < TG; ++k) old[k][e] = J.slab[k][si[e]];
             }
-            atomicAdd(reinterpret_cast<float4*>(J.tgt[t] + off + q0), make_float4(iv[0], iv[1], iv[2], iv[3]));
+        }
+#pragma unroll
+        for (int k = 0; k < TG; ++k) {
+            float v[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                v[e] = increment(p.dt, KIND == JOB_NORMAL ? normal_coef(a[e], b[e], k == J.diag) : a[e], d[e]);
+                if (slab >> e & 1) {
+                    const float sn = __fmul_rn(P[e], __fmaf_rn(P[e], old[k][e], v[e]));  // s <- P (P s + inc)
+                    J.slab[k][si[e]] = sn;
+                    v[e] = __fsub_rn(sn, old[k][e]);
+                }
+            }
+            atomicAdd(reinterpret_cast<float4*>(tgt[k]) + i, make_float4(v[0], v[1], v[2], v[3]));
         }
     }
 }
@@ -1642,10 +1658,8 @@ pass_x_any(const __grid_constant__ PassParams p)
         if (CELLS % NT != 0 && it >= CELLS) break;
         const int r = 4 * ((it >> 5) & 7) + ((it >> 3) & 3), xx = 8 * (it >> 8) + (it & 7);
         if (xx >= N) continue;
-        float v = 0.f;
-        if (r < nl && ES_INB(p, off + (size_t)(line0 + r) * N + xx, p.ext_f))
-            v = __ldg(src + (size_t)(line0 + r) * N + xx);
-        bf[x_at<N>(xx, r)] = v;
+        const bool ok = r < nl && ES_INB(p, off + (size_t)(line0 + r) * N + xx, p.ext_f);
+        cp_async<4>(bf + x_at<N>(xx, r), ok ? src + (size_t)(line0 + r) * N + xx : src, ok);
     }
     // the tile's coefficient lines (contiguous, N lines of 128 bytes) into L2
     if (J.coef[0]) {
@@ -1658,6 +1672,7 @@ pass_x_any(const __grid_constant__ PassParams p)
         }
     }
     load_tables<N>(p, J, s_tw, s_h, tid, NT);
+    cp_async_commit_wait_all();
     __syncthreads();
     auto at = [&](int e) { return e * PAIRS + (c ^ x_swz<N>(e)); };
     near_part<N, RN>(
@@ -1691,8 +1706,10 @@ pass_x_any(const __grid_constant__ PassParams p)
     if (J.kind == JOB_NORMAL) vec = vec && a16(J.tgt[1] + off) && a16(J.tgt[2] + off) && a16(J.coef[1]);
     if (J.kind != JOB_STORE) vec = vec && a16(J.coef[0]);
     const int nq = vec ? nf / 4 : 0;
-    for (int i = tid; i < nq; i += NT)
-        epilogue_quad_flat<N>(p, J, q0 + 4 * (size_t)i, 4 * i, line0, reinterpret_cast<const float4*>(bf)[i], off, soff);
+    auto line_of = [](int f) { return f / N; };
+    if (J.kind == JOB_STORE) x_quads_flat<NT, JOB_STORE>(p, J, bf, q0, line0, nq, N, off, soff, line_of);
+    else if (J.kind == JOB_SINGLE) x_quads_flat<NT, JOB_SINGLE>(p, J, bf, q0, line0, nq, N, off, soff, line_of);
+    else x_quads_flat<NT, JOB_NORMAL>(p, J, bf, q0, line0, nq, N, off, soff, line_of);
     // what is left: a last, partial tile's cells past its last full chunk
     for (int f = 4 * nq + tid; f < nf; f += NT) {
         const int r = f / N, x = f - r * N, line = line0 + r;

@@ -108,12 +108,13 @@ cudaError_t prepare_pass_kernels()
 #undef ES_PREP
     if ((e = prepare_strided2()) != cudaSuccess) return e;
     if ((e = prepare_strided1()) != cudaSuccess) return e;
+    if ((e = prepare_conv_kernels()) != cudaSuccess) return e;
     return prepare_circ_kernels();
 }
 
 cudaError_t launch_pass(const PassParams& p, cudaStream_t st)
 {
-    if (p.circ) return launch_circ(p, st);
+    if (p.circ) return p.m > 0 && !circ_tc_eligible(p) ? launch_conv(p, st) : launch_circ(p, st);
     std::call_once(g_init, init_choice);
     const int kind = p.axis == 0 ? 0 : 1;
     if (p.n < 1 || p.n > 256 || g_choice[kind][p.n] < 0) return cudaErrorInvalidValue;

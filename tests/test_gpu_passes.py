@@ -51,3 +51,43 @@ def test_slab_widths_that_are_not_whole_quads(es, orc, nx, pml):
     assert trace_errors(gpu, ref["traces"]).max() < 1e-4
     for f in range(9):
         assert rel_l2(st[f], ref["state"][f]) < 1e-4, f
+
+
+# every transform length of the convolution passes at both ends of its range (2 n <= length), the
+# shortest axis they take and the one below, an axis past what one tile of CTAs holds
+@pytest.mark.parametrize("n", [15, 16, 31, 33, 50, 51, 79, 81, 127, 129, 158, 161, 200, 201, 250, 251, 301, 312, 313, 512])
+@pytest.mark.parametrize("axis,others", [(0, (7, 9)), (1, (5, 36)), (2, (6, 35))])
+def test_convolution_lengths(es, orc, n, axis, others):
+    """A derivative rounds its input, its taps and about 4 log2 (padded length)
+    butterflies at 2 % weight: a few 1e-7; water-to-rock-like steps in the data."""
+    import torch
+    shape = {0: (others[0], others[1], n), 1: (others[0], n, others[1]), 2: (n, others[0], others[1])}[axis]
+    rng = np.random.default_rng(n + axis)
+    f = rng.standard_normal(shape).astype(np.float32)
+    f[shape[0] // 2:] *= 50.0
+    out = torch.empty(shape, device="cuda")
+    for shift in (1, -1):
+        es.es_derivative(torch.from_numpy(f).cuda(), axis, 10.0, shift, out)
+        ref = orc.deriv(f.astype(np.float64), axis, 10.0, shift)
+        assert rel_l2(out.cpu().numpy(), ref) < 5e-7
+
+
+def test_run_on_convolution_axes(es, orc):
+    """A batch on three axes without a plan (33 x 30 x 27: odd nx) and PML, the
+    first simulation against the oracle, the second against a run of its own."""
+    shape, pml, nt = (27, 30, 33), 4, 100
+    rho, cp, cs = synth.two_layer_model(shape=shape, water_cells=6)
+    dt = cfl_dt(cp, 10.0)
+    w = synth.ricker(nt, dt, 25.0)
+    pos = np.array([[16, 15, 14], [14, 13, 15]], np.int32)
+    mts = np.stack([synth.explosive(), synth.clvd()])
+    rcv = orc.seabed_receivers(cs, pml, 3, 3)
+    with es.Model(rho, cp, cs, dx=10.0, pml=pml) as m:
+        m.batch_set(pos, mts, np.stack([w, w]))
+        got = m.run(nt, dt, rcv)
+    ref = orc.simulate(rho, cp, cs, dx=10.0, dt=dt, nt=nt, pml=pml,
+                       sources=[dict(kind="moment", pos=tuple(pos[0]), m=mts[0], w=w)], receivers=rcv)["traces"]
+    assert trace_errors(got[0], ref).max() < 1e-4
+    with es.Model(rho, cp, cs, dx=10.0, pml=pml) as m:
+        m.source_set(pos[1], mts[1], w)
+        assert np.array_equal(m.run(nt, dt, rcv), got[1])
