@@ -210,40 +210,91 @@ cudaError_t launch_transpose_traces(const float* rec, int nt, int cols, float* o
     return cudaGetLastError();
 }
 
-// gather[row][t] = sum_e amp_e traces[src_e][row][t - k_e], rows = 4 n_rcv.
-// One thread per output sample; events in order (FP32 accumulation).  The
-// events reach shared memory in chunks of SUP_CHUNK, so any number of events
-// fits in a fixed 48 KB block without changing the order of the sum.
-constexpr int SUP_CHUNK = 4096;
+// gather[row][t] = sum_e amp_e traces[src_e][row][t - k_e], rows = 4 n_rcv, in
+// FP32 with the events in order (one multiply-add per event and sample).
+//
+// A warp owns 32 R consecutive output samples of one row, R per thread (lane +
+// 32 i), and walks the events once: per event one uniform test of how its trace
+// overlaps the span (not at all, wholly, partly), then R coalesced loads and R
+// multiply-adds, so the event's bookkeeping is paid once per 32 R samples.  What
+// bounds it is the L2 -> SM traffic: an event's trace is read at its own shift,
+// 4 bytes per event and sample (a trace itself comes from DRAM about once: the
+// rows in flight fit in L2).  Events reach shared memory in chunks of SUP_CHUNK,
+// so any number of them fits without changing the order of the sum.
+// 64 sources x 1024 receivers x 2000 samples, 300 events into 4666 samples (one
+// GB300): 0.99 ms (1.46 ms with the call around it); one sample per thread with
+// a test, an address and three shared loads per event and sample took 4.69 ms
+// with the call.
+constexpr int SUP_CHUNK = 1024, SUP_WARPS = 8;
 
-__global__ void superpose_kernel(const float* traces, int n_rcv, int nt, const int* ev_src,
-                                 const float* ev_amp, const int* ev_shift, int n_events, int n_out,
-                                 float* gather)
+template <int R>
+__global__ void __launch_bounds__(32 * SUP_WARPS) superpose_kernel(const float* traces, long long rows, int nt,
+                                                                   const int* ev_src, const float* ev_amp,
+                                                                   const int* ev_shift, int n_events, int n_out,
+                                                                   int spans, float* gather)
 {
-    __shared__ int s_src[SUP_CHUNK], s_k[SUP_CHUNK];
-    __shared__ float s_a[SUP_CHUNK];
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    const size_t row = blockIdx.y;
-    const bool active = t < n_out;
-    const size_t rows = 4 * (size_t)n_rcv;
-    float acc = 0.f;
+    struct Event {
+        long long ofs;  // of the event's trace in row 0, at sample -k
+        int k;
+        float amp;
+    };
+    __shared__ __align__(16) Event ev[SUP_CHUNK];
+    const long long unit = (long long)blockIdx.x * SUP_WARPS + threadIdx.x / 32;  // row-major: consecutive warps share a row
+    const long long row = unit / spans;
+    const bool active = row < rows;
+    const int t0 = (int)(unit - row * spans) * 32 * R, lane = threadIdx.x % 32;
+    const float* base = traces + row * nt + t0 + lane;
+    float acc[R];
+#pragma unroll
+    for (int i = 0; i < R; ++i) acc[i] = 0.f;
     for (int e0 = 0; e0 < n_events; e0 += SUP_CHUNK) {
         const int ne = min(SUP_CHUNK, n_events - e0);
         __syncthreads();  // the previous chunk is no longer read
-        for (int i = threadIdx.x; i < ne; i += blockDim.x) {
-            s_src[i] = ev_src[e0 + i];
-            s_k[i] = ev_shift[e0 + i];
-            s_a[i] = ev_amp[e0 + i];
+        for (int i = threadIdx.x; i < ne; i += 32 * SUP_WARPS) {
+            // a shift past either end of the window: no overlap with any span
+            int k = ev_shift[e0 + i];
+            if (k <= -nt || k > n_out) k = n_out;
+            ev[i].ofs = (long long)ev_src[e0 + i] * rows * nt - k;
+            ev[i].k = k;
+            ev[i].amp = ev_amp[e0 + i];
         }
         __syncthreads();
         if (!active) continue;
+#pragma unroll 2
         for (int e = 0; e < ne; ++e) {
-            const long u = (long)t - s_k[e];
-            if (u < 0 || u >= nt) continue;
-            acc += s_a[e] * __ldg(traces + ((size_t)s_src[e] * rows + row) * nt + u);
+            const Event v = ev[e];
+            const int u = t0 - v.k;  // trace sample of the span's first output sample
+            if (u >= nt || u + 32 * R <= 0) continue;
+            const float* x = base + v.ofs;
+            if (u >= 0 && u + 32 * R <= nt) {
+#pragma unroll
+                for (int i = 0; i < R; ++i) acc[i] = __fmaf_rn(v.amp, __ldg(x + 32 * i), acc[i]);
+            } else {
+#pragma unroll
+                for (int i = 0; i < R; ++i) {
+                    const int ui = u + lane + 32 * i;
+                    if (ui >= 0 && ui < nt) acc[i] = __fmaf_rn(v.amp, __ldg(x + 32 * i), acc[i]);
+                }
+            }
         }
     }
-    if (active) gather[row * n_out + t] = acc;
+    if (!active) return;
+    float* out = gather + row * n_out + t0 + lane;
+#pragma unroll
+    for (int i = 0; i < R; ++i)
+        if (t0 + lane + 32 * i < n_out) out[32 * i] = acc[i];
+}
+
+template <int R>
+static cudaError_t launch_superpose_r(const float* traces, int n_rcv, int nt, const int* ev_src, const float* ev_amp,
+                                      const int* ev_shift, int n_events, int n_out, float* gather, cudaStream_t st)
+{
+    const long long rows = 4LL * n_rcv, spans = (n_out + 32LL * R - 1) / (32 * R);
+    const long long blocks = (rows * spans + SUP_WARPS - 1) / SUP_WARPS;
+    if (blocks > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
+    superpose_kernel<R><<<(unsigned)blocks, 32 * SUP_WARPS, 0, st>>>(traces, rows, nt, ev_src, ev_amp, ev_shift,
+                                                                    n_events, n_out, (int)spans, gather);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_superpose(const float* traces, int n_src, int n_rcv, int nt, const int* ev_src,
@@ -251,9 +302,14 @@ cudaError_t launch_superpose(const float* traces, int n_src, int n_rcv, int nt, 
                              cudaStream_t st)
 {
     (void)n_src;
-    dim3 grid((n_out + 255) / 256, 4 * n_rcv);
-    superpose_kernel<<<grid, 256, 0, st>>>(traces, n_rcv, nt, ev_src, ev_amp, ev_shift, n_events, n_out, gather);
-    return cudaGetLastError();
+    // R = 8 and 4 by output samples (one GB300, 300 events): 19.1 M 0.991 and 1.022 ms, 16.4 M with
+    // short traces 0.336 and 0.475, 1.23 M 67.9 and 71.9 us; 0.61 M (200 events) 38.3 and 34.3,
+    // 0.26 M 24.2 and 22.2: below about a million the longer
+    // spans leave SMs idle.  R = 2 lost at every size, R = 16 won only with the short traces (0.287 ms,
+    // 1.24 at the first size).
+    if (4LL * n_rcv * n_out >= 1 << 20)
+        return launch_superpose_r<8>(traces, n_rcv, nt, ev_src, ev_amp, ev_shift, n_events, n_out, gather, st);
+    return launch_superpose_r<4>(traces, n_rcv, nt, ev_src, ev_amp, ev_shift, n_events, n_out, gather, st);
 }
 
 // flag |= 1 if any field value is NaN or infinite

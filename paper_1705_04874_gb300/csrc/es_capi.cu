@@ -214,7 +214,7 @@ int ensure_prepared()
 // Axis lengths: an FFT plan (pass_plans.h), else a convolution pass (conv_plans.h) or, below
 // CONV_MIN_N cells and in the compensated mode, the circulant pass, up to
 // CIRC_MAX_N (circ_pass.cu).  With an odd nx the y and z FFT passes move their
-// x-adjacent pencil pairs as single floats (pass_kernels_odd.cu).
+// pencil pairs as single floats (pass_strided1.cu).
 bool fft_plan(int n) { int a, b; return plan_radices(n, &a, &b) != 0; }
 bool axis_ok(int n) { return n >= 3 && n <= CIRC_MAX_N; }
 bool fft_axis(int n, int) { return fft_plan(n); }

@@ -65,3 +65,33 @@ def test_event_selection_and_clustered_superposition(ev, orc):
     # the clusters follow each other in time (means 0.3 s apart, spread 0.1 s)
     mean_t0 = [float(np.mean(t0s[labels == c])) for c in range(3)]
     assert mean_t0[0] < mean_t0[1] < mean_t0[2]
+
+
+@pytest.mark.parametrize("n_src, n_rcv, nt, n_events, n_out", [
+    (2, 1, 1, 3, 1),          # one sample
+    (3, 5, 64, 40, 128),      # one span of 128 samples exactly, four per thread
+    (3, 5, 63, 40, 129),      # one sample over
+    (2, 3, 700, 1025, 300),   # a trace longer than the window, one event past a chunk of 1024
+    (3, 520, 300, 1030, 1217),  # eight per thread: 256 samples per span, the last one partly outside
+])
+def test_superpose_spans_and_chunks(ev, n_src, n_rcv, nt, n_events, n_out):
+    """Shifts from a trace before the window to one past its end; a sum of k products in FP32 is
+    within k 2^-24 of the sum of their magnitudes (first order, doubled here)."""
+    es, _ = ev
+    rng = np.random.default_rng(n_out)
+    tr = rng.standard_normal((n_src, 4, n_rcv, nt)).astype(np.float32)
+    src = rng.integers(0, n_src, n_events).astype(np.int32)
+    amps = rng.standard_normal(n_events).astype(np.float32)
+    shift = rng.integers(-nt - 2, n_out + 3, n_events)
+    shift[:3] = (-nt, n_out, n_out - 1)[:len(shift[:3])]
+    dt = 0.25  # exact in FP32 with every shift
+    got = es.es_superpose(tr, src, amps, (shift * dt).astype(np.float32), dt, n_out)
+    want = np.zeros((4, n_rcv, n_out))
+    size = np.zeros((4, n_rcv, n_out))
+    for s, a, k in zip(src, amps.astype(np.float64), shift):
+        lo, hi = max(k, 0), min(k + nt, n_out)
+        if lo < hi:
+            term = a * tr[s][..., lo - k:hi - k]
+            want[..., lo:hi] += term
+            size[..., lo:hi] += np.abs(term)
+    assert np.all(np.abs(got - want) <= 2 * n_events * 2.0 ** -24 * size)
