@@ -105,8 +105,9 @@ int forward(es_sur* s, const float* pos, const float* mt, int B, float* out = nu
     return ES_OK;
 }
 
-// gradients into s->g, given s->dUb from the loss
-int backward(es_sur* s, const float* mt, int B)
+// gradients into s->g, given s->dUb from the loss; the decoder's only with `decoder` (a training
+// step takes it in the GEMM that updates the decoder)
+int backward(es_sur* s, const float* mt, int B, bool decoder = true)
 {
     const int K6 = 6 * s->K, D = (int)s->D;
     const __nv_bfloat16* W2 = s->pb + s->oW2;
@@ -116,7 +117,8 @@ int backward(es_sur* s, const float* mt, int B)
     // (long K = D: split-K)
     CKS(transpose_bf16(s->Zb, B, K6, s->ZT, s->st));
     CKS(transpose_bf16(s->dUb, B, D, s->dUT, s->st));
-    CKS(gemm_bf16(K6, D, B, s->ZT, B, false, s->dUT, B, true, s->g + s->oWd, D, 1.f, 0.f, 1, s->st));
+    if (decoder)
+        CKS(gemm_bf16(K6, D, B, s->ZT, B, false, s->dUT, B, true, s->g + s->oWd, D, 1.f, 0.f, 1, s->st));
     const int split = (int)std::max<long long>(1, std::min<long long>(256, s->D / 2048));
     CKS(gemm_bf16(B, K6, D, s->dUb, D, false, Wd, D, true, s->dZ, K6, 1.f, 0.f, split, s->st));
     CKS(sur_contract(mt, s->dZ, B, s->K, s->dA, s->dAb, s->st));
@@ -167,7 +169,7 @@ int es_sur_create(const es_sur_config* cfg, es_sur** out)
     s->oWd = seg((size_t)6 * s->K * s->D);
     s->P = o;
     const size_t B = s->B, P = s->P, H = s->H, K = s->K, D = s->D, F = s->F;
-    const size_t f32 = 4 * (4 * P + 4 + B * (2 * H + K + D + 6 * K + K + 2 * H + 2) + 128);
+    const size_t f32 = 4 * (4 * P + 4 + B * (2 * H + K + D + 6 * K + K + 2 * H + 8) + 128);
     const size_t b16 = 2 * (P + B * (F + 2 * H + 6 * K + D + K + 2 * H) + B * (6 * K + D)) + 2048;
     if (cudaMalloc(&s->pool, f32 + b16) != cudaSuccess) {
         delete s;
@@ -189,7 +191,7 @@ int es_sur_create(const es_sur_config* cfg, es_sur** out)
     s->dH2 = takef(B * H);
     s->dH1 = takef(B * H);
     s->loss = takef(8);
-    s->acc = takef(2 * B);
+    s->acc = takef(8 * B);
     __nv_bfloat16* bp = reinterpret_cast<__nv_bfloat16*>(fp);
     auto takeb = [&](size_t n) { __nv_bfloat16* r = bp; bp += (n + 7) / 8 * 8; return r; };
     s->pb = takeb(P);
@@ -320,14 +322,14 @@ int es_sur_train_step(es_sur* s, const float* pos, const float* mt, const float*
     cudaGetLastError();
     if ((rc = forward(s, pos, mt, B)) != ES_OK) return rc;
     CKS(sur_loss(s->U, target, s->scale, B, s->D / 4, 1e-30f, s->dUb, s->loss, s->acc, nullptr, s->st));
-    if ((rc = backward(s, mt, B)) != ES_OK) return rc;
+    if ((rc = backward(s, mt, B, false)) != ES_OK) return rc;
     s->t += 1;
-    // the MLP's parameters, then the decoder (the last segment) with its K-major copy refreshed
-    // in the same pass
-    const size_t K6 = 6 * (size_t)s->K;
-    CKS(sur_adam(s->p, s->g, s->m, s->v, s->oWd, lr, 0.9f, 0.999f, 1e-8f, s->t, s->pb, s->st));
-    CKS(sur_adam_t(s->p + s->oWd, s->g + s->oWd, s->m + s->oWd, s->v + s->oWd, (long long)K6, s->D, lr, 0.9f, 0.999f,
-                   1e-8f, s->t, s->pb + s->oWd, s->WdT, s->st));
+    // the decoder (the last segment) in the GEMM that forms its gradient, both BF16 copies with it;
+    // then the MLP's parameters
+    const size_t wd = s->oWd;
+    CKS(gemm_adam_tc(6 * s->K, (int)s->D, B, s->ZT, B, s->dUT, B, s->p + wd, s->m + wd, s->v + wd, lr, 0.9f, 0.999f,
+                     1e-8f, s->t, s->pb + wd, s->WdT, s->st));
+    CKS(sur_adam(s->p, s->g, s->m, s->v, wd, lr, 0.9f, 0.999f, 1e-8f, s->t, s->pb, s->st));
     s->ver += 1;
     s->wdt_ver = s->ver;
     if (loss) {

@@ -34,6 +34,7 @@
 
 #include <mutex>
 
+#include "sur_adam.cuh"
 #include "sur_internal.h"
 #include "tc_ptx.cuh"
 
@@ -288,6 +289,341 @@ __global__ void __launch_bounds__(THREADS, 1)
     }
 }
 
+// ---------------------------------------------------------------------------
+// dW = A B^T with the Adam step in the epilogue: the gradient of a weight block
+// W[M][N] goes from tensor memory straight into the update of p, m and v, and of
+// the two BF16 copies (row-major pb, transposed pt), and is never stored.
+//
+// What bounds it is HBM: 28 bytes per weight (p, m, v read and written, two BF16
+// copies written) against 36 with the gradient written by one kernel and read by
+// the next.  A tile is 128 x 128 and K is one batch, a few k-blocks, so one
+// operand stage is enough (the MMAs run a tile ahead of the epilogue) and the
+// rest of shared memory moves the weights: each of eight epilogue warps walks
+// 32 x 32 blocks of p, m and v through two places of its own, one block arriving
+// by TMA while the other is updated in place and leaves by TMA.  A lane holds a
+// row, as tcgen05.ld delivers the gradient, so nothing is turned around but the
+// row-major BF16 copy: the 128-byte swizzle keeps the 16-byte accesses free of
+// bank conflicts, and the transposed copy is written by columns (32 lanes, 64
+// contiguous bytes).
+// 4608 x 262144 weights, batch 256 (one GB300): 5.8 ms, 5.8 TB/s, where the two
+// kernels took 7.0 (1.26 and 5.7, at 6.8 TB/s; 8.65 -> 7.46 ms per training
+// step).  Of the step times on the way: operands through registers 10.5 (the
+// kernel spilled, which waits for each load where it is issued), blocks of 16
+// columns 9.0 (TMA moves a row of 64 bytes no faster than one of 128), the
+// row-major copy stored 16 bytes a row 8.2, the two column blocks of a row not
+// side by side 7.9; prefetching into L2 was slower (8.5).  Without the copies
+// it runs at the same 5.8 TB/s: the rest is DRAM's rate for this pattern.
+constexpr int AD_TN = 128, AD_STAGES = 1, AD_WARPS = 8, AD_THREADS = 32 * (2 + AD_WARPS);
+constexpr int AD_STAGE_BYTES = A_BYTES + AD_TN * TK * 2;
+constexpr int AD_COLS = 32, AD_RING = 2;             // columns of a block, blocks of a warp's ring
+constexpr int AD_ARRAY = 32 * AD_COLS * 4;           // one array's block: 32 rows of 128 bytes
+constexpr int AD_SMEM = AD_STAGES * AD_STAGE_BYTES + AD_WARPS * AD_RING * 3 * AD_ARRAY + 1024;
+constexpr int AD_BLOCKS = AD_TN / 2 / AD_COLS;       // blocks of a warp in a tile: 32 rows, every other column block
+constexpr uint32_t AD_IDESC = (IDESC & ~(0x3fu << 17)) | ((uint32_t)(AD_TN >> 3) << 17);
+static_assert(AD_RING - 1 <= AD_BLOCKS, "blocks ahead reach the next tile at most");
+static_assert(AD_STAGE_BYTES % 1024 == 0 && AD_ARRAY % 1024 == 0, "swizzle atoms must stay aligned");
+
+struct AdamBlock {
+    __nv_bfloat16 *pb, *pt;
+    AdamStep step;
+};
+
+// Tiles in strips of AD_STRIP columns, columns fastest within a strip: the CTAs at work are two rows
+// of tiles, 38 KB contiguous in each row of the weights, and the strip's part of B stays in L2 while
+// the rows go by.  ms per step at the size above by strip width: 5 7.64, 19 7.54, 38 7.50, 76 7.46,
+// 152 7.53; row tiles fastest over the whole matrix 7.66.
+constexpr int AD_STRIP = 76;
+__device__ __forceinline__ void adam_tile(int t, int mt, int ntl, int* mi, int* ni)
+{
+    const int s = t / (AD_STRIP * mt), r = t - s * AD_STRIP * mt, w = min(AD_STRIP, ntl - s * AD_STRIP);
+    *mi = r / w;
+    *ni = s * AD_STRIP + r - *mi * w;
+}
+
+// 4 x 4 transpose of 16-byte pieces among four neighbouring lanes: lane i's piece k becomes lane k's piece i
+__device__ __forceinline__ void turn_four(uint4 (&x)[4], int lane)
+{
+#pragma unroll
+    for (int d = 1; d <= 2; d *= 2) {
+        const bool up = lane & d;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            if (k & d) continue;
+            uint4 give = up ? x[k] : x[k | d];
+            give.x = __shfl_xor_sync(0xffffffffu, give.x, d);
+            give.y = __shfl_xor_sync(0xffffffffu, give.y, d);
+            give.z = __shfl_xor_sync(0xffffffffu, give.z, d);
+            give.w = __shfl_xor_sync(0xffffffffu, give.w, d);
+            if (up) x[k] = give;
+            else x[k | d] = give;
+        }
+    }
+}
+
+__device__ __forceinline__ void tma_store_2d(const CUtensorMap* map, uint32_t src, int x, int y)
+{
+    asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%2, %3}], [%1];" ::"l"(
+                     reinterpret_cast<uint64_t>(map)),
+                 "r"(src), "r"(x), "r"(y)
+                 : "memory");
+}
+
+__global__ void __launch_bounds__(AD_THREADS, 1)
+    gemm_adam_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,
+                     const __grid_constant__ CUtensorMap mapP, const __grid_constant__ CUtensorMap mapM,
+                     const __grid_constant__ CUtensorMap mapV, int M, int N, int nkb, int mt, int ntl, const AdamBlock w)
+{
+    extern __shared__ uint8_t dyn[];
+    __shared__ __align__(8) uint64_t full[AD_STAGES], empty[AD_STAGES], acc_full[2], acc_empty[2], mma_done;
+    __shared__ __align__(8) uint64_t arrived[AD_WARPS * AD_RING];
+    __shared__ uint32_t tmem_slot;
+    __shared__ int s_issued, s_consumed;
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t base = (smem_u32(dyn) + 1023u) & ~1023u;
+    const int ntiles = mt * ntl;
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < AD_STAGES; ++s) {
+            mbar_init(&full[s], 1);
+            mbar_init(&empty[s], 1);
+        }
+        for (int b = 0; b < 2; ++b) {
+            mbar_init(&acc_full[b], 1);
+            mbar_init(&acc_empty[b], AD_WARPS);  // one arrival per epilogue warp
+        }
+        for (int s = 0; s < AD_WARPS * AD_RING; ++s) mbar_init(&arrived[s], 1);
+        mbar_init(&mma_done, 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        s_issued = 0;
+        s_consumed = 0;
+    }
+    __syncwarp();
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)),
+                     "r"(2 * AD_TN)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = tmem_slot;
+
+    if (warp == 0) {
+        if (lane == 0) {
+            int it = 0;
+            bool ok = true;
+            for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
+                int mi, ni;
+                adam_tile(t, mt, ntl, &mi, &ni);
+                for (int kb = 0; kb < nkb; ++kb, ++it) {
+                    const int s = it % AD_STAGES;
+                    if (!mbar_wait(&empty[s], ((it / AD_STAGES) & 1) ^ 1)) {
+                        atomicOr(&g_tc_status, 1u);
+                        ok = false;
+                        break;
+                    }
+                    const uint32_t sa = base + s * AD_STAGE_BYTES;
+                    mbar_expect_tx(&full[s], AD_STAGE_BYTES);
+                    tma_load_2d(sa, &mapA, &full[s], kb * TK, mi * TM);
+                    tma_load_2d(sa + A_BYTES, &mapB, &full[s], kb * TK, ni * AD_TN);
+                }
+            }
+            s_issued = it;
+        }
+    } else if (warp == 1) {
+        if (lane == 0) {
+            int it = 0, lt = 0;
+            bool ok = true;
+            for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x, ++lt) {
+                const int b = lt & 1;
+                if (!mbar_wait(&acc_empty[b], ((lt >> 1) & 1) ^ 1)) {
+                    atomicOr(&g_tc_status, 2u);
+                    break;
+                }
+                tc_fence_after();
+                const uint32_t acc = tmem + (uint32_t)(b * AD_TN);
+                for (int kb = 0; kb < nkb; ++kb, ++it) {
+                    const int s = it % AD_STAGES;
+                    if (!mbar_wait(&full[s], (it / AD_STAGES) & 1)) {
+                        atomicOr(&g_tc_status, 2u);
+                        ok = false;
+                        break;
+                    }
+                    tc_fence_after();
+                    const uint32_t sa = base + s * AD_STAGE_BYTES;
+                    const uint64_t da = sw128_desc(sa), db = sw128_desc(sa + A_BYTES);
+#pragma unroll
+                    for (int k = 0; k < TK / UK; ++k) {
+                        const uint64_t step = (uint64_t)((k * UK * 2) >> 4);
+                        tc_mma(acc, da + step, db + step, AD_IDESC, (kb | k) != 0);
+                    }
+                    tc_commit(&empty[s]);
+                }
+                if (ok) tc_commit(&acc_full[b]);
+            }
+            s_consumed = it;
+            tc_commit(&mma_done);
+        }
+    } else {
+        // epilogue warp: TMEM lane quarter q (tile rows 32 q ..), column blocks h, h + 2 of the tile
+        const int q = warp & 3, h = (warp - 2) >> 2;
+        const uint32_t ring = base + AD_STAGES * AD_STAGE_BYTES + (uint32_t)(warp - 2) * (AD_RING * 3 * AD_ARRAY);
+        uint64_t* const bar = arrived + (warp - 2) * AD_RING;
+        const int mine = (ntiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;  // tiles of this CTA
+        const int blocks = mine * AD_BLOCKS;
+        // one lane: block j of the tile at (row, col) into place s (past the edge zeros arrive)
+        auto load = [&](int s, int row, int col, int j) {
+            const uint32_t dst = ring + s * 3 * AD_ARRAY;
+            mbar_expect_tx(&bar[s], 3 * AD_ARRAY);
+            tma_load_2d(dst, &mapP, &bar[s], col + 2 * j * AD_COLS, row);
+            tma_load_2d(dst + AD_ARRAY, &mapM, &bar[s], col + 2 * j * AD_COLS, row);
+            tma_load_2d(dst + 2 * AD_ARRAY, &mapV, &bar[s], col + 2 * j * AD_COLS, row);
+        };
+        // corner of this warp's part of tile t
+        auto corner = [&](int t, int* row, int* col) {
+            int mi, ni;
+            adam_tile(t, mt, ntl, &mi, &ni);
+            *row = mi * TM + q * 32;
+            *col = ni * AD_TN + h * AD_COLS;
+        };
+        int row0, col_t;
+        corner(blockIdx.x, &row0, &col_t);
+        int issued = 0, used = 0;
+        for (; issued < AD_RING - 1 && issued < blocks; ++issued)
+            if (lane == 0) load(issued, row0, col_t, issued);
+        bool ok = true;
+        for (int lt = 0; lt < mine && ok; ++lt) {
+            const int b = lt & 1;
+            // one lane waits and the warp follows its result: tcgen05.ld below needs the whole warp
+            int got = 0;
+            if (lane == 0) got = mbar_wait(&acc_full[b], (lt >> 1) & 1) ? 1 : 0;
+            got = __shfl_sync(0xffffffffu, got, 0);
+            if (!got) {
+                if (lane == 0) atomicOr(&g_tc_status, 4u);
+                break;
+            }
+            tc_fence_after();
+            int row_n = 0, col_n = 0;  // the next tile's
+            if (lt + 1 < mine) corner(blockIdx.x + (lt + 1) * gridDim.x, &row_n, &col_n);
+            const int row = row0 + lane;
+#pragma unroll 1
+            for (int j = 0; j < AD_BLOCKS; ++j, ++used) {
+                const int s = used % AD_RING;
+                got = mbar_wait(&bar[s], (used / AD_RING) & 1) ? 1 : 0;  // every lane: it reads what TMA wrote
+                if (!__all_sync(0xffffffffu, got)) {
+                    if (lane == 0) atomicOr(&g_tc_status, 4u);
+                    ok = false;
+                    break;
+                }
+                __syncwarp();
+                uint32_t r[32];
+                tmem_ld32(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(b * AD_TN + (2 * j + h) * AD_COLS), r);
+                const int col0 = col_t + 2 * j * AD_COLS;
+                __nv_bfloat16* pt = w.pt + (size_t)col0 * M + row;
+                uint8_t* const blk = dyn + (ring + s * 3 * AD_ARRAY - smem_u32(dyn)) + lane * 128;
+                uint4 piece[4];  // the row's BF16 copy, eight columns each
+#pragma unroll
+                for (int c = 0; c < AD_COLS / 8; ++c) {  // eight columns at a time: two 16-byte pieces, swizzled
+                    float4* const at[2] = {reinterpret_cast<float4*>(blk + 16 * ((2 * c) ^ (lane & 7))),
+                                           reinterpret_cast<float4*>(blk + 16 * ((2 * c + 1) ^ (lane & 7)))};
+                    constexpr int ARRAY = AD_ARRAY / 16;
+                    float p[8], g[8], m[8], v[8];
+#pragma unroll
+                    for (int i = 0; i < 2; ++i) {
+                        *reinterpret_cast<float4*>(p + 4 * i) = at[i][0];
+                        *reinterpret_cast<float4*>(m + 4 * i) = at[i][ARRAY];
+                        *reinterpret_cast<float4*>(v + 4 * i) = at[i][2 * ARRAY];
+                    }
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) g[i] = __uint_as_float(r[8 * c + i]);
+                    adam_many<8>(p, g, m, v, w.step);
+#pragma unroll
+                    for (int i = 0; i < 2; ++i) {
+                        at[i][0] = *reinterpret_cast<const float4*>(p + 4 * i);
+                        at[i][ARRAY] = *reinterpret_cast<const float4*>(m + 4 * i);
+                        at[i][2 * ARRAY] = *reinterpret_cast<const float4*>(v + 4 * i);
+                    }
+                    const int col = col0 + 8 * c;
+                    const uint2 lo = pack_bf16x4(make_float4(p[0], p[1], p[2], p[3])),
+                                hi = pack_bf16x4(make_float4(p[4], p[5], p[6], p[7]));
+                    piece[c] = make_uint4(lo.x, lo.y, hi.x, hi.y);
+                    if (row < M && col < N) {  // N is a multiple of 8
+                        const __nv_bfloat16* e = reinterpret_cast<const __nv_bfloat16*>(&piece[c]);
+#pragma unroll
+                        for (int k = 0; k < 8; ++k, pt += M) *pt = e[k];
+                    }
+                    if (c == 0) {
+                        // the other place is free once the block before has been read from it
+                        if (lane == 0 && issued < blocks) {
+                            asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+                            const int ahead = j + AD_RING - 1;  // blocks into this tile, or the next
+                            if (ahead < AD_BLOCKS) load(issued % AD_RING, row0, col_t, ahead);
+                            else load(issued % AD_RING, row_n, col_n, ahead - AD_BLOCKS);
+                        }
+                        if (issued < blocks) ++issued;
+                    }
+                }
+                // the row-major copy, turned around among four lanes: a store covers 64 bytes of eight rows
+                // (pieces of 16 bytes a row at a time would write half sectors)
+                turn_four(piece, lane);
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const int rr = row0 + (lane & ~3) + k, col = col0 + 8 * (lane & 3);
+                    if (rr < M && col < N) *reinterpret_cast<uint4*>(w.pb + (size_t)rr * N + col) = piece[k];
+                }
+                // the block leaves; the place of the one before is free once it has been read
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                __syncwarp();
+                if (lane == 0) {
+                    if (row0 < M && col0 < N) {
+                        const uint32_t src = ring + s * 3 * AD_ARRAY;
+                        tma_store_2d(&mapP, src, col0, row0);
+                        tma_store_2d(&mapM, src + AD_ARRAY, col0, row0);
+                        tma_store_2d(&mapV, src + 2 * AD_ARRAY, col0, row0);
+                    }
+                    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+                }
+                if (j == AD_BLOCKS - 1) {  // every tcgen05.ld of this warp has completed: hand the accumulator back
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&acc_empty[b]);
+                }
+            }
+            row0 = row_n;
+            col_t = col_n;
+        }
+        if (lane == 0) {
+            // blocks that were asked for and not used (only after a wait gave up) must land before the CTA
+            // exits, and the last ones must have left shared memory
+            for (; used < issued; ++used)
+                if (!mbar_wait(&bar[used % AD_RING], (used / AD_RING) & 1)) {
+                    atomicOr(&g_tc_status, 16u);
+                    break;
+                }
+            asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+        }
+    }
+
+    __syncwarp();
+    tc_fence_before();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        if (!mbar_wait(&mma_done, 0)) atomicOr(&g_tc_status, 8u);
+        for (int it = s_consumed; it < s_issued; ++it)
+            if (!mbar_wait(&full[it % AD_STAGES], (it / AD_STAGES) & 1)) {
+                atomicOr(&g_tc_status, 16u);
+                break;
+            }
+    }
+    __syncthreads();
+    if (warp == 0) {
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * AD_TN) : "memory");
+    }
+}
+
 }  // namespace
 
 cudaError_t gemm_bf16_tc(int M, int N, int K, const __nv_bfloat16* A, int lda, const __nv_bfloat16* B, int ldb,
@@ -326,6 +662,47 @@ cudaError_t gemm_bf16_tc(int M, int N, int K, const __nv_bfloat16* A, int lda, c
     gemm_tc_kernel<<<(unsigned)grid, THREADS, SMEM_BYTES, st>>>(mapA, mapB, M, N, nkb, kb_per, mt, ntl, (int)ntiles,
                                                                C, ldc, alpha, beta, split_k > 1 ? 1 : 0, av,
                                                                alpha4 ? span : 0);
+    return cudaGetLastError();
+}
+
+// a row-major FP32 [rows][cols] array in blocks of 32 x AD_COLS, 128-byte swizzle
+static bool make_map_f32(EncodeTiled fn, CUtensorMap* map, float* ptr, int rows, int cols)
+{
+    const cuuint64_t dim[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
+    const cuuint64_t stride[1] = {(cuuint64_t)cols * 4};
+    const cuuint32_t box[2] = {(cuuint32_t)AD_COLS, 32u};
+    const cuuint32_t estride[2] = {1, 1};
+    return fn(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, ptr, dim, stride, box, estride, CU_TENSOR_MAP_INTERLEAVE_NONE,
+              CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) ==
+           CUDA_SUCCESS;
+}
+
+cudaError_t gemm_adam_tc(int M, int N, int K, const __nv_bfloat16* A, int lda, const __nv_bfloat16* B, int ldb, float* p,
+                         float* m, float* v, float lr, float b1, float b2, float eps, int t, __nv_bfloat16* pb,
+                         __nv_bfloat16* pt, cudaStream_t st)
+{
+    if (M <= 0 || N <= 0 || K <= 0 || N % 8) return cudaErrorInvalidValue;
+    const uintptr_t al = reinterpret_cast<uintptr_t>(p) | reinterpret_cast<uintptr_t>(m) | reinterpret_cast<uintptr_t>(v) |
+                         reinterpret_cast<uintptr_t>(pb) | reinterpret_cast<uintptr_t>(A) | reinterpret_cast<uintptr_t>(B);
+    if (al & 15) return cudaErrorInvalidValue;
+    if (lda % 8 || ldb % 8 || lda < K || ldb < K) return cudaErrorInvalidValue;
+    EncodeTiled fn = encode_tiled();
+    if (!fn) return cudaErrorNotSupported;
+    alignas(64) CUtensorMap mapA, mapB, mapP, mapM, mapV;
+    if (!make_map(fn, &mapA, A, M, K, lda, TM) || !make_map(fn, &mapB, B, N, K, ldb, AD_TN) ||
+        !make_map_f32(fn, &mapP, p, M, N) || !make_map_f32(fn, &mapM, m, M, N) || !make_map_f32(fn, &mapV, v, M, N))
+        return cudaErrorInvalidValue;
+    const int mt = (M + TM - 1) / TM;
+    const long long ntiles = (long long)mt * ((N + AD_TN - 1) / AD_TN);
+    if (ntiles > 0x7fffffffLL - 4096) return cudaErrorInvalidValue;
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(gemm_adam_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, AD_SMEM);
+    if (e != cudaSuccess) return e;
+    const AdamBlock w = {pb, pt, adam_step(lr, b1, b2, eps, t)};
+    const long long grid = ntiles < sms ? ntiles : sms;
+    gemm_adam_kernel<<<(unsigned)grid, AD_THREADS, AD_SMEM, st>>>(mapA, mapB, mapP, mapM, mapV, M, N, (K + TK - 1) / TK, mt, (N + AD_TN - 1) / AD_TN, w);
     return cudaGetLastError();
 }
 

@@ -16,6 +16,12 @@ cudaError_t gemm_bf16(int M, int N, int K, const __nv_bfloat16* A, int lda, bool
 cudaError_t gemm_bf16_tc(int M, int N, int K, const __nv_bfloat16* A, int lda, const __nv_bfloat16* B, int ldb,
                          float* C, int ldc, float alpha, float beta, int split_k, cudaStream_t st,
                          const float* alpha4 = nullptr, int span = 0);
+// The Adam step of a row-major weight block W[M][N] (p, its moments m, v) with the gradient A[M][K]
+// B[N][K]^T taken from tensor memory and never stored; writes the BF16 copy row-major (pb) and
+// transposed (pt, [N][M]).  N a multiple of 8, arrays 16-byte aligned; see sur_gemm_tc.cu.
+cudaError_t gemm_adam_tc(int M, int N, int K, const __nv_bfloat16* A, int lda, const __nv_bfloat16* B, int ldb, float* p,
+                         float* m, float* v, float lr, float b1, float b2, float eps, int t, __nv_bfloat16* pb,
+                         __nv_bfloat16* pt, cudaStream_t st);
 // reads and clears the tcgen05 GEMM's device status word (bits set by waits that gave up)
 cudaError_t gemm_tc_status(unsigned* status);
 // Launches one kernel whose bounded wait on a barrier nothing completes gives
@@ -42,7 +48,7 @@ cudaError_t sur_contract(const float* M6, const float* dZ, int B, int K, float* 
 // l_b = sum_c |u_c - tau_c|^2 / (sum_c |tau_c|^2 + eps) (squared relative L2 of
 // the component-scaled seismogram), loss = mean_b l_b (device float),
 // per_sample (optional, device [B]) = l_b, dU = dloss/du in BF16 (skipped when
-// null); acc: device scratch of 2 B floats
+// null); acc: device scratch of 8 B floats, 8-byte aligned
 cudaError_t sur_loss(const float* U, const float* T, const float* scale, int B, long long Dc, float eps,
                      __nv_bfloat16* dU, float* loss, float* acc, float* per_sample, cudaStream_t st);
 cudaError_t sur_init_normal(float* p, size_t n, float std, unsigned long long seed, cudaStream_t st);
@@ -56,11 +62,5 @@ cudaError_t sur_colsum(const float* G, int B, int N, float* db, cudaStream_t st)
 // Adam step (bias-corrected, lr, b1, b2, eps) on FP32 params, refreshing the BF16 copy (may be null)
 cudaError_t sur_adam(float* p, const float* g, float* m, float* v, size_t n, float lr, float b1, float b2, float eps,
                      int t, __nv_bfloat16* pb, cudaStream_t st);
-// The same step on a row-major [rows][cols] block (the decoder; cols a multiple
-// of 4, 16-byte aligned), writing the BF16 copy both row-major (pb) and
-// transposed (pt, [cols][rows]) -- one pass over the parameters instead of a
-// step plus a transpose.
-cudaError_t sur_adam_t(float* p, const float* g, float* m, float* v, long long rows, long long cols, float lr,
-                       float b1, float b2, float eps, int t, __nv_bfloat16* pb, __nv_bfloat16* pt, cudaStream_t st);
 
 }  // namespace es

@@ -7,6 +7,7 @@
 
 #include <algorithm>
 
+#include "sur_adam.cuh"
 #include "sur_internal.h"
 
 namespace es {
@@ -91,9 +92,11 @@ __global__ void contract_kernel(const float* M6, const float* dZ, int B, int K, 
 // Loss in component-scaled units: with y = s_c u and tau = t / s_c,
 // l_b = sum_c |u_c - tau_c|^2 / (sum_c |tau_c|^2 + eps) -- the relative L2
 // error (squared) of the whole 4C seismogram after each component is divided
-// by its scale.  Pass 1 (one block per sample and component) accumulates the
-// two sums per sample; pass 2 writes l_b, the mean loss and dL/du.
-__global__ void loss_sums_kernel(const float* U, const float* T, const float* scale, long long Dc, float* acc)
+// by its scale.  Pass 1 (one block per sample and component) forms the two sums
+// of each, in a fixed order, so that two calls see the same dL/du to the last
+// bit of its BF16 rounding; pass 2 adds the components and writes l_b, the mean
+// loss and dL/du.
+__global__ void loss_sums_kernel(const float* U, const float* T, const float* scale, long long Dc, float2* acc)
 {
     const int b = blockIdx.x, c = blockIdx.y;
     const size_t base = ((size_t)b * 4 + c) * Dc;
@@ -109,19 +112,27 @@ __global__ void loss_sums_kernel(const float* U, const float* T, const float* sc
         se += __shfl_down_sync(0xffffffffu, se, o);
         st += __shfl_down_sync(0xffffffffu, st, o);
     }
-    if ((threadIdx.x & 31) == 0) {
-        atomicAdd(acc + 2 * b, se);
-        atomicAdd(acc + 2 * b + 1, st);
+    __shared__ float2 part[8];
+    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = make_float2(se, st);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        float2 sum = part[0];
+        for (int i = 1; i < 8; ++i) {
+            sum.x += part[i].x;
+            sum.y += part[i].y;
+        }
+        acc[4 * b + c] = sum;
     }
 }
 
 __global__ void loss_grad_kernel(const float* U, const float* T, const float* scale, int B, long long Dc, float eps,
-                                 const float* acc, __nv_bfloat16* dU, float* loss, float* per_sample)
+                                 const float2* acc, __nv_bfloat16* dU, float* loss, float* per_sample)
 {
     const int b = blockIdx.x, c = blockIdx.y;
-    const float den = acc[2 * b + 1] + eps;
+    const float2 a0 = acc[4 * b], a1 = acc[4 * b + 1], a2 = acc[4 * b + 2], a3 = acc[4 * b + 3];
+    const float den = a0.y + a1.y + a2.y + a3.y + eps;
     if (c == 0 && threadIdx.x == 0) {
-        const float lb = acc[2 * b] / den;
+        const float lb = (a0.x + a1.x + a2.x + a3.x) / den;
         if (per_sample) per_sample[b] = lb;
         atomicAdd(loss, lb / B);
     }
@@ -178,16 +189,6 @@ __global__ void colsum_kernel(const float* G, int B, int N, float* db)
     db[n] = s;
 }
 
-// one Adam update (bias corrections c1 = 1 - b1^t, c2 = 1 - b2^t); returns the new parameter
-__device__ __forceinline__ float adam_one(float& p, float g, float& m, float& v, float lr, float b1, float b2,
-                                          float eps, float c1, float c2)
-{
-    m = b1 * m + (1.f - b1) * g;
-    v = b2 * v + (1.f - b2) * g * g;
-    p = p - lr * (m / c1) / (sqrtf(v / c2) + eps);
-    return p;
-}
-
 __global__ void adam_kernel(float* p, const float* g, float* m, float* v, size_t n, float lr, float b1, float b2,
                             float eps, float c1, float c2, __nv_bfloat16* pb)
 {
@@ -201,76 +202,17 @@ __global__ void adam_kernel(float* p, const float* g, float* m, float* v, size_t
     }
 }
 
-__device__ __forceinline__ void adam_four(float4& p, float4 g, float4& m, float4& v, float lr, float b1, float b2,
-                                          float eps, float c1, float c2)
-{
-    adam_one(p.x, g.x, m.x, v.x, lr, b1, b2, eps, c1, c2);
-    adam_one(p.y, g.y, m.y, v.y, lr, b1, b2, eps, c1, c2);
-    adam_one(p.z, g.z, m.z, v.z, lr, b1, b2, eps, c1, c2);
-    adam_one(p.w, g.w, m.w, v.w, lr, b1, b2, eps, c1, c2);
-}
-
-__device__ __forceinline__ uint2 pack_bf16x4(float4 p)
-{
-    const __nv_bfloat162 lo = __floats2bfloat162_rn(p.x, p.y), hi = __floats2bfloat162_rn(p.z, p.w);
-    return make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
-}
-
 // four parameters per thread and iteration (n4 groups of four, 16-byte aligned)
-__global__ void adam4_kernel(float4* p, const float4* g, float4* m, float4* v, size_t n4, float lr, float b1,
-                             float b2, float eps, float c1, float c2, uint2* pb)
+__global__ void adam4_kernel(float4* p, const float4* g, float4* m, float4* v, size_t n4,
+                             const AdamStep w, uint2* pb)
 {
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n4; i += (size_t)gridDim.x * blockDim.x) {
         float4 pi = p[i], mi = m[i], vi = v[i];
-        adam_four(pi, g[i], mi, vi, lr, b1, b2, eps, c1, c2);
+        adam_four(pi, g[i], mi, vi, w);
         m[i] = mi;
         v[i] = vi;
         p[i] = pi;
         if (pb) pb[i] = pack_bf16x4(pi);
-    }
-}
-
-// 64 x 64 tiles of a row-major [rows][cols] block: the update and the
-// row-major BF16 copy four columns per thread, the transposed copy through a
-// shared [column][row] tile, four rows per thread (8-byte stores)
-constexpr int AT = 64, AT_LD = AT + 4;
-__global__ void adam_t_kernel(float* p, const float* g, float* m, float* v, long long rows, long long cols, float lr,
-                              float b1, float b2, float eps, float c1, float c2, __nv_bfloat16* pb,
-                              __nv_bfloat16* pt)
-{
-    __shared__ __align__(16) __nv_bfloat16 tt[AT][AT_LD];
-    const long long c0 = (long long)blockIdx.x * AT, r0 = (long long)blockIdx.y * AT;
-    const int cq = threadIdx.x & 15, rq = threadIdx.x >> 4;  // 16 column quads x 16 rows per sweep
-    for (int i = rq; i < AT; i += 16) {
-        const long long r = r0 + i, c = c0 + 4 * cq;
-        float4 pi = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (r < rows && c < cols) {
-            const size_t k = (size_t)r * cols + c;
-            pi = *reinterpret_cast<const float4*>(p + k);
-            float4 mi = *reinterpret_cast<const float4*>(m + k), vi = *reinterpret_cast<const float4*>(v + k);
-            adam_four(pi, *reinterpret_cast<const float4*>(g + k), mi, vi, lr, b1, b2, eps, c1, c2);
-            *reinterpret_cast<float4*>(m + k) = mi;
-            *reinterpret_cast<float4*>(v + k) = vi;
-            *reinterpret_cast<float4*>(p + k) = pi;
-            *reinterpret_cast<uint2*>(pb + k) = pack_bf16x4(pi);
-        }
-        tt[4 * cq][i] = __float2bfloat16(pi.x);
-        tt[4 * cq + 1][i] = __float2bfloat16(pi.y);
-        tt[4 * cq + 2][i] = __float2bfloat16(pi.z);
-        tt[4 * cq + 3][i] = __float2bfloat16(pi.w);
-    }
-    __syncthreads();
-    for (int j = rq; j < AT; j += 16) {
-        const long long c = c0 + j, r = r0 + 4 * cq;
-        if (c >= cols || r >= rows) continue;
-        const uint2 q = *reinterpret_cast<const uint2*>(&tt[j][4 * cq]);
-        __nv_bfloat16* dst = pt + (size_t)c * rows + r;
-        if (r + 4 <= rows && (rows & 3) == 0) {
-            *reinterpret_cast<uint2*>(dst) = q;
-        } else {
-            const __nv_bfloat16* e = reinterpret_cast<const __nv_bfloat16*>(&q);
-            for (int k = 0; k < 4 && r + k < rows; ++k) dst[k] = e[k];
-        }
     }
 }
 
@@ -354,10 +296,10 @@ cudaError_t sur_loss(const float* U, const float* T, const float* scale, int B, 
                      __nv_bfloat16* dU, float* loss, float* acc, float* per_sample, cudaStream_t st)
 {
     cudaError_t e = cudaMemsetAsync(loss, 0, sizeof(float), st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(acc, 0, 2 * sizeof(float) * B, st);
     if (e != cudaSuccess) return e;
-    loss_sums_kernel<<<dim3(B, 4), 256, 0, st>>>(U, T, scale, Dc, acc);
-    loss_grad_kernel<<<dim3(B, 4), 256, 0, st>>>(U, T, scale, B, Dc, eps, acc, dU, loss, per_sample);
+    float2* sums = reinterpret_cast<float2*>(acc);
+    loss_sums_kernel<<<dim3(B, 4), 256, 0, st>>>(U, T, scale, Dc, sums);
+    loss_grad_kernel<<<dim3(B, 4), 256, 0, st>>>(U, T, scale, B, Dc, eps, sums, dU, loss, per_sample);
     return cudaGetLastError();
 }
 
@@ -392,33 +334,17 @@ cudaError_t sur_colsum(const float* G, int B, int N, float* db, cudaStream_t st)
 cudaError_t sur_adam(float* p, const float* g, float* m, float* v, size_t n, float lr, float b1, float b2, float eps,
                      int t, __nv_bfloat16* pb, cudaStream_t st)
 {
-    const float c1 = 1.f - powf(b1, (float)t), c2 = 1.f - powf(b2, (float)t);
+    const AdamStep w = adam_step(lr, b1, b2, eps, t);
     const uintptr_t al = reinterpret_cast<uintptr_t>(p) | reinterpret_cast<uintptr_t>(g) |
                          reinterpret_cast<uintptr_t>(m) | reinterpret_cast<uintptr_t>(v);
     if (n % 4 == 0 && (al & 15) == 0 && (reinterpret_cast<uintptr_t>(pb) & 7) == 0) {
         adam4_kernel<<<blocks_for(n / 4), 256, 0, st>>>(
             reinterpret_cast<float4*>(p), reinterpret_cast<const float4*>(g), reinterpret_cast<float4*>(m),
-            reinterpret_cast<float4*>(v), n / 4, lr, b1, b2, eps, c1, c2, reinterpret_cast<uint2*>(pb));
+            reinterpret_cast<float4*>(v), n / 4, w,
+            reinterpret_cast<uint2*>(pb));
     } else {
-        adam_kernel<<<blocks_for(n), 256, 0, st>>>(p, g, m, v, n, lr, b1, b2, eps, c1, c2, pb);
+        adam_kernel<<<blocks_for(n), 256, 0, st>>>(p, g, m, v, n, lr, b1, b2, eps, w.c1, w.c2, pb);
     }
-    return cudaGetLastError();
-}
-
-cudaError_t sur_adam_t(float* p, const float* g, float* m, float* v, long long rows, long long cols, float lr,
-                       float b1, float b2, float eps, int t, __nv_bfloat16* pb, __nv_bfloat16* pt, cudaStream_t st)
-{
-    if (rows <= 0 || cols <= 0) return cudaSuccess;
-    const uintptr_t al = reinterpret_cast<uintptr_t>(p) | reinterpret_cast<uintptr_t>(g) |
-                         reinterpret_cast<uintptr_t>(m) | reinterpret_cast<uintptr_t>(v);
-    if (cols % 4 || (al & 15) || (reinterpret_cast<uintptr_t>(pb) & 7) || (reinterpret_cast<uintptr_t>(pt) & 7) ||
-        !pb || !pt)
-        return cudaErrorInvalidValue;
-    const long long gx = (cols + AT - 1) / AT, gy = (rows + AT - 1) / AT;
-    if (gx > 0x7fffffffLL || gy > 65535) return cudaErrorInvalidValue;
-    const float c1 = 1.f - powf(b1, (float)t), c2 = 1.f - powf(b2, (float)t);
-    adam_t_kernel<<<dim3((unsigned)gx, (unsigned)gy), 256, 0, st>>>(p, g, m, v, rows, cols, lr, b1, b2, eps, c1, c2,
-                                                                     pb, pt);
     return cudaGetLastError();
 }
 

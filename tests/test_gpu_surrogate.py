@@ -323,3 +323,44 @@ def test_sources_away_from_the_catalog(env):
             assert used.any() and (~used[:8]).sum() == trusted[:8].sum()
         finally:
             s.close()
+
+
+def test_decoder_step_inside_its_gradient_gemm(env):
+    """The decoder takes its Adam step in the GEMM that forms the gradient, here with more 128 x 128
+    tiles than SMs: 144 x 9824 (ragged row and column tiles, a 16-row remainder of a 32-row block), a batch
+    of 24 (a part of a K slab).  Two steps against Adam in FP64 on the gradients that loss_grad
+    returns.  The two FP32 accumulations of at most 24 products differ by about 1e-6 of their size,
+    so where |g| > 0.1 rms in both steps a step m / sqrt(v) agrees to 1e-3.  Then both BF16 copies
+    of the decoder equal those of a network that is given the parameters."""
+    es, sur, torch = env
+    args = dict(nfreq=2, hidden=64, latent=24, max_batch=24)
+    n_rcv, nt, B, lr = 307, 8, 24, 1e-2
+    D, K6 = 4 * n_rcv * nt, 6 * 24
+    s, f = sur.Surrogate(n_rcv, nt, seed=3, **args), sur.Surrogate(n_rcv, nt, seed=4, **args)
+    try:
+        rng = np.random.default_rng(17)
+        cu = lambda a: torch.from_numpy(a.astype(np.float32)).cuda()
+        pos, mt = cu(rng.uniform(-1, 1, (B, 3))), cu(rng.standard_normal((B, 6)))
+        tgt = cu(rng.standard_normal((B, D)))
+        p = (rng.standard_normal(s.num_params()) * 0.2).astype(np.float32)
+        s.set_params(p)
+        wd = slice(len(p) - K6 * D, len(p))
+        m = v = 0.0
+        sure = True
+        for t in (1, 2):
+            before = s.get_params()[wd].astype(np.float64)
+            g = s.loss_grad(pos, mt, tgt)[2].cpu().numpy()[wd].astype(np.float64)
+            s.train_step(pos, mt, tgt, lr)
+            after = s.get_params()[wd].astype(np.float64)
+            m, v = 0.9 * m + 0.1 * g, 0.999 * v + 0.001 * g * g
+            want = -lr * (m / (1 - 0.9 ** t)) / (np.sqrt(v / (1 - 0.999 ** t)) + 1e-8)
+            sure = sure & (np.abs(g) > 0.1 * np.sqrt(np.mean(g * g)))
+            assert sure.mean() > 0.5
+            assert np.abs(after - before - want)[sure].max() <= 1e-3 * lr
+        f.set_params(s.get_params())
+        assert torch.equal(s.predict(pos, mt), f.predict(pos, mt))
+        a, b = (x.loss_grad(pos, mt, tgt)[2][:wd.start] for x in (s, f))  # through the row-major copy
+        assert float((a - b).norm()) <= 1e-5 * float(b.norm())
+    finally:
+        s.close()
+        f.close()
