@@ -28,7 +28,7 @@ struct es_sur {
     float scale_h[4] = {1.f, 1.f, 1.f, 1.f};  // host copy (GEMM alpha of the fused inference output)
     __nv_bfloat16 *X, *H1b, *H2b, *Zb, *dUb, *dAb, *dH2b, *dH1b;
     __nv_bfloat16 *ZT, *dUT;  // z^T [6K][B] and dU^T [D][B]: K-major operands of dWd = z^T dU
-    float *H1, *H2, *A, *U, *dZ, *dA, *dH2, *dH1, *loss, *acc;
+    float *H1, *H2, *U, *dZ, *dA, *dH2, *dH1, *loss, *acc;
     int t = 0;
     // inference copy of the decoder, K-major for the tcgen05 GEMM: WdT [D][6K],
     // rebuilt from the BF16 mirror whenever the parameters changed (ver)
@@ -88,13 +88,18 @@ int forward(es_sur* s, const float* pos, const float* mt, int B, float* out = nu
     const __nv_bfloat16* W2 = s->pb + s->oW2;
     const __nv_bfloat16* W3 = s->pb + s->oW3;
     CKS(sur_features(pos, B, s->cfg.nfreq, s->F, s->X, s->st));
-    CKS(gemm_bf16(B, s->H, s->F, s->X, s->F, false, W1, s->H, false, s->H1, s->H, 1.f, 0.f, 1, s->st));
-    CKS(sur_bias_act(s->H1, s->p + s->ob1, B, s->H, true, s->H1b, s->st));
-    CKS(gemm_bf16(B, s->H, s->H, s->H1b, s->H, false, W2, s->H, false, s->H2, s->H, 1.f, 0.f, 1, s->st));
-    CKS(sur_bias_act(s->H2, s->p + s->ob2, B, s->H, true, s->H2b, s->st));
-    CKS(gemm_bf16(B, s->K, s->H, s->H2b, s->H, false, W3, s->K, false, s->A, s->K, 1.f, 0.f, 1, s->st));
-    CKS(sur_bias_act(s->A, s->p + s->ob3, B, s->K, false, nullptr, s->st));
-    CKS(sur_outer(mt, s->A, B, s->K, s->Zb, s->st));
+    MlpEpilogue l1, l2, l3;
+    l1.bias = s->p + s->ob1;
+    l2.bias = s->p + s->ob2;
+    l1.relu = l2.relu = true;
+    l1.copy = s->H1b;
+    l2.copy = s->H2b;
+    l3.bias = s->p + s->ob3;
+    l3.m6 = mt;
+    l3.outer = s->Zb;
+    CKS(gemm_layer(B, s->H, s->F, s->X, s->F, false, W1, s->H, false, s->H1, l1, s->st));
+    CKS(gemm_layer(B, s->H, s->H, s->H1b, s->H, false, W2, s->H, false, s->H2, l2, s->st));
+    CKS(gemm_layer(B, s->K, s->H, s->H2b, s->H, false, W3, s->K, false, nullptr, l3, s->st));
     if (out) {
         // one product over all four components, each column block scaled by its component's RMS
         CKS(gemm_bf16_tc(B, (int)s->D, 6 * s->K, s->Zb, 6 * s->K, s->WdT, 6 * s->K, out, (int)s->D, 1.f, 0.f, 1, s->st,
@@ -124,17 +129,21 @@ int backward(es_sur* s, const float* mt, int B, bool decoder = true)
     CKS(sur_contract(mt, s->dZ, B, s->K, s->dA, s->dAb, s->st));
     // latent layer
     CKS(sur_colsum(s->dA, B, s->K, s->g + s->ob3, s->st));
-    CKS(gemm_bf16(s->H, s->K, B, s->H2b, s->H, true, s->dAb, s->K, false, s->g + s->oW3, s->K, 1.f, 0.f, 1, s->st));
-    CKS(gemm_bf16(B, s->H, s->K, s->dAb, s->K, false, W3, s->K, true, s->dH2, s->H, 1.f, 0.f, 1, s->st));
-    CKS(sur_relu_grad(s->dH2, s->H2, (size_t)B * s->H, s->dH2b, s->st));
+    const MlpEpilogue none;
+    CKS(gemm_layer(s->H, s->K, B, s->H2b, s->H, true, s->dAb, s->K, false, s->g + s->oW3, none, s->st));
+    MlpEpilogue d2, d1;
+    d2.mask = s->H2;
+    d2.copy = s->dH2b;
+    d1.mask = s->H1;
+    d1.copy = s->dH1b;
+    CKS(gemm_layer(B, s->H, s->K, s->dAb, s->K, false, W3, s->K, true, s->dH2, d2, s->st));
     // hidden 2
     CKS(sur_colsum(s->dH2, B, s->H, s->g + s->ob2, s->st));
-    CKS(gemm_bf16(s->H, s->H, B, s->H1b, s->H, true, s->dH2b, s->H, false, s->g + s->oW2, s->H, 1.f, 0.f, 1, s->st));
-    CKS(gemm_bf16(B, s->H, s->H, s->dH2b, s->H, false, W2, s->H, true, s->dH1, s->H, 1.f, 0.f, 1, s->st));
-    CKS(sur_relu_grad(s->dH1, s->H1, (size_t)B * s->H, s->dH1b, s->st));
+    CKS(gemm_layer(s->H, s->H, B, s->H1b, s->H, true, s->dH2b, s->H, false, s->g + s->oW2, none, s->st));
+    CKS(gemm_layer(B, s->H, s->H, s->dH2b, s->H, false, W2, s->H, true, s->dH1, d1, s->st));
     // hidden 1
     CKS(sur_colsum(s->dH1, B, s->H, s->g + s->ob1, s->st));
-    CKS(gemm_bf16(s->F, s->H, B, s->X, s->F, true, s->dH1b, s->H, false, s->g + s->oW1, s->H, 1.f, 0.f, 1, s->st));
+    CKS(gemm_layer(s->F, s->H, B, s->X, s->F, true, s->dH1b, s->H, false, s->g + s->oW1, none, s->st));
     return ES_OK;
 }
 
@@ -169,7 +178,7 @@ int es_sur_create(const es_sur_config* cfg, es_sur** out)
     s->oWd = seg((size_t)6 * s->K * s->D);
     s->P = o;
     const size_t B = s->B, P = s->P, H = s->H, K = s->K, D = s->D, F = s->F;
-    const size_t f32 = 4 * (4 * P + 4 + B * (2 * H + K + D + 6 * K + K + 2 * H + 8) + 128);
+    const size_t f32 = 4 * (4 * P + 4 + B * (2 * H + D + 6 * K + K + 2 * H + 8) + 128);
     const size_t b16 = 2 * (P + B * (F + 2 * H + 6 * K + D + K + 2 * H) + B * (6 * K + D)) + 2048;
     if (cudaMalloc(&s->pool, f32 + b16) != cudaSuccess) {
         delete s;
@@ -184,7 +193,6 @@ int es_sur_create(const es_sur_config* cfg, es_sur** out)
     s->scale = takef(4);
     s->H1 = takef(B * H);
     s->H2 = takef(B * H);
-    s->A = takef(B * K);
     s->U = takef(B * D);
     s->dZ = takef(B * 6 * K);
     s->dA = takef(B * K);

@@ -10,6 +10,20 @@ namespace es {
 cudaError_t gemm_bf16(int M, int N, int K, const __nv_bfloat16* A, int lda, bool a_t, const __nv_bfloat16* B,
                       int ldb, bool b_nk, float* C, int ldc, float alpha, float beta, int split_k, cudaStream_t st);
 
+// What a layer of the encoder does with its product x (row r, column c), in this order; null: not
+struct MlpEpilogue {
+    const float* bias = nullptr;      // x += bias[c]
+    bool relu = false;                // x = max(x, 0)
+    const float* mask = nullptr;      // x = 0 where mask[r][c] <= 0
+    __nv_bfloat16* copy = nullptr;    // BF16 copy [M][N]
+    const float* m6 = nullptr;        // with outer: outer[r][k N + c] = m6[r][k] x, k < 6 (BF16)
+    __nv_bfloat16* outer = nullptr;
+};
+// C[M][N] = op(A) op(B) through the epilogue (C may be null; N a multiple of 8), for products too
+// small to fill the device in 128 x 128 tiles; see layer_kernel in sur_gemm.cu
+cudaError_t gemm_layer(int M, int N, int K, const __nv_bfloat16* A, int lda, bool a_t, const __nv_bfloat16* B, int ldb,
+                       bool b_nk, float* C, const MlpEpilogue& ep, cudaStream_t st);
+
 // the K-major case (A [M][K], B [N][K]) on tcgen05 tensor cores; see sur_gemm_tc.cu.
 // alpha4 (host, 4 values) with span > 0: column n of C takes alpha4[n / span] instead of
 // alpha (4 span >= N), e.g. one scale per output component of the decoder
@@ -35,12 +49,6 @@ cudaError_t scale_f32(float* C, int M, int N, int ldc, float s, cudaStream_t st)
 cudaError_t cast_bf16(const float* x, __nv_bfloat16* y, size_t n, cudaStream_t st);
 // position features: [p, sin(2^j pi p), cos(2^j pi p)], j < nfreq, zero padded to width
 cudaError_t sur_features(const float* pos, int B, int nfreq, int width, __nv_bfloat16* X, cudaStream_t st);
-// Y = relu(Y + bias) (in place, FP32) and its BF16 copy; relu = false: bias only
-cudaError_t sur_bias_act(float* Y, const float* bias, int B, int N, bool relu, __nv_bfloat16* Yb, cudaStream_t st);
-// G = G * (H > 0) in place, with its BF16 copy
-cudaError_t sur_relu_grad(float* G, const float* H, size_t n, __nv_bfloat16* Gb, cudaStream_t st);
-// Z[b][c K + k] = M[b][c] A[b][k] (BF16)
-cudaError_t sur_outer(const float* M6, const float* A, int B, int K, __nv_bfloat16* Z, cudaStream_t st);
 // dA[b][k] = sum_c M[b][c] dZ[b][c K + k], FP32 and BF16
 cudaError_t sur_contract(const float* M6, const float* dZ, int B, int K, float* dA, __nv_bfloat16* dAb,
                          cudaStream_t st);

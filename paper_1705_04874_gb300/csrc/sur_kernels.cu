@@ -33,48 +33,21 @@ __global__ void cast_kernel(const float* x, __nv_bfloat16* y, size_t n)
         y[i] = __float2bfloat16(x[i]);
 }
 
+// one thread per sine and cosine pair of a position, and one for its three coordinates and the padding
 __global__ void features_kernel(const float* pos, int B, int nfreq, int width, __nv_bfloat16* X)
 {
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
+    const int per = 3 * nfreq + 1, i = blockIdx.x * blockDim.x + threadIdx.x;
+    const int b = i / per, q = i - b * per;
     if (b >= B) return;
     __nv_bfloat16* row = X + (size_t)b * width;
-    int k = 0;
-    for (int a = 0; a < 3; ++a) row[k++] = __float2bfloat16(pos[3 * b + a]);
-    for (int j = 0; j < nfreq; ++j)
-        for (int a = 0; a < 3; ++a) {
-            float s, c;
-            sincospif(ldexpf(pos[3 * b + a], j), &s, &c);  // sin, cos of 2^j pi p
-            row[k++] = __float2bfloat16(s);
-            row[k++] = __float2bfloat16(c);
-        }
-    for (; k < width; ++k) row[k] = __float2bfloat16(0.f);
-}
-
-__global__ void bias_act_kernel(float* Y, const float* bias, int B, int N, bool relu, __nv_bfloat16* Yb)
-{
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < (size_t)B * N; i += (size_t)gridDim.x * blockDim.x) {
-        float v = Y[i] + bias[i % N];
-        if (relu) v = fmaxf(v, 0.f);
-        Y[i] = v;
-        if (Yb) Yb[i] = __float2bfloat16(v);
-    }
-}
-
-__global__ void relu_grad_kernel(float* G, const float* H, size_t n, __nv_bfloat16* Gb)
-{
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-        const float g = H[i] > 0.f ? G[i] : 0.f;
-        G[i] = g;
-        Gb[i] = __float2bfloat16(g);
-    }
-}
-
-__global__ void outer_kernel(const float* M6, const float* A, int B, int K, __nv_bfloat16* Z)
-{
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < (size_t)B * 6 * K; i += (size_t)gridDim.x * blockDim.x) {
-        const size_t b = i / (6 * (size_t)K), r = i % (6 * (size_t)K);
-        const int c = (int)(r / K), k = (int)(r % K);
-        Z[i] = __float2bfloat16(M6[6 * b + c] * A[b * K + k]);
+    if (q < 3 * nfreq) {
+        float s, c;
+        sincospif(ldexpf(pos[3 * b + q % 3], q / 3), &s, &c);  // sin, cos of 2^j pi p
+        row[3 + 2 * q] = __float2bfloat16(s);
+        row[4 + 2 * q] = __float2bfloat16(c);
+    } else {
+        for (int a = 0; a < 3; ++a) row[a] = __float2bfloat16(pos[3 * b + a]);
+        for (int k = 3 + 6 * nfreq; k < width; ++k) row[k] = __float2bfloat16(0.f);
     }
 }
 
@@ -180,12 +153,19 @@ __global__ void combine_kernel(const float* G, long long D, const int* loc, cons
                                  m5 * g[5 * D + d];
 }
 
+// 32 columns per block; warp w sums rows w, w + 8, ... in order, then the warps' sums are added in order
 __global__ void colsum_kernel(const float* G, int B, int N, float* db)
 {
-    const int n = blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= N) return;
+    __shared__ float part[8][32];
+    const int n = blockIdx.x * 32 + threadIdx.x % 32, w = threadIdx.x / 32;
     float s = 0.f;
-    for (int b = 0; b < B; ++b) s += G[(size_t)b * N + n];
+    if (n < N)
+#pragma unroll 8
+        for (int b = w; b < B; b += 8) s += G[(size_t)b * N + n];
+    part[w][threadIdx.x % 32] = s;
+    __syncthreads();
+    if (w > 0 || n >= N) return;
+    for (int i = 1; i < 8; ++i) s += part[i][threadIdx.x];
     db[n] = s;
 }
 
@@ -264,25 +244,7 @@ cudaError_t cast_bf16(const float* x, __nv_bfloat16* y, size_t n, cudaStream_t s
 cudaError_t sur_features(const float* pos, int B, int nfreq, int width, __nv_bfloat16* X, cudaStream_t st)
 {
     if (3 + 6 * nfreq > width) return cudaErrorInvalidValue;
-    features_kernel<<<(B + 127) / 128, 128, 0, st>>>(pos, B, nfreq, width, X);
-    return cudaGetLastError();
-}
-
-cudaError_t sur_bias_act(float* Y, const float* bias, int B, int N, bool relu, __nv_bfloat16* Yb, cudaStream_t st)
-{
-    bias_act_kernel<<<blocks_for((size_t)B * N), 256, 0, st>>>(Y, bias, B, N, relu, Yb);
-    return cudaGetLastError();
-}
-
-cudaError_t sur_relu_grad(float* G, const float* H, size_t n, __nv_bfloat16* Gb, cudaStream_t st)
-{
-    relu_grad_kernel<<<blocks_for(n), 256, 0, st>>>(G, H, n, Gb);
-    return cudaGetLastError();
-}
-
-cudaError_t sur_outer(const float* M6, const float* A, int B, int K, __nv_bfloat16* Z, cudaStream_t st)
-{
-    outer_kernel<<<blocks_for((size_t)B * 6 * K), 256, 0, st>>>(M6, A, B, K, Z);
+    features_kernel<<<(B * (3 * nfreq + 1) + 127) / 128, 128, 0, st>>>(pos, B, nfreq, width, X);
     return cudaGetLastError();
 }
 
@@ -327,7 +289,7 @@ cudaError_t sur_combine(const float* G, long long D, const int* loc, const float
 
 cudaError_t sur_colsum(const float* G, int B, int N, float* db, cudaStream_t st)
 {
-    colsum_kernel<<<(N + 255) / 256, 256, 0, st>>>(G, B, N, db);
+    colsum_kernel<<<(N + 31) / 32, 256, 0, st>>>(G, B, N, db);
     return cudaGetLastError();
 }
 

@@ -364,3 +364,50 @@ def test_decoder_step_inside_its_gradient_gemm(env):
     finally:
         s.close()
         f.close()
+
+
+@pytest.mark.parametrize("hidden, latent, B, nfreq", [(8, 8, 8, 0), (64, 64, 32, 9), (328, 40, 40, 3), (392, 136, 72, 16)])
+def test_encoder_layers_at_ragged_sizes(env, hidden, latent, B, nfreq):
+    """The 32 x 64 x 64 tiles of the layer kernel: less than one of each, exact ones, remainders of 8
+    in every direction and more k-slabs than the ring holds, against the oracle's formulas in FP64
+    with every operand rounded to BF16 where the GPU rounds it.  What is left are FP32 sums, about
+    1e-6 off, and the BF16 roundings they flip: one in some 2^8 1e-5 of the values by 2^-8, 2e-4 of
+    a norm per rounding, five of them on the way to the first layer, doubled."""
+    es, sur, torch = env
+    from oracle import surrogate as osur
+    cfg = dict(nfreq=nfreq, hidden=hidden, latent=latent, n_rcv=4, nt=16)
+    s = sur.Surrogate(4, 16, nfreq=nfreq, hidden=hidden, latent=latent, max_batch=B, seed=3)
+    try:
+        rng = np.random.default_rng(hidden)
+        lay, P, F, D = osur.layout(**cfg)
+        params = (rng.standard_normal(P) / np.sqrt(hidden)).astype(np.float32)
+        s.set_params(params)
+        scale = [1.5, 0.7, 0.9, 1.1]
+        s.set_output_scale(scale)
+        pos = rng.uniform(-1, 1, (B, 3)).astype(np.float32)
+        mt = rng.standard_normal((B, 6)).astype(np.float32)
+        tgt = rng.standard_normal((B, D)).astype(np.float32)
+        cu = lambda a: torch.from_numpy(a).cuda()
+        got = s.loss_grad(cu(pos), cu(mt), cu(tgt))[2].cpu().numpy().astype(np.float64)
+        bf = lambda a: torch.from_numpy(np.asarray(a, np.float64)).float().to(torch.bfloat16).double().numpy()
+        w = osur.unpack(params, lay)
+        W1, W2, W3, Wd = (bf(w[k]) for k in ("W1", "W2", "W3", "Wd"))
+        X = bf(osur.features(pos, nfreq, F))
+        H1 = np.maximum(X @ W1 + w["b1"], 0)
+        H2 = np.maximum(bf(H1) @ W2 + w["b2"], 0)
+        A = bf(H2) @ W3 + w["b3"]
+        m6 = mt.astype(np.float64)
+        Z = bf((m6[:, :, None] * A[:, None, :]).reshape(B, -1))
+        sc = np.repeat(scale, D // 4)
+        den = np.sum((tgt / sc) ** 2, axis=1, keepdims=True)
+        dU = bf(2 * (Z @ Wd - tgt / sc) / (B * den))
+        dA = np.einsum("bc,bck->bk", m6, (dU @ Wd.T).reshape(B, 6, latent))
+        dH2 = (bf(dA) @ W3.T) * (H2 > 0)
+        dH1 = (bf(dH2) @ W2.T) * (H1 > 0)
+        want = dict(Wd=Z.T @ dU, b3=dA.sum(0), W3=bf(H2).T @ bf(dA), b2=dH2.sum(0), W2=bf(H1).T @ bf(dH2),
+                    b1=dH1.sum(0), W1=X.T @ bf(dH1))
+        for name, (o, shp) in lay.items():
+            a, b = got[o:o + int(np.prod(shp))], want[name].ravel()
+            assert np.linalg.norm(a - b) <= 2e-3 * np.linalg.norm(b), name
+    finally:
+        s.close()
