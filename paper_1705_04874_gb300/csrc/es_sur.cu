@@ -110,7 +110,7 @@ int forward(es_sur* s, const float* pos, const float* mt, int B, float* out = nu
     return ES_OK;
 }
 
-// gradients into s->g, given s->dUb from the loss; the decoder's only with `decoder` (a training
+// gradients into s->g, given s->dUb and s->dUT from the loss; the decoder's only with `decoder` (a training
 // step takes it in the GEMM that updates the decoder)
 int backward(es_sur* s, const float* mt, int B, bool decoder = true)
 {
@@ -121,7 +121,6 @@ int backward(es_sur* s, const float* mt, int B, bool decoder = true)
     // decoder: dWd = z^T dU through the K-major transposes (both on tcgen05), dz = dU Wd^T
     // (long K = D: split-K)
     CKS(transpose_bf16(s->Zb, B, K6, s->ZT, s->st));
-    CKS(transpose_bf16(s->dUb, B, D, s->dUT, s->st));
     if (decoder)
         CKS(gemm_bf16(K6, D, B, s->ZT, B, false, s->dUT, B, true, s->g + s->oWd, D, 1.f, 0.f, 1, s->st));
     const int split = (int)std::max<long long>(1, std::min<long long>(256, s->D / 2048));
@@ -311,7 +310,7 @@ int es_sur_loss_grad(es_sur* s, const float* pos, const float* mt, const float* 
         return ES_ERR_ARG;
     cudaGetLastError();
     if ((rc = forward(s, pos, mt, B)) != ES_OK) return rc;
-    CKS(sur_loss(s->U, target, s->scale, B, s->D / 4, 1e-30f, grads ? s->dUb : nullptr, s->loss, s->acc, per_sample,
+    CKS(sur_loss(s->U, target, s->scale, B, s->D / 4, 1e-30f, grads ? s->dUb : nullptr, s->dUT, s->loss, s->acc, per_sample,
                  s->st));
     if (grads) {
         if ((rc = backward(s, mt, B)) != ES_OK) return rc;
@@ -329,7 +328,7 @@ int es_sur_train_step(es_sur* s, const float* pos, const float* mt, const float*
     if (!target || !dev_ptr(target) || !(lr > 0)) return ES_ERR_ARG;
     cudaGetLastError();
     if ((rc = forward(s, pos, mt, B)) != ES_OK) return rc;
-    CKS(sur_loss(s->U, target, s->scale, B, s->D / 4, 1e-30f, s->dUb, s->loss, s->acc, nullptr, s->st));
+    CKS(sur_loss(s->U, target, s->scale, B, s->D / 4, 1e-30f, s->dUb, s->dUT, s->loss, s->acc, nullptr, s->st));
     if ((rc = backward(s, mt, B, false)) != ES_OK) return rc;
     s->t += 1;
     // the decoder (the last segment) in the GEMM that forms its gradient, both BF16 copies with it;

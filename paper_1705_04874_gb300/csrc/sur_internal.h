@@ -55,10 +55,10 @@ cudaError_t sur_contract(const float* M6, const float* dZ, int B, int K, float* 
 // outputs [B][4][Dc], y = scale[c] u, tau = t / scale[c]: per sample
 // l_b = sum_c |u_c - tau_c|^2 / (sum_c |tau_c|^2 + eps) (squared relative L2 of
 // the component-scaled seismogram), loss = mean_b l_b (device float),
-// per_sample (optional, device [B]) = l_b, dU = dloss/du in BF16 (skipped when
-// null); acc: device scratch of 8 B floats, 8-byte aligned
+// per_sample (optional, device [B]) = l_b, dU = dloss/du in BF16 and dUT its
+// transpose (skipped when null); Dc and B multiples of 8; acc: device scratch of 8 B floats, 8-byte aligned
 cudaError_t sur_loss(const float* U, const float* T, const float* scale, int B, long long Dc, float eps,
-                     __nv_bfloat16* dU, float* loss, float* acc, float* per_sample, cudaStream_t st);
+                     __nv_bfloat16* dU, __nv_bfloat16* dUT, float* loss, float* acc, float* per_sample, cudaStream_t st);
 cudaError_t sur_init_normal(float* p, size_t n, float std, unsigned long long seed, cudaStream_t st);
 // ss[c] = sum of squares of component c over n samples [n][4][Dc]
 cudaError_t sur_comp_sumsq(const float* T, int n, long long Dc, float* ss, cudaStream_t st);

@@ -67,8 +67,7 @@ __global__ void contract_kernel(const float* M6, const float* dZ, int B, int K, 
 // error (squared) of the whole 4C seismogram after each component is divided
 // by its scale.  Pass 1 (one block per sample and component) forms the two sums
 // of each, in a fixed order, so that two calls see the same dL/du to the last
-// bit of its BF16 rounding; pass 2 adds the components and writes l_b, the mean
-// loss and dL/du.
+// bit of its BF16 rounding.
 __global__ void loss_sums_kernel(const float* U, const float* T, const float* scale, long long Dc, float2* acc)
 {
     const int b = blockIdx.x, c = blockIdx.y;
@@ -98,22 +97,59 @@ __global__ void loss_sums_kernel(const float* U, const float* T, const float* sc
     }
 }
 
-__global__ void loss_grad_kernel(const float* U, const float* T, const float* scale, int B, long long Dc, float eps,
-                                 const float2* acc, __nv_bfloat16* dU, float* loss, float* per_sample)
+// Pass 2 on tiles of 64 samples x 64 columns: dL/du in BF16 both row-major and
+// transposed (the K-major operand of the decoder's gradient), the second through a
+// shared [column][sample] tile; the first column tile also writes the losses.
+// What bounds it is HBM.  256 x 262144 (one GB300): 120 us, 164 with two-byte
+// stores and 136 more for a transpose kernel that read them back.
+constexpr int LT = 64, LT_LD = LT + 2;
+__global__ void __launch_bounds__(256) loss_grad_kernel(const float* U, const float* T, const float* scale, int B,
+                                                        long long Dc, float eps, const float2* acc, __nv_bfloat16* dU,
+                                                        __nv_bfloat16* dUT, float* loss, float* per_sample, bool vec)
 {
-    const int b = blockIdx.x, c = blockIdx.y;
-    const float2 a0 = acc[4 * b], a1 = acc[4 * b + 1], a2 = acc[4 * b + 2], a3 = acc[4 * b + 3];
-    const float den = a0.y + a1.y + a2.y + a3.y + eps;
-    if (c == 0 && threadIdx.x == 0) {
-        const float lb = (a0.x + a1.x + a2.x + a3.x) / den;
-        if (per_sample) per_sample[b] = lb;
-        atomicAdd(loss, lb / B);
+    __shared__ __align__(16) __nv_bfloat16 tt[LT][LT_LD];
+    __shared__ float g[LT];
+    const long long D = 4 * Dc, d0 = (long long)blockIdx.x * LT;
+    const int b0 = blockIdx.y * LT;
+    if (threadIdx.x < LT && b0 + (int)threadIdx.x < B) {
+        const int b = b0 + threadIdx.x;
+        const float2 a0 = acc[4 * b], a1 = acc[4 * b + 1], a2 = acc[4 * b + 2], a3 = acc[4 * b + 3];
+        const float den = a0.y + a1.y + a2.y + a3.y + eps;
+        g[threadIdx.x] = 2.f / ((float)B * den);
+        if (blockIdx.x == 0) {
+            const float lb = (a0.x + a1.x + a2.x + a3.x) / den;
+            if (per_sample) per_sample[b] = lb;
+            atomicAdd(loss, lb / B);
+        }
     }
     if (!dU) return;
-    const size_t base = ((size_t)b * 4 + c) * Dc;
-    const float inv = 1.f / scale[c];
-    const float g = 2.f / ((float)B * den);
-    for (long long i = threadIdx.x; i < Dc; i += blockDim.x) dU[base + i] = __float2bfloat16(g * (U[base + i] - T[base + i] * inv));
+    __syncthreads();
+    const int q = threadIdx.x & 15, r = threadIdx.x >> 4;  // 16 column quads x 16 samples per sweep
+    const long long d = d0 + 4 * q;
+    if (d < D) {  // Dc is a multiple of 8: a quad lies within one component
+        const float inv = 1.f / scale[d / Dc];
+#pragma unroll
+        for (int i = r; i < LT; i += 16) {
+            if (b0 + i >= B) break;
+            const size_t at = (size_t)(b0 + i) * D + d;
+            const float4 u = *reinterpret_cast<const float4*>(U + at);
+            const float4 t = vec ? *reinterpret_cast<const float4*>(T + at)
+                                 : make_float4(T[at], T[at + 1], T[at + 2], T[at + 3]);
+            const float4 v = make_float4(g[i] * (u.x - t.x * inv), g[i] * (u.y - t.y * inv), g[i] * (u.z - t.z * inv),
+                                         g[i] * (u.w - t.w * inv));
+            const uint2 w = pack_bf16x4(v);
+            *reinterpret_cast<uint2*>(dU + at) = w;
+            const __nv_bfloat16* e = reinterpret_cast<const __nv_bfloat16*>(&w);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) tt[4 * q + k][i] = e[k];
+        }
+    }
+    __syncthreads();
+    for (int j = r; j < LT; j += 16) {  // four samples of column d0 + j (B is a multiple of 8)
+        if (d0 + j >= D || b0 + 4 * q >= B) continue;
+        const uint32_t* w = reinterpret_cast<const uint32_t*>(&tt[j][4 * q]);
+        *reinterpret_cast<uint2*>(dUT + (size_t)(d0 + j) * B + b0 + 4 * q) = make_uint2(w[0], w[1]);
+    }
 }
 
 // x ~ N(0, std^2) from a counter-based hash (splitmix64 of seed + index) and Box-Muller
@@ -255,13 +291,16 @@ cudaError_t sur_contract(const float* M6, const float* dZ, int B, int K, float* 
 }
 
 cudaError_t sur_loss(const float* U, const float* T, const float* scale, int B, long long Dc, float eps,
-                     __nv_bfloat16* dU, float* loss, float* acc, float* per_sample, cudaStream_t st)
+                     __nv_bfloat16* dU, __nv_bfloat16* dUT, float* loss, float* acc, float* per_sample, cudaStream_t st)
 {
     cudaError_t e = cudaMemsetAsync(loss, 0, sizeof(float), st);
     if (e != cudaSuccess) return e;
     float2* sums = reinterpret_cast<float2*>(acc);
     loss_sums_kernel<<<dim3(B, 4), 256, 0, st>>>(U, T, scale, Dc, sums);
-    loss_grad_kernel<<<dim3(B, 4), 256, 0, st>>>(U, T, scale, B, Dc, eps, sums, dU, loss, per_sample);
+    const long long nx = dU ? (4 * Dc + LT - 1) / LT : 1;
+    if (nx > 0x7fffffffLL) return cudaErrorInvalidValue;
+    loss_grad_kernel<<<dim3((unsigned)nx, (B + LT - 1) / LT), 256, 0, st>>>(
+        U, T, scale, B, Dc, eps, sums, dU, dUT, loss, per_sample, (reinterpret_cast<uintptr_t>(T) & 15) == 0);
     return cudaGetLastError();
 }
 

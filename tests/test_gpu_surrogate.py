@@ -411,3 +411,21 @@ def test_encoder_layers_at_ragged_sizes(env, hidden, latent, B, nfreq):
             assert np.linalg.norm(a - b) <= 2e-3 * np.linalg.norm(b), name
     finally:
         s.close()
+
+
+@pytest.mark.parametrize("B", [8, 64, 72])
+def test_target_on_any_word_boundary(env, B):
+    """A target off the 16-byte boundary gives the same loss and gradients to the last bit (D = 288 is
+    a multiple of neither tile side; one split, so every sum has a fixed order)."""
+    es, sur, torch = env
+    s = sur.Surrogate(3, 24, nfreq=1, hidden=16, latent=8, max_batch=B, seed=3)
+    try:
+        g = torch.Generator().manual_seed(B)
+        r = lambda *n: torch.randn(*n, generator=g).cuda()
+        pos, mt, tgt = r(B, 3).clamp(-1, 1), r(B, 6), r(B, 4 * 3 * 24)
+        shifted = torch.empty(tgt.numel() + 1, device="cuda")[1:].view_as(tgt).copy_(tgt)
+        a, b = s.loss_grad(pos, mt, tgt), s.loss_grad(pos, mt, shifted)
+        assert abs(a[0] - b[0]) <= 1e-6 * abs(a[0])  # the mean over samples is added in any order
+        assert torch.equal(a[1], b[1]) and torch.equal(a[2], b[2])
+    finally:
+        s.close()
