@@ -3,7 +3,7 @@
 //   C[M][N] = alpha * A[M][K] * B[N][K]^T + beta * C
 // A row-major [M][K] (lda), B row-major [N][K] (ldb), C FP32 row-major (ldc).
 //
-// Persistent: one CTA per SM walks the 128 x 256 output tiles (x split_k
+// Persistent: one CTA per SM (or a pair of them, see below) walks the 128 x 256 output tiles (x split_k
 // slices of K) with stride gridDim.x, 6 warps:
 //   warp 0, one thread: TMA producer -- 64-wide K slabs of A (128 rows) and
 //       B (256 rows) into a 4-stage ring of 128-byte-swizzled shared tiles,
@@ -21,6 +21,17 @@
 //       segments, and writes alpha * acc + beta * C (split_k > 1: atomically
 //       adds alpha * acc onto a C that already holds beta * C), then returns
 //       the accumulator; the next tile's MMAs run in the other one meanwhile.
+// With an even number of row tiles two CTAs (a cluster) work on two of them as one
+// 256 x 256 tile: each loads its 128 rows of A and half of B's rows, the first one's
+// issuer runs tcgen05.mma.cta_group::2 (M 256) over both, and each reads its own
+// 128 rows back.  Shared memory is what bounds a CTA on its own: it must take in
+// and give to the tensor core 384 rows per 64 of K, a CTA of a pair 256 (and the
+// ring is 6 stages deep in the same memory).  One GB300, N = 262144, K = 4608:
+// 256 rows 504 -> 443 us; 1024 rows, a serving batch with its encoder 1.78 -> 1.69
+// ms; 256 x 4608 with K = 262144 in 128 slices 560 -> 477 us.  (The pair sharing B by
+// TMA multicast alone, each CTA with its own MMAs: 506, 1.80 and 544.)  An odd
+// number of row tiles stays with single CTAs: an empty half would cost what the
+// pair gains at 8 tiles and more, far more below.
 // Rows, columns and K past the matrix edge are zero-filled by TMA and masked
 // in the epilogue.  Every mbarrier wait gives up after WAIT_NS of global
 // time, records the role that gave up in a device status word (read and
@@ -67,6 +78,12 @@ static_assert(TK == 64, "make_map boxes are 64 BF16 wide");
 constexpr uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(TN >> 3) << 17) |
                            ((uint32_t)(TM >> 4) << 24);
 
+// of a pair of CTAs: M is that of both
+constexpr uint32_t IDESC_PAIR = (IDESC & ~(0x1fu << 24)) | ((uint32_t)(2 * TM >> 4) << 24);
+// a CTA of a pair holds half of B's rows, so the ring is deeper
+template <int CL>
+__host__ __device__ constexpr int tc_stages() { return STAGES * STAGE_BYTES / (A_BYTES + B_BYTES / CL); }
+
 __device__ unsigned g_tc_status;  // bit 0 producer, 1 MMA, 2 epilogue, 3 MMA drain, 4 TMA drain, 5 probe gave up
 
 // The timeout path of the bounded waits, on demand: one thread waits, through
@@ -82,27 +99,33 @@ __global__ void wait_probe_kernel(unsigned long long limit_ns)
     }
 }
 
-__global__ void __launch_bounds__(THREADS, 1)
+template <int CL>
+__global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(THREADS, 1)
     gemm_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB, int M, int N,
                    int nkb, int kb_per, int mt, int ntl, int ntiles, float* __restrict__ C, int ldc, float alpha,
                    float beta, int atomic, float4 alpha4, int span)
 {
     extern __shared__ uint8_t dyn[];
-    __shared__ __align__(8) uint64_t full[STAGES], empty[STAGES], acc_full[2], acc_empty[2], mma_done;
+    constexpr int ST = tc_stages<CL>(), BYTES = A_BYTES + B_BYTES / CL;  // a stage of this CTA
+    __shared__ __align__(8) uint64_t full[ST], empty[ST], acc_full[2], acc_empty[2], mma_done;
     __shared__ uint32_t tmem_slot;
     __shared__ int s_issued, s_consumed;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t base = (smem_u32(dyn) + 1023u) & ~1023u;
+    // CTA r of a cluster takes row tile CL p + r of the cluster's tiles
+    const int r = CL > 1 ? (int)cluster_rank() : 0, first = blockIdx.x / CL, stride = gridDim.x / CL;
+    ntiles /= CL;
+    mt /= CL;
 
     if (threadIdx.x == 0) {
-        for (int s = 0; s < STAGES; ++s) {
+        for (int s = 0; s < ST; ++s) {
             mbar_init(&full[s], 1);
             mbar_init(&empty[s], 1);
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(&acc_full[b], 1);
-            mbar_init(&acc_empty[b], 4);  // one arrival per epilogue warp
+            mbar_init(&acc_empty[b], 4 * CL);  // one arrival per epilogue warp of the cluster
         }
         mbar_init(&mma_done, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -111,46 +134,65 @@ __global__ void __launch_bounds__(THREADS, 1)
     }
     __syncwarp();
     if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)),
-                     "r"(TMEM_COLS)
-                     : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+        if constexpr (CL == 1) {
+            asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)),
+                         "r"(TMEM_COLS)
+                         : "memory");
+            asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+        } else {
+            asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)),
+                         "r"(TMEM_COLS)
+                         : "memory");
+            asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+        }
     }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    if (CL > 1) cluster_sync();  // the barriers of every CTA are there
     const uint32_t tmem = tmem_slot;
+    auto commit = [](uint64_t* bar) {
+        if constexpr (CL == 1) tc_commit(bar);
+        else tc_commit_pair(bar);
+    };
 
     if (warp == 0) {
         if (lane == 0) {
             // producer: every k-block of every tile of this CTA, through the ring
             int it = 0;
             bool ok = true;
-            for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
-                const int mi = t % mt, rest = t / mt;
+            for (int t = first; t < ntiles && ok; t += stride) {
+                const int mi = t % mt * CL + r, rest = t / mt;
                 const int ni = rest % ntl, kb0 = (rest / ntl) * kb_per;
                 const int nk = min(nkb, kb0 + kb_per) - kb0;
                 for (int kb = 0; kb < nk; ++kb, ++it) {
-                    const int s = it % STAGES;
-                    if (!mbar_wait(&empty[s], ((it / STAGES) & 1) ^ 1)) {
+                    const int s = it % ST;
+                    if (!mbar_wait(&empty[s], ((it / ST) & 1) ^ 1)) {
                         atomicOr(&g_tc_status, 1u);
                         ok = false;
                         break;
                     }
-                    const uint32_t sa = base + s * STAGE_BYTES;
-                    mbar_expect_tx(&full[s], STAGE_BYTES);
-                    tma_load_2d(sa, &mapA, &full[s], (kb0 + kb) * TK, mi * TM);
-                    tma_load_2d(sa + A_BYTES, &mapB, &full[s], (kb0 + kb) * TK, ni * TN);
+                    const uint32_t sa = base + s * BYTES;
+                    if constexpr (CL == 1) {
+                        mbar_expect_tx(&full[s], BYTES);
+                        tma_load_2d(sa, &mapA, &full[s], (kb0 + kb) * TK, mi * TM);
+                        tma_load_2d(sa + A_BYTES, &mapB, &full[s], (kb0 + kb) * TK, ni * TN);
+                    } else {  // each CTA its rows of A and of B; the issuing CTA's barrier hears of both
+                        if (r == 0) mbar_expect_tx(&full[s], CL * BYTES);
+                        const uint32_t bar = cluster_addr(&full[s], 0);
+                        tma_load_2d_pair(sa, &mapA, bar, (kb0 + kb) * TK, mi * TM);
+                        tma_load_2d_pair(sa + A_BYTES, &mapB, bar, (kb0 + kb) * TK, ni * TN + r * (TN / CL));
+                    }
                 }
             }
             s_issued = it;
         }
     } else if (warp == 1) {
-        if (lane == 0) {
-            // MMA issuer: accumulator b = local tile index mod 2
+        if (lane == 0 && r == 0) {
+            // MMA issuer (of a cluster: its first CTA's): accumulator b = local tile index mod 2
             int it = 0, lt = 0;
             bool ok = true;
-            for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x, ++lt) {
+            for (int t = first; t < ntiles && ok; t += stride, ++lt) {
                 const int rest = t / mt;
                 const int kb0 = (rest / ntl) * kb_per;
                 const int nk = min(nkb, kb0 + kb_per) - kb0;
@@ -162,34 +204,35 @@ __global__ void __launch_bounds__(THREADS, 1)
                 tc_fence_after();
                 const uint32_t acc = tmem + (uint32_t)(b * TN);
                 for (int kb = 0; kb < nk; ++kb, ++it) {
-                    const int s = it % STAGES;
-                    if (!mbar_wait(&full[s], (it / STAGES) & 1)) {
+                    const int s = it % ST;
+                    if (!mbar_wait(&full[s], (it / ST) & 1)) {
                         atomicOr(&g_tc_status, 2u);
                         ok = false;
                         break;
                     }
                     tc_fence_after();
-                    const uint32_t sa = base + s * STAGE_BYTES;
+                    const uint32_t sa = base + s * BYTES;
                     const uint64_t da = sw128_desc(sa), db = sw128_desc(sa + A_BYTES);
 #pragma unroll
                     for (int k = 0; k < TK / UK; ++k) {
                         const uint64_t step = (uint64_t)((k * UK * 2) >> 4);  // 32 bytes along the swizzled row
-                        tc_mma(acc, da + step, db + step, IDESC, (kb | k) != 0);
+                        if constexpr (CL == 1) tc_mma(acc, da + step, db + step, IDESC, (kb | k) != 0);
+                        else tc_mma_pair(acc, da + step, db + step, IDESC_PAIR, (kb | k) != 0);
                     }
-                    tc_commit(&empty[s]);
+                    commit(&empty[s]);
                 }
-                if (ok) tc_commit(&acc_full[b]);
+                if (ok) commit(&acc_full[b]);
             }
             s_consumed = it;
-            tc_commit(&mma_done);  // arrives when every MMA issued above has completed
+            commit(&mma_done);  // arrives when every MMA issued above has completed
         }
     } else {
         // epilogue warps 2..5: TMEM lane quarter q = warp mod 4
         const int q = warp & 3;
         const bool vec = (ldc & 3) == 0 && (reinterpret_cast<uintptr_t>(C) & 15) == 0;
         int lt = 0;
-        for (int t = blockIdx.x; t < ntiles; t += gridDim.x, ++lt) {
-            const int mi = t % mt, ni = (t / mt) % ntl;
+        for (int t = first; t < ntiles; t += stride, ++lt) {
+            const int mi = t % mt * CL + r, ni = (t / mt) % ntl;
             const int b = lt & 1;
             // one lane waits and the warp follows its result: tcgen05.ld below needs the whole warp
             int got = 0;
@@ -202,13 +245,13 @@ __global__ void __launch_bounds__(THREADS, 1)
             tc_fence_after();
             const int n0 = ni * TN, row0 = mi * TM + q * 32;
             // this warp's staging block: row r (TMEM lane) at stage + r * EPI_LD
-            float* stage = reinterpret_cast<float*>(dyn + (base - smem_u32(dyn)) + STAGES * STAGE_BYTES) +
+            float* stage = reinterpret_cast<float*>(dyn + (base - smem_u32(dyn)) + ST * BYTES) +
                            q * 32 * EPI_LD;
             for (int c0 = 0; c0 < TN; c0 += 32) {
                 if (n0 + c0 >= N) break;  // uniform over the warp
                 __syncwarp();               // the previous block's reads of the staging rows are done
-                uint32_t r[32];
-                tmem_ld32(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(b * TN + c0), r);
+                uint32_t acc[32];
+                tmem_ld32(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(b * TN + c0), acc);
                 float4* srow = reinterpret_cast<float4*>(stage + lane * EPI_LD);
                 if (span) {
                     // per-column alpha: columns [c span, (c + 1) span) of C take component c of alpha4
@@ -218,15 +261,15 @@ __global__ void __launch_bounds__(THREADS, 1)
                         const int col = n0 + c0 + j;
                         a[j] = (col < span ? alpha4.x : col < 2 * span ? alpha4.y : col < 3 * span ? alpha4.z
                                                                                                   : alpha4.w) *
-                               __uint_as_float(r[j]);
+                               __uint_as_float(acc[j]);
                     }
 #pragma unroll
                     for (int j = 0; j < 8; ++j) srow[j] = make_float4(a[4 * j], a[4 * j + 1], a[4 * j + 2], a[4 * j + 3]);
                 } else {
 #pragma unroll
                     for (int j = 0; j < 8; ++j)
-                        srow[j] = make_float4(alpha * __uint_as_float(r[4 * j]), alpha * __uint_as_float(r[4 * j + 1]),
-                                              alpha * __uint_as_float(r[4 * j + 2]), alpha * __uint_as_float(r[4 * j + 3]));
+                        srow[j] = make_float4(alpha * __uint_as_float(acc[4 * j]), alpha * __uint_as_float(acc[4 * j + 1]),
+                                              alpha * __uint_as_float(acc[4 * j + 2]), alpha * __uint_as_float(acc[4 * j + 3]));
                 }
                 __syncwarp();
                 // lane l stores columns 4 (l mod 8) .. +3 of row 4 i + l / 8: a warp instruction writes
@@ -266,7 +309,10 @@ __global__ void __launch_bounds__(THREADS, 1)
             // every tcgen05.ld of this warp has completed (tmem_ld32 waits): hand the accumulator back
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive(&acc_empty[b]);
+            if (lane == 0) {
+                if constexpr (CL == 1) mbar_arrive(&acc_empty[b]);
+                else mbar_arrive_cluster(cluster_addr(&acc_empty[b], 0));
+            }
         }
     }
 
@@ -276,16 +322,20 @@ __global__ void __launch_bounds__(THREADS, 1)
     if (threadIdx.x == 0) {
         if (!mbar_wait(&mma_done, 0)) atomicOr(&g_tc_status, 8u);
         // copies issued but never consumed (only after a wait gave up) must land before the CTA exits
-        for (int it = s_consumed; it < s_issued; ++it)
-            if (!mbar_wait(&full[it % STAGES], (it / STAGES) & 1)) {
+        for (int it = s_consumed; r == 0 && it < s_issued; ++it)
+            if (!mbar_wait(&full[it % ST], (it / ST) & 1)) {
                 atomicOr(&g_tc_status, 16u);
                 break;
             }
     }
     __syncthreads();
+    if (CL > 1) cluster_sync();  // no CTA leaves while another may write to it or to its barriers
     if (warp == 0) {
         tc_fence_after();
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS) : "memory");
+        if constexpr (CL == 1)
+            asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS) : "memory");
+        else
+            asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS) : "memory");
     }
 }
 
@@ -638,7 +688,8 @@ cudaError_t gemm_bf16_tc(int M, int N, int K, const __nv_bfloat16* A, int lda, c
     EncodeTiled fn = encode_tiled();
     if (!fn) return cudaErrorNotSupported;
     alignas(64) CUtensorMap mapA, mapB;
-    if (!make_map(fn, &mapA, A, M, K, lda, TM) || !make_map(fn, &mapB, B, N, K, ldb, TN))
+    const bool pair = (M + TM - 1) / TM % 2 == 0;
+    if (!make_map(fn, &mapA, A, M, K, lda, TM) || !make_map(fn, &mapB, B, N, K, ldb, pair ? TN / 2 : TN))
         return cudaErrorInvalidValue;
     const int nkb = (K + TK - 1) / TK;
     if (split_k < 1) split_k = 1;
@@ -652,16 +703,16 @@ cudaError_t gemm_bf16_tc(int M, int N, int K, const __nv_bfloat16* A, int lda, c
     cudaError_t e0 = cudaGetDevice(&dev);
     if (e0 == cudaSuccess) e0 = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e0 != cudaSuccess) return e0;
-    const long long grid = ntiles < sms ? ntiles : sms;
+    const long long grid = ntiles < sms ? ntiles : (pair ? sms / 2 * 2 : sms);
     if (split_k > 1 && beta != 1.f) {
         cudaError_t e = scale_f32(C, M, N, ldc, beta, st);
         if (e != cudaSuccess) return e;
     }
-    cudaError_t e = cudaFuncSetAttribute(gemm_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
+    const auto kernel = pair ? gemm_tc_kernel<2> : gemm_tc_kernel<1>;
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
     if (e != cudaSuccess) return e;
-    gemm_tc_kernel<<<(unsigned)grid, THREADS, SMEM_BYTES, st>>>(mapA, mapB, M, N, nkb, kb_per, mt, ntl, (int)ntiles,
-                                                               C, ldc, alpha, beta, split_k > 1 ? 1 : 0, av,
-                                                               alpha4 ? span : 0);
+    kernel<<<(unsigned)grid, THREADS, SMEM_BYTES, st>>>(mapA, mapB, M, N, nkb, kb_per, mt, ntl, (int)ntiles, C, ldc, alpha,
+                                                       beta, split_k > 1 ? 1 : 0, av, alpha4 ? span : 0);
     return cudaGetLastError();
 }
 
