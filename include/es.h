@@ -23,10 +23,10 @@
  * - Axis lengths run from 3 to 512; anything else is ES_ERR_SIZE.  The
  *   lengths 16, 32, 48, 64, 75, 80, 96, 125, 128, 160, 192 and 256 take the
  *   fused FFT passes (two-stage plans R1 x R2, three-stage ones for 75 and
- *   125); every other length from 16 on -- odd or non-smooth ones such as the
- *   301 of the paper's 125 x 75 x 301 grid (Sec. III) -- takes the same
- *   passes as a zero-padded convolution through a longer FFT, and the
- *   shortest axes a direct sum; both apply the same staggered spectral
+ *   125); every other length from 64 on (an odd nx from 96 on) -- odd or
+ *   non-smooth ones such as the 301 of the paper's 125 x 75 x 301 grid
+ *   (Sec. III) -- takes the same passes as a zero-padded convolution through
+ *   a longer FFT, and the shorter ones a direct sum; both apply the same staggered spectral
  *   derivative as an exact periodic convolution.
  */
 #ifndef ES_H
@@ -67,7 +67,7 @@ int es_model_create(const float* rho, const float* cp, const float* cs, int nx, 
  * derivative as a 10-point near stencil in FP32 plus the FFT of the rest of
  * the operator, which confines FP32 FFT roundoff to about 1 % of its plain
  * size), elsewhere the same derivative as a zero-padded convolution (direct
- * circulant sums below 16 cells).
+ * circulant sums below 64 cells, for an odd nx below 96).
  * ES_PREC_COMPENSATED: every axis through the circulant passes with
  * error-free transformations (each product split exactly by one FMA, Knuth's
  * TwoSum on the running sum, the kernel row as FP32 high plus low parts), so

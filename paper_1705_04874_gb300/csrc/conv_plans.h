@@ -6,8 +6,6 @@
 #pragma once
 
 #define ES_CONV_PLANS(X)                                                                            \
-    X(64, 8, 8, 1, 8, 16)                                                                           \
-    X(100, 10, 10, 1, 10, 16)                                                                       \
     X(160, 16, 10, 1, 10, 16)                                                                       \
     X(256, 16, 16, 1, 16, 16)                                                                       \
     X(320, 20, 16, 1, 20, 8)                                                                        \

@@ -4,9 +4,9 @@
 
 namespace es {
 
-int conv_length(int n)
+int conv_length(int n, int axis)
 {
-    if (n < CONV_MIN_N) return 0;
+    if (n < CONV_MIN_N || (axis == 0 && n % 2 && n < CONV_MIN_ODD_X)) return 0;
     // the plans in ascending order: the first with room for the zero padding
 #define ES_CASE(len, a, b, c, t, pr) if (2 * n <= len) return len;
     ES_CONV_PLANS(ES_CASE)

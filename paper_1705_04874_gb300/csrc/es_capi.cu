@@ -212,7 +212,7 @@ int ensure_prepared()
 }
 
 // Axis lengths: an FFT plan (pass_plans.h), else a convolution pass (conv_plans.h) or, below
-// CONV_MIN_N cells and in the compensated mode, the circulant pass, up to
+// CONV_MIN_N cells (an odd x axis: CONV_MIN_ODD_X) and in the compensated mode, the direct sum, up to
 // CIRC_MAX_N (circ_pass.cu).  With an odd nx the y and z FFT passes move their
 // pencil pairs as single floats (pass_strided1.cu).
 bool fft_plan(int n) { int a, b; return plan_radices(n, &a, &b) != 0; }
@@ -491,7 +491,7 @@ cudaError_t upload_axis_tables(es_model* m, int a)
     std::vector<float2> tw, hp, hm;
     std::vector<double> ckp, ckm;
     const bool circ = circ_axis(m, a);
-    axis_tables(n, m->d[a], circ ? conv_length(n) : 0, tw, hp, hm, m->gp[a], m->gm[a], circ ? &ckp : nullptr,
+    axis_tables(n, m->d[a], circ ? conv_length(n, a) : 0, tw, hp, hm, m->gp[a], m->gm[a], circ ? &ckp : nullptr,
                 circ ? &ckm : nullptr);
     cudaError_t e = cudaMemcpy(m->tw[a], tw.data(), tw.size() * 8, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(m->hp[a], hp.data(), hp.size() * 8, cudaMemcpyHostToDevice);
@@ -639,7 +639,7 @@ PassParams make_pass(const es_model* m, int axis, bool stress, float dt)
     p.scratch = m->prec == ES_PREC_FP32_TC ? m->ctc_scratch : nullptr;
     p.circ = circ_axis(m, axis) ? 1 : 0;
     p.comp = m->prec == ES_PREC_COMPENSATED ? 1 : 0;
-    p.m = !p.circ ? p.n : (p.comp ? 0 : conv_length(p.n));
+    p.m = !p.circ ? p.n : (p.comp ? 0 : conv_length(p.n, axis));
     p.pc = m->pc[axis];
     p.ps = m->ps[axis];
     p.L = m->L;
@@ -915,12 +915,12 @@ struct AxisTables {
     float gp[NEAR_TAPS], gm[NEAR_TAPS];
 };
 
-AxisTables pack_axis(int n, int nx, double d, std::vector<float>& h)
+AxisTables pack_axis(int axis, int n, int nx, double d, std::vector<float>& h)
 {
     AxisTables t;
     t.n = n;
     t.circ = !fft_axis(n, nx);
-    t.m = t.circ ? conv_length(n) : n;
+    t.m = t.circ ? conv_length(n, axis) : n;
     std::vector<float2> tw, hp, hm;
     std::vector<double> ckp64, ckm64;
     axis_tables(n, d, t.circ ? t.m : 0, tw, hp, hm, t.gp, t.gm, t.circ ? &ckp64 : nullptr, t.circ ? &ckm64 : nullptr);
@@ -1088,7 +1088,7 @@ int es_model_create(const float* rho, const float* cp, const float* cs, int nx, 
     auto up = [&](size_t b) { return (b + A - 1) / A * A; };
     size_t bytes = up(n * 4) * NMAT;
     // an FFT's tables have the axis length, a convolution pass's the padded length
-    auto table_len = [&](int a) { return (size_t)std::max(axis_len(m, a), conv_length(axis_len(m, a))); };
+    auto table_len = [&](int a) { return (size_t)std::max(axis_len(m, a), conv_length(axis_len(m, a), a)); };
     for (int a = 0; a < 3; ++a) bytes += 3 * up(table_len(a) * 8) + 6 * up(axis_len(m, a) * 4);
     bytes += up(16) + up(NFIELD * sizeof(float*));
     cudaError_t e = dev_alloc(&m->pool, bytes);
@@ -1795,7 +1795,7 @@ int es_derivative(const float* f, int nx, int ny, int nz, int axis, double d, in
     if (rc != ES_OK) return rc;
     cudaStream_t st = (cudaStream_t)stream;
     std::vector<float> h;
-    const AxisTables t = pack_axis(axis == 0 ? nx : (axis == 1 ? ny : nz), nx, d, h);
+    const AxisTables t = pack_axis(axis, axis == 0 ? nx : (axis == 1 ? ny : nz), nx, d, h);
     float* tab = nullptr;
     CK(dev_alloc(&tab, h.size() * sizeof(float)));
     cudaError_t e = cudaMemcpyAsync(tab, h.data(), h.size() * sizeof(float), cudaMemcpyHostToDevice, st);
@@ -1827,8 +1827,10 @@ int es_laplacian(const float* f, int nx, int ny, int nz, double dx, double dy, d
     AxisTables t[3];
     for (int a = 0; a < 3; ++a) {
         int same = 0;
-        while (same < a && !(len[same] == len[a] && d[same] == d[a])) ++same;
-        t[a] = same < a ? t[same] : pack_axis(len[a], nx, d[a], h);
+        while (same < a && !(len[same] == len[a] && d[same] == d[a] &&
+                             conv_length(len[same], same) == conv_length(len[a], a)))
+            ++same;
+        t[a] = same < a ? t[same] : pack_axis(a, len[a], nx, d[a], h);
     }
     float* tmp = nullptr;
     CK(dev_alloc(&tmp, (2 * n_al + h.size()) * sizeof(float)));

@@ -162,11 +162,15 @@ cudaError_t launch_strided1(int ra, int rb, int rc, int ntiles, const PassParams
 cudaError_t prepare_strided2();
 cudaError_t prepare_strided1();
 // Axis lengths without a plan, FP32 mode: zero-padded convolution passes (conv_pass.cuh) with
-// transforms of conv_length(n) points (0: none, the circulant pass), from CONV_MIN_N cells on:
-// below, the near stencil's window would wrap round the axis more than once, and 17 cells
-// already take the same time either way (2.5 against 2.5-2.7 ms per 17 M cells along z).
-constexpr int CONV_MIN_N = 16;
-int conv_length(int n);
+// transforms of conv_length(n, axis) points (0: none, the direct sum), from CONV_MIN_N cells on.  ms
+// per 17 M cells, a step's two x passes + its four y and z passes, direct and as a convolution: 33
+// cells 1.02 + 3.21 and 1.15 + 4.07, 45 0.95 + 2.19 and 1.04 + 2.48, 63 0.90 + 1.61 and 1.25 + 1.72,
+// 66 1.04 + 2.65 and 0.86 + 2.27, 72 1.02 + 2.37 and 0.81 + 1.91, 104 1.07 + 2.47 and 0.76 + 1.59
+// (24, 28 and 50 cells, just below a transform length, also gained, up to 14 %; the others lost).  An
+// odd x axis, whose tiles start off 16-byte boundaries: 81 cells 1.03 and 1.06, 127 1.09 and 0.97,
+// so from CONV_MIN_ODD_X on.
+constexpr int CONV_MIN_N = 64, CONV_MIN_ODD_X = 96;
+int conv_length(int n, int axis);
 cudaError_t launch_conv(const PassParams& p, cudaStream_t st);
 cudaError_t launch_conv_strided1(const PassParams& p, cudaStream_t st);  // nx odd
 cudaError_t launch_conv_strided2(const PassParams& p, cudaStream_t st);  // nx even

@@ -3,8 +3,8 @@
 //   C[M][N] = alpha * A[M][K] * B[N][K]^T + beta * C
 // A row-major [M][K] (lda), B row-major [N][K] (ldb), C FP32 row-major (ldc).
 //
-// Persistent: one CTA per SM (or a pair of them, see below) walks the 128 x 256 output tiles (x split_k
-// slices of K) with stride gridDim.x, 6 warps:
+// Persistent: one CTA per SM (or pairs of them, below) walks the 128 x 256 output
+// tiles (x split_k slices of K) with stride gridDim.x, 6 warps:
 //   warp 0, one thread: TMA producer -- 64-wide K slabs of A (128 rows) and
 //       B (256 rows) into a 4-stage ring of 128-byte-swizzled shared tiles,
 //       completion tracked by transaction-count mbarriers; it runs ahead
@@ -30,8 +30,8 @@
 // 256 rows 504 -> 443 us; 1024 rows, a serving batch with its encoder 1.78 -> 1.69
 // ms; 256 x 4608 with K = 262144 in 128 slices 560 -> 477 us.  (The pair sharing B by
 // TMA multicast alone, each CTA with its own MMAs: 506, 1.80 and 544.)  An odd
-// number of row tiles stays with single CTAs: an empty half would cost what the
-// pair gains at 8 tiles and more, far more below.
+// number of row tiles stays with single CTAs: a pair's empty half is work for
+// nothing, half of it all at a single row tile.
 // Rows, columns and K past the matrix edge are zero-filled by TMA and masked
 // in the epilogue.  Every mbarrier wait gives up after WAIT_NS of global
 // time, records the role that gave up in a device status word (read and

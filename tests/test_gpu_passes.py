@@ -72,10 +72,11 @@ def test_convolution_lengths(es, orc, n, axis, others):
         assert rel_l2(out.cpu().numpy(), ref) < 5e-7
 
 
-def test_run_on_convolution_axes(es, orc):
-    """A batch on three axes without a plan (33 x 30 x 27: odd nx) and PML, the
+@pytest.mark.parametrize("shape", [(27, 30, 33), (66, 65, 97), (70, 27, 95)])
+def test_run_on_convolution_axes(es, orc, shape):
+    """A batch on three axes without a plan (odd nx; convolutions, direct sums and both) and PML, the
     first simulation against the oracle, the second against a run of its own."""
-    shape, pml, nt = (27, 30, 33), 4, 100
+    pml, nt = 4, 100
     rho, cp, cs = synth.two_layer_model(shape=shape, water_cells=6)
     dt = cfl_dt(cp, 10.0)
     w = synth.ricker(nt, dt, 25.0)
