@@ -559,7 +559,7 @@ def measure_train(args):
 def measure_paper(args):
     """The paper's own workload shape: 125 x 75 x 301 cells (12.5 / 12.5 / 10 m), PML 10, a double
     couple in the reservoir box, Ricker 30 Hz, 2000 steps (--nt overrides), 105 x 55 seabed receivers
-    (every interior x-y point).  No axis length has an FFT plan, so every pass is a circulant pass.
+    (every interior x-y point).  x and y have FFT plans, z runs as a zero-padded FFT convolution.
     Device time of whole es_run calls, --steps timed after --warmup."""
     import torch
     from paper_1705_04874_gb300 import es
@@ -605,7 +605,7 @@ def measure_paper(args):
                       "data": "synthetic",
                       "config": {"workload": "the paper's grid 125x75x301, 12.5/12.5/10 m, PML 10, "
                                              f"{nt} steps, 105x55 seabed receivers; x (125 = 5x5x5) and y (75 = 5x15) "
-                                             "through the FFT passes, z (301 = 7x43) through the circulant "
+                                             "through the FFT passes, z (301 = 7x43) through the convolution "
                                              "passes"},
                       "paths": out}))
     return 0
@@ -672,7 +672,7 @@ def measure_configs(args):
                "Mcell_steps_per_s": round(float(n) * nt / (ms * 1e-3) / 1e6, 1)}
         if kind == "paper":
             # the paper's per-source times on this grid (2000 samples): K20 ~1313 s, C2075 ~2091 s
-            rec["passes"] = "x 125 (5x5x5) and y 75 (5x15) FFT, z 301 = 7 x 43 circulant"
+            rec["passes"] = "x 125 (5x5x5) and y 75 (5x15) FFT, z 301 = 7 x 43 as a convolution"
             rec["s_per_source"] = round(ms * 1e-3, 3)
             rec["vs_paper_k20_s_per_source"] = round(1313.0 / (ms * 1e-3), 1)
         if name == "C1":

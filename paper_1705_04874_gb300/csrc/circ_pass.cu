@@ -1,6 +1,7 @@
 // Staggered spectral derivative passes as direct circulant sums: the axes too
-// short for the convolution passes (conv_pass.cuh, n < CONV_MIN_N), and every
-// axis in the compensated mode.  Along a periodic axis the operator
+// short for the convolution passes (conv_pass.cuh; n < CONV_MIN_N, an odd x axis
+// n < CONV_MIN_ODD_X), and every axis in the compensated mode.  Along a periodic
+// axis the operator
 //   D(+/-) f = IFFT( i kappa exp(+/- i kappa d / 2) FFT(f) )
 // is a real circulant matrix: (D f)_i = sum_j c[(i - j) mod n] f_j with
 // c_l = sum_m H_m exp(2 pi i m l / n), computed once on the host in FP64
