@@ -712,11 +712,15 @@ __host__ __device__ constexpr size_t pass_smem_x()
     return N % 16 == 0 ? pass_smem_strided<N, T>() : 2 * sizeof(float2) * N * PAIRS + 2 * sizeof(float2) * N;
 }
 
-// tensor memory as a per-thread store: K consecutive columns of the thread's lane
+// Tensor memory as a per-thread store: K consecutive columns of the thread's lane.
+// The instructions are .aligned, all 32 lanes at once, while the loops around them
+// branch by lane (a ragged tile's missing lines, PML rows): each helper brings the
+// warp together first.
 template <int K>
 __device__ __forceinline__ void tmem_st(uint32_t addr, const float* v)
 {
     static_assert(K == 4 || K == 8, "");
+    __syncwarp();
     if constexpr (K == 8)
         asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"r"(addr),
                      "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7])
@@ -726,11 +730,16 @@ __device__ __forceinline__ void tmem_st(uint32_t addr, const float* v)
                      "f"(v[2]), "f"(v[3])
                      : "memory");
 }
-__device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+__device__ __forceinline__ void tmem_st_wait()
+{
+    __syncwarp();
+    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+}
 template <int K>
 __device__ __forceinline__ void tmem_ld(uint32_t addr, float* v)
 {
     static_assert(K == 4 || K == 8, "");
+    __syncwarp();
     if constexpr (K == 8)
         asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];\n"
                      "tcgen05.wait::ld.sync.aligned;"
@@ -747,6 +756,7 @@ __device__ __forceinline__ void tmem_ld(uint32_t addr, float* v)
 // give them back without waiting for this one) and publishes the address
 __device__ __forceinline__ void tmem_alloc(uint32_t* slot, unsigned columns)
 {
+    __syncwarp();
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                      (uint32_t)__cvta_generic_to_shared(slot)),
                  "r"(columns)
@@ -755,6 +765,7 @@ __device__ __forceinline__ void tmem_alloc(uint32_t* slot, unsigned columns)
 }
 __device__ __forceinline__ void tmem_free(uint32_t addr, unsigned columns)
 {
+    __syncwarp();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(addr), "r"(columns) : "memory");
 }
 

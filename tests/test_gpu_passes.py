@@ -92,3 +92,24 @@ def test_run_on_convolution_axes(es, orc, shape):
     with es.Model(rho, cp, cs, dx=10.0, pml=pml) as m:
         m.source_set(pos[1], mts[1], w)
         assert np.array_equal(m.run(nt, dt, rcv), got[1])
+
+
+@pytest.mark.parametrize("shape,pml", [((19, 17, 96), 5), ((17, 19, 128), 3), ((48, 64, 45), 6), ((64, 48, 50), 5)])
+def test_ragged_tiles_with_near_parts_in_tensor_memory(es, orc, shape, pml):
+    """Lanes of one warp on either side of every branch between two reads of tensor memory: a last x tile of
+    three lines, half a tile of columns (nx odd and even) and PML rows that start inside a warp's
+    positions, on axes whose near parts wait there."""
+    rho, cp, cs = synth.two_layer_model(shape=shape, water_cells=6)
+    nt, dt = 60, cfl_dt(cp, 10.0)
+    w = synth.ricker(nt, dt, 25.0)
+    pos = (shape[2] // 2, shape[1] // 2, max(9, shape[0] // 2))
+    rcv = orc.seabed_receivers(cs, pml, 3, 3)
+    with es.Model(rho, cp, cs, dx=10.0, pml=pml) as m:
+        m.source_set(pos, synth.explosive(), w)
+        gpu = m.run(nt, dt, rcv)
+        st = m.state_get()
+    ref = orc.simulate(rho, cp, cs, dx=10.0, dt=dt, nt=nt, pml=pml, receivers=rcv, state=np.zeros((9,) + shape),
+                       sources=[dict(kind="moment", pos=pos, m=synth.explosive(), w=w)])
+    assert trace_errors(gpu, ref["traces"]).max() < 1e-4
+    for f in range(9):
+        assert rel_l2(st[f], ref["state"][f]) < 1e-4, f
