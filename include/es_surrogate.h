@@ -108,6 +108,14 @@ int es_gemm_status(void);
  * (seconds out of range) or ES_ERR_CUDA. */
 int es_gemm_wait_probe(double seconds, void* stream);
 
+/* The same for a pair of CTAs that share one product's tiles: the copies of
+ * CTA `rank` (0 or 1) stop before k-block `stage` (0 .. 19), every other wait
+ * of the two runs out after 50 ms, and the kernel ends once the copies that
+ * either had started have landed.  Synchronizes the stream.  ES_OK if so (the
+ * next es_gemm_status() reports ES_ERR_TIMEOUT), ES_ERR_STATE if copies were
+ * left in flight, ES_ERR_ARG or ES_ERR_CUDA. */
+int es_gemm_pair_probe(int rank, int stage, void* stream);
+
 #ifdef __cplusplus
 }
 #endif

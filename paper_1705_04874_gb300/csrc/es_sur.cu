@@ -373,6 +373,15 @@ int es_gemm_wait_probe(double seconds, void* stream)
     return ES_OK;
 }
 
+int es_gemm_pair_probe(int rank, int stage, void* stream)
+{
+    if (rank < 0 || rank > 1 || stage < 0 || stage >= 20) return ES_ERR_ARG;
+    cudaGetLastError();
+    unsigned v = 0;
+    CKS(gemm_pair_probe(rank, stage, &v, static_cast<cudaStream_t>(stream)));
+    return (v & 7u) && !(v & 24u) ? ES_OK : ES_ERR_STATE;
+}
+
 int es_gemm_bf16(int M, int N, int K, const void* A, int lda, int a_t, const void* B, int ldb, int b_nk, float* C,
                  int ldc, float alpha, float beta, int split_k, void* stream)
 {

@@ -37,7 +37,11 @@
 // time, records the role that gave up in a device status word (read and
 // cleared by gemm_tc_status) and lets the CTA finish: the MMAs issued are
 // awaited, TMA copies still in flight are awaited (both bounded) and the
-// tensor memory is always freed.
+// tensor memory is always freed.  A pair's copies are counted stage by stage by
+// the first CTA's barriers, which complete when both CTAs' shares have landed: at
+// the end the CTAs compare how many stages each has started, the one that gave up
+// earlier starts the missing ones too (nothing reads them any more), and the first
+// one waits for them all before either leaves.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -99,12 +103,16 @@ __global__ void wait_probe_kernel(unsigned long long limit_ns)
     }
 }
 
-template <int CL>
+// PROBE (pairs): the producer of CTA `span` mod 2 gives up before its stage `span` / 2, as after a wait
+// that ran out, and the other roles' waits run out after PROBE_NS (gemm_pair_probe)
+constexpr unsigned long long PROBE_NS = 50000000ull;
+template <int CL, bool PROBE = false>
 __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(THREADS, 1)
     gemm_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB, int M, int N,
                    int nkb, int kb_per, int mt, int ntl, int ntiles, float* __restrict__ C, int ldc, float alpha,
                    float beta, int atomic, float4 alpha4, int span)
 {
+    constexpr unsigned long long LIMIT = PROBE ? PROBE_NS : WAIT_NS;
     extern __shared__ uint8_t dyn[];
     constexpr int ST = tc_stages<CL>(), BYTES = A_BYTES + B_BYTES / CL;  // a stage of this CTA
     __shared__ __align__(8) uint64_t full[ST], empty[ST], acc_full[2], acc_empty[2], mma_done;
@@ -155,6 +163,20 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(THREADS, 1)
         if constexpr (CL == 1) tc_commit(bar);
         else tc_commit_pair(bar);
     };
+    // this CTA's copies into stage s: 64 of K from x on, A's rows from ya and B's from yb on
+    auto load = [&](int s, int x, int ya, int yb) {
+        const uint32_t sa = base + s * BYTES;
+        if constexpr (CL == 1) {
+            mbar_expect_tx(&full[s], BYTES);
+            tma_load_2d(sa, &mapA, &full[s], x, ya);
+            tma_load_2d(sa + A_BYTES, &mapB, &full[s], x, yb);
+        } else {  // each CTA its rows of A and of B; the issuing CTA's barrier hears of both
+            if (r == 0) mbar_expect_tx(&full[s], CL * BYTES);
+            const uint32_t bar = cluster_addr(&full[s], 0);
+            tma_load_2d_pair(sa, &mapA, bar, x, ya);
+            tma_load_2d_pair(sa + A_BYTES, &mapB, bar, x, yb);
+        }
+    };
 
     if (warp == 0) {
         if (lane == 0) {
@@ -167,22 +189,12 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(THREADS, 1)
                 const int nk = min(nkb, kb0 + kb_per) - kb0;
                 for (int kb = 0; kb < nk; ++kb, ++it) {
                     const int s = it % ST;
-                    if (!mbar_wait(&empty[s], ((it / ST) & 1) ^ 1)) {
+                    if ((PROBE && span == 2 * it + r) || !mbar_wait(&empty[s], ((it / ST) & 1) ^ 1, LIMIT)) {
                         atomicOr(&g_tc_status, 1u);
                         ok = false;
                         break;
                     }
-                    const uint32_t sa = base + s * BYTES;
-                    if constexpr (CL == 1) {
-                        mbar_expect_tx(&full[s], BYTES);
-                        tma_load_2d(sa, &mapA, &full[s], (kb0 + kb) * TK, mi * TM);
-                        tma_load_2d(sa + A_BYTES, &mapB, &full[s], (kb0 + kb) * TK, ni * TN);
-                    } else {  // each CTA its rows of A and of B; the issuing CTA's barrier hears of both
-                        if (r == 0) mbar_expect_tx(&full[s], CL * BYTES);
-                        const uint32_t bar = cluster_addr(&full[s], 0);
-                        tma_load_2d_pair(sa, &mapA, bar, (kb0 + kb) * TK, mi * TM);
-                        tma_load_2d_pair(sa + A_BYTES, &mapB, bar, (kb0 + kb) * TK, ni * TN + r * (TN / CL));
-                    }
+                    load(s, (kb0 + kb) * TK, mi * TM, ni * TN + r * (TN / CL));
                 }
             }
             s_issued = it;
@@ -197,7 +209,7 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(THREADS, 1)
                 const int kb0 = (rest / ntl) * kb_per;
                 const int nk = min(nkb, kb0 + kb_per) - kb0;
                 const int b = lt & 1;
-                if (!mbar_wait(&acc_empty[b], ((lt >> 1) & 1) ^ 1)) {
+                if (!mbar_wait(&acc_empty[b], ((lt >> 1) & 1) ^ 1, LIMIT)) {
                     atomicOr(&g_tc_status, 2u);
                     break;
                 }
@@ -205,7 +217,7 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(THREADS, 1)
                 const uint32_t acc = tmem + (uint32_t)(b * TN);
                 for (int kb = 0; kb < nk; ++kb, ++it) {
                     const int s = it % ST;
-                    if (!mbar_wait(&full[s], (it / ST) & 1)) {
+                    if (!mbar_wait(&full[s], (it / ST) & 1, LIMIT)) {
                         atomicOr(&g_tc_status, 2u);
                         ok = false;
                         break;
@@ -236,7 +248,7 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(THREADS, 1)
             const int b = lt & 1;
             // one lane waits and the warp follows its result: tcgen05.ld below needs the whole warp
             int got = 0;
-            if (lane == 0) got = mbar_wait(&acc_full[b], (lt >> 1) & 1) ? 1 : 0;
+            if (lane == 0) got = mbar_wait(&acc_full[b], (lt >> 1) & 1, LIMIT) ? 1 : 0;
             got = __shfl_sync(0xffffffffu, got, 0);
             if (!got) {
                 if (lane == 0) atomicOr(&g_tc_status, 4u);
@@ -253,7 +265,7 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(THREADS, 1)
                 uint32_t acc[32];
                 tmem_ld32(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(b * TN + c0), acc);
                 float4* srow = reinterpret_cast<float4*>(stage + lane * EPI_LD);
-                if (span) {
+                if (!PROBE && span) {
                     // per-column alpha: columns [c span, (c + 1) span) of C take component c of alpha4
                     float a[32];
 #pragma unroll
@@ -319,14 +331,18 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(THREADS, 1)
     __syncwarp();
     tc_fence_before();
     __syncthreads();
+    if (CL > 1) cluster_sync();  // both producers have stopped
     if (threadIdx.x == 0) {
         if (!mbar_wait(&mma_done, 0)) atomicOr(&g_tc_status, 8u);
         // copies issued but never consumed (only after a wait gave up) must land before the CTA exits
-        for (int it = s_consumed; r == 0 && it < s_issued; ++it)
-            if (!mbar_wait(&full[it % ST], (it / ST) & 1)) {
-                atomicOr(&g_tc_status, 16u);
-                break;
-            }
+        int issued = s_issued;
+        if constexpr (CL > 1) {
+            // stages the other CTA started alone: their places here are free (it saw them released by the
+            // MMAs, which read both CTAs' memory)
+            for (const int other = cluster_load(&s_issued, r ^ 1); issued < other; ++issued) load(issued % ST, 0, 0, 0);
+        }
+        for (int it = s_consumed; r == 0 && it < issued; ++it)
+            if (!mbar_wait(&full[it % ST], (it / ST) & 1)) atomicOr(&g_tc_status, 16u);
     }
     __syncthreads();
     if (CL > 1) cluster_sync();  // no CTA leaves while another may write to it or to its barriers
@@ -762,6 +778,33 @@ cudaError_t gemm_wait_probe(double seconds, cudaStream_t st)
     if (!(seconds > 0.0) || seconds > 2.0) return cudaErrorInvalidValue;
     wait_probe_kernel<<<1, 32, 0, st>>>((unsigned long long)(seconds * 1e9));
     return cudaGetLastError();
+}
+
+cudaError_t gemm_pair_probe(int rank, int stage, unsigned* status, cudaStream_t st)
+{
+    constexpr int K = 20 * TK;
+    if (rank < 0 || rank > 1 || stage < 0 || stage >= 20) return cudaErrorInvalidValue;
+    EncodeTiled fn = encode_tiled();
+    if (!fn) return cudaErrorNotSupported;
+    const size_t ab = (size_t)2 * TM * K * sizeof(__nv_bfloat16), c = (size_t)2 * TM * TN * sizeof(float);
+    char* mem = nullptr;
+    cudaError_t e = cudaMalloc(&mem, 2 * ab + c);
+    if (e != cudaSuccess) return e;
+    alignas(64) CUtensorMap mapA, mapB;
+    const __nv_bfloat16 *A = reinterpret_cast<__nv_bfloat16*>(mem), *B = reinterpret_cast<__nv_bfloat16*>(mem + ab);
+    if (!make_map(fn, &mapA, A, 2 * TM, K, K, TM) || !make_map(fn, &mapB, B, TN, K, K, TN / 2)) e = cudaErrorInvalidValue;
+    if (e == cudaSuccess) e = cudaMemsetAsync(mem, 0, 2 * ab + c, st);
+    const auto kernel = gemm_tc_kernel<2, true>;
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
+    if (e == cudaSuccess) {
+        kernel<<<2, THREADS, SMEM_BYTES, st>>>(mapA, mapB, 2 * TM, TN, 20, 20, 2, 1, 2, reinterpret_cast<float*>(mem + 2 * ab),
+                                               TN, 1.f, 0.f, 0, make_float4(0.f, 0.f, 0.f, 0.f), 2 * stage + rank);
+        e = cudaGetLastError();
+    }
+    const cudaError_t e2 = cudaStreamSynchronize(st);
+    cudaFree(mem);
+    if (e == cudaSuccess) e = e2;
+    return e == cudaSuccess ? cudaMemcpyFromSymbol(status, g_tc_status, sizeof *status) : e;
 }
 
 cudaError_t gemm_tc_status(unsigned* status)

@@ -41,6 +41,10 @@ cudaError_t gemm_tc_status(unsigned* status);
 // Launches one kernel whose bounded wait on a barrier nothing completes gives
 // up after `seconds` (0 < seconds <= 2) and sets the status word.
 cudaError_t gemm_wait_probe(double seconds, cudaStream_t st);
+// The give-up path of a pair of CTAs: one pair on a 256 x 256 x 1280 product of zeros whose producer in
+// CTA `rank` stops before k-block `stage` < 20, the other waits running out after 50 ms; synchronizes
+// and returns the status word (not cleared): bits 3 and 4 stay clear if the copies were all awaited.
+cudaError_t gemm_pair_probe(int rank, int stage, unsigned* status, cudaStream_t st);
 // out[c][r] = in[r][c] for a rows x cols BF16 matrix (row-major both)
 cudaError_t transpose_bf16(const __nv_bfloat16* in, long long rows, long long cols, __nv_bfloat16* out,
                            cudaStream_t st);

@@ -53,6 +53,7 @@ def _lib():
             "es_gemm_bf16": ([ci, ci, ci, vp, ci, ci, vp, ci, ci, vp, ci, cf, cf, ci, vp], ci),
             "es_gemm_status": ([], ci),
             "es_gemm_wait_probe": ([ctypes.c_double, vp], ci),
+            "es_gemm_pair_probe": ([ci, ci, vp], ci),
             "es_sur_combine": ([vp, ci, ctypes.c_longlong, vp, vp, ci, vp, vp], ci),
         }
         for name, (args, res) in sig.items():
@@ -86,6 +87,12 @@ def es_gemm_wait_probe(seconds, stream=None):
     one wait on a barrier nothing completes gives up after `seconds`; the next
     es_gemm_status() raises EsError(ES_ERR_TIMEOUT)."""
     _check(_lib().es_gemm_wait_probe(float(seconds), _es._stream_handle(stream)), "es_gemm_wait_probe")
+
+
+def es_gemm_pair_probe(rank, stage, stream=None):
+    """Runs the failure path of a CTA pair's bounded waits (es_gemm_pair_probe): raises EsError unless
+    every copy in flight was awaited; the next es_gemm_status() raises EsError(ES_ERR_TIMEOUT)."""
+    _check(_lib().es_gemm_pair_probe(int(rank), int(stage), _es._stream_handle(stream)), "es_gemm_pair_probe")
 
 
 def es_gemm_bf16(A, B, C, a_t=False, b_nk=False, alpha=1.0, beta=0.0, split_k=1, stream=None):

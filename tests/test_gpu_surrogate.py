@@ -429,3 +429,24 @@ def test_target_on_any_word_boundary(env, B):
         assert torch.equal(a[1], b[1]) and torch.equal(a[2], b[2])
     finally:
         s.close()
+
+
+@pytest.mark.parametrize("rank, stage", [(0, 0), (1, 0), (0, 3), (1, 3), (0, 6), (1, 13), (0, 19), (1, 19)])
+def test_a_pair_that_gives_up_awaits_its_copies(env, rank, stage):
+    """The failure path of a CTA pair, without a fault or a hang: one CTA's producer stops (at the first
+    k-block, within the ring of six, a turn later, at the last), every wait runs out within its bound,
+    and the copies that only the other CTA had started are awaited too.  The status word reports it once,
+    and the next product on pairs is right."""
+    es, sur, torch = env
+    sur.es_gemm_status()
+    sur.es_gemm_pair_probe(rank, stage)
+    with pytest.raises(es.EsError) as err:
+        sur.es_gemm_status()
+    assert err.value.status == es.ES_ERR_TIMEOUT
+    rng = np.random.default_rng(stage)
+    A, B = _bf(torch, rng.standard_normal((256, 1280))), _bf(torch, rng.standard_normal((512, 1280)))
+    C = torch.zeros((256, 512), device="cuda")
+    sur.es_gemm_bf16(A, B, C, b_nk=True)
+    sur.es_gemm_status()
+    ref = A.float().cpu().numpy().astype(np.float64) @ B.float().cpu().numpy().astype(np.float64).T
+    assert np.abs(C.cpu().numpy() - ref).max() <= 2e-5 * np.abs(ref).max()
