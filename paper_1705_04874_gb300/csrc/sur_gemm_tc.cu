@@ -21,7 +21,8 @@
 //       segments, and writes alpha * acc + beta * C (split_k > 1: atomically
 //       adds alpha * acc onto a C that already holds beta * C), then returns
 //       the accumulator; the next tile's MMAs run in the other one meanwhile.
-// With an even number of row tiles two CTAs (a cluster) work on two of them as one
+// With an even number of row tiles, and enough work (PAIR_MIN_K, PAIR_MIN_WORK), two
+// CTAs (a cluster) work on two of them as one
 // 256 x 256 tile: each loads its 128 rows of A and half of B's rows, the first one's
 // issuer runs tcgen05.mma.cta_group::2 (M 256) over both, and each reads its own
 // 128 rows back.  Shared memory is what bounds a CTA on its own: it must take in
@@ -84,6 +85,14 @@ constexpr uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(TN >
 
 // of a pair of CTAs: M is that of both
 constexpr uint32_t IDESC_PAIR = (IDESC & ~(0x1fu << 24)) | ((uint32_t)(2 * TM >> 4) << 24);
+// Pairs where a tile has PAIR_MIN_K k-blocks or more and each SM's share of all tiles' k-blocks is at
+// least PAIR_MIN_WORK.  A pair costs 1 to 2 us a launch (the cluster's launch and its two barriers), and
+// with few k-blocks a tile is bound by its output, not its operands.  us, single CTAs and pairs (one GB300;
+// tiles x k-blocks): 2 x 4 10.8 and 12.5, 512 x 12 37.1 and 37.3, 2048 x 12 104 and 103, 384 x 16 30.6 and
+// 30.9, 608 x 16 41.7 and 39.7, 1024 x 16 65.8 and 61.2, 256 x 24 28.9 and 28.7, 512 x 24 55.4 and 48.4, 64 x
+// 72 31.0 and 33.0, 152 x 72 41.0 and 37.1, 512 x 72 125 and 105; past both lines pairs won every one of 108
+// sizes but one (16 x 128 k-blocks in 8 row tiles, 2 % lost), by 14 % on average.
+constexpr int PAIR_MIN_K = 16, PAIR_MIN_WORK = 64;
 // a CTA of a pair holds half of B's rows, so the ring is deeper
 template <int CL>
 __host__ __device__ constexpr int tc_stages() { return STAGES * STAGE_BYTES / (A_BYTES + B_BYTES / CL); }
@@ -107,7 +116,7 @@ __global__ void wait_probe_kernel(unsigned long long limit_ns)
 // that ran out, and the other roles' waits run out after PROBE_NS (gemm_pair_probe)
 constexpr unsigned long long PROBE_NS = 50000000ull;
 template <int CL, bool PROBE = false>
-__global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(THREADS, 1)
+__global__ void __launch_bounds__(THREADS, 1)
     gemm_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB, int M, int N,
                    int nkb, int kb_per, int mt, int ntl, int ntiles, float* __restrict__ C, int ldc, float alpha,
                    float beta, int atomic, float4 alpha4, int span)
@@ -122,7 +131,7 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(THREADS, 1)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t base = (smem_u32(dyn) + 1023u) & ~1023u;
     // CTA r of a cluster takes row tile CL p + r of the cluster's tiles
-    const int r = CL > 1 ? (int)cluster_rank() : 0, first = blockIdx.x / CL, stride = gridDim.x / CL;
+    const int r = CL > 1 ? (int)cluster_rank() : 0;
     ntiles /= CL;
     mt /= CL;
 
@@ -183,7 +192,7 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(THREADS, 1)
             // producer: every k-block of every tile of this CTA, through the ring
             int it = 0;
             bool ok = true;
-            for (int t = first; t < ntiles && ok; t += stride) {
+            for (int t = blockIdx.x / CL; t < ntiles && ok; t += gridDim.x / CL) {
                 const int mi = t % mt * CL + r, rest = t / mt;
                 const int ni = rest % ntl, kb0 = (rest / ntl) * kb_per;
                 const int nk = min(nkb, kb0 + kb_per) - kb0;
@@ -204,7 +213,7 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(THREADS, 1)
             // MMA issuer (of a cluster: its first CTA's): accumulator b = local tile index mod 2
             int it = 0, lt = 0;
             bool ok = true;
-            for (int t = first; t < ntiles && ok; t += stride, ++lt) {
+            for (int t = blockIdx.x / CL; t < ntiles && ok; t += gridDim.x / CL, ++lt) {
                 const int rest = t / mt;
                 const int kb0 = (rest / ntl) * kb_per;
                 const int nk = min(nkb, kb0 + kb_per) - kb0;
@@ -243,7 +252,7 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(THREADS, 1)
         const int q = warp & 3;
         const bool vec = (ldc & 3) == 0 && (reinterpret_cast<uintptr_t>(C) & 15) == 0;
         int lt = 0;
-        for (int t = first; t < ntiles; t += stride, ++lt) {
+        for (int t = blockIdx.x / CL; t < ntiles; t += gridDim.x / CL, ++lt) {
             const int mi = t % mt * CL + r, ni = (t / mt) % ntl;
             const int b = lt & 1;
             // one lane waits and the warp follows its result: tcgen05.ld below needs the whole warp
@@ -692,6 +701,26 @@ __global__ void __launch_bounds__(AD_THREADS, 1)
 
 }  // namespace
 
+// gemm_tc_kernel on `grid` CTAs, in clusters of CL
+template <int CL, bool PROBE = false, class... Args>
+static cudaError_t launch_gemm(unsigned grid, cudaStream_t st, Args... args)
+{
+    cudaError_t e = cudaFuncSetAttribute(gemm_tc_kernel<CL, PROBE>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(THREADS);
+    cfg.dynamicSmemBytes = SMEM_BYTES;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = CL;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = CL > 1 ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, gemm_tc_kernel<CL, PROBE>, args...);
+}
+
 cudaError_t gemm_bf16_tc(int M, int N, int K, const __nv_bfloat16* A, int lda, const __nv_bfloat16* B, int ldb,
                          float* C, int ldc, float alpha, float beta, int split_k, cudaStream_t st,
                          const float* alpha4, int span)
@@ -703,10 +732,6 @@ cudaError_t gemm_bf16_tc(int M, int N, int K, const __nv_bfloat16* A, int lda, c
     if (lda % 8 || ldb % 8 || lda < K || ldb < K || ldc < N) return cudaErrorInvalidValue;
     EncodeTiled fn = encode_tiled();
     if (!fn) return cudaErrorNotSupported;
-    alignas(64) CUtensorMap mapA, mapB;
-    const bool pair = (M + TM - 1) / TM % 2 == 0;
-    if (!make_map(fn, &mapA, A, M, K, lda, TM) || !make_map(fn, &mapB, B, N, K, ldb, pair ? TN / 2 : TN))
-        return cudaErrorInvalidValue;
     const int nkb = (K + TK - 1) / TK;
     if (split_k < 1) split_k = 1;
     if (split_k > nkb) split_k = nkb;
@@ -716,20 +741,18 @@ cudaError_t gemm_bf16_tc(int M, int N, int K, const __nv_bfloat16* A, int lda, c
     const long long ntiles = (long long)mt * ntl * split_k;
     if (ntiles > 0x7fffffffLL) return cudaErrorInvalidValue;
     int dev = 0, sms = 0;
-    cudaError_t e0 = cudaGetDevice(&dev);
-    if (e0 == cudaSuccess) e0 = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e0 != cudaSuccess) return e0;
-    const long long grid = ntiles < sms ? ntiles : (pair ? sms / 2 * 2 : sms);
-    if (split_k > 1 && beta != 1.f) {
-        cudaError_t e = scale_f32(C, M, N, ldc, beta, st);
-        if (e != cudaSuccess) return e;
-    }
-    const auto kernel = pair ? gemm_tc_kernel<2> : gemm_tc_kernel<1>;
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
-    kernel<<<(unsigned)grid, THREADS, SMEM_BYTES, st>>>(mapA, mapB, M, N, nkb, kb_per, mt, ntl, (int)ntiles, C, ldc, alpha,
-                                                       beta, split_k > 1 ? 1 : 0, av, alpha4 ? span : 0);
-    return cudaGetLastError();
+    const bool pair = mt % 2 == 0 && kb_per >= PAIR_MIN_K && ntiles * kb_per >= (long long)PAIR_MIN_WORK * sms;
+    alignas(64) CUtensorMap mapA, mapB;
+    if (!make_map(fn, &mapA, A, M, K, lda, TM) || !make_map(fn, &mapB, B, N, K, ldb, pair ? TN / 2 : TN))
+        return cudaErrorInvalidValue;
+    if (split_k > 1 && beta != 1.f && (e = scale_f32(C, M, N, ldc, beta, st)) != cudaSuccess) return e;
+    const unsigned grid = (unsigned)(ntiles < sms ? ntiles : (pair ? sms / 2 * 2 : sms));
+    const int atomic = split_k > 1 ? 1 : 0, sp = alpha4 ? span : 0;
+    return pair ? launch_gemm<2>(grid, st, mapA, mapB, M, N, nkb, kb_per, mt, ntl, (int)ntiles, C, ldc, alpha, beta, atomic, av, sp)
+                : launch_gemm<1>(grid, st, mapA, mapB, M, N, nkb, kb_per, mt, ntl, (int)ntiles, C, ldc, alpha, beta, atomic, av, sp);
 }
 
 // a row-major FP32 [rows][cols] array in blocks of 32 x AD_COLS, 128-byte swizzle
@@ -794,13 +817,9 @@ cudaError_t gemm_pair_probe(int rank, int stage, unsigned* status, cudaStream_t 
     const __nv_bfloat16 *A = reinterpret_cast<__nv_bfloat16*>(mem), *B = reinterpret_cast<__nv_bfloat16*>(mem + ab);
     if (!make_map(fn, &mapA, A, 2 * TM, K, K, TM) || !make_map(fn, &mapB, B, TN, K, K, TN / 2)) e = cudaErrorInvalidValue;
     if (e == cudaSuccess) e = cudaMemsetAsync(mem, 0, 2 * ab + c, st);
-    const auto kernel = gemm_tc_kernel<2, true>;
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
-    if (e == cudaSuccess) {
-        kernel<<<2, THREADS, SMEM_BYTES, st>>>(mapA, mapB, 2 * TM, TN, 20, 20, 2, 1, 2, reinterpret_cast<float*>(mem + 2 * ab),
-                                               TN, 1.f, 0.f, 0, make_float4(0.f, 0.f, 0.f, 0.f), 2 * stage + rank);
-        e = cudaGetLastError();
-    }
+    if (e == cudaSuccess)
+        e = launch_gemm<2, true>(2, st, mapA, mapB, 2 * TM, TN, 20, 20, 2, 1, 2, reinterpret_cast<float*>(mem + 2 * ab), TN, 1.f,
+                                 0.f, 0, make_float4(0.f, 0.f, 0.f, 0.f), 2 * stage + rank);
     const cudaError_t e2 = cudaStreamSynchronize(st);
     cudaFree(mem);
     if (e == cudaSuccess) e = e2;

@@ -436,7 +436,7 @@ def test_a_pair_that_gives_up_awaits_its_copies(env, rank, stage):
     """The failure path of a CTA pair, without a fault or a hang: one CTA's producer stops (at the first
     k-block, within the ring of six, a turn later, at the last), every wait runs out within its bound,
     and the copies that only the other CTA had started are awaited too.  The status word reports it once,
-    and the next product on pairs is right."""
+    and the next product is right."""
     es, sur, torch = env
     sur.es_gemm_status()
     sur.es_gemm_pair_probe(rank, stage)
@@ -450,3 +450,26 @@ def test_a_pair_that_gives_up_awaits_its_copies(env, rank, stage):
     sur.es_gemm_status()
     ref = A.float().cpu().numpy().astype(np.float64) @ B.float().cpu().numpy().astype(np.float64).T
     assert np.abs(C.cpu().numpy() - ref).max() <= 2e-5 * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("M, N, K, split, beta", [
+    (256, 77824, 1024, 1, 0.0),   # 608 tiles of 16 k-blocks: 64 for each of 152 SMs, the fewest that run on pairs
+    (256, 77824, 960, 1, 0.0),    # 15 k-blocks: single CTAs
+    (200, 77800, 1000, 1, 0.5),   # ragged rows, columns and K on pairs
+    (1024, 20000, 1096, 1, 0.0),  # eight row tiles, several tiles per pair
+    (250, 4600, 100000, 32, 1.0), # slices of K added by atomics
+])
+def test_products_large_enough_for_pairs(env, M, N, K, split, beta):
+    """Products on either side of the rule that puts them on pairs of CTAs, against FP64.  K products of
+    N(0, 1) operands summed in FP32 are within 2e-5 of the largest sum (about 6 sqrt(K))."""
+    es, sur, torch = env
+    g = torch.Generator(device="cuda").manual_seed(M + N)
+    A = torch.randn((M, K), device="cuda", generator=g).bfloat16()
+    B = torch.randn((N, K), device="cuda", generator=g).bfloat16()
+    C = torch.randn((M, N), device="cuda", generator=g)
+    want = beta * C.double()
+    for n in range(0, N, 8192):
+        want[:, n:n + 8192] += A.double() @ B[n:n + 8192].double().T
+    sur.es_gemm_bf16(A, B, C, b_nk=True, beta=beta, split_k=split)
+    sur.es_gemm_status()
+    assert float((C - want).abs().max()) <= 2e-5 * float(want.abs().max())
