@@ -221,13 +221,16 @@ cudaError_t launch_transpose_traces(const float* rec, int nt, int cols, float* o
 // 4 bytes per event and sample (a trace itself comes from DRAM about once: the
 // rows in flight fit in L2).  Events reach shared memory in chunks of SUP_CHUNK,
 // so any number of them fits without changing the order of the sum.
+// Small gathers do not have the warps to hide an event's load behind other
+// warps: there the events that overlap the span go U at a time, the loads of all
+// of them before the first multiply-add.
 // 64 sources x 1024 receivers x 2000 samples, 300 events into 4666 samples (one
 // GB300): 0.99 ms (1.46 ms with the call around it); one sample per thread with
 // a test, an address and three shared loads per event and sample took 4.69 ms
 // with the call.
 constexpr int SUP_CHUNK = 1024, SUP_WARPS = 8;
 
-template <int R>
+template <int R, int U>
 __global__ void __launch_bounds__(32 * SUP_WARPS) superpose_kernel(const float* traces, long long rows, int nt,
                                                                    const int* ev_src, const float* ev_amp,
                                                                    const int* ev_shift, int n_events, int n_out,
@@ -238,7 +241,7 @@ __global__ void __launch_bounds__(32 * SUP_WARPS) superpose_kernel(const float* 
         int k;
         float amp;
     };
-    __shared__ __align__(16) Event ev[SUP_CHUNK];
+    __shared__ __align__(16) Event ev[SUP_CHUNK + (U > 1 ? 1 : 0)];
     const long long unit = (long long)blockIdx.x * SUP_WARPS + threadIdx.x / 32;  // row-major: consecutive warps share a row
     const long long row = unit / spans;
     const bool active = row < rows;
@@ -258,8 +261,39 @@ __global__ void __launch_bounds__(32 * SUP_WARPS) superpose_kernel(const float* 
             ev[i].k = k;
             ev[i].amp = ev_amp[e0 + i];
         }
+        // what fills up a group: an event past the window (row 0 of source 0, at a shift of n_out)
+        if (U > 1 && threadIdx.x == 0) ev[SUP_CHUNK] = {-(long long)n_out, n_out, 0.f};
         __syncthreads();
         if (!active) continue;
+        if constexpr (U > 1) {
+#pragma unroll 1
+            for (int g = 0; g < ne; g += 32) {  // a lane tests one event of 32, the warp walks those that overlap
+                const int k0 = t0 - (g + lane < ne ? ev[g + lane].k : n_out);
+                unsigned todo = __ballot_sync(0xffffffffu, g + lane < ne && k0 < nt && k0 + 32 * R > 0);
+#pragma unroll 1
+                while (todo) {
+                    float x[U][R], amp[U];
+                    bool in[U][R];
+#pragma unroll
+                    for (int j = 0; j < U; ++j) {
+                        const Event v = ev[todo ? g + __ffs(todo) - 1 : SUP_CHUNK];
+                        todo &= todo - 1;
+                        const int u = t0 - v.k + lane;
+                        amp[j] = v.amp;
+#pragma unroll
+                        for (int i = 0; i < R; ++i) {
+                            in[j][i] = u + 32 * i >= 0 && u + 32 * i < nt;
+                            x[j][i] = in[j][i] ? __ldg(base + v.ofs + 32 * i) : 0.f;
+                        }
+                    }
+#pragma unroll
+                    for (int j = 0; j < U; ++j)
+#pragma unroll
+                        for (int i = 0; i < R; ++i) acc[i] = in[j][i] ? __fmaf_rn(amp[j], x[j][i], acc[i]) : acc[i];
+                }
+            }
+            continue;
+        }
 #pragma unroll 2
         for (int e = 0; e < ne; ++e) {
             const Event v = ev[e];
@@ -285,14 +319,14 @@ __global__ void __launch_bounds__(32 * SUP_WARPS) superpose_kernel(const float* 
         if (t0 + lane + 32 * i < n_out) out[32 * i] = acc[i];
 }
 
-template <int R>
+template <int R, int U>
 static cudaError_t launch_superpose_r(const float* traces, int n_rcv, int nt, const int* ev_src, const float* ev_amp,
                                       const int* ev_shift, int n_events, int n_out, float* gather, cudaStream_t st)
 {
     const long long rows = 4LL * n_rcv, spans = (n_out + 32LL * R - 1) / (32 * R);
     const long long blocks = (rows * spans + SUP_WARPS - 1) / SUP_WARPS;
     if (blocks > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-    superpose_kernel<R><<<(unsigned)blocks, 32 * SUP_WARPS, 0, st>>>(traces, rows, nt, ev_src, ev_amp, ev_shift,
+    superpose_kernel<R, U><<<(unsigned)blocks, 32 * SUP_WARPS, 0, st>>>(traces, rows, nt, ev_src, ev_amp, ev_shift,
                                                                     n_events, n_out, (int)spans, gather);
     return cudaGetLastError();
 }
@@ -304,12 +338,16 @@ cudaError_t launch_superpose(const float* traces, int n_src, int n_rcv, int nt, 
     (void)n_src;
     // R = 8 and 4 by output samples (one GB300, 300 events): 19.1 M 0.991 and 1.022 ms, 16.4 M with
     // short traces 0.336 and 0.475, 1.23 M 67.9 and 71.9 us; 0.61 M (200 events) 38.3 and 34.3,
-    // 0.26 M 24.2 and 22.2: below about a million the longer
-    // spans leave SMs idle.  R = 2 lost at every size, R = 16 won only with the short traces (0.287 ms,
-    // 1.24 at the first size).
+    // 0.26 M 24.2 and 22.2: below about a million the longer spans leave SMs idle.  R = 16 won only with the
+    // short traces (0.287 ms, 1.24 at the first size).  Below half a million R = 4 leaves them idle too: us
+    // a call with R = 4 and with R = 2 and events eight at a time (one sample per thread), 384 K 59.1 and 51
+    // (118), 307 K 88.6 and 63 (113), 96 K 50.7 and 47 (55), 32 K 86.1 and 40 (43), 8 K with 60,000 events
+    // 3732 and 1577 (2672); 1.02 M 74.9 and 77 (252).
     if (4LL * n_rcv * n_out >= 1 << 20)
-        return launch_superpose_r<8>(traces, n_rcv, nt, ev_src, ev_amp, ev_shift, n_events, n_out, gather, st);
-    return launch_superpose_r<4>(traces, n_rcv, nt, ev_src, ev_amp, ev_shift, n_events, n_out, gather, st);
+        return launch_superpose_r<8, 1>(traces, n_rcv, nt, ev_src, ev_amp, ev_shift, n_events, n_out, gather, st);
+    if (4LL * n_rcv * n_out >= 1 << 19)
+        return launch_superpose_r<4, 1>(traces, n_rcv, nt, ev_src, ev_amp, ev_shift, n_events, n_out, gather, st);
+    return launch_superpose_r<2, 8>(traces, n_rcv, nt, ev_src, ev_amp, ev_shift, n_events, n_out, gather, st);
 }
 
 // flag |= 1 if any field value is NaN or infinite

@@ -95,3 +95,37 @@ def test_superpose_spans_and_chunks(ev, n_src, n_rcv, nt, n_events, n_out):
             want[..., lo:hi] += term
             size[..., lo:hi] += np.abs(term)
     assert np.all(np.abs(got - want) <= 2 * n_events * 2.0 ** -24 * size)
+
+
+@pytest.mark.parametrize("n_src, n_rcv, nt, n_events, n_out", [
+    (1, 1, 5, 1, 1), (2, 1, 64, 8, 64), (2, 3, 40, 15, 65),  # part of a group, a whole one, one sample over a span
+    (3, 2, 900, 1065, 300),       # a trace longer than the window, 41 events past a chunk
+    (2, 1, 30, 400, 60000),       # most groups overlap no sample of a span
+    (3, 64, 100, 61, 2047),       # 524,032 samples: the most that take groups of events
+    (3, 64, 100, 61, 2048),       # 524,288: the fewest that do not
+])
+def test_superpose_events_in_groups(ev, n_src, n_rcv, nt, n_events, n_out):
+    """Small gathers take the events eight at a time: remainders of a group, of a span and of a chunk, and both
+    sides of the rule, with the largest amplitudes on events outside the window, which must add nothing.  The
+    sum of k products in FP32 is within k 2^-24 of the sum of their magnitudes (doubled)."""
+    es, _ = ev
+    rng = np.random.default_rng(n_out + n_events)
+    tr = rng.standard_normal((n_src, 4, n_rcv, nt)).astype(np.float32)
+    src = rng.integers(0, n_src, n_events).astype(np.int32)
+    amps = rng.standard_normal(n_events).astype(np.float32)
+    shift = rng.integers(-nt + 1, n_out, n_events)
+    out = rng.integers(0, n_events, max(1, n_events // 5))
+    if n_events > 1:
+        shift[out] = rng.choice([-nt, -nt - 3, n_out, n_out + 31], len(out))
+        amps[out] = 3e38
+    dt = 0.25  # exact in FP32 with every shift
+    got = es.es_superpose(tr, src, amps, (shift * dt).astype(np.float32), dt, n_out)
+    want = np.zeros((4, n_rcv, n_out))
+    size = np.zeros((4, n_rcv, n_out))
+    for s, a, k in zip(src, amps.astype(np.float64), shift):
+        lo, hi = max(k, 0), min(k + nt, n_out)
+        if lo < hi:
+            term = a * tr[s][..., lo - k:hi - k]
+            want[..., lo:hi] += term
+            size[..., lo:hi] += np.abs(term)
+    assert np.all(np.abs(got - want) <= 2 * n_events * 2.0 ** -24 * size)
