@@ -552,11 +552,11 @@ bool fused_sources(const es_model* m)
     return std::none_of(m->srcs.begin(), m->srcs.end(), [](const Src& s) { return s.smooth != 0; });
 }
 
-// The per-CTA cell lists of the fused passes (PassParams::sp_off / sp): for the velocity z pass
+// The per-tile cell lists of the fused passes (PassParams::sp_off / sp): for the velocity z pass
 // (SP_VEL_Z) the point forces, then the receivers; for the stress y pass (SP_STR_Y) the moment
-// sources; for the stress z pass (SP_STR_Z) the moment sources, then the receivers.  A y or z pass
-// CTA owns 32 consecutive x at one z (y pass) or one y (z pass) of one simulation: blockIdx.x =
-// sim + nsim (x / 32 + ntx outer).  Sources keep their order (the order the injection kernel adds
+// sources; for the stress z pass (SP_STR_Z) the moment sources, then the receivers.  A tile of a y or z
+// pass is 32 consecutive x at one z (y pass) or one y (z pass) of one simulation, and its list
+// (StridedTile::list) sim + nsim (x / 32 + ntx outer).  Sources keep their order (the order the injection kernel adds
 // them in).
 int build_special(es_model* m, const std::vector<long long>& rcv_cells)
 {

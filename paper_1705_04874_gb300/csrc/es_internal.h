@@ -112,7 +112,7 @@ struct PassParams {
     // step advances the device step counter (step_counter); the velocity z pass injects the
     // point forces and records the velocities, the stress y pass injects Mxy, the stress z pass
     // the other moment components and records the pressure.  sp_off[b] .. sp_off[b + 1] are
-    // CTA b's (blockIdx.x) cells in sp, in source order, then receivers.  The step index is
+    // the cells of tile b (StridedTile::list) in sp, in source order, then receivers.  The step index is
     // *step_now - 1; samples go to rec[(n - rec_start) nsim + sim][4][n_rcv].
     int* step_counter;
     const int* step_now;

@@ -32,7 +32,8 @@
 // |H_far| / |H| (about 1 %), so far-away receivers no longer see the FP32
 // noise of the pencil's largest values.
 //
-// The passes are persistent: while a CTA works on one tile, the next one's
+// The passes (but for the y and z passes of the shortest and the odd lengths,
+// pass_strided_once) are persistent: while a CTA works on one tile, the next one's
 // source arrives in shared memory (cp.async), so that the 3 CTAs an SM holds at
 // n = 256 (72 KB each) have 6 tiles in hand.  What bounds them is memory: at
 // 256^3 (one GB300, 6.68 TB/s copy rate) the y / z velocity passes move 844 MB
@@ -356,9 +357,9 @@ __device__ __forceinline__ void red_pair(float* q, float2 v, bool two)
     }
 }
 
-// Epilogue for one cell (odd nx in the y / z passes, any length in the x pass,
-// the circulant passes): the same arithmetic as the pass epilogues,
-// one cell at a time.
+// Epilogue for one cell (what is left of an x pass's tile past its whole quads, or
+// all of it where its arrays are not on 16-byte boundaries; the circulant passes):
+// the same arithmetic as the pass epilogues, one cell at a time.
 __device__ __forceinline__ void epilogue_one(const PassParams& p, const PassJob& J, size_t q, int pos, int x, int y,
                                              int z, float d, size_t off, size_t soff)
 {
@@ -692,7 +693,8 @@ __host__ __device__ constexpr unsigned tmem_columns()
 template <int RN>
 __host__ __device__ constexpr int epi_batch()
 {
-    return RN % 4 == 0 ? 4 : (RN % 5 == 0 ? 5 : (RN % 3 == 0 ? 3 : 2));
+    static_assert(RN % 4 == 0 || RN % 5 == 0, "whole batches");
+    return RN % 4 == 0 ? 4 : 5;
 }
 
 // shared bytes of the y / z passes: two tiles [N][PAIRS] (the current one,
@@ -838,9 +840,10 @@ inline cudaError_t persistent_grid(K kernel, int threads, size_t smem, int units
 // reductions visible to the CTA; the reads go through L2), thread 0 adds the
 // sources in their order, and after a second barrier every receiver is
 // recorded by a thread of its own -- the arithmetic of the separate injection
-// and recording kernels (inject_kernel, record_kernel).  job = the CTA's job
-// (blockIdx.y): the velocity z pass's job c updates v_c, the stress y pass's
-// job 1 sxy, the stress z pass's job 0 sxx syy szz, job 1 sxz, job 2 syz.
+// and recording kernels (inject_kernel, record_kernel).  job and tile: those of
+// the tile just updated (StridedTile::job, ::list): the velocity z pass's job c updates
+// v_c, the stress y pass's job 1 sxy, the stress z pass's job 0 sxx syy szz, job 1
+// sxz, job 2 syz.
 __device__ __forceinline__ void special_phase(const PassParams& p, const PassJob& J, int job, int tile)
 {
     const int b0 = p.sp_off[tile], b1 = p.sp_off[tile + 1];
@@ -1278,6 +1281,150 @@ pass_strided(const __grid_constant__ PassParams p, int ntiles)
         __syncthreads();
         if (tid < 32) tmem_free(tmem_slot, tmem_columns<N, T>());
     }
+}
+
+// The same passes with one tile per CTA (blockIdx.x) and job (blockIdx.y), for the shortest lengths and
+// the odd ones: the source goes straight into registers and comes again, from L2, for the stencil once
+// the FFT is done with the one shared tile, so a CTA takes a third of the shared memory and more of them
+// hide each other's chain of loads and stages.  A thread keeps the elements its first stage reads, j + q
+// N / RA, to the end.  Which lengths: one_tile(), pass_strided.cuh.
+constexpr int HALO = 5;  // rows of wrap-around copies on each side of that tile
+static_assert(-near_ofs(-1) <= HALO && near_ofs(+1) + NEAR_TAPS - 1 <= HALO, "near taps reach beyond the halo");
+template <int RA, int RB, int RC>
+__host__ __device__ constexpr int once_threads() { return RB * RC * PAIRS; }
+// (more threads than the register file holds at 64 each, but for the butterflies that need those: 75 = 5 x
+// 15 with four and five CTAs per SM 70.6 and 65.4 ps per cell, 64 = 16 x 4 with 16 and 18 50.9 and 59.5)
+template <int RA, int RB, int RC>
+__host__ __device__ constexpr int once_blocks() { return (RA <= 12 ? 1200 : 1024) / once_threads<RA, RB, RC>(); }
+template <int RA, int RB, int RC>
+__host__ __device__ constexpr size_t once_smem()
+{
+    return sizeof(float2) * ((size_t)(RA * RB * RC + 2 * HALO) * PAIRS + 2 * (size_t)RA * RB * RC);
+}
+
+// Update of one pair of cells: offsets of its first cell in a field (f), a coefficient array (cf) and a slab
+// array (s: of slab coordinate 0, est per coordinate), position pos along the axis.
+template <int V>
+__device__ __forceinline__ void update_pair(const PassParams& p, const PassJob& J, size_t f, size_t cf, size_t s, unsigned est,
+                                            int pos, float2 d, bool two)
+{
+    const int last = V == 2 ? 1 : (two ? PAIRS : 0);
+    if (!ES_INB(p, f + last, p.ext_f)) return;
+    if (J.kind == JOB_STORE) {
+        st_pair<V, PAIRS>(J.tgt[0] + f, d, two);
+        return;
+    }
+    if (!ES_INB(p, cf + last, p.ext_c)) return;
+    const bool slab = in_slab(pos, p.n, p.L);
+    float P = 1.f;
+    if (slab) {
+        s += (size_t)((unsigned)slab_pos(pos, p.n, p.L, p.S) * est);
+        if (!ES_INB(p, s + last, p.ext_s)) return;
+        P = __ldg((J.stag ? p.ps : p.pc) + pos);
+    }
+    auto add = [&](int k, float2 c) {
+        float2 inc = make_float2(increment(p.dt, c.x, d.x), increment(p.dt, c.y, d.y));
+        if (slab) {  // s <- P (P s + inc); the total takes the split's change
+            const float2 sv = ld_pair<V, PAIRS>(J.slab[k] + s, two);
+            const float2 sn = make_float2(__fmul_rn(P, __fmaf_rn(P, sv.x, inc.x)), __fmul_rn(P, __fmaf_rn(P, sv.y, inc.y)));
+            st_pair<V, PAIRS>(J.slab[k] + s, sn, two);
+            inc = make_float2(__fsub_rn(sn.x, sv.x), __fsub_rn(sn.y, sv.y));
+        }
+        red_pair<V, PAIRS>(J.tgt[k] + f, inc, two);
+    };
+    const float2 c0 = ldg_pair<V, PAIRS>(J.coef[0] + cf, two);
+    if (J.kind == JOB_SINGLE) {
+        add(0, c0);
+    } else {
+        const float2 c1 = ldg_pair<V, PAIRS>(J.coef[1] + cf, two);
+#pragma unroll
+        for (int k = 0; k < 3; ++k)
+            add(k, make_float2(normal_coef(c0.x, c1.x, k == J.diag), normal_coef(c0.y, c1.y, k == J.diag)));
+    }
+}
+
+template <int RA, int RB, int RC, int V>
+__global__ void __launch_bounds__(once_threads<RA, RB, RC>(), once_blocks<RA, RB, RC>())
+pass_strided_once(const __grid_constant__ PassParams p, int ntiles)
+{
+    constexpr int T = RB * RC, NT = T * PAIRS;
+    using C = CoreOf<RA, RB, RC, T>;
+    constexpr int N = C::N, BA = C::BA;
+    static_assert(C::MA == 1, "a thread's elements are j + q BA");
+    extern __shared__ __align__(16) float2 smem[];
+    float2* buf = smem;  // FFT rows 0 .. N-1; then the source tile at rows HALO + pos (wrapped)
+    float2* s_tw = buf + (N + 2 * HALO) * PAIRS;
+    float2* s_h = s_tw + N;
+    const int tid = threadIdx.x;
+    const int c = tid % PAIRS, j = tid / PAIRS;
+    const PassJob& J = p.job[blockIdx.y];
+    pdl_begin(p.pdl);
+    const unsigned est = p.axis == 1 ? (unsigned)p.nx : (unsigned)p.nx * p.ny, step = BA * est;
+    const StridedTile t = strided_tile(p, blockIdx.x, ntiles);
+    const bool valid = t.x0 + V * c < p.nx, two = V == 2 || t.x0 + PAIRS + c < p.nx;
+    const int last = V == 2 ? 1 : (two ? PAIRS : 0);
+    const size_t f0 = t.off + t.base + V * c;
+    const float* src = J.src + f0;
+    float2 a[1][RA];
+#pragma unroll
+    for (int q = 0; q < RA; ++q)
+        a[0][q] = valid && ES_INB(p, f0 + (j + q * BA) * est + last, p.ext_f)
+                      ? ldg_pair<V, PAIRS>(src + (j + q * BA) * est, two)
+                      : make_float2(0.f, 0.f);
+    // coefficient rows of this tile (128 bytes each) into L2 for the epilogue
+    if (J.coef[0])
+        for (int i = tid; i < N; i += NT) {
+            const unsigned o = (unsigned)i * est;
+            if (ES_INB(p, t.base + o, p.ext_c)) {
+                prefetch_l2(J.coef[0] + t.base + o);
+                if (J.coef[1]) prefetch_l2(J.coef[1] + t.base + o);
+            }
+        }
+    load_tables<N>(p, J, s_tw, s_h, tid, NT);
+    Dft<RA>::run(a[0]);
+    C::stageA_store(a, buf, j, c);
+    __syncthreads();
+    C::middle(buf, s_tw, s_h, j, c);
+    __syncthreads();
+    C::stageA_inv(buf, s_tw, a, j, c);
+    __syncthreads();  // the FFT's rows have been read
+    auto copy = [&](float2* d, unsigned o) {
+        if (!ES_INB(p, f0 + o + last, p.ext_f)) return;
+        if constexpr (V == 2) {
+            cp_async<8>(d, src + o, true);
+        } else {
+            cp_async<4>(&d->x, src + o, true);
+            cp_async<4>(&d->y, two ? src + o + PAIRS : src, two);
+        }
+    };
+    if (valid) {
+        unsigned o = (unsigned)j * est;
+        float2* d = buf + (j + HALO) * PAIRS + c;
+#pragma unroll 1
+        for (int q = 0; q < RA; ++q, o += step, d += BA * PAIRS) copy(d, o);
+        for (int h = j; h < 2 * HALO; h += T) {
+            const int pos = h < HALO ? N - HALO + h : h - HALO;
+            copy(buf + (h < HALO ? h : N + h) * PAIRS + c, (unsigned)pos * est);
+        }
+    }
+    cp_async_commit_wait_all();
+    __syncthreads();
+    if (valid) {
+        const float2* w = buf + (j + HALO + near_ofs(J.sign)) * PAIRS + c;
+#pragma unroll
+        for (int q = 0; q < RA; ++q) {
+            float2 s = make_float2(0.f, 0.f);
+#pragma unroll
+            for (int k = 0; k < NEAR_TAPS; ++k) s = fma2(rep2(J.g[k]), w[(q * BA + k) * PAIRS], s);
+            a[0][q] = make_float2(__fadd_rn(a[0][q].x, s.x), __fsub_rn(s.y, a[0][q].y));  // far (conj) + near
+        }
+        if (p.pdl == 1) pdl_wait();  // the previous pass's updates of the targets come first
+        const size_t s0 = t.soff + t.x0 + V * c + (p.axis == 1 ? (size_t)p.nx * p.S * t.outer : (size_t)p.nx * t.outer);
+#pragma unroll
+        for (int q = 0; q < RA; ++q)
+            update_pair<V>(p, J, f0 + (j + q * BA) * est, t.base + V * c + (j + q * BA) * est, s0, est, j + q * BA, a[0][q], two);
+    }
+    if (p.sp_mode != SP_NONE) special_phase(p, J, blockIdx.y, t.list);
 }
 
 // x pass: cell (position x, line r of the tile) of a turned-around tile is

@@ -113,3 +113,56 @@ def test_ragged_tiles_with_near_parts_in_tensor_memory(es, orc, shape, pml):
     assert trace_errors(gpu, ref["traces"]).max() < 1e-4
     for f in range(9):
         assert rel_l2(st[f], ref["state"][f]) < 1e-4, f
+
+
+ONE_TILE = [(16, 4, 4), (32, 8, 4), (48, 12, 4), (64, 16, 4), (64, 8, 8), (75, 5, 15), (75, 3, 25), (75, 15, 5), (125, 5, 25)]
+
+
+@pytest.mark.parametrize("n,ra,rb", ONE_TILE)
+@pytest.mark.parametrize("nx", [3, 33, 34, 64, 66])  # part of a tile, one or two columns of a second one, whole ones
+def test_one_tile_per_cta(es, orc, n, ra, rb, nx):
+    """The y and z passes that run one tile per CTA, both directions, stored and accumulated (the Laplacian
+    along the other axes adds to what the first one stored).  Bounds as in test_many_tiles_per_cta; the second
+    derivative's error is twice a derivative's."""
+    import torch
+    if nx == 64 and n == 64:
+        pytest.skip("persistent")
+    default = es.es_fft_plan(1, n)
+    es.es_fft_plan_select(1, n, ra, rb)
+    try:
+        rng = np.random.default_rng(n + nx)
+        for axis, shape in ((1, (5, n, nx)), (2, (n, 7, nx))):
+            f = rng.standard_normal(shape).astype(np.float32)
+            d = torch.from_numpy(f).cuda()
+            out = torch.empty(shape, device="cuda")
+            for shift in (1, -1):
+                es.es_derivative(d, axis, 10.0, shift, out)
+                assert rel_l2(out.cpu().numpy(), orc.deriv(f.astype(np.float64), axis, 10.0, shift)) < 5e-7
+            es.es_laplacian(d, (10.0, 10.0, 10.0), out)
+            want = sum(orc.deriv(orc.deriv(f.astype(np.float64), a, 10.0, -1), a, 10.0, 1) for a in range(3))
+            assert rel_l2(out.cpu().numpy(), want) < 1e-6
+    finally:
+        es.es_fft_plan_select(1, n, *default)
+
+
+@pytest.mark.parametrize("shape,pml", [((16, 32, 34), 4), ((48, 16, 61), 3), ((125, 75, 20), 5), ((75, 64, 62), 10)])
+def test_runs_on_one_tile_passes(es, orc, shape, pml):
+    """A batch with PML, sources and receivers in these passes: the first simulation against the oracle, the second
+    against a run of its own."""
+    nt = 60
+    rho, cp, cs = synth.two_layer_model(shape=shape, water_cells=6)
+    dt = cfl_dt(cp, 10.0)
+    w = synth.ricker(nt, dt, 25.0)
+    nz, ny, nx = shape
+    pos = np.array([[nx // 2, ny // 2, max(8, nz // 3)], [nx // 2 - 1, ny // 2 - 1, max(9, nz // 3)]], np.int32)
+    mts = np.stack([synth.explosive(), synth.clvd()])
+    rcv = orc.seabed_receivers(cs, pml, 3, 3)
+    with es.Model(rho, cp, cs, dx=10.0, pml=pml) as m:
+        m.batch_set(pos, mts, np.stack([w, w]))
+        got = m.run(nt, dt, rcv)
+    ref = orc.simulate(rho, cp, cs, dx=10.0, dt=dt, nt=nt, pml=pml, receivers=rcv,
+                       sources=[dict(kind="moment", pos=tuple(pos[0]), m=mts[0], w=w)])["traces"]
+    assert trace_errors(got[0], ref).max() < 1e-4
+    with es.Model(rho, cp, cs, dx=10.0, pml=pml) as m:
+        m.source_set(pos[1], mts[1], w)
+        assert np.array_equal(m.run(nt, dt, rcv), got[1])
