@@ -110,6 +110,16 @@ int forward(es_sur* s, const float* pos, const float* mt, int B, float* out = nu
     return ES_OK;
 }
 
+// Whether a training step takes the decoder's Adam step in the GEMM that forms its gradient, which has
+// one stage for its operands: a tile's k-blocks (64 of the batch) come one after another, and past seven of
+// them take longer than the weights they hide behind.  Above that the gradient is written and read by the
+// element-wise step, as it was before the two were one.  ms a training step in one and in two (one GB300;
+// 4608 x 262144 weights): batch 256 7.03 and 8.43, 384 8.71 and 9.11, 448 9.41 and 9.27, 512 9.96 and 9.38, 1024
+// 15.56 and 11.57 (13.40 before both); 384 x 65536: 384 0.439 and 0.453, 448 0.467 and 0.470, 512 0.493 and
+// 0.489.  Weights that stay in L2 (1536 x 2048): 512 0.206 and 0.211, 768 0.2295 and 0.2298, 1024 0.264 and
+// 0.257.
+bool adam_in_gemm(long long weights, int batch) { return batch < 448 || (batch <= 768 && weights <= 1LL << 23); }
+
 // gradients into s->g, given s->dUb and s->dUT from the loss; the decoder's only with `decoder` (a training
 // step takes it in the GEMM that updates the decoder)
 int backward(es_sur* s, const float* mt, int B, bool decoder = true)
@@ -329,13 +339,18 @@ int es_sur_train_step(es_sur* s, const float* pos, const float* mt, const float*
     cudaGetLastError();
     if ((rc = forward(s, pos, mt, B)) != ES_OK) return rc;
     CKS(sur_loss(s->U, target, s->scale, B, s->D / 4, 1e-30f, s->dUb, s->dUT, s->loss, s->acc, nullptr, s->st));
-    if ((rc = backward(s, mt, B, false)) != ES_OK) return rc;
+    const bool fused = adam_in_gemm(6LL * s->K * s->D, B);
+    if ((rc = backward(s, mt, B, !fused)) != ES_OK) return rc;
     s->t += 1;
-    // the decoder (the last segment) in the GEMM that forms its gradient, both BF16 copies with it;
-    // then the MLP's parameters
+    // the decoder (the last segment) in the GEMM that forms its gradient, or after it, both BF16 copies
+    // with it; then the MLP's parameters
     const size_t wd = s->oWd;
-    CKS(gemm_adam_tc(6 * s->K, (int)s->D, B, s->ZT, B, s->dUT, B, s->p + wd, s->m + wd, s->v + wd, lr, 0.9f, 0.999f,
-                     1e-8f, s->t, s->pb + wd, s->WdT, s->st));
+    if (fused)
+        CKS(gemm_adam_tc(6 * s->K, (int)s->D, B, s->ZT, B, s->dUT, B, s->p + wd, s->m + wd, s->v + wd, lr, 0.9f, 0.999f,
+                         1e-8f, s->t, s->pb + wd, s->WdT, s->st));
+    else
+        CKS(sur_adam_t(s->p + wd, s->g + wd, s->m + wd, s->v + wd, 6 * s->K, s->D, lr, 0.9f, 0.999f, 1e-8f, s->t,
+                       s->pb + wd, s->WdT, s->st));
     CKS(sur_adam(s->p, s->g, s->m, s->v, wd, lr, 0.9f, 0.999f, 1e-8f, s->t, s->pb, s->st));
     s->ver += 1;
     s->wdt_ver = s->ver;

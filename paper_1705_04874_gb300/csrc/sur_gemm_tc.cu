@@ -371,9 +371,10 @@ __global__ void __launch_bounds__(THREADS, 1)
 //
 // What bounds it is HBM: 28 bytes per weight (p, m, v read and written, two BF16
 // copies written) against 36 with the gradient written by one kernel and read by
-// the next.  A tile is 128 x 128 and K is one batch, a few k-blocks, so one
-// operand stage is enough (the MMAs run a tile ahead of the epilogue) and the
-// rest of shared memory moves the weights: each of eight epilogue warps walks
+// the next.  A tile is 128 x 128 and K is one batch: up to seven k-blocks (larger
+// batches go to two kernels, adam_in_gemm in es_sur.cu) one operand stage is
+// enough (the MMAs run a tile ahead of the epilogue) and the rest of shared
+// memory moves the weights: each of eight epilogue warps walks
 // 32 x 32 blocks of p, m and v through two places of its own, one block arriving
 // by TMA while the other is updated in place and leaves by TMA.  A lane holds a
 // row, as tcgen05.ld delivers the gradient, so nothing is turned around but the

@@ -473,3 +473,41 @@ def test_products_large_enough_for_pairs(env, M, N, K, split, beta):
     sur.es_gemm_bf16(A, B, C, b_nk=True, beta=beta, split_k=split)
     sur.es_gemm_status()
     assert float((C - want).abs().max()) <= 2e-5 * float(want.abs().max())
+
+
+@pytest.mark.parametrize("latent, n_rcv, nt, B", [
+    (8, 3, 24, 768),      # the largest batch whose step stays in the gradient GEMM while the weights fit in L2
+    (8, 3, 24, 776),      # the smallest past it: gradient and step apart
+    (48, 37, 208, 440),   # 8.9 M weights: in the GEMM below 448
+    (48, 37, 208, 448),   # and apart from there on; 288 rows and 30784 columns, ragged tiles of 64
+])
+def test_decoder_step_on_both_sides_of_its_rule(env, latent, n_rcv, nt, B):
+    """One training step against Adam in FP64 on the gradient that loss_grad returns, where that is not tiny
+    (|g| > 0.1 rms): the two FP32 sums of at most 776 products differ by about 1e-6 of their size, so the first
+    step, lr g / |g|, agrees to 1e-3.  Then both BF16 copies equal those of a network given the parameters."""
+    es, sur, torch = env
+    args = dict(nfreq=1, hidden=16, latent=latent, max_batch=B)
+    s, f = sur.Surrogate(n_rcv, nt, seed=3, **args), sur.Surrogate(n_rcv, nt, seed=4, **args)
+    D, lr = 4 * n_rcv * nt, 1e-2
+    try:
+        g = torch.Generator().manual_seed(B)
+        r = lambda *n: torch.randn(*n, generator=g).cuda()
+        pos, mt, tgt = r(B, 3).clamp(-1, 1), r(B, 6), r(B, D)
+        s.set_params((np.random.default_rng(B).standard_normal(s.num_params()) * 0.2).astype(np.float32))
+        wd = slice(s.num_params() - 6 * latent * D, s.num_params())
+        before = s.get_params()[wd].astype(np.float64)
+        grad = s.loss_grad(pos, mt, tgt)[2].cpu().numpy()[wd].astype(np.float64)
+        s.train_step(pos, mt, tgt, lr)
+        after = s.get_params()[wd].astype(np.float64)
+        m, v = 0.1 * grad, 0.001 * grad * grad
+        want = -lr * (m / (1 - 0.9)) / (np.sqrt(v / (1 - 0.999)) + 1e-8)
+        sure = np.abs(grad) > 0.1 * np.sqrt(np.mean(grad * grad))
+        assert sure.mean() > 0.5
+        assert np.abs(after - before - want)[sure].max() <= 1e-3 * lr
+        f.set_params(s.get_params())
+        assert torch.equal(s.predict(pos, mt), f.predict(pos, mt))
+        a, b = (x.loss_grad(pos, mt, tgt)[2][:wd.start] for x in (s, f))  # through the row-major copy
+        assert float((a - b).norm()) <= 1e-5 * float(b.norm())
+    finally:
+        s.close()
+        f.close()
