@@ -203,6 +203,8 @@ __global__ void __launch_bounds__(THREADS) gemm_bf16_kernel(int M, int N, int K,
 // against 11.2 (weights) and 9.4 against 14.6 + 3.8 (tcgen05, 6 CTAs; rows).  A
 // training step of a small network (hidden layers of 128, decoder 96 x 256) falls
 // from 218 to 149 us, a serving batch of 1024 at full size from 1.82 to 1.78 ms.
+// Products with many tiles go to the general kernels and a pass of their own for
+// the elementwise step (small_layer).
 constexpr int LM = 32, LN = 64, LK = 64, LS = 5, LTHREADS = 128;
 
 template <bool AT, bool BNK>
@@ -326,6 +328,48 @@ layer_kernel(int M, int N, int K, const __nv_bfloat16* __restrict__ A, int lda, 
         }
 }
 
+// The elementwise step of a layer on its stored product, four columns per thread (N a multiple of 8)
+__global__ void mlp_epilogue_kernel(float* C, size_t n4, int N, const MlpEpilogue ep)
+{
+    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n4; i += (size_t)gridDim.x * blockDim.x) {
+        float4 x = reinterpret_cast<const float4*>(C)[i];
+        if (ep.bias) {
+            const float* b = ep.bias + 4 * i % N;
+            x = make_float4(x.x + b[0], x.y + b[1], x.z + b[2], x.w + b[3]);
+        }
+        if (ep.relu) x = make_float4(fmaxf(x.x, 0.f), fmaxf(x.y, 0.f), fmaxf(x.z, 0.f), fmaxf(x.w, 0.f));
+        if (ep.mask) {
+            const float4 k = reinterpret_cast<const float4*>(ep.mask)[i];
+            x = make_float4(k.x > 0.f ? x.x : 0.f, k.y > 0.f ? x.y : 0.f, k.z > 0.f ? x.z : 0.f, k.w > 0.f ? x.w : 0.f);
+        }
+        reinterpret_cast<float4*>(C)[i] = x;
+        if (ep.copy) {
+            reinterpret_cast<__nv_bfloat162*>(ep.copy)[2 * i] = __floats2bfloat162_rn(x.x, x.y);
+            reinterpret_cast<__nv_bfloat162*>(ep.copy)[2 * i + 1] = __floats2bfloat162_rn(x.z, x.w);
+        }
+    }
+}
+
+// Whether a product runs in 32 x 64 tiles, by how many CTAs that takes.  The device holds three per SM at
+// once; past that the general kernels' larger tiles pay, the deeper the product the sooner.  General kernel
+// and element-wise step / this one (one GB300, 152 SMs; CTAs x K): rows [M][K] times [K][N] 768 x 4096 1.04,
+// 768 x 512 1.25, 1024 x 512 0.92 .. 1.03, 1024 x 4096 0.80, 32768 x 256 1.16, 32768 x 4096 0.61; weight
+// gradients (A transposed) 576 x 4096 1.02, 768 x 1024 0.95, 1024 x 1024 0.72; B transposed (tcgen05) 384 x
+// 4096 1.00, 576 x 768 1.00, 768 x 512 1.23, 1024 x 512 0.95, 1536 x 256 1.00, 4096 x 64 1.10, 2048 x 4096 0.30.
+// The outer product's six copies are worth the epilogue at every size (32768 x 4096: 0.95).
+cudaError_t small_layer(int M, int N, int K, bool a_t, bool b_nk, const MlpEpilogue& ep, bool* small)
+{
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const long long ctas = (long long)((M + LM - 1) / LM) * ((N + LN - 1) / LN);
+    if (ep.outer) *small = true;
+    else if (a_t) *small = ctas <= 4LL * sms;
+    else if (b_nk) *small = ctas <= 3LL * sms || ctas * K <= 2560LL * sms;
+    else *small = ctas <= 6LL * sms || K <= 256;
+    return e;
+}
+
 template <bool AT, bool BNK>
 cudaError_t launch_layer(int M, int N, int K, const __nv_bfloat16* A, int lda, const __nv_bfloat16* B, int ldb, float* C,
                          const MlpEpilogue& ep, cudaStream_t st)
@@ -344,7 +388,18 @@ cudaError_t gemm_layer(int M, int N, int K, const __nv_bfloat16* A, int lda, boo
                        bool b_nk, float* C, const MlpEpilogue& ep, cudaStream_t st)
 {
     if (M <= 0 || N <= 0 || K <= 0) return cudaSuccess;
-    if (N % 8 || (a_t && b_nk)) return cudaErrorInvalidValue;
+    if (N % 8 || (a_t && b_nk) || (!C && !ep.outer)) return cudaErrorInvalidValue;
+    bool small = true;
+    cudaError_t e = small_layer(M, N, K, a_t, b_nk, ep, &small);
+    if (e != cudaSuccess) return e;
+    if (!small) {
+        e = gemm_bf16(M, N, K, A, lda, a_t, B, ldb, b_nk, C, N, 1.f, 0.f, 1, st);
+        if (e != cudaSuccess || !(ep.bias || ep.relu || ep.mask || ep.copy)) return e;
+        const size_t n4 = (size_t)M * N / 4;
+        const size_t blocks = (n4 + 255) / 256;
+        mlp_epilogue_kernel<<<(unsigned)(blocks < 65536 ? blocks : 65536), 256, 0, st>>>(C, n4, N, ep);
+        return cudaGetLastError();
+    }
     if (a_t) return launch_layer<true, false>(M, N, K, A, lda, B, ldb, C, ep, st);
     if (b_nk) return launch_layer<false, true>(M, N, K, A, lda, B, ldb, C, ep, st);
     return launch_layer<false, false>(M, N, K, A, lda, B, ldb, C, ep, st);

@@ -19,8 +19,9 @@ struct MlpEpilogue {
     const float* m6 = nullptr;        // with outer: outer[r][k N + c] = m6[r][k] x, k < 6 (BF16)
     __nv_bfloat16* outer = nullptr;
 };
-// C[M][N] = op(A) op(B) through the epilogue (C may be null; N a multiple of 8), for products too
-// small to fill the device in 128 x 128 tiles; see layer_kernel in sur_gemm.cu
+// C[M][N] = op(A) op(B) through the epilogue (N a multiple of 8; C may be null with an outer product), for
+// products too small to fill the device in 128 x 128 tiles by layer_kernel in sur_gemm.cu, the others by the
+// general kernels
 cudaError_t gemm_layer(int M, int N, int K, const __nv_bfloat16* A, int lda, bool a_t, const __nv_bfloat16* B, int ldb,
                        bool b_nk, float* C, const MlpEpilogue& ep, cudaStream_t st);
 

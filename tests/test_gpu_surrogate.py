@@ -511,3 +511,10 @@ def test_decoder_step_on_both_sides_of_its_rule(env, latent, n_rcv, nt, B):
     finally:
         s.close()
         f.close()
+
+
+def test_encoder_layers_past_the_small_tiles(env):
+    """Hidden layers of 1544 units and a batch of 1280: the second layer, its weight gradient and the gradient of
+    its input (1000, 1225 and 1000 small tiles, 1544, 1280 and 1544 deep) each run through a general kernel and
+    the element-wise pass, the other products in small tiles; same formulas and bound as above."""
+    test_encoder_layers_at_ragged_sizes(env, 1544, 24, 1280, 3)
