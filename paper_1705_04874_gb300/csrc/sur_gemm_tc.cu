@@ -274,8 +274,13 @@ __global__ void __launch_bounds__(THREADS, 1)
                 uint32_t acc[32];
                 tmem_ld32(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(b * TN + c0), acc);
                 float4* srow = reinterpret_cast<float4*>(stage + lane * EPI_LD);
-                if (!PROBE && span) {
-                    // per-column alpha: columns [c span, (c + 1) span) of C take component c of alpha4
+                // per-column alpha: columns [c span, (c + 1) span) of C take component c of alpha4, one choice
+                // for a block that lies within a component (64 sources x 262144 outputs with 192 inputs, one
+                // GB300: a serving batch 78 us, 137 and 151 with a choice per column)
+                auto comp = [&](int col) { return (col >= span) + (col >= 2 * span) + (col >= 3 * span); };
+                const int first = n0 + c0, c4 = !PROBE && span ? comp(first) : -1;
+                const float one = c4 < 0 ? alpha : c4 == 0 ? alpha4.x : c4 == 1 ? alpha4.y : c4 == 2 ? alpha4.z : alpha4.w;
+                if (c4 >= 0 && comp(first + 31) != c4) {  // (a block on a component's edge)
                     float a[32];
 #pragma unroll
                     for (int j = 0; j < 32; ++j) {
@@ -289,8 +294,8 @@ __global__ void __launch_bounds__(THREADS, 1)
                 } else {
 #pragma unroll
                     for (int j = 0; j < 8; ++j)
-                        srow[j] = make_float4(alpha * __uint_as_float(acc[4 * j]), alpha * __uint_as_float(acc[4 * j + 1]),
-                                              alpha * __uint_as_float(acc[4 * j + 2]), alpha * __uint_as_float(acc[4 * j + 3]));
+                        srow[j] = make_float4(one * __uint_as_float(acc[4 * j]), one * __uint_as_float(acc[4 * j + 1]),
+                                              one * __uint_as_float(acc[4 * j + 2]), one * __uint_as_float(acc[4 * j + 3]));
                 }
                 __syncwarp();
                 // lane l stores columns 4 (l mod 8) .. +3 of row 4 i + l / 8: a warp instruction writes

@@ -518,3 +518,23 @@ def test_encoder_layers_past_the_small_tiles(env):
     its input (1000, 1225 and 1000 small tiles, 1544, 1280 and 1544 deep) each run through a general kernel and
     the element-wise pass, the other products in small tiles; same formulas and bound as above."""
     test_encoder_layers_at_ragged_sizes(env, 1544, 24, 1280, 3)
+
+
+@pytest.mark.parametrize("n_rcv, nt", [(1, 8), (3, 24), (5, 40), (4, 64)])
+@pytest.mark.parametrize("B", [8, 136])
+def test_component_scales_across_column_blocks(env, n_rcv, nt, B):
+    """Served outputs take their component's scale 32 columns at a time, or column by column in a block on a
+    component's edge (components of 8, 72 and 200 columns; of 256, none).  Scales that are powers of two
+    change nothing else, so the outputs are exact multiples."""
+    es, sur, torch = env
+    s = sur.Surrogate(n_rcv, nt, nfreq=1, hidden=16, latent=8, max_batch=B, seed=5)
+    try:
+        g = torch.Generator().manual_seed(B + nt)
+        pos, mt = torch.randn(B, 3, generator=g).clamp(-1, 1).cuda(), torch.randn(B, 6, generator=g).cuda()
+        one = s.predict(pos, mt)
+        scale = [2.0, 0.25, 8.0, 0.5]
+        s.set_output_scale(scale)
+        want = one.view(B, 4, -1) * torch.tensor(scale, device="cuda")[None, :, None]
+        assert torch.equal(s.predict(pos, mt).view(B, 4, -1), want)
+    finally:
+        s.close()
