@@ -223,7 +223,8 @@ layer_kernel(int M, int N, int K, const __nv_bfloat16* __restrict__ A, int lda, 
     extern __shared__ __align__(128) __nv_bfloat16 ring[];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int wm = warp >> 1, wn = warp & 1;
-    const int m0 = blockIdx.y * LM, n0 = blockIdx.x * LN;
+    const int ntn = (N + LN - 1) / LN;  // tiles in a row of them; rows in one dimension, which takes any batch
+    const int m0 = (int)(blockIdx.x / ntn) * LM, n0 = (int)(blockIdx.x % ntn) * LN;
     const int nk = (K + LK - 1) / LK;
 
     auto load = [&](int t) {
@@ -377,8 +378,9 @@ cudaError_t launch_layer(int M, int N, int K, const __nv_bfloat16* A, int lda, c
     constexpr int bytes = LayerTile<AT, BNK>::BYTES;
     const cudaError_t e = cudaFuncSetAttribute(layer_kernel<AT, BNK>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
     if (e != cudaSuccess) return e;
-    const dim3 grid((N + LN - 1) / LN, (M + LM - 1) / LM);
-    layer_kernel<AT, BNK><<<grid, LTHREADS, bytes, st>>>(M, N, K, A, lda, B, ldb, C, ep);
+    const long long ctas = (long long)((M + LM - 1) / LM) * ((N + LN - 1) / LN);
+    if (ctas > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
+    layer_kernel<AT, BNK><<<(unsigned)ctas, LTHREADS, bytes, st>>>(M, N, K, A, lda, B, ldb, C, ep);
     return cudaGetLastError();
 }
 

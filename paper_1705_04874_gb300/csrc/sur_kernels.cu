@@ -105,18 +105,21 @@ __global__ void loss_sums_kernel(const float* U, const float* T, const float* sc
 constexpr int LT = 64, LT_LD = LT + 2;
 __global__ void __launch_bounds__(256) loss_grad_kernel(const float* U, const float* T, const float* scale, int B,
                                                         long long Dc, float eps, const float2* acc, __nv_bfloat16* dU,
-                                                        __nv_bfloat16* dUT, float* loss, float* per_sample, bool vec)
+                                                        __nv_bfloat16* dUT, float* loss, float* per_sample, bool vec,
+                                                        int nx)
 {
     __shared__ __align__(16) __nv_bfloat16 tt[LT][LT_LD];
     __shared__ float g[LT];
-    const long long D = 4 * Dc, d0 = (long long)blockIdx.x * LT;
-    const int b0 = blockIdx.y * LT;
+    // column tiles fastest, in one dimension (any number of samples)
+    const int tx = blockIdx.x % nx;
+    const long long D = 4 * Dc, d0 = (long long)tx * LT;
+    const int b0 = (int)(blockIdx.x / nx) * LT;
     if (threadIdx.x < LT && b0 + (int)threadIdx.x < B) {
         const int b = b0 + threadIdx.x;
         const float2 a0 = acc[4 * b], a1 = acc[4 * b + 1], a2 = acc[4 * b + 2], a3 = acc[4 * b + 3];
         const float den = a0.y + a1.y + a2.y + a3.y + eps;
         g[threadIdx.x] = 2.f / ((float)B * den);
-        if (blockIdx.x == 0) {
+        if (tx == 0) {
             const float lb = (a0.x + a1.x + a2.x + a3.x) / den;
             if (per_sample) per_sample[b] = lb;
             atomicAdd(loss, lb / B);
@@ -331,9 +334,10 @@ cudaError_t sur_loss(const float* U, const float* T, const float* scale, int B, 
     float2* sums = reinterpret_cast<float2*>(acc);
     loss_sums_kernel<<<dim3(B, 4), 256, 0, st>>>(U, T, scale, Dc, sums);
     const long long nx = dU ? (4 * Dc + LT - 1) / LT : 1;
-    if (nx > 0x7fffffffLL) return cudaErrorInvalidValue;
-    loss_grad_kernel<<<dim3((unsigned)nx, (B + LT - 1) / LT), 256, 0, st>>>(
-        U, T, scale, B, Dc, eps, sums, dU, dUT, loss, per_sample, (reinterpret_cast<uintptr_t>(T) & 15) == 0);
+    const long long tiles = nx * ((B + LT - 1) / LT);
+    if (tiles > 0x7fffffffLL) return cudaErrorInvalidValue;
+    loss_grad_kernel<<<(unsigned)tiles, 256, 0, st>>>(U, T, scale, B, Dc, eps, sums, dU, dUT, loss, per_sample,
+                                                     (reinterpret_cast<uintptr_t>(T) & 15) == 0, (int)nx);
     return cudaGetLastError();
 }
 

@@ -538,3 +538,29 @@ def test_component_scales_across_column_blocks(env, n_rcv, nt, B):
         assert torch.equal(s.predict(pos, mt).view(B, 4, -1), want)
     finally:
         s.close()
+
+
+def test_batches_of_millions(env):
+    """A small network serves 2.2 million sources at once (68,750 row tiles of the encoder) and takes the losses
+    of 4.3 million (67,188 tiles of the loss): each sample's result is that of a batch of 64."""
+    es, sur, torch = env
+    for B in (2_200_000, 4_300_000):
+        s = sur.Surrogate(1, 8, nfreq=0, hidden=8, latent=8, max_batch=B, seed=2)
+        try:
+            g = torch.Generator(device="cuda").manual_seed(1)
+            pos = torch.rand((B, 3), device="cuda", generator=g) * 2 - 1
+            mt = torch.randn((B, 6), device="cuda", generator=g)
+            tgt = torch.randn((B, s.D), device="cuda", generator=g)
+            ends = [slice(0, 64), slice(B - 64, B)]
+            if B < 3_000_000:
+                out = s.predict(pos, mt)
+                for e in ends:
+                    assert torch.equal(out[e], s.predict(pos[e].contiguous(), mt[e].contiguous()))
+            else:
+                per = s.loss_grad(pos, mt, tgt, grads=False)[1]
+                for e in ends:
+                    assert torch.equal(per[e], s.loss_grad(pos[e].contiguous(), mt[e].contiguous(), tgt[e].contiguous(),
+                                                           grads=False)[1])
+        finally:
+            s.close()
+            torch.cuda.empty_cache()
