@@ -90,3 +90,28 @@ def test_bounds_checked_build_runs_clean():
         assert v["bad"] == 0, (case, v["bad"] >> 40, v["bad"] & ((1 << 40) - 1))
         if "err" in v:
             assert v["err"] < 1e-4, (case, v["err"])
+
+
+def test_convolution_axes_with_pml_stay_in_bounds():
+    """Convolution axes with PML, sources and receivers in the bounds-checked build: x (even and odd lengths), y
+    and z, a batch whose simulations start off 16-byte boundaries, a ragged last tile, the longest transform."""
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    child = CHILD[:CHILD.index("out['fft_even']")] + r"""
+out['conv_xyz'] = run((66, 65, 98), 5, 30)
+out['conv_odd_x'] = run((70, 67, 97), 4, 30, d=(12.5, 12.5, 10.0))
+out['conv_batch'] = run((65, 27, 101), 5, 15, nb=3, oracle=False)
+out['conv_long'] = run((17, 19, 331), 4, 20)
+out['conv_long_z'] = run((313, 16, 34), 4, 20)
+print('RESULT ' + json.dumps(out))
+"""
+    env = dict(os.environ, ES_BOUNDS="1")
+    r = subprocess.run([sys.executable, "-c", "ROOT = %r\n" % ROOT + child], env=env, capture_output=True, text=True,
+                       timeout=1500)
+    assert r.returncode == 0, r.stdout[-2000:] + r.stderr[-4000:]
+    res = json.loads([l for l in r.stdout.splitlines() if l.startswith("RESULT ")][-1][len("RESULT "):])
+    for case, v in res.items():
+        assert v["bad"] == 0, (case, v["bad"] >> 40, v["bad"] & ((1 << 40) - 1))
+        if "err" in v:
+            assert v["err"] < 1e-4, (case, v["err"])
