@@ -166,3 +166,26 @@ def test_runs_on_one_tile_passes(es, orc, shape, pml):
     with es.Model(rho, cp, cs, dx=10.0, pml=pml) as m:
         m.source_set(pos[1], mts[1], w)
         assert np.array_equal(m.run(nt, dt, rcv), got[1])
+
+
+# either side of the shortest convolution axes (64 cells, an odd x axis 96) and both ends of every transform's range
+@pytest.mark.parametrize("n", [63, 65, 66, 78, 95, 97, 98, 126, 159, 162, 202, 252, 314, 511])
+@pytest.mark.parametrize("axis,others", [(0, (7, 9)), (1, (5, 36)), (2, (6, 35))])
+def test_quiet_half_beside_a_loud_one(es, orc, n, axis, others):
+    """Half of every line is 50 times louder, in space a step along the transformed axis.  The near taps round
+    locally; the far part's roundoff, at 2 % of the operator's weight and some 4 log2(1024) = 40 roundings,
+    spreads over the line, so the quiet half sees 50 x 0.02 x 40 x 2^-24 = 2.4e-6 of its own derivative, and the
+    few 1e-7 of its own rounding."""
+    import torch
+    shape = {0: (others[0], others[1], n), 1: (others[0], n, others[1]), 2: (n, others[0], others[1])}[axis]
+    f = np.random.default_rng(3 * n + axis).standard_normal(shape).astype(np.float32)
+    quiet, loud = [slice(None)] * 3, [slice(None)] * 3
+    quiet[2 - axis], loud[2 - axis] = slice(8, n // 2 - 8), slice(n // 2, n)
+    f[tuple(loud)] *= 50.0
+    out = torch.empty(shape, device="cuda")
+    for shift in (1, -1):
+        es.es_derivative(torch.from_numpy(f).cuda(), axis, 10.0, shift, out)
+        ref = orc.deriv(f.astype(np.float64), axis, 10.0, shift)
+        got = out.cpu().numpy()
+        assert rel_l2(got, ref) < 5e-7
+        assert rel_l2(got[tuple(quiet)], ref[tuple(quiet)]) < 3e-6
