@@ -24,25 +24,39 @@ constexpr bool one_tile(int n, int ra, int rb, int nx)
     return n % 2 ? ra < 25 : ra >= rb && (n < 64 || (n == 64 && nx % 4 != 0));
 }
 
+// ... unless all tiles fit on the device at once: then there is nothing to overlap, and the second trip to L2
+// for the stencil is what the one-tile kernel waits for.  us a step, one tile per CTA and persistent (tiles x
+// jobs of a y or z pass): 32^3 (96) 32.9 and 30.5, eight of them (768) 48.4 and 41.8, 32 (3072, past one round)
+// 98.3 and 116.1; 48^3 (288) 48.3 and 45.0, two (576) 53.4 and 47.7, eight (2304, past it) 78.8 and 104.7; 64 x 64
+// x 62 (384) 89.9 and 77.0, four (1536) 129.2 and 126.4, eight 234 and 238; 16^3 21.8 and 21.3.  Below 48 cells a
+// tile of few columns costs the persistent kernel more than that (32 x 32 x 34, two (384) 55.2 and 56.2, eight
+// 67.2 and 72.2), unless there are no more than two tiles per SM (one (192) 53.5 and 47.2).
+constexpr bool short_of_tiles(int n, int nx, int units, int sms)
+{
+    return n % 2 == 0 && (n >= 48 || nx % 32 == 0 || units <= 2 * sms);
+}
+
 template <int RA, int RB, int RC, int T, int V>
 static cudaError_t launch_strided_plan(int ntiles, const PassParams& p, cudaStream_t st)
 {
     constexpr int N = RA * RB * RC;
-    // the kernel of an nx that is a multiple of V and not of 4, and of one that is (V = 2 only)
-    constexpr bool once = one_tile(N, RA, RB, V), persists = !once || (V == 2 && !one_tile(N, RA, RB, 4));
-    if constexpr (once) {
-        if (one_tile(N, RA, RB, p.nx))
-            return launch_pass_kernel(pass_strided_once<RA, RB, RC, V>, dim3((unsigned)ntiles, (unsigned)p.njobs),
-                                      once_threads<RA, RB, RC>(), once_smem<RA, RB, RC>(), st, p, ntiles);
-    }
-    if constexpr (persists) {
+    const int units = ntiles * p.njobs;
+    bool once = one_tile(N, RA, RB, p.nx);
+    if constexpr (N % 2 == 0 || !one_tile(N, RA, RB, V)) {
         constexpr int threads = pass_threads<T>();
         constexpr size_t smem = pass_smem_strided<N, T>();
-        int grid = 0;
-        const cudaError_t e = persistent_grid(pass_strided<RA, RB, RC, T, V>, threads, smem, ntiles * p.njobs, &grid);
+        int grid = 0, dev = 0, sms = 0;
+        cudaError_t e = persistent_grid(pass_strided<RA, RB, RC, T, V>, threads, smem, units, &grid);
+        if (e == cudaSuccess) e = cudaGetDevice(&dev);
+        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         if (e != cudaSuccess) return e;
-        return launch_pass_kernel(pass_strided<RA, RB, RC, T, V>, dim3((unsigned)grid), threads, smem, st, p, ntiles);
+        if (once && grid == units && short_of_tiles(N, p.nx, units, sms)) once = false;
+        if (!once)
+            return launch_pass_kernel(pass_strided<RA, RB, RC, T, V>, dim3((unsigned)grid), threads, smem, st, p, ntiles);
     }
+    if constexpr (one_tile(N, RA, RB, V))
+        return launch_pass_kernel(pass_strided_once<RA, RB, RC, V>, dim3((unsigned)ntiles, (unsigned)p.njobs),
+                                  once_threads<RA, RB, RC>(), once_smem<RA, RB, RC>(), st, p, ntiles);
     return cudaErrorInvalidValue;
 }
 
@@ -61,7 +75,7 @@ static cudaError_t prepare_strided_plans()
 {
     cudaError_t e = cudaSuccess;
 #define ES_PREP(n, a, b, c, t)                                                                               \
-    if constexpr (!one_tile(n, a, b, V == 2 ? 4 : 1))                                                        \
+    if constexpr (n % 2 == 0 || !one_tile(n, a, b, V))                                                        \
         if (e == cudaSuccess)                                                                                 \
             e = cudaFuncSetAttribute(pass_strided<a, b, c, t, V>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
                                      (int)pass_smem_strided<n, t>());
