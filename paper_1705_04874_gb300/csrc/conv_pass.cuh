@@ -14,8 +14,13 @@
 // 5 log2 m operations, twice.  190^3 (m = 400), velocity / stress pass: x 0.307 /
 // 0.330 -> 0.187 / 0.199 ms, y and z 0.285 / 0.301 -> 0.146 / 0.160 ms; the
 // 301-cell z axis of the 125 x 75 x 301 grid (m = 625): 0.156 / 0.168 -> 0.078 /
-// 0.084 ms.  What bounds them is the shared memory a tile takes ((m + 2 n) rows),
-// which leaves 2 to 4 CTAs per SM, and the padded half of the transforms.
+// 0.084 ms.  What bounds them is the shared memory a tile takes ((m + 2 n) rows) and
+// the padded half of the transforms.  At the longest axis of each transform the y and z
+// passes have 5 CTAs on an SM (160 points), 4 (320), 3 (256 and 400), 2 (500 and 625)
+// and one (1024 points, every axis from 313 cells on: 130 to 156 KB).  Even that one
+// is ahead of the direct sum, ps per cell, velocity / stress: y and z 313 cells 55 / 58
+// -> 36 / 38, 400 64 / 69 -> 29 / 31, 512 72 / 74 -> 24 / 26; x 313 64 / 67 -> 41 / 43,
+// 512 125 / 133 -> 31 / 33.
 //
 // A CTA keeps the arriving tile (n rows), the FFT's rows (m) and the near parts
 // (n) in shared memory and is persistent, as the y and z passes are; the next
@@ -178,8 +183,7 @@ conv_strided(const __grid_constant__ PassParams p, int ntiles)
 // x pass: a tile is 2 PR consecutive x-lines, one contiguous block of memory;
 // blockIdx.y = job.  Staged and turned around four lines x eight cells per warp
 // (any length, any alignment); the derivatives go back to memory order through
-// the FFT's rows and out four cells per thread where every array they touch is
-// on a 16-byte boundary.
+// the FFT's rows and out four cells per thread (x_quads).
 template <int PR>
 __device__ __forceinline__ int conv_x_swz(int x)
 {
@@ -251,21 +255,15 @@ conv_x(const __grid_constant__ PassParams p)
     __syncthreads();
     if (p.pdl == 1) pdl_wait();  // the previous pass's updates of the targets come first
     const int nf = nl * n;
-    auto a16 = [](const float* q) { return ((uintptr_t)q & 15) == 0; };
-    bool vec = a16(J.tgt[0] + off + q0);
-    if (J.kind == JOB_NORMAL) vec = vec && a16(J.tgt[1] + off + q0) && a16(J.tgt[2] + off + q0) && a16(J.coef[1] + q0);
-    if (J.kind != JOB_STORE) vec = vec && a16(J.coef[0] + q0);
-    const int nq = vec ? nf / 4 : 0;
+    const XQuads xq = x_quads(J, off, q0, nf);
     const float inv = 1.f / (float)n;
     // line of the tile's cell f: floor((f + 1/2) / n), exact for these f < 2^15 (the nearest
     // multiple of 1 / n is at least 1 / (2 n) away, far above the rounding)
     auto line_of = [&](int f) { return (int)(((float)f + 0.5f) * inv); };
-    if (J.kind == JOB_STORE) x_quads_flat<NT, JOB_STORE>(p, J, bf, q0, line0, nq, n, off, soff, line_of);
-    else if (J.kind == JOB_SINGLE) x_quads_flat<NT, JOB_SINGLE>(p, J, bf, q0, line0, nq, n, off, soff, line_of);
-    else x_quads_flat<NT, JOB_NORMAL>(p, J, bf, q0, line0, nq, n, off, soff, line_of);
-    // what is left: unaligned tiles, a last, partial tile's cells past its last full chunk
-    for (int f = 4 * nq + tid; f < nf; f += NT) {
-        const int r = line_of(f), x = f - r * n, line = line0 + r;
+    x_quads_update<NT>(p, J, bf, q0, line0, xq, n, off, soff, line_of);
+    // what is left: the cells before the first chunk and past the last one
+    for (int i = tid; i < nf - 4 * xq.nq; i += NT) {
+        const int f = i < xq.h ? i : i + 4 * xq.nq, r = line_of(f), x = f - r * n, line = line0 + r;
         // the slab index along x is sp + S (y + ny z) = sp + S line: the line goes in as y, with z = 0
         epilogue_one(p, J, q0 + f, x, x, line, 0, bf[f], off, soff);
     }

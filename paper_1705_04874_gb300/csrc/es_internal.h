@@ -167,8 +167,9 @@ cudaError_t prepare_strided1();
 // cells 1.02 + 3.21 and 1.15 + 4.07, 45 0.95 + 2.19 and 1.04 + 2.48, 63 0.90 + 1.61 and 1.25 + 1.72,
 // 66 1.04 + 2.65 and 0.86 + 2.27, 72 1.02 + 2.37 and 0.81 + 1.91, 104 1.07 + 2.47 and 0.76 + 1.59
 // (24, 28 and 50 cells, just below a transform length, also gained, up to 14 %; the others lost).  An
-// odd x axis, whose tiles start off 16-byte boundaries: 81 cells 1.03 and 1.06, 127 1.09 and 0.97,
-// so from CONV_MIN_ODD_X on.
+// odd x axis in batches, whose simulations start off 16-byte boundaries: 81 cells 1.03 and 1.06, 127 1.09 and
+// 0.97, so from CONV_MIN_ODD_X on (with such tiles cell by cell; x_quads has since taken a quarter off the
+// longer ones).
 constexpr int CONV_MIN_N = 64, CONV_MIN_ODD_X = 96;
 int conv_length(int n, int axis);
 cudaError_t launch_conv(const PassParams& p, cudaStream_t st);
@@ -182,12 +183,13 @@ constexpr int CIRC_MAX_N = 512;
 // From this length on, the compensated circulant passes along y and z run their epilogue from
 // the registers.
 constexpr int CIRC_DIRECT_N = 192;
-// From this length on, circulant passes in FP32 mode run on the tensor cores (circ_tc.cu):
-// below it the CUDA-core pass is faster (measured at 75 and 125 cells: the scratch round trip
-// and the separate update kernel cost more than the O(n) multiply-adds they replace).
+// From this length on, axes without a plan run on the tensor cores in the opt-in mode (circ_tc.cu).  The line
+// is from when the alternative was the direct sum (below it the scratch round trip and the separate update
+// kernel cost more than the O(n) multiply-adds they replace).  The default mode's convolutions are the faster
+// ones at every length: z velocity + stress ps per cell, 301 cells 51 against 85, 512 cells 50 against 80.
 constexpr int CIRC_TC_N = 192;
 cudaError_t launch_circ(const PassParams& p, cudaStream_t st);
-// The circulant pass on the tensor cores (long z axes, FP32 mode; circ_tc.cu).
+// The circulant pass on the tensor cores (long axes, opt-in mode; circ_tc.cu).
 bool circ_tc_eligible(const PassParams& p);
 cudaError_t launch_circ_tc(const PassParams& p, cudaStream_t st);
 // reads and clears its device status word (bits set by waits that gave up)

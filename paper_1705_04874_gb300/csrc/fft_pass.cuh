@@ -1459,30 +1459,64 @@ __device__ __forceinline__ void x_item(int it, int* r, int* xx)
     *xx = 4 * (it / (CL * 2 * PAIRS) * CL + lo);
 }
 
-// Update of nq chunks of 4 consecutive cells of an x-pass tile in memory order
-// (16-byte aligned from linear index q0 on), the next chunk's coefficients in
-// flight.  A chunk may span two lines, so every cell takes its own x and line for
-// the PML split.
-template <int NT, int KIND, class LineOf>
+// The cells of an x-pass tile in memory order that are updated four at a time: nq chunks of four from the
+// h-th of its nf cells on, where the targets reach a 16-byte boundary (a simulation of an odd cell count
+// starts off one); on: from the first cell on, and the coefficients are on one too.  Tiles off a boundary
+// went cell by cell, a chain of coefficient, split and target for each: us a velocity and a stress x pass
+// (one GB300), five simulations of 14 x 75 x 75 28.2 and 33.4 -> 18.5 and 20.3, two of 75^3 36.2 and 40.9 -> 25.7
+// and 26.6; batches of 66 and 127 cells as convolutions 32.1 and 36.7 -> 25.6 and 27.8, 26.7 and 31.0 -> 19.6 and
+// 21.6 ps per cell.  The loops stay apart: one for both cost aligned 125-cell tiles 8 % in registers.
+struct XQuads {
+    int h, nq;
+    bool on;
+};
+__device__ __forceinline__ XQuads x_quads(const PassJob& J, size_t off, size_t q0, int nf)
+{
+    auto mis = [](const float* q) { return (int)((uintptr_t)q >> 2) & 3; };  // floats past the last boundary
+    const int m = mis(J.tgt[0] + off + q0);
+    XQuads x = {min((4 - m) & 3, nf), 0, m == 0};
+    bool same = true;
+    if (J.kind == JOB_NORMAL) {
+        same = mis(J.tgt[1] + off + q0) == m && mis(J.tgt[2] + off + q0) == m;
+        x.on = x.on && mis(J.coef[1] + q0) == 0;
+    }
+    if (J.kind != JOB_STORE) x.on = x.on && mis(J.coef[0] + q0) == 0;
+    if (same) x.nq = (nf - x.h) / 4;
+    else x.h = 0;
+    return x;
+}
+
+// Update of those chunks, the next one's coefficients in flight (ON: XQuads::on; else four loads each).  A
+// chunk may span two lines, so every cell takes its own x and line for the PML split.
+template <int NT, int KIND, bool ON, class LineOf>
 __device__ __forceinline__ void x_quads_flat(const PassParams& p, const PassJob& J, const float* bf, size_t q0, int line0,
-                                             int nq, int n, size_t off, size_t soff, LineOf line_of)
+                                             const XQuads& xq, int n, size_t off, size_t soff, LineOf line_of)
 {
     constexpr int TG = KIND == JOB_NORMAL ? 3 : 1;
+    const int nq = xq.nq, h = ON ? 0 : xq.h;
+    q0 += h;
+    bf += h;
     const float *co0 = J.coef[0] + q0, *co1 = J.coef[1] + q0;
     const float* prof = J.stag ? p.ps : p.pc;
     float* tgt[TG];
 #pragma unroll
     for (int k = 0; k < TG; ++k) tgt[k] = J.tgt[k] + off + q0;
     float4 c0 = make_float4(0.f, 0.f, 0.f, 0.f), c1 = c0;
+    auto four = [](const float* q) {
+        if constexpr (ON) return __ldg(reinterpret_cast<const float4*>(q));
+        else return make_float4(__ldg(q), __ldg(q + 1), __ldg(q + 2), __ldg(q + 3));
+    };
     auto coefs = [&](int i) {
         if (KIND == JOB_STORE || i >= nq || !ES_INB(p, q0 + 4 * i + 3, p.ext_c)) return;
-        c0 = __ldg(reinterpret_cast<const float4*>(co0) + i);
-        if (KIND == JOB_NORMAL) c1 = __ldg(reinterpret_cast<const float4*>(co1) + i);
+        c0 = four(co0 + 4 * i);
+        if (KIND == JOB_NORMAL) c1 = four(co1 + 4 * i);
     };
     coefs(threadIdx.x);
 #pragma unroll 1
     for (int i = threadIdx.x; i < nq; i += NT) {
-        const float4 d4 = reinterpret_cast<const float4*>(bf)[i], a4 = c0, b4 = c1;
+        const float4 a4 = c0, b4 = c1;
+        const float4 d4 = ON ? reinterpret_cast<const float4*>(bf)[i]
+                             : make_float4(bf[4 * i], bf[4 * i + 1], bf[4 * i + 2], bf[4 * i + 3]);
         coefs(i + NT);
         if (!ES_INB(p, off + q0 + 4 * i + 3, p.ext_f)) continue;
         if (KIND == JOB_STORE) {
@@ -1495,7 +1529,7 @@ __device__ __forceinline__ void x_quads_flat(const PassParams& p, const PassJob&
         float P[4], old[TG][4];
         unsigned slab = 0;
         if (p.L > 0) {
-            const int f = 4 * i, r = line_of(f), x = f - r * n;
+            const int f = h + 4 * i, r = line_of(f), x = f - r * n;
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
                 const int xe = x + e < n ? x + e : x + e - n, re = x + e < n ? r : r + 1;
@@ -1523,6 +1557,19 @@ __device__ __forceinline__ void x_quads_flat(const PassParams& p, const PassJob&
             atomicAdd(reinterpret_cast<float4*>(tgt[k]) + i, make_float4(v[0], v[1], v[2], v[3]));
         }
     }
+}
+
+// the same by the tile's alignment and the kind of job
+template <int NT, class LineOf>
+__device__ __forceinline__ void x_quads_update(const PassParams& p, const PassJob& J, const float* bf, size_t q0, int line0,
+                                               const XQuads& xq, int n, size_t off, size_t soff, LineOf line_of)
+{
+    if (J.kind == JOB_STORE && xq.on) x_quads_flat<NT, JOB_STORE, true>(p, J, bf, q0, line0, xq, n, off, soff, line_of);
+    else if (J.kind == JOB_STORE) x_quads_flat<NT, JOB_STORE, false>(p, J, bf, q0, line0, xq, n, off, soff, line_of);
+    else if (J.kind == JOB_SINGLE && xq.on) x_quads_flat<NT, JOB_SINGLE, true>(p, J, bf, q0, line0, xq, n, off, soff, line_of);
+    else if (J.kind == JOB_SINGLE) x_quads_flat<NT, JOB_SINGLE, false>(p, J, bf, q0, line0, xq, n, off, soff, line_of);
+    else if (xq.on) x_quads_flat<NT, JOB_NORMAL, true>(p, J, bf, q0, line0, xq, n, off, soff, line_of);
+    else x_quads_flat<NT, JOB_NORMAL, false>(p, J, bf, q0, line0, xq, n, off, soff, line_of);
 }
 
 // Epilogue of a tile of the x pass (lengths that are a multiple of 16): item by
@@ -1781,9 +1828,9 @@ pass_x(const __grid_constant__ PassParams p, int ntiles)
 
 // x pass for other lengths: blockIdx.x = tile of 32 consecutive x-lines,
 // blockIdx.y = job.  After the inverse transform the derivatives are turned
-// around through shared memory into memory order (the tile, 32 n floats from
-// line 32 k, starts on a 16-byte boundary), and a thread updates four
-// consecutive cells with 16-byte accesses where every array allows it.
+// around through shared memory into memory order, and a thread updates four
+// consecutive cells with 16-byte accesses from the targets' first 16-byte
+// boundary on (x_quads).
 template <int RA, int RB, int RC, int T>
 __global__ void __launch_bounds__(pass_threads<T>(), pass_min_blocks<RA, RB, RC, T>(1250))
 pass_x_any(const __grid_constant__ PassParams p)
@@ -1854,23 +1901,12 @@ pass_x_any(const __grid_constant__ PassParams p)
     if (p.pdl == 1) pdl_wait();
     const size_t q0 = (size_t)line0 * N;
     const int nf = nl * N;
-    // 16-byte chunks need every array they touch on a 16-byte boundary at the
-    // tile (the tile's own offset q0 is a multiple of 4 cells): the targets
-    // at this simulation's offset (an odd cell count per simulation leaves
-    // every other one unaligned) and the coefficient arrays, which a caller
-    // may pass at any 4-byte offset
-    auto a16 = [](const float* q) { return ((uintptr_t)q & 15) == 0; };
-    bool vec = a16(J.tgt[0] + off);
-    if (J.kind == JOB_NORMAL) vec = vec && a16(J.tgt[1] + off) && a16(J.tgt[2] + off) && a16(J.coef[1]);
-    if (J.kind != JOB_STORE) vec = vec && a16(J.coef[0]);
-    const int nq = vec ? nf / 4 : 0;
+    const XQuads xq = x_quads(J, off, q0, nf);
     auto line_of = [](int f) { return f / N; };
-    if (J.kind == JOB_STORE) x_quads_flat<NT, JOB_STORE>(p, J, bf, q0, line0, nq, N, off, soff, line_of);
-    else if (J.kind == JOB_SINGLE) x_quads_flat<NT, JOB_SINGLE>(p, J, bf, q0, line0, nq, N, off, soff, line_of);
-    else x_quads_flat<NT, JOB_NORMAL>(p, J, bf, q0, line0, nq, N, off, soff, line_of);
-    // what is left: a last, partial tile's cells past its last full chunk
-    for (int f = 4 * nq + tid; f < nf; f += NT) {
-        const int r = f / N, x = f - r * N, line = line0 + r;
+    x_quads_update<NT>(p, J, bf, q0, line0, xq, N, off, soff, line_of);
+    // what is left: the cells before the first chunk and past the last one
+    for (int i = tid; i < nf - 4 * xq.nq; i += NT) {
+        const int f = i < xq.h ? i : i + 4 * xq.nq, r = f / N, x = f - r * N, line = line0 + r;
         epilogue_one(p, J, q0 + f, x, x, line % p.ny, line / p.ny, bf[f], off, soff);
     }
 }
