@@ -364,7 +364,7 @@ __global__ void circ_tc_update_xy_kernel(const __grid_constant__ PassParams p)
             }
             float s = 0.f;
 #pragma unroll
-            for (int t = 0; t < NEAR_PAIRS; ++t) s = __fmaf_rn(J.g[t], __fsub_rn(v[t], v[NEAR_TAPS - 1 - t]), s);
+            for (int t = 0; t < NEAR_PAIRS; ++t) s = __fmaf_rn(J.g[NEAR_AT + t], __fsub_rn(v[t], v[NEAR_TAPS - 1 - t]), s);
             s = __fadd_rn(dv[k], s);
             if (p.axis == 0)
                 update_cell(p, J, q, (int)x, (int)x, (int)line, 0, s, off, soff);
@@ -403,7 +403,7 @@ __global__ void circ_tc_update_kernel(const __grid_constant__ PassParams p)
     for (int k = 0; k < UPD_Z; ++k) {
         float s = 0.f;
 #pragma unroll
-        for (int t = 0; t < NEAR_PAIRS; ++t) s = __fmaf_rn(J.g[t], __fsub_rn(v[k + t], v[k + NEAR_TAPS - 1 - t]), s);
+        for (int t = 0; t < NEAR_PAIRS; ++t) s = __fmaf_rn(J.g[NEAR_AT + t], __fsub_rn(v[k + t], v[k + NEAR_TAPS - 1 - t]), s);
         dv[k] = __fadd_rn(dv[k], s);
     }
 #pragma unroll

@@ -7,20 +7,20 @@
 // pass is the FFT pass of fft_pass.cuh with transforms of a length m that has a
 // plan, a multiplier that is the m-point transform of the (far) kernel, n rows
 // of input and n of output; the kernel is real, so two pencils still share a
-// complex line.  The near stencil is the same, wrapped at n.
+// complex line.  The near stencil is longer (CONV_TAPS, es_internal.h) and wraps at n.
 //
 // Against the direct O(n) sum (circ_pass.cu, which the shortest axes and the
 // compensated mode keep) the work per cell falls from n multiply-adds to about
-// 5 log2 m operations, twice.  190^3 (m = 400), velocity / stress pass: x 0.307 /
-// 0.330 -> 0.187 / 0.199 ms, y and z 0.285 / 0.301 -> 0.146 / 0.160 ms; the
-// 301-cell z axis of the 125 x 75 x 301 grid (m = 625): 0.156 / 0.168 -> 0.078 /
-// 0.084 ms.  What bounds them is the shared memory a tile takes ((m + 2 n) rows) and
-// the padded half of the transforms.  At the longest axis of each transform the y and z
-// passes have 5 CTAs on an SM (160 points), 4 (320), 3 (256 and 400), 2 (500 and 625)
-// and one (1024 points, every axis from 313 cells on: 130 to 156 KB).  Even that one
-// is ahead of the direct sum, ps per cell, velocity / stress: y and z 313 cells 55 / 58
-// -> 36 / 38, 400 64 / 69 -> 29 / 31, 512 72 / 74 -> 24 / 26; x 313 64 / 67 -> 41 / 43,
-// 512 125 / 133 -> 31 / 33.
+// 5 log2 m operations, twice.  190^3 (m = 400), velocity / stress pass: x 0.312 /
+// 0.335 -> 0.211 / 0.221 ms, y and z 0.288 / 0.303 -> 0.166 / 0.176 ms; the
+// 301-cell z axis of the 125 x 75 x 301 grid (m = 625): 0.176 / 0.187 -> 0.086 /
+// 0.092 ms.  What bounds them is the shared memory a tile takes ((m + 2 n) rows) and
+// the registers of the radix-16 to 25 stages, which leave the y and z passes 4 CTAs on
+// an SM (160 points), 3 (256, 320 and 400), 2 (500 and 625) or one (1024 points, every
+// axis from 313 cells on: 130 to 156 KB), and the padded half of the transforms.  Even
+// the one is ahead of the direct sum, ps per cell, velocity / stress: y and z 313 cells
+// 55 / 58 -> 39 / 41, 400 64 / 69 -> 32 / 34, 512 72 / 74 -> 26 / 28; x 313 64 / 67 ->
+// 44 / 46, 512 125 / 133 -> 34 / 36.
 //
 // A CTA keeps the arriving tile (n rows), the FFT's rows (m) and the near parts
 // (n) in shared memory and is persistent, as the y and z passes are; the next
@@ -64,25 +64,25 @@ __host__ __device__ constexpr size_t conv_smem_x(int n)
     return sizeof(float2) * ((size_t)M * PR + (size_t)n * PR + 2 * (size_t)M);
 }
 
-// near_part for an axis length known at run time, R rows from e0 on, wrapped at n
+// near_part for an axis length known at run time, R rows from e0 on, wrapped at n: every row that is
+// read goes to all the sums that it has a tap in, so that R sums are live and not CONV_TAPS rows
 template <int R, class Row, class Put>
 __device__ __forceinline__ void near_part_n(const PassJob& J, int e0, int n, Row row, Put put)
 {
-    const int ofs = near_ofs(J.sign);
-    float2 w[R + NEAR_TAPS - 1];
+    const int ofs = conv_near_ofs(J.sign);
+    float2 s[R];
 #pragma unroll
-    for (int k = 0; k < R + NEAR_TAPS - 1; ++k) {
+    for (int q = 0; q < R; ++q) s[q] = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int k = 0; k < R + CONV_TAPS - 1; ++k) {
         int e = e0 + ofs + k;
         e = e < 0 ? e + n : e;
         e = e >= n ? e - n : e;
-        w[k] = e < n ? row(e) : make_float2(0.f, 0.f);
-        if (k >= NEAR_TAPS - 1) {
-            const int q = k - (NEAR_TAPS - 1);
-            float2 s = make_float2(0.f, 0.f);
+        const float2 w = e < n ? row(e) : make_float2(0.f, 0.f);
 #pragma unroll
-            for (int t = 0; t < NEAR_TAPS; ++t) s = fma2(rep2(J.g[t]), w[q + t], s);
-            if (e0 + q < n) put(e0 + q, s);
-        }
+        for (int q = 0; q < R; ++q)
+            if (k >= q && k - q < CONV_TAPS) s[q] = fma2(rep2(J.g[k - q]), w, s[q]);
+        if (k >= CONV_TAPS - 1 && e0 + k - (CONV_TAPS - 1) < n) put(e0 + k - (CONV_TAPS - 1), s[k - (CONV_TAPS - 1)]);
     }
 }
 

@@ -272,18 +272,20 @@ void axis_tables(int n, double d, int m_conv, std::vector<float2>& tw, std::vect
         }
         return acc;
     };
+    const int taps = m_conv > 0 ? CONV_TAPS : NEAR_TAPS;
+    auto tap_ofs = [&](int s) { return m_conv > 0 ? conv_near_ofs(s == 0 ? +1 : -1) : near_ofs(s == 0 ? +1 : -1); };
     for (int s = 0; s < 2; ++s) {
         float* g = s == 0 ? gp : gm;
-        const int ofs = near_ofs(s == 0 ? +1 : -1);
-        // the taps in antisymmetric pairs, g[NEAR_TAPS - 1 - t] = -g[t] (exact for the staggered
+        const int ofs = tap_ofs(s);
+        // the taps in antisymmetric pairs, g[taps - 1 - t] = -g[t] (exact for the staggered
         // kernel up to FP64 roundoff; enforced here so the passes can sum differences)
-        for (int t = 0; t < NEAR_PAIRS; ++t) {
-            g[t] = g[NEAR_TAPS - 1 - t] = 0.f;
-            if (n <= NEAR_TAPS) continue;
+        for (int t = 0; t < taps / 2; ++t) {
+            g[t] = g[taps - 1 - t] = 0.f;
+            if (n <= taps) continue;
             const double lo = kernel_entry(s, ((-(ofs + t)) % n + n) % n);  // (D f)_i = sum_l c_l f_{i - l}
-            const double hi = kernel_entry(s, ((-(ofs + NEAR_TAPS - 1 - t)) % n + n) % n);
+            const double hi = kernel_entry(s, ((-(ofs + taps - 1 - t)) % n + n) % n);
             g[t] = (float)(0.5 * (lo - hi));
-            g[NEAR_TAPS - 1 - t] = -g[t];
+            g[taps - 1 - t] = -g[t];
         }
     }
     if (ckp && ckm) {
@@ -304,8 +306,8 @@ void axis_tables(int n, double d, int m_conv, std::vector<float2>& tw, std::vect
         for (int s = 0; s < 2; ++s) {
             std::vector<double> far = s == 0 ? *ckp : *ckm;
             const float* g = s == 0 ? gp : gm;
-            for (int t = 0; t < NEAR_TAPS; ++t) {
-                const int delta = near_ofs(s == 0 ? +1 : -1) + t;  // (N f)_i gains g_t f_{i + delta}
+            for (int t = 0; t < taps; ++t) {
+                const int delta = tap_ofs(s) + t;  // (N f)_i gains g_t f_{i + delta}
                 far[((-delta) % n + n) % n] -= (double)g[t];
             }
             // lags 0 .. n-1 at 0 .. n-1, lags -1 .. -(n-1) at len-1 .. len-(n-1)
@@ -373,7 +375,7 @@ struct es_model {
     float* mat[NMAT] = {};
     float** d_fields = nullptr;
     float2 *tw[3] = {}, *hp[3] = {}, *hm[3] = {};
-    float gp[3][NEAR_TAPS] = {}, gm[3][NEAR_TAPS] = {};  // near taps of D(+), D(-) per axis (FFT passes)
+    float gp[3][CONV_TAPS] = {}, gm[3][CONV_TAPS] = {};  // near taps of D(+), D(-) per axis (FFT passes)
     float *ckp[3] = {}, *ckm[3] = {};  // circulant kernels (axes without an FFT pass)
     float *ckp_lo[3] = {}, *ckm_lo[3] = {};  // their low parts (compensated mode)
     __nv_bfloat16* ctc[3] = {};               // long circulant axes: kernel matrices split in three BF16 parts
@@ -519,7 +521,7 @@ cudaError_t upload_axis_tables(es_model* m, int a)
             std::vector<__nv_bfloat16> sp(6 * mat, __float2bfloat16(0.f));
             for (int sgn = 0; sgn < 2; ++sgn) {
                 std::vector<double> ck = sgn == 0 ? ckp : ckm;
-                const float* g = sgn == 0 ? m->gp[a] : m->gm[a];
+                const float* g = (sgn == 0 ? m->gp[a] : m->gm[a]) + NEAR_AT;
                 for (int t = 0; t < NEAR_TAPS; ++t) {
                     const int delta = near_ofs(sgn == 0 ? +1 : -1) + t;  // (N f)_o gains g_t f_{o + delta}
                     ck[(size_t)(((-delta) % n) + n) % n] -= (double)g[t];
@@ -653,7 +655,7 @@ PassParams make_pass(const es_model* m, int axis, bool stress, float dt)
     p.ext_c = p.fstride;
     p.bad = bounds_word();
     auto taps = [&](PassJob& J) {
-        for (int t = 0; t < NEAR_TAPS; ++t) J.g[t] = J.sign > 0 ? m->gp[axis][t] : m->gm[axis][t];
+        std::copy_n(J.sign > 0 ? m->gp[axis] : m->gm[axis], CONV_TAPS, J.g);
     };
     auto single = [&](PassJob& J, int src, int sign, int tgt, int coef) {
         J.src = m->f[src];
@@ -912,12 +914,12 @@ struct AxisTables {
     int n, m;
     bool circ;
     size_t at, len;  // at: twiddles, the two multipliers (len float2 each), circ: the two kernels (n floats each)
-    float gp[NEAR_TAPS], gm[NEAR_TAPS];
+    float gp[CONV_TAPS], gm[CONV_TAPS];
 };
 
 AxisTables pack_axis(int axis, int n, int nx, double d, std::vector<float>& h)
 {
-    AxisTables t;
+    AxisTables t = {};
     t.n = n;
     t.circ = !fft_axis(n, nx);
     t.m = t.circ ? conv_length(n, axis) : n;
@@ -968,7 +970,7 @@ cudaError_t derivative_pass(const AxisTables& t, const float* tab, const float* 
     p.job[0].kind = acc ? JOB_SINGLE : JOB_STORE;
     p.job[0].coef[0] = acc;
     p.job[0].sign = shift;
-    for (int k = 0; k < NEAR_TAPS; ++k) p.job[0].g[k] = shift > 0 ? t.gp[k] : t.gm[k];
+    std::copy_n(shift > 0 ? t.gp : t.gm, CONV_TAPS, p.job[0].g);
     return launch_pass(p, st);
 }
 

@@ -33,6 +33,15 @@ constexpr int NEAR_TAPS = 10;
 constexpr int NEAR_PAIRS = NEAR_TAPS / 2;
 // first tap offset o: D(+) (result at i + 1/2) reads i-4 .. i+5, D(-) reads i-5 .. i+4
 __host__ __device__ constexpr int near_ofs(int sign) { return sign > 0 ? -4 : -5; }
+// The convolution passes (axes without an FFT plan) take more of the kernel's centre.  The direct sums
+// that they stand in for round in proportion to a kernel that falls off as 1/l^2, so where the wave has
+// not arrived they are quiet; the far part's roundoff is the same at every distance, and with 10 taps
+// such traces were up to 53 times further from FP64 than the direct sum's (a 151-cell cube, 30 steps:
+// 9e-7 and 5e-5; with 24 taps 7e-6, with 32 and 48 4e-6 and 3e-6).  Four more taps cost a
+// convolution pass about 3 %: steps of 190^3 take 1.00 ms with 10, 1.12 with 24, direct 1.83.
+constexpr int CONV_TAPS = 24;
+constexpr int NEAR_AT = (CONV_TAPS - NEAR_TAPS) / 2;  // where the NEAR_TAPS central ones stand among them
+__host__ __device__ constexpr int conv_near_ofs(int sign) { return near_ofs(sign) - NEAR_AT; }
 
 // Storage of the split parts inside a PML slab: [0, L) and [n-1-L, n) along the
 // axis, every point whose whole- or half-index factor differs from 1.  y and z
@@ -54,7 +63,8 @@ struct PassJob {
     int sign;             // +1: D(+) (result at +d/2), -1: D(-)
     int stag;             // targets sit at half indices along this axis
     int diag;             // JOB_NORMAL: target index receiving lambda + 2 mu
-    float g[NEAR_TAPS];   // FFT passes: near taps of D(sign) (the multiplier tables hold H_far / n)
+    float g[CONV_TAPS];   // near taps of D(sign) (the multiplier tables hold H_far / n): CONV_TAPS of
+                          // them in a convolution pass, NEAR_TAPS in the others
 };
 
 struct SourceDev {
@@ -163,13 +173,12 @@ cudaError_t prepare_strided2();
 cudaError_t prepare_strided1();
 // Axis lengths without a plan, FP32 mode: zero-padded convolution passes (conv_pass.cuh) with
 // transforms of conv_length(n, axis) points (0: none, the direct sum), from CONV_MIN_N cells on.  ms
-// per 17 M cells, a step's two x passes + its four y and z passes, direct and as a convolution: 33
-// cells 1.02 + 3.21 and 1.15 + 4.07, 45 0.95 + 2.19 and 1.04 + 2.48, 63 0.90 + 1.61 and 1.25 + 1.72,
-// 66 1.04 + 2.65 and 0.86 + 2.27, 72 1.02 + 2.37 and 0.81 + 1.91, 104 1.07 + 2.47 and 0.76 + 1.59
-// (24, 28 and 50 cells, just below a transform length, also gained, up to 14 %; the others lost).  An
-// odd x axis in batches, whose simulations start off 16-byte boundaries: 81 cells 1.03 and 1.06, 127 1.09 and
-// 0.97, so from CONV_MIN_ODD_X on (with such tiles cell by cell; x_quads has since taken a quarter off the
-// longer ones).
+// per 17 M cells, a step's two x passes + its four y and z passes, direct and as a convolution: 66 cells
+// 1.05 + 2.63 and 0.94 + 2.56, 72 1.02 + 2.38 and 0.90 + 2.18, 104 1.06 + 2.44 and 0.82 + 1.82.  Shorter ones
+// lose, here with 10 taps: 33 cells 1.02 + 3.21 and 1.15 + 4.07, 45 0.95 + 2.19 and 1.04 + 2.48, 63 0.90 + 1.61
+// and 1.25 + 1.72 (24, 28 and 50, just below a transform length, gained up to 14 %).  An odd x axis in
+// batches, whose simulations start off 16-byte boundaries: 97 cells 1.11 and 0.90, 127 1.06 and 0.72; 81 were
+// even with 10 taps and such tiles cell by cell, so it is one from CONV_MIN_ODD_X on.
 constexpr int CONV_MIN_N = 64, CONV_MIN_ODD_X = 96;
 int conv_length(int n, int axis);
 cudaError_t launch_conv(const PassParams& p, cudaStream_t st);
@@ -186,7 +195,7 @@ constexpr int CIRC_DIRECT_N = 192;
 // From this length on, axes without a plan run on the tensor cores in the opt-in mode (circ_tc.cu).  The line
 // is from when the alternative was the direct sum (below it the scratch round trip and the separate update
 // kernel cost more than the O(n) multiply-adds they replace).  The default mode's convolutions are the faster
-// ones at every length: z velocity + stress ps per cell, 301 cells 51 against 85, 512 cells 50 against 80.
+// ones at every length: z velocity + stress ps per cell, 301 cells 55 against 85, 512 cells 55 against 80.
 constexpr int CIRC_TC_N = 192;
 cudaError_t launch_circ(const PassParams& p, cudaStream_t st);
 // The circulant pass on the tensor cores (long axes, opt-in mode; circ_tc.cu).

@@ -212,3 +212,31 @@ def test_x_tiles_off_every_boundary(es, orc, shape):
     ref = orc.simulate(rho, cp, cs, dx=10.0, dt=dt, nt=nt, pml=pml, receivers=rcv,
                        sources=[dict(kind="moment", pos=pos, m=synth.explosive(), w=w)])["traces"]
     assert trace_errors(one, ref).max() < 1e-4
+
+
+# both ends of every transform of the convolution passes
+@pytest.mark.parametrize("n,m", [(66, 160), (78, 160), (98, 256), (103, 256), (126, 256), (151, 320), (199, 400),
+                                 (202, 500), (252, 625), (314, 1024), (511, 1024)])
+@pytest.mark.parametrize("axis", [0, 1, 2])
+def test_silence_far_from_a_pulse(es, orc, n, m, axis):
+    """What a pulse leaves where its derivative is as good as zero, past the near taps (24).  An FFT of m points
+    leaves a few 2^-24 of the pulse's norm over sqrt(m), times the norm of the kernel's far part, in every row:
+    1.5 to 2.4 of them with this pulse, transforms and tables in 32 bits and a radix-free FFT on the host, so at
+    most 4.  (A near part of 10 taps leaves 3 to 4 times as much, 5 at the least.)"""
+    import torch
+    rng = np.random.default_rng(7 * n + axis)
+    x = np.arange(n)[:, None]
+    f = np.exp(-((x - n // 2 - rng.uniform(-1, 1, 320)) / rng.uniform(2, 4, 320)) ** 2) * rng.uniform(0.5, 2, 320)
+    f = np.where(abs(x - n // 2) <= 12, f, 0).astype(np.float32)
+    a = np.moveaxis(f.reshape(n, 10, 32), 0, 2 - axis).copy()
+    out = torch.empty(a.shape, device="cuda")
+    quiet = abs(x[:, 0] - n // 2) > 26
+    delta = np.moveaxis(np.eye(1, n)[0].reshape(n, 1, 1), 0, 2 - axis)
+    for shift in (1, -1):
+        c = np.moveaxis(orc.deriv(delta, axis, 10.0, shift), 2 - axis, 0).ravel()  # the circulant kernel
+        far = np.sort(abs(c))[:-24]
+        es.es_derivative(torch.from_numpy(a).cuda(), axis, 10.0, shift, out)
+        err = out.cpu().numpy() - orc.deriv(a.astype(np.float64), axis, 10.0, shift)
+        err = np.moveaxis(err, 2 - axis, 0)[quiet]
+        rms = np.sqrt((f.astype(np.float64) ** 2).sum(0).mean())
+        assert np.sqrt((err ** 2).mean()) < 4 * 2.0 ** -24 * rms * np.linalg.norm(far) / np.sqrt(m)
