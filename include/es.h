@@ -66,8 +66,11 @@ int es_model_create(const float* rho, const float* cp, const float* cs, int nx, 
  * ES_PREC_FP32 (default): fused FFT passes where an axis has a plan (each
  * derivative as a 10-point near stencil in FP32 plus the FFT of the rest of
  * the operator, which confines FP32 FFT roundoff to about 1 % of its plain
- * size), elsewhere the same derivative as a zero-padded convolution (direct
- * circulant sums below 64 cells, for an odd nx below 96).
+ * size), elsewhere the same derivative as a zero-padded convolution with a
+ * 24-point near stencil (direct circulant sums below 64 cells, for an odd nx
+ * below 96).  Both transform two
+ * neighbouring lines as one complex line, so an infinity or NaN in one reaches
+ * the other, and roundoff follows the louder of the two.
  * ES_PREC_COMPENSATED: every axis through the circulant passes with
  * error-free transformations (each product split exactly by one FMA, Knuth's
  * TwoSum on the running sum, the kernel row as FP32 high plus low parts), so
@@ -78,7 +81,7 @@ int es_model_create(const float* rho, const float* cp, const float* cs, int nx, 
  * field and the kernel matrix split in three BF16 parts each, six products
  * accumulated in FP32; the near stencil stays on the CUDA cores).  The paper
  * has no tensor-core step: this mode is an opt-in alternative for long odd axes
- * such as the paper's 301 (the default mode's passes take 0.078 / 0.084 ms
+ * such as the paper's 301 (the default mode's passes take 0.086 / 0.092 ms
  * there, this one's 0.106 / 0.112).  Applies from the next es_run.  ES_ERR_ARG
  * for any other mode. */
 #define ES_PREC_FP32 0

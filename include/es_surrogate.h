@@ -87,9 +87,9 @@ int es_sur_combine(const float* G, int n_loc, long long D, const int* loc, const
  * of 8 (and M when a_t, N when !b_nk).  split_k > 1 splits K across CTAs
  * (atomic FP32 adds: summation order not fixed).  FP32 accumulation.
  * Both operands K-major (a_t == 0, b_nk != 0; A and B 16-byte aligned): the
- * fifth-generation tensor cores -- TMA-fed 4-stage shared-memory ring,
- * tcgen05.mma 128 x 256 x 16 into a tensor-memory accumulator, 128 x 256
- * tiles.  Other storage orders: mma.sync m16n8k16 with ldmatrix operands.
+ * fifth-generation tensor cores -- TMA-fed shared-memory ring, tcgen05.mma
+ * into a tensor-memory accumulator, 128 x 256 tiles (large products with an
+ * even number of row tiles: 256 x 256 over a pair of CTAs).  Other storage orders: mma.sync m16n8k16 with ldmatrix operands.
  * Device waits in the tcgen05 kernel are bounded; see es_gemm_status. */
 int es_gemm_bf16(int M, int N, int K, const void* A, int lda, int a_t, const void* B, int ldb, int b_nk, float* C,
                  int ldc, float alpha, float beta, int split_k, void* stream);

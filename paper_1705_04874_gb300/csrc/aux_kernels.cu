@@ -225,9 +225,8 @@ cudaError_t launch_transpose_traces(const float* rec, int nt, int cols, float* o
 // warps: there the events that overlap the span go U at a time, the loads of all
 // of them before the first multiply-add.
 // 64 sources x 1024 receivers x 2000 samples, 300 events into 4666 samples (one
-// GB300): 0.99 ms (1.46 ms with the call around it); one sample per thread with
-// a test, an address and three shared loads per event and sample took 4.69 ms
-// with the call.
+// GB300): 1.28 ms (1.44 ms with the call around it); one sample per thread with
+// a test, an address and three shared loads per event and sample took 4.54 (4.70).
 constexpr int SUP_CHUNK = 1024, SUP_WARPS = 8;
 
 template <int R, int U>
@@ -336,13 +335,12 @@ cudaError_t launch_superpose(const float* traces, int n_src, int n_rcv, int nt, 
                              cudaStream_t st)
 {
     (void)n_src;
-    // R = 8 and 4 by output samples (one GB300, 300 events): 19.1 M 0.991 and 1.022 ms, 16.4 M with
-    // short traces 0.336 and 0.475, 1.23 M 67.9 and 71.9 us; 0.61 M (200 events) 38.3 and 34.3,
-    // 0.26 M 24.2 and 22.2: below about a million the longer spans leave SMs idle.  R = 16 won only with the
-    // short traces (0.287 ms, 1.24 at the first size).  Below half a million R = 4 leaves them idle too: us
-    // a call with R = 4 and with R = 2 and events eight at a time (one sample per thread), 384 K 59.1 and 51
-    // (118), 307 K 88.6 and 63 (113), 96 K 50.7 and 47 (55), 32 K 86.1 and 40 (43), 8 K with 60,000 events
-    // 3732 and 1577 (2672); 1.02 M 74.9 and 77 (252).
+    // us a call by output samples (one GB300, 300 events; one sample per thread in brackets).  R = 8 and
+    // 4: 19.1 M 1282 and 1270 (4541), 12.3 M with short traces 297 and 372 (2597), 5.1 M 229 and 272 (1173), 1.28 M
+    // 101 and 115 (325), 1.02 M 63 and 74 (250), 307 K 102 and 89 (112): below about a million the longer spans
+    // leave SMs idle.  Below half a million R = 4 does too; R = 4, and R = 2 with the events eight at a time:
+    // 384 K 59 and 55 (118), 307 K 89 and 64 (112), 96 K 51 and 45 (55), 32 K 86 and 42 (42), 8 K with 60,000
+    // events 3732 and 1577 (2672); 1.02 M 75 and 77.
     if (4LL * n_rcv * n_out >= 1 << 20)
         return launch_superpose_r<8, 1>(traces, n_rcv, nt, ev_src, ev_amp, ev_shift, n_events, n_out, gather, st);
     if (4LL * n_rcv * n_out >= 1 << 19)
