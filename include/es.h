@@ -82,7 +82,7 @@ int es_model_create(const float* rho, const float* cp, const float* cs, int nx, 
  * accumulated in FP32; the near stencil stays on the CUDA cores).  The paper
  * has no tensor-core step: this mode is an opt-in alternative for long odd axes
  * such as the paper's 301 (the default mode's passes take 0.086 / 0.092 ms
- * there, this one's 0.106 / 0.112).  Applies from the next es_run.  ES_ERR_ARG
+ * there, this one's 0.103 / 0.112).  Applies from the next es_run.  ES_ERR_ARG
  * for any other mode. */
 #define ES_PREC_FP32 0
 #define ES_PREC_COMPENSATED 1
